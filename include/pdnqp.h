@@ -314,35 +314,20 @@ typedef struct {
  * pointer to 4 doubles.  A point passes at tolerances (eps_a, eps_r) when
  * r_p <= eps_a + eps_r s_p and r_d <= eps_a + eps_r s_d (Eq. outer-termination).  The work is issued on `stream` (cudaStream_t,
  * NULL = legacy default stream) and the call returns after the stream has
- * finished it.  Scratch for the block partial sums (5 x 1216 doubles) is
- * allocated with cudaMalloc and freed inside the call.  Returns 0 or a
+ * finished it.  No scratch is used.  Returns 0 or a
  * negative error code; the message is available from pdnqp_kkt_last_error
  * (thread-local). */
 PDNQP_API int pdnqp_kkt_residuals(const pdnqp_device_problem *P, const double *x, const double *y, double *out,
                                   void *stream);
 PDNQP_API const char *pdnqp_kkt_last_error(void);
 
-/* The same external KKT test without any device allocation, for callers that
- * cannot call cudaMalloc / cudaFree: for example code running inside a
- * runtime whose memory manager owns all device memory, or latency-critical
- * loops that cannot take the device-wide synchronisation of cudaFree.  The
- * paper has no counterpart; it is a variant of pdnqp_kkt_residuals.
- * Differences from pdnqp_kkt_residuals:
- *   - Scratch: a file-scope __device__ array of 5 x 1216 doubles (48,640
- *     bytes) that every GPU loading the library holds until the process
- *     exits.  Every problem that fits the int32 CSR layout is accepted (the
- *     kernels stride over rows with at most 1216 blocks); larger ones are
- *     rejected with PDNQP_ERR_ARG and a message.
- *   - Set-up: the first call on each device looks up the device address of
- *     that array (cudaGetSymbolAddress) with the device current and keeps it
- *     for the life of the process; make that first call before any stream
- *     capture.  A cudaDeviceReset unloads the library's device code, so the
- *     kept address is no longer valid afterwards: a process that resets a
- *     device must not call this entry point on that device again.
- *   - All calls on a device share the array and it keeps the last call's
- *     contents (no clearing is needed: each call writes every entry it
- *     reads).  Calls that overlap on the GPU (other streams, other host
- *     threads) race on it and must be serialised by the caller.
+/* The same external KKT test without waiting, for callers that cannot
+ * synchronise: for example latency-critical loops or a stream that is being
+ * captured.  The paper has no counterpart; it is a variant of
+ * pdnqp_kkt_residuals.
+ *   - No device memory is allocated or held: the residuals are joined in `out`
+ *     itself, so calls on other streams or host threads do not disturb each
+ *     other (each with its own out).
  *   - Asynchronous: the work is enqueued on `stream` and the call returns
  *     without waiting; out holds the residuals once the stream has reached
  *     this work, and execution errors surface at the next synchronisation.

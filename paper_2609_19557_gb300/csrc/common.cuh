@@ -504,6 +504,240 @@ __device__ __forceinline__ Acc tile_row_max(const int *__restrict__ rp, const in
   return tile_stream<K, true, Acc>(rp, ci, val, tile, nrows, f);
 }
 
+// Tests and comparisons of doubles on the integer pipes, a few instructions
+// each, instead of 16 cycles of the SM's FP64 pipe.  They work on the two words
+// (from the intrinsics: on the 64-bit pattern the compiler recognises the
+// floating-point test and emits it again).
+typedef unsigned long long u64;
+constexpr u64 kInfBits = 0x7ff0000000000000ull;
+__device__ __forceinline__ u64 abs_bits(double v) {
+  return ((u64)(unsigned)(__double2hiint(v) & 0x7fffffff) << 32) | (unsigned)__double2loint(v);
+}
+__device__ __forceinline__ bool nonfinite(double v) { return (__double2hiint(v) & 0x7fffffff) >= 0x7ff00000; }
+__device__ __forceinline__ bool is_nan_bits(double v) {
+  const int h = __double2hiint(v) & 0x7fffffff;
+  return h > 0x7ff00000 || (h == 0x7ff00000 && __double2loint(v) != 0);
+}
+// Order-preserving key (-0 before +0; NaN beyond the infinity of its sign).
+__device__ __forceinline__ long long order_key(double v) {
+  const int h = __double2hiint(v), s = h >> 31;
+  return ((long long)(h ^ (s & 0x7fffffff)) << 32) | (unsigned)(__double2loint(v) ^ s);
+}
+// a < b; false when either is NaN.
+__device__ __forceinline__ bool less_bits(double a, double b) {
+  return order_key(a) < order_key(b) && !is_nan_bits(a) && !is_nan_bits(b);
+}
+
+// ---------------------------------------------------------------------------
+// Row reductions of CSR matrices, one warp per tile of consecutive rows.  Lane
+// l brings the entry range [rb, re) of row tile + l (empty past the matrix)
+// and gets that row's sum (or maximum): F::gather(col) loads what an entry
+// multiplies, F::add(acc, val, x) adds the entry.  The order of every sum is
+// fixed (entry order in tile_rows; the halving order in tile_long_rows).
+//
+// What the two forms are built around: gathers are bound by memory latency, so
+// a warp issues the 8 index and value loads of a round, then the 8 gathers (16
+// with two matrices) before it uses any; and an FP64 instruction occupies its
+// SM's pipe for 16 cycles however many lanes are active, so no step may run
+// with few of them.
+// ---------------------------------------------------------------------------
+template <typename Acc>
+struct __align__(2 * sizeof(Acc)) Slot {
+  Acc a, x;
+};
+constexpr int kSlotLd = 9;                     // slots of a row in a round's buffer (8 and one of padding)
+constexpr int kTileSlots = 32 * kSlotLd;       // slots of one warp and matrix
+constexpr int kLongRowEntries = 32;            // longer rows are summed by the whole warp
+
+template <bool IsMax, typename A>
+__device__ __forceinline__ A acc_join(A a, A b) {
+  return IsMax ? (a < b ? b : a) : a + b;
+}
+
+// One row of any length by the whole warp, 256 entries a round; every lane
+// gets the result.
+template <bool IsMax, typename Acc, typename T, typename F>
+__device__ __forceinline__ Acc warp_row(const int *__restrict__ ci, const T *__restrict__ val, int b, int e,
+                                        const F &f) {
+  Acc acc = Acc(0);
+  for (int k0 = b + (int)(threadIdx.x & 31); k0 - (int)(threadIdx.x & 31) < e; k0 += 256) {
+    int c[8];
+    T a[8];
+    Acc p[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const bool ok = k0 + 32 * u < e;
+      c[u] = ok ? __ldg(ci + k0 + 32 * u) : -1;
+      a[u] = ok ? __ldg(val + k0 + 32 * u) : T(0);
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) p[u] = c[u] >= 0 ? f.gather(c[u]) : Acc(0);
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (k0 - (int)(threadIdx.x & 31) + 32 * u < e) {  // the same for the whole warp
+        if (c[u] >= 0) f.add(acc, Acc(a[u]), p[u]);
+      }
+  }
+#pragma unroll
+  for (int w = 16; w > 0; w >>= 1) acc = acc_join<IsMax>(acc, __shfl_xor_sync(0xffffffffu, acc, w));
+  return acc;
+}
+
+// Short rows (32 of them, NM matrices with the same rows).  A round takes 8
+// entries of every row: groups of 4 lanes load them (two steps of 8 rows x 4
+// entries per quarter of the tile, so the loads of a step are consecutive in
+// memory), gather, and leave value and operand in the warp's buffer, from
+// which lane l adds its own row's entries in order, one multiply-add each:
+// per round and matrix at most 8 FP64 steps, all with the rows that still have
+// entries, where sums across lanes would add idle lanes and a reduction.
+// Rows of more than kLongRowEntries entries are left out of the rounds and
+// summed by warp_row, so that one of them does not hold up its tile.  buf: NM
+// x kTileSlots slots of this warp.
+template <int NM, bool IsMax, typename Acc, typename T, typename F>
+__device__ __forceinline__ void tile_rows(const int *const (&ci)[NM], const T *const (&val)[NM], const int (&rb)[NM],
+                                          const int (&re)[NM], const F (&f)[NM], Slot<Acc> *buf, Acc (&out)[NM]) {
+  const int lane = threadIdx.x & 31, sub = lane >> 2, lg = lane & 3;
+  int se[NM], most = 0;
+  bool lng = false;
+#pragma unroll
+  for (int m = 0; m < NM; ++m) {
+    const bool l = re[m] - rb[m] > kLongRowEntries;
+    lng |= l;
+    se[m] = l ? rb[m] : re[m];
+    most = max(most, se[m] - rb[m]);
+    out[m] = Acc(0);
+  }
+  const int longest = (int)__reduce_max_sync(0xffffffffu, (unsigned)most);
+  for (int s = 0; s < longest; s += 8) {
+    int c[NM][4][2];
+    T a[NM][4][2];
+#pragma unroll
+    for (int m = 0; m < NM; ++m)
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int p = __shfl_sync(0xffffffffu, rb[m], t * 8 + sub) + s + lg;
+        const int e = __shfl_sync(0xffffffffu, se[m], t * 8 + sub);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const bool ok = p + 4 * u < e;
+          c[m][t][u] = ok ? __ldg(ci[m] + p + 4 * u) : -1;
+          a[m][t][u] = ok ? __ldg(val[m] + p + 4 * u) : T(0);
+        }
+      }
+    Acc x[NM][4][2];
+#pragma unroll
+    for (int m = 0; m < NM; ++m)
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) x[m][t][u] = c[m][t][u] >= 0 ? f[m].gather(c[m][t][u]) : Acc(0);
+    __syncwarp();  // the last round's slots have been read
+#pragma unroll
+    for (int m = 0; m < NM; ++m)
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+          if (c[m][t][u] >= 0)
+            buf[m * kTileSlots + (t * 8 + sub) * kSlotLd + 4 * u + lg] = Slot<Acc>{Acc(a[m][t][u]), x[m][t][u]};
+    __syncwarp();
+#pragma unroll
+    for (int m = 0; m < NM; ++m) {
+      const int n = se[m] - rb[m] - s;
+      const Slot<Acc> *row = buf + m * kTileSlots + lane * kSlotLd;
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (j < longest - s) {  // the same for the whole warp
+          if (j < n) f[m].add(out[m], row[j].a, row[j].x);
+        }
+    }
+  }
+  unsigned todo = __ballot_sync(0xffffffffu, lng);
+  while (todo) {
+    const int l = __ffs(todo) - 1;
+    todo &= todo - 1;
+#pragma unroll
+    for (int m = 0; m < NM; ++m) {
+      const int b = __shfl_sync(0xffffffffu, rb[m], l), e = __shfl_sync(0xffffffffu, re[m], l);
+      if (e - b > kLongRowEntries) {
+        const Acc v = warp_row<IsMax, Acc>(ci[m], val[m], b, e, f[m]);
+        if (lane == l) out[m] = v;
+      }
+    }
+  }
+  __syncwarp();  // the slots may be written again
+}
+
+// One matrix.
+template <bool IsMax, typename Acc, typename T, typename F>
+__device__ __forceinline__ Acc tile_rows1(const int *ci, const T *val, int rb, int re, const F &f, Slot<Acc> *buf) {
+  const int *const ca[1] = {ci};
+  const T *const va[1] = {val};
+  const int ba[1] = {rb}, ea[1] = {re};
+  const F fa[1] = {f};
+  Acc out[1];
+  tile_rows<1, IsMax, Acc, T, F>(ca, va, ba, ea, fa, buf, out);
+  return out[0];
+}
+
+// Long rows (8 of them, lanes 0..7): all 32 lanes on each row, the 8 rows
+// together (a round takes 32 entries of each).  The lanes' partial sums are
+// reduced by halving: at every level a lane hands over half of its rows and
+// adds the other half, 9 additions for the 8 rows instead of 40.
+template <bool IsMax, typename Acc, typename T, typename F>
+__device__ __forceinline__ Acc tile_long_rows(const int *__restrict__ ci, const T *__restrict__ val, int rb, int re,
+                                              const F &f) {
+  const int lane = threadIdx.x & 31;
+  const int longest = (int)__reduce_max_sync(0xffffffffu, (unsigned)(re - rb));
+  int pos[8], end[8];
+  Acc acc[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    pos[t] = __shfl_sync(0xffffffffu, rb, t) + lane;
+    end[t] = __shfl_sync(0xffffffffu, re, t);
+    acc[t] = Acc(0);
+  }
+  for (int s = 0; s < longest; s += 32) {
+    int c[8];
+    T a[8];
+    Acc p[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const bool ok = pos[t] + s < end[t];
+      c[t] = ok ? __ldg(ci + pos[t] + s) : -1;
+      a[t] = ok ? __ldg(val + pos[t] + s) : T(0);
+    }
+#pragma unroll
+    for (int t = 0; t < 8; ++t) p[t] = c[t] >= 0 ? f.gather(c[t]) : Acc(0);
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+      if (pos[t] - lane + s < end[t]) {  // the same for the whole warp
+        if (c[t] >= 0) f.add(acc[t], Acc(a[t]), p[t]);
+      }
+  }
+  int w = 16;
+#pragma unroll
+  for (int h = 4; h > 0; h >>= 1, w >>= 1) {
+    const bool up = (lane & w) != 0;
+#pragma unroll
+    for (int t = 0; t < h; ++t) {
+      const Acc keep = up ? acc[t + h] : acc[t], give = up ? acc[t] : acc[t + h];
+      acc[t] = acc_join<IsMax>(keep, __shfl_xor_sync(0xffffffffu, give, w));
+    }
+  }
+#pragma unroll
+  for (int v = 2; v > 0; v >>= 1) acc[0] = acc_join<IsMax>(acc[0], __shfl_xor_sync(0xffffffffu, acc[0], v));
+  return __shfl_sync(0xffffffffu, acc[0], (lane & 7) * 4);  // row l ended in lanes 4 l .. 4 l + 3
+}
+
+// Product with a vector that no block writes meanwhile.
+template <typename T>
+struct MulLdg {
+  const T *x;
+  __device__ __forceinline__ T gather(int k) const { return __ldg(x + k); }
+  __device__ __forceinline__ void add(T &acc, T a, T v) const { acc += a * v; }
+};
+
 inline int grid_for(long long work_items, int per_block) {
   long long b = (work_items + per_block - 1) / per_block;
   if (b < 1) b = 1;

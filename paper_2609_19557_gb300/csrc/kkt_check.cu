@@ -3,8 +3,8 @@
 // original (unscaled) problem, with variable-bound violations counted in r_p.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
-#include <mutex>
 #include <string>
 
 #include "../../include/pdnqp.h"
@@ -41,63 +41,32 @@ int check_problem(const pdnqp_device_problem *P, const double *x, const double *
   return 0;
 }
 
-int launch_kkt(const pdnqp_device_problem *P, const double *x, const double *y, double *out, double *scratch,
-               cudaStream_t s) {
+int launch_kkt(const pdnqp_device_problem *P, const double *x, const double *y, double *out, cudaStream_t s) {
   const int n = P->Q.n_rows, m = P->A.n_rows;
-  const int nb_r = grid_for(m > 0 ? m : 1, kBlock), nb_c = grid_for(n, kBlock);
-  if (m > 0)
-    k_kkt_rows<<<nb_r, kBlock, 0, s>>>(m, P->A.row_ptr, P->A.col_idx, P->A.val, P->l_c, P->u_c, x, scratch);
+  const KktCsr Q{P->Q.row_ptr, P->Q.col_idx, P->Q.val};
+  KktCsr A{nullptr, nullptr, nullptr}, At = A;
+  if (m > 0) {
+    A = KktCsr{P->A.row_ptr, P->A.col_idx, P->A.val};
+    At = KktCsr{P->At.row_ptr, P->At.col_idx, P->At.val};
+  }
+  // Rows of Q (the matrix that carries the entries) of more than 24 on average:
+  // tiles of 8 rows, else of 32 (whose long rows go one at a time).
+  const bool lng = P->Q.nnz > 24 * (int64_t)n;
+  const int tr = lng ? 8 : 32;
+  const long long tiles = ((long long)n + tr - 1) / tr + ((long long)m + tr - 1) / tr;
+  // As many blocks as are resident together (3 on each of 152 SMs): a grid of
+  // 1216 ran 2.67 waves of unequal length (114 us instead of 105 at n = 1e6).
+  const int nb = std::min(grid_for(tiles, kBlock / 32), 3 * 152);
+  k_kkt_init<<<1, 32, 0, s>>>(out);
+  if (lng)
+    k_kkt<true><<<nb, kBlock, 0, s>>>(n, m, Q, At, A, P->c, P->l_c, P->u_c, P->l_x, P->u_x, x, y, out);
   else
-    k_kkt_rows<<<1, kBlock, 0, s>>>(0, nullptr, nullptr, nullptr, nullptr, nullptr, x, scratch);
-  k_kkt_cols<<<nb_c, kBlock, 0, s>>>(n, P->Q.row_ptr, P->Q.col_idx, P->Q.val, m > 0 ? P->At.row_ptr : nullptr,
-                                     m > 0 ? P->At.col_idx : nullptr, m > 0 ? P->At.val : nullptr, P->c, P->l_x,
-                                     P->u_x, x, y, scratch);
-  k_kkt_final<<<1, kRedThreads, 0, s>>>(scratch, m > 0 ? nb_r : 1, nb_c, out);
+    k_kkt<false><<<nb, kBlock, 0, s>>>(n, m, Q, At, A, P->c, P->l_c, P->u_c, P->l_x, P->u_x, x, y, out);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     g_kkt_err = std::string("kernel launch: ") + cudaGetErrorString(e);
     return PDNQP_ERR_CUDA;
   }
-  return 0;
-}
-
-// Scratch of pdnqp_kkt_residuals_noalloc: the block partial sums of one call,
-// kKktQ quantities x kMaxBlocks blocks = 5 x 1216 doubles (48,640 bytes).
-// Every device that loads the library holds this array until the process
-// exits; all calls on a device share it.
-static __device__ __align__(256) double g_kkt_noalloc_scratch[kKktQ * kMaxBlocks];
-
-constexpr int kMaxDevices = 64;
-std::mutex g_noalloc_mu;
-double *g_noalloc_ptr[kMaxDevices] = {};
-
-// Device address of the static scratch on the current device.  In host code
-// the array's name is only a host-side stand-in, so the address is looked up
-// once per device (with that device current) and cached for the life of the
-// process (a cudaDeviceReset, which unloads the module, invalidates it; the
-// header tells callers not to use this entry point on a reset device).
-int noalloc_scratch(double **out) {
-  int dev = -1;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) {
-    g_kkt_err = std::string("cudaGetDevice: ") + cudaGetErrorString(e);
-    return PDNQP_ERR_CUDA;
-  }
-  if (dev < 0 || dev >= kMaxDevices) {
-    g_kkt_err = "device ordinal out of range for the static scratch table";
-    return PDNQP_ERR_ARG;
-  }
-  std::lock_guard<std::mutex> lock(g_noalloc_mu);
-  if (!g_noalloc_ptr[dev]) {
-    void *p = nullptr;
-    e = cudaGetSymbolAddress(&p, g_kkt_noalloc_scratch);
-    if (e != cudaSuccess || !p) {
-      g_kkt_err = std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e);
-      return PDNQP_ERR_CUDA;
-    }
-    g_noalloc_ptr[dev] = (double *)p;
-  }
-  *out = g_noalloc_ptr[dev];
   return 0;
 }
 
@@ -111,20 +80,7 @@ int pdnqp_kkt_residuals_noalloc(const pdnqp_device_problem *P, const double *x, 
   using namespace pdq;
   int rc = check_problem(P, x, y, out);
   if (rc) return rc;
-  // Each pass launches at most kMaxBlocks blocks (grid-stride over rows), so
-  // the partial sums of any problem that fits the int32 CSR layout fit the
-  // static array; a grid that would not fit is rejected.
-  const int nb_r = grid_for(P->A.n_rows > 0 ? P->A.n_rows : 1, kBlock), nb_c = grid_for(P->Q.n_rows, kBlock);
-  if (nb_r > kMaxBlocks || nb_c > kMaxBlocks) {
-    g_kkt_err = "problem needs more partial sums than the static scratch holds (5 x 1216)";
-    return PDNQP_ERR_ARG;
-  }
-  double *scratch = nullptr;
-  rc = noalloc_scratch(&scratch);
-  if (rc) return rc;
-  // Every block writes its partial sums before the final kernel reads exactly
-  // those entries, so nothing left by a previous call needs clearing.
-  return launch_kkt(P, x, y, out, scratch, (cudaStream_t)stream);
+  return launch_kkt(P, x, y, out, (cudaStream_t)stream);
 }
 
 int pdnqp_kkt_residuals(const pdnqp_device_problem *P, const double *x, const double *y, double *out,
@@ -132,16 +88,8 @@ int pdnqp_kkt_residuals(const pdnqp_device_problem *P, const double *x, const do
   using namespace pdq;
   int rc = check_problem(P, x, y, out);
   if (rc) return rc;
-  cudaStream_t s = (cudaStream_t)stream;
-  double *scratch = nullptr;
-  cudaError_t e = cudaMalloc(&scratch, sizeof(double) * kKktQ * kMaxBlocks);
-  if (e != cudaSuccess) {
-    g_kkt_err = std::string("cudaMalloc: ") + cudaGetErrorString(e);
-    return PDNQP_ERR_OOM;
-  }
-  rc = launch_kkt(P, x, y, out, scratch, s);
-  e = cudaStreamSynchronize(s);
-  cudaFree(scratch);
+  rc = launch_kkt(P, x, y, out, (cudaStream_t)stream);
+  const cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
   if (rc) return rc;
   if (e != cudaSuccess) {
     g_kkt_err = std::string("cudaStreamSynchronize: ") + cudaGetErrorString(e);
