@@ -56,7 +56,51 @@ struct DevState {
   double shrink;       // kappa factor on rejection
   double beta_suff, beta_nec, beta_art;
   double chk[16];      // reductions of the last check (diagnostics)
+  // Scalars of the next trial, formed once where t, kappa, omega or alpha_acc
+  // change (refresh_scalars): alpha, 1 - alpha, beta, kappa / omega, kappa
+  // omega, alpha_acc, 1 - alpha_acc, in both storage types.  Formed by every
+  // thread of every pass they took 4 FP64 divisions a thread (5 us a pass with
+  // 24 warps on an SM's FP64 pipe).
+  double sd[8];
+  float sf[8];
 };
+
+// Scalars of one trial in the storage type T.
+template <typename T>
+struct Scal {
+  T alpha, oma, beta, sct, sce, ap, omap;
+  __device__ __forceinline__ explicit Scal(const DevState *st) {
+    const T *v = pick(st, T(0));
+    alpha = v[0];
+    oma = v[1];
+    beta = v[2];
+    sct = v[3];
+    sce = v[4];
+    ap = v[5];
+    omap = v[6];
+  }
+  static __device__ __forceinline__ const double *pick(const DevState *st, double) { return st->sd; }
+  static __device__ __forceinline__ const float *pick(const DevState *st, float) { return st->sf; }
+};
+
+__host__ __device__ inline void refresh_scalars(DevState *S) {
+  const double t = (double)S->t;
+  const double v[5] = {2.0 / (t + 2.0), t / (t + 1.0), S->kappa / S->omega, S->kappa * S->omega, S->alpha_acc};
+  S->sd[0] = v[0];
+  S->sd[2] = v[1];
+  S->sd[3] = v[2];
+  S->sd[4] = v[3];
+  S->sd[5] = v[4];
+  S->sf[0] = (float)v[0];
+  S->sf[2] = (float)v[1];
+  S->sf[3] = (float)v[2];
+  S->sf[4] = (float)v[3];
+  S->sf[5] = (float)v[4];
+  S->sd[1] = 1.0 - S->sd[0];
+  S->sd[6] = 1.0 - S->sd[5];
+  S->sf[1] = 1.0f - S->sf[0];
+  S->sf[6] = 1.0f - S->sf[5];
+}
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -256,6 +300,11 @@ __device__ __forceinline__ bool grid_sync(unsigned *bar, F lead) {
   __shared__ int role;  // 0 released, 1 leader, 2 fault
   unsigned gen = 0;
   __syncthreads();
+  if (gridDim.x == 1) {  // nobody to wait for
+    lead();
+    __syncthreads();
+    return true;
+  }
   if (threadIdx.x == 0) {
     gen = ld_acquire_gpu(bar + kBarGen);
     __threadfence();
@@ -274,12 +323,12 @@ __device__ __forceinline__ bool grid_sync(unsigned *bar, F lead) {
   } else if (threadIdx.x == 0) {
     unsigned it = 0;
     while (ld_acquire_gpu(bar + kBarGen) == gen) {
-      if (ld_acquire_gpu(bar + kBarFault) != 0u || ++it > kSpinLimit) {
+      // The fault flag every 64 polls: each of the two reads is a round trip to L2.
+      if (++it > kSpinLimit || ((it & 63u) == 0u && ld_acquire_gpu(bar + kBarFault) != 0u)) {
         atomicExch(bar + kBarFault, 1u);
         role = 2;
         break;
       }
-      __nanosleep(32);
     }
     __threadfence();
   }
@@ -533,7 +582,7 @@ __device__ __forceinline__ bool less_bits(double a, double b) {
 // l brings the entry range [rb, re) of row tile + l (empty past the matrix)
 // and gets that row's sum (or maximum): F::gather(col) loads what an entry
 // multiplies, F::add(acc, val, x) adds the entry.  The order of every sum is
-// fixed (entry order in tile_rows; the halving order in tile_long_rows).
+// fixed.
 //
 // What the two forms are built around: gathers are bound by memory latency, so
 // a warp issues the 8 index and value loads of a round, then the 8 gathers (16
@@ -586,13 +635,17 @@ __device__ __forceinline__ Acc warp_row(const int *__restrict__ ci, const T *__r
 // Short rows (32 of them, NM matrices with the same rows).  A round takes 8
 // entries of every row: groups of 4 lanes load them (two steps of 8 rows x 4
 // entries per quarter of the tile, so the loads of a step are consecutive in
-// memory), gather, and leave value and operand in the warp's buffer, from
-// which lane l adds its own row's entries in order, one multiply-add each:
-// per round and matrix at most 8 FP64 steps, all with the rows that still have
-// entries, where sums across lanes would add idle lanes and a reduction.
+// memory) and gather.
+//   FP64: value and operand go to the warp's buffer, from which lane l adds its
+// own row's entries in order, one multiply-add each: per round and matrix at
+// most 8 FP64 steps, all with the rows that still have entries, where sums
+// across lanes would add idle lanes and a reduction.
+//   FP32: the lanes add their entries, and the 4 partial sums of a row are
+// joined by halving (3 additions and 4 shuffles for the 32 rows): arithmetic is
+// cheap, and the buffer would cost 16 shared-memory accesses a round.
 // Rows of more than kLongRowEntries entries are left out of the rounds and
 // summed by warp_row, so that one of them does not hold up its tile.  buf: NM
-// x kTileSlots slots of this warp.
+// x kTileSlots slots of this warp (FP32: unused).
 template <int NM, bool IsMax, typename Acc, typename T, typename F>
 __device__ __forceinline__ void tile_rows(const int *const (&ci)[NM], const T *const (&val)[NM], const int (&rb)[NM],
                                           const int (&re)[NM], const F (&f)[NM], Slot<Acc> *buf, Acc (&out)[NM]) {
@@ -608,6 +661,12 @@ __device__ __forceinline__ void tile_rows(const int *const (&ci)[NM], const T *c
     out[m] = Acc(0);
   }
   const int longest = (int)__reduce_max_sync(0xffffffffu, (unsigned)most);
+  constexpr bool kHalve = sizeof(Acc) == 4;
+  Acc part[NM][4];
+#pragma unroll
+  for (int m = 0; m < NM; ++m)
+#pragma unroll
+    for (int t = 0; t < 4; ++t) part[m][t] = Acc(0);
   for (int s = 0; s < longest; s += 8) {
     int c[NM][4][2];
     T a[NM][4][2];
@@ -631,6 +690,16 @@ __device__ __forceinline__ void tile_rows(const int *const (&ci)[NM], const T *c
       for (int t = 0; t < 4; ++t)
 #pragma unroll
         for (int u = 0; u < 2; ++u) x[m][t][u] = c[m][t][u] >= 0 ? f[m].gather(c[m][t][u]) : Acc(0);
+    if (kHalve) {
+#pragma unroll
+      for (int m = 0; m < NM; ++m)
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+#pragma unroll
+          for (int u = 0; u < 2; ++u)
+            if (c[m][t][u] >= 0) f[m].add(part[m][t], Acc(a[m][t][u]), x[m][t][u]);
+      continue;
+    }
     __syncwarp();  // the last round's slots have been read
 #pragma unroll
     for (int m = 0; m < NM; ++m)
@@ -650,6 +719,22 @@ __device__ __forceinline__ void tile_rows(const int *const (&ci)[NM], const T *c
         if (j < longest - s) {  // the same for the whole warp
           if (j < n) f[m].add(out[m], row[j].a, row[j].x);
         }
+    }
+  }
+  if (kHalve) {
+    // Lane lg of a group keeps quarter lg: hands over two quarters, then one.
+    const bool u2 = (lg & 2) != 0, u1 = (lg & 1) != 0;
+#pragma unroll
+    for (int m = 0; m < NM; ++m) {
+      Acc v[2];
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        const Acc keep = u2 ? part[m][t + 2] : part[m][t], give = u2 ? part[m][t] : part[m][t + 2];
+        v[t] = acc_join<IsMax>(keep, __shfl_xor_sync(0xffffffffu, give, 2));
+      }
+      const Acc keep = u1 ? v[1] : v[0], give = u1 ? v[0] : v[1];
+      const Acc r = acc_join<IsMax>(keep, __shfl_xor_sync(0xffffffffu, give, 1));
+      out[m] = __shfl_sync(0xffffffffu, r, (lane & 7) * 4 + (lane >> 3));  // row 8 lg + sub
     }
   }
   unsigned todo = __ballot_sync(0xffffffffu, lng);
@@ -729,6 +814,15 @@ __device__ __forceinline__ Acc tile_long_rows(const int *__restrict__ ci, const 
   for (int v = 2; v > 0; v >>= 1) acc[0] = acc_join<IsMax>(acc[0], __shfl_xor_sync(0xffffffffu, acc[0], v));
   return __shfl_sync(0xffffffffu, acc[0], (lane & 7) * 4);  // row l ended in lanes 4 l .. 4 l + 3
 }
+
+// Product with a vector that other blocks wrote before the last grid barrier of
+// the same launch (not through the read-only path).
+template <typename T>
+struct MulLd {
+  const T *x;
+  __device__ __forceinline__ T gather(int k) const { return x[k]; }
+  __device__ __forceinline__ void add(T &acc, T a, T v) const { acc += a * v; }
+};
 
 // Product with a vector that no block writes meanwhile.
 template <typename T>

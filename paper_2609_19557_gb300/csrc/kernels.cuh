@@ -35,6 +35,7 @@ constexpr int P_TR_R = 0;    // trial, row kernel: lhs_tau, lhs_eta, rhs_h, rhs_
 constexpr int P_TR_C = 4;    // trial, column kernel (same 4)
 constexpr int P_CK_R = 8;    // check, row kernel: 16 quantities
 constexpr int P_CK_C = 24;   // check, column kernel: 16 quantities
+constexpr int P_TRP = 40;    // persistent loop: 8 sums (4 of the row pass, 4 of the column pass) per block, block-major
 constexpr unsigned CK_MAXMASK = 0x0F0Fu;  // quantities 0-3 and 8-11 of a check are maxima
 // Counter words (d.ctr): [0] column last-block counter, [1] check last-block
 // counter, [2] row last-block counter (long rows), [kCtrBar, kCtrBar + kBarWords) the grid barrier of the persistent loop.
@@ -75,6 +76,7 @@ struct Dev {
   // FP64 base point and outer data
   const double *xb, *yb, *sb, *rb;  // base: outer x, inner y, warm-start s and r
   const double *lam, *sig;          // multipliers and row penalties
+  T *sg;                            // the row penalties in the storage type (constant during an inner solve)
   double *part;
   // Dense coupling rows (more than kLongRowMin entries): their products are
   // split evenly over the blocks of the row pass, and the block that
@@ -102,6 +104,15 @@ __device__ __forceinline__ T clampv(T v, T lo, T hi) {
   v = v < lo ? lo : v;
   v = v > hi ? hi : v;
   return v;
+}
+
+// FP64: the same on the integer pipes (a comparison on the FP64 pipe costs as much as a multiply-add).
+template <>
+__device__ __forceinline__ double clampv<double>(double v, double lo, double hi) {
+  const long long k = order_key(v);
+  const bool below = k < order_key(lo), above = k > order_key(hi);
+  const double p = above ? hi : (below ? lo : v);
+  return is_nan_bits(v) ? v : p;
 }
 
 // Per-thread accumulator of the acceptance sums: FP64 in the FP64 form; in
@@ -208,11 +219,8 @@ struct Pack {
 template <typename T>
 __device__ __forceinline__ void primal_phase(const Dev<T> &d, const DevState *st, GridCtx g = hw_grid()) {
   const int cur = st->cur, a0 = st->acur, acc = st->accepted;
-  const double t = (double)st->t;
-  const T alpha = T(2.0 / (t + 2.0));
-  const T oma = T(1) - alpha;
-  const T sc = T(st->kappa / st->omega);
-  const T ap = T(st->alpha_acc), omap = T(1) - ap;
+  const Scal<T> k0(st);
+  const T alpha = k0.alpha, oma = k0.oma, sc = k0.sct, ap = k0.ap, omap = k0.omap;
   const T *x = d.x[cur];
   const T *Hx = d.Hx[cur];
   const T *Aty = d.Aty[cur];
@@ -287,13 +295,13 @@ __device__ __forceinline__ long long lr_cut(long long L, int b, int nb) { return
 
 // Sum of one double per thread, in a fixed order; the result is in thread 0.
 __device__ __forceinline__ double block_sum_fixed(double v) {
-  __shared__ double ws[kBlock / 32];
+  __shared__ double ws[32];
   v = warp_sum(v);
   if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
   __syncthreads();
   double a = 0.0;
   if (threadIdx.x == 0)
-    for (int w = 0; w < kBlock / 32; ++w) a += ws[w];
+    for (int w = 0; w < (int)blockDim.x / 32; ++w) a += ws[w];
   __syncthreads();
   return a;
 }
@@ -310,7 +318,7 @@ __device__ __forceinline__ void long_rows_partial(const Dev<T> &d, const T *xt, 
     const long long a0 = e0 > d.lr_ptr[s] ? e0 : d.lr_ptr[s];
     const long long a1 = e1 < d.lr_ptr[s + 1] ? e1 : d.lr_ptr[s + 1];
     T acc = T(0);
-    for (long long k = a0 + threadIdx.x; k < a1; k += kBlock) acc += d.lr_val[k] * __ldcg(xt + d.lr_ci[k]);
+    for (long long k = a0 + threadIdx.x; k < a1; k += blockDim.x) acc += d.lr_val[k] * __ldcg(xt + d.lr_ci[k]);
     const double v = block_sum_fixed(double(acc));
     if (threadIdx.x == 0) d.lr_part[(long long)s * kMaxBlocks + b] = v;
   }
@@ -322,11 +330,8 @@ template <typename T>
 __device__ __forceinline__ void row_update_one(const Dev<T> &d, const DevState *st, long long j, T ax, T &Lt, T &Le,
                                                T &RH, T &RB) {
   const int cur = st->cur, nx = 1 - cur, a0 = st->acur, acc = st->accepted;
-  const double t = (double)st->t;
-  const T alpha = T(2.0 / (t + 2.0)), oma = T(1) - alpha;
-  const T beta = T(t / (t + 1.0));
-  const T sct = T(st->kappa / st->omega), sce = T(st->kappa * st->omega);
-  const T ap = T(st->alpha_acc), omap = T(1) - ap;
+  const Scal<T> k0(st);
+  const T alpha = k0.alpha, oma = k0.oma, beta = k0.beta, sct = k0.sct, sce = k0.sce, ap = k0.ap, omap = k0.omap;
   const bool ineq = j >= d.mE;
   const T y = d.y[cur][j], r = d.r[cur][j];
   T rb;
@@ -361,15 +366,15 @@ __device__ __forceinline__ void row_update_one(const Dev<T> &d, const DevState *
 }
 
 // Run by one whole block once every block's partials are visible (nb = the
-// row pass's grid size).  Warp w takes long rows w, w + 8, ...; the four
+// row pass's grid size).  The warps take the long rows in turn; the four
 // acceptance-sum terms go to lr_acc (warps combined in order).
 template <typename T>
 __device__ void long_rows_finish(const Dev<T> &d, const DevState *st, int nb) {
-  __shared__ double wacc[kBlock / 32][4];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  __shared__ double wacc[32][4];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const long long L = d.lr_nnz;
   T Lt = T(0), Le = T(0), RH = T(0), RB = T(0);
-  for (int s = w; s < d.nlr; s += kBlock / 32) {
+  for (int s = w; s < d.nlr; s += nw) {
     const long long p0 = d.lr_ptr[s], p1 = d.lr_ptr[s + 1];
     double a = 0.0;
     for (int b = lane; b < nb; b += 32) {
@@ -388,7 +393,7 @@ __device__ void long_rows_finish(const Dev<T> &d, const DevState *st, int nb) {
   __syncthreads();
   if (threadIdx.x < 4) {
     double v = 0.0;
-    for (int k = 0; k < kBlock / 32; ++k) v += wacc[k][threadIdx.x];
+    for (int k = 0; k < nw; ++k) v += wacc[k][threadIdx.x];
     d.lr_acc[threadIdx.x] = v;
   }
   __syncthreads();
@@ -403,11 +408,8 @@ __device__ void long_rows_finish(const Dev<T> &d, const DevState *st, int nb) {
 template <typename T, int G>
 __device__ __forceinline__ void rows_phase(const Dev<T> &d, const DevState *st, GridCtx g = hw_grid()) {
   const int cur = st->cur, nx = 1 - cur, a0 = st->acur, acc = st->accepted;
-  const double t = (double)st->t;
-  const T alpha = T(2.0 / (t + 2.0)), oma = T(1) - alpha;
-  const T beta = T(t / (t + 1.0));
-  const T sct = T(st->kappa / st->omega), sce = T(st->kappa * st->omega);
-  const T ap = T(st->alpha_acc), omap = T(1) - ap;
+  const Scal<T> k0(st);
+  const T alpha = k0.alpha, oma = k0.oma, beta = k0.beta, sct = k0.sct, sce = k0.sce, ap = k0.ap, omap = k0.omap;
   const T *xt = d.x[nx];
   T Lt = T(0), Le = T(0), RH = T(0), RB = T(0);
   TileIter ti(g);
@@ -539,409 +541,291 @@ __global__ void __launch_bounds__(kBlock) k_cols(Dev<T> d, int nb_r) {
 }
 
 // ===========================================================================
-// Panel stream of the persistent loop.  The rows of one or two CSR matrices
-// with the same row set are cut into panels of kBlock rows; each block takes
-// panels blockIdx.x, blockIdx.x + gridDim.x, ...  For each panel one thread
-// issues bulk copies of the panel's column-index and value ranges (rounded
-// to 16 bytes) into one of two shared-memory stages while the block works on
-// the other stage, so the matrix stream runs ahead of the arithmetic instead
-// of behind a chain of dependent loads.  In a stage, the block first forms
-// the products a_k x[col_k] over the panel's entries (coalesced, many
-// independent gathers per thread, written in place of the values), then
-// thread t sums the products of row panel + t in entry order.  A panel whose
-// entries do not fit a stage is read directly from global memory (same
-// order).  Per row: pre(r, valid) runs before the wait (its loads overlap the
-// copies) and returns a context; post(r, valid, ctx, sums) runs after.
+// Persistent trial loop.  One block per SM (fewer for small problems), whose
+// warps take tiles of consecutive rows (columns) and work independently: per
+// tile the row-local operands, the entries and the gathers are all in flight
+// before the first is used, and the arithmetic and the stores follow.  Block
+// barriers only at the end of a pass.
 // ===========================================================================
-constexpr int kStageEntries = 3072;  // entries (index + value) per stage, all matrices of a panel
+// Threads of a block: as many as the registers of the two passes allow (FP32
+// 80 a thread, FP64 128); few blocks make the grid barrier and the final
+// reduction of the acceptance sums cheap.
 template <typename T>
-constexpr unsigned stage_bytes() {
-  return kStageEntries * (4u + (unsigned)sizeof(T));
-}
-// Dynamic shared memory of the persistent loop: two stages.  (Shared memory
-// taken here is L1 capacity lost to the in-flight loads of every pass, so
-// the products are formed in place.)
+constexpr int kTrialThreads = sizeof(T) == 4 ? 768 : 512;
+// Slots of tile_rows (FP64: two matrices a warp).
 template <typename T>
-constexpr unsigned stream_smem_bytes() {
-  return 2 * stage_bytes<T>();
+constexpr unsigned trials_smem_bytes() {
+  return sizeof(T) == 4 ? 0u : kTrialThreads<T> / 32 * 2 * kTileSlots * (unsigned)sizeof(Slot<T>);
 }
 
-struct StreamCtl {
-  unsigned long long bar[2];
-  int done[2];     // per stage: warps finished with the panel in it
-  int base[2][2];  // per stage and matrix: first entry copied (multiple of 4)
-  int cnt[2][2];   // entries copied (multiple of 4)
-  int off[2][2];   // byte offset of the index array in the stage (values follow)
-  int fits[2];
+// The tiles of this warp: tile w gridDim + b first, so that the last, partial
+// round of a pass is spread over all SMs.
+struct WarpTiles {
+  long long first, step;
+  int lane;
+  __device__ __forceinline__ WarpTiles() {
+    lane = threadIdx.x & 31;
+    first = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    step = (long long)(blockDim.x >> 5) * gridDim.x;
+  }
 };
 
-__device__ __forceinline__ void stream_init(StreamCtl &ctl) {
-  if (threadIdx.x == 0) {
-    mbar_init(&ctl.bar[0], 1);
-    mbar_init(&ctl.bar[1], 1);
-    mbar_init_fence();
-  }
-  __syncthreads();
+// A FP32 sum as a double without the conversion instruction (which runs on the
+// FP64 pipe): exact; zeros, denormals, infinities and NaN take the instruction.
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v) {
+  const unsigned u = __float_as_uint(v), e = u & 0x7f800000u;
+  if (e == 0u || e == 0x7f800000u) return double(v);
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
 }
 
-// Row bounds of panel p (thread 0 loads them one panel ahead of the issue).
-template <typename T, int NM>
-__device__ __forceinline__ void panel_bounds(const Mat<T> *M, long long p, long long nrows, int *lo, int *hi) {
-  const long long r0 = p * kBlock;
-  const long long r1 = r0 + kBlock < nrows ? r0 + kBlock : nrows;
+// End of a pass: this block's four sums to part[0..3] (fixed order), then the
+// grid barrier; the last block to arrive runs lead() before it releases the
+// others.  Per warp the four quantities are reduced together by halving (6 FP64
+// additions), then warp 0 adds the warps' sums.
+template <typename F>
+__device__ __forceinline__ bool sums_and_sync(double (&v)[4], double *part, unsigned *bar, F lead) {
+  __shared__ double ws[4][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  {
+    const bool hi = (lane & 16) != 0;
+    double a0 = hi ? v[2] : v[0], a1 = hi ? v[3] : v[1];
+    a0 += __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[2], 16);
+    a1 += __shfl_xor_sync(0xffffffffu, hi ? v[1] : v[3], 16);
+    const bool lo = (lane & 8) != 0;
+    double b = lo ? a1 : a0;
+    b += __shfl_xor_sync(0xffffffffu, lo ? a0 : a1, 8);
 #pragma unroll
-  for (int m = 0; m < NM; ++m) {
-    lo[m] = M[m].rp[r0];
-    hi[m] = M[m].rp[r1];
-  }
-}
-
-template <typename T, int NM>
-__device__ __forceinline__ void stream_issue(StreamCtl &ctl, unsigned char *buf, int st, const Mat<T> *M,
-                                             const int *lo, const int *hi) {
-  unsigned total = 0;
-  int a[NM], c[NM], o[NM];
-#pragma unroll
-  for (int m = 0; m < NM; ++m) {
-    a[m] = lo[m] & ~3;
-    c[m] = ((hi[m] + 3) & ~3) - a[m];
-    o[m] = (int)total;
-    total += (unsigned)c[m] * (4u + (unsigned)sizeof(T));
-  }
-  const int fits = total <= stage_bytes<T>() ? 1 : 0;
-#pragma unroll
-  for (int m = 0; m < NM; ++m) {
-    ctl.base[st][m] = a[m];
-    ctl.cnt[st][m] = c[m];
-    ctl.off[st][m] = o[m];
-  }
-  ctl.fits[st] = fits;
-  unsigned char *dst = buf + (size_t)st * stage_bytes<T>();
-  fence_proxy_async_smem();
-  mbar_arrive_expect_tx(&ctl.bar[st], fits ? total : 0u);
-  if (fits) {
-    const unsigned long long pol = l2_evict_first_policy();
-#pragma unroll
-    for (int m = 0; m < NM; ++m) {
-      if (c[m] > 0) {
-        bulk_g2s_hint(dst + o[m], M[m].ci + a[m], (unsigned)c[m] * 4u, &ctl.bar[st], pol);
-        bulk_g2s_hint(dst + o[m] + 4 * c[m], M[m].val + a[m], (unsigned)c[m] * (unsigned)sizeof(T), &ctl.bar[st], pol);
-      }
-    }
-  }
-}
-
-// Warps work through the panels independently: warp w owns rows 32w..32w+31
-// of every panel, waits for the panel's copy on the stage's mbarrier, forms
-// the products of its own entry ranges (contiguous slices of the stage) and
-// the row sums, and reports on the stage's counter; the last warp to finish
-// with a stage refills it with the panel two ahead.  Per panel a warp makes a
-// single round of dependent memory accesses: load(r) issues the row-local
-// loads before the wait, the gathers of all matrices go out in one batch,
-// and finish(r, raw, sums) does all the arithmetic and the stores at the end.
-// The only block-wide barriers are at the start and end of the pass.  On a
-// fault (a copy that never lands) the warps run out the loop without
-// touching the stages, the copies in flight get a bounded wait, and the pass
-// returns false.
-template <typename T, int NM, int GB, typename Load, typename Finish>
-__device__ __forceinline__ bool stream_panels(StreamCtl &ctl, unsigned char *buf, unsigned &ph, unsigned *fault,
-                                              const Mat<T> *M, const T *const *gx, long long nrows, Load load,
-                                              Finish finish) {
-  constexpr int kWarps = kBlock / 32;
-  const long long np = (nrows + kBlock - 1) / kBlock;
-  const long long p0 = blockIdx.x, nb = gridDim.x;
-  if (p0 >= np) return true;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (threadIdx.x == 0) {
-    ctl.done[0] = 0;
-    ctl.done[1] = 0;
-    int lo[NM], hi[NM];
-    panel_bounds<T, NM>(M, p0, nrows, lo, hi);
-    stream_issue<T, NM>(ctl, buf, 0, M, lo, hi);
-    if (p0 + nb < np) {
-      panel_bounds<T, NM>(M, p0 + nb, nrows, lo, hi);
-      stream_issue<T, NM>(ctl, buf, 1, M, lo, hi);
-    }
+    for (int o = 4; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+    if ((lane & 7) == 0) ws[lane >> 3][w] = b;  // quantity lane / 8
   }
   __syncthreads();
-  bool ok = true;
-  for (long long k = 0, p = p0; p < np; ++k, p += nb) {
-    const int st = (int)(k & 1);
-    const long long r = p * kBlock + threadIdx.x;
-    const bool valid = r < nrows;
-    int rb[NM], re[NM];
+  if (w == 0) {
+    const int q = lane >> 3;
+    double b = 0.0;
+    for (int k = lane & 7; k < nw; k += 8) b += ws[q][k];
 #pragma unroll
-    for (int m = 0; m < NM; ++m) {
-      rb[m] = valid ? M[m].rp[r] : 0;
-      re[m] = valid ? M[m].rp[r + 1] : 0;
-    }
-    const auto raw = load(r, valid);
-    // This warp's rows: [rw, rw + 32) clipped to nrows.
-    const long long rw = p * kBlock + 32 * w;
-    const int last = rw < nrows ? (int)((nrows - 1 - rw) < 31 ? (nrows - 1 - rw) : 31) : -1;
-    T sum[NM];
-#pragma unroll
-    for (int m = 0; m < NM; ++m) sum[m] = T(0);
-    if (ok) ok = mbar_wait_warp(&ctl.bar[st], (ph >> st) & 1u, fault);
-    ph ^= 1u << st;
-    if (ok && last >= 0) {
-      if (ctl.fits[st]) {
-        unsigned char *sb = buf + (size_t)st * stage_bytes<T>();
-        int wb[NM], we[NM], b0[NM];
-        const int *sci[NM];
-        T *sv[NM];
-#pragma unroll
-        for (int m = 0; m < NM; ++m) {
-          const int cnt = ctl.cnt[st][m];
-          b0[m] = ctl.base[st][m];
-          sci[m] = reinterpret_cast<const int *>(sb + ctl.off[st][m]);
-          sv[m] = reinterpret_cast<T *>(sb + ctl.off[st][m] + 4 * cnt);
-          // The warp's entries [wb, we) (rows of invalid lanes are empty).
-          wb[m] = __shfl_sync(0xffffffffu, rb[m], 0) - b0[m];
-          we[m] = __shfl_sync(0xffffffffu, re[m], last) - b0[m];
-        }
-        // Products in batches of GB entries per lane and matrix: all index
-        // and value reads and all gathers of a batch (every matrix) are
-        // issued before its stores.
-        for (int j0 = lane;; j0 += GB * 32) {
-          bool more = false;
-#pragma unroll
-          for (int m = 0; m < NM; ++m) more |= wb[m] + j0 < we[m];
-          if (!__any_sync(0xffffffffu, more)) break;
-          int ci[NM][GB];
-          T a[NM][GB], xg[NM][GB];
-#pragma unroll
-          for (int m = 0; m < NM; ++m)
-#pragma unroll
-            for (int u = 0; u < GB; ++u) {
-              const int e = wb[m] + j0 + u * 32;
-              ci[m][u] = e < we[m] ? sci[m][e] : 0;
-              a[m][u] = e < we[m] ? sv[m][e] : T(0);
-            }
-#pragma unroll
-          for (int m = 0; m < NM; ++m)
-#pragma unroll
-            for (int u = 0; u < GB; ++u) xg[m][u] = __ldcg(gx[m] + ci[m][u]);
-#pragma unroll
-          for (int m = 0; m < NM; ++m)
-#pragma unroll
-            for (int u = 0; u < GB; ++u) {
-              const int e = wb[m] + j0 + u * 32;
-              if (e < we[m]) sv[m][e] = a[m][u] * xg[m][u];
-            }
-        }
-        __syncwarp();
-#pragma unroll
-        for (int m = 0; m < NM; ++m) {
-          T a = T(0);
-          for (int k2 = rb[m]; k2 < re[m]; ++k2) a += sv[m][k2 - b0[m]];
-          sum[m] = a;
-        }
-      } else {
-        // The panel does not fit a stage: read it from global memory.  Rows of
-        // at most kLongRow entries are summed by their own lane in entry order;
-        // longer rows (dense coupling rows) by the whole warp, lane-strided,
-        // then a fixed butterfly (deterministic).
-        constexpr int kLongRow = 64;
-#pragma unroll
-        for (int m = 0; m < NM; ++m) {
-          const bool lng = valid && re[m] - rb[m] > kLongRow;
-          T a = T(0);
-          if (!lng)
-            for (int k2 = rb[m]; k2 < re[m]; ++k2) a += M[m].val[k2] * __ldcg(gx[m] + M[m].ci[k2]);
-          unsigned todo = __ballot_sync(0xffffffffu, lng);
-          while (todo) {
-            const int l = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const int b = __shfl_sync(0xffffffffu, rb[m], l), e = __shfl_sync(0xffffffffu, re[m], l);
-            T w = T(0);
-            for (int k2 = b + lane; k2 < e; k2 += 32) w += M[m].val[k2] * __ldcg(gx[m] + M[m].ci[k2]);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-            if (lane == l) a = w;
-          }
-          sum[m] = a;
-        }
-      }
-    }
-    // Done with the stage: the last warp refills it with the panel two ahead.
-    // The fences on both sides of the counter order every warp's reads and
-    // in-place writes of the stage before the refill's copy.
-    __syncwarp();
-    bool refill = false;
-    if (ok && lane == 0) {
-      __threadfence_block();
-      refill = atomicAdd(&ctl.done[st], 1) == kWarps - 1;
-    }
-    if (refill) {
-      __threadfence_block();
-      ctl.done[st] = 0;
-      const long long p2 = p + 2 * nb;
-      if (p2 < np) {
-        int lo[NM], hi[NM];
-        panel_bounds<T, NM>(M, p2, nrows, lo, hi);
-        stream_issue<T, NM>(ctl, buf, st, M, lo, hi);
-      }
-    }
-    finish(r, valid, raw, sum);
+    for (int o = 4; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+    if ((lane & 7) == 0) part[q] = b;
   }
-  __syncthreads();
-  if (!ok && threadIdx.x == 0) {
-    // Bounded wait for copies that may still be in flight.
-    for (int s2 = 0; s2 < 2; ++s2)
-      for (unsigned it = 0; it <= kSpinLimitTx && !mbar_test(&ctl.bar[s2], (ph >> s2) & 1u); ++it) __nanosleep(32);
-  }
-  __syncthreads();
-  return ok;
+  return grid_sync(bar, lead);
 }
 
-// Row pass of the persistent loop: the per-row arithmetic of rows_phase with
-// (A x_tr) from the panel stream.
-template <typename T, bool LR>
-__device__ __forceinline__ bool rows_phase_stream(const Dev<T> &d, const DevState *st, StreamCtl &ctl,
-                                                  unsigned char *buf, unsigned &ph, unsigned *fault) {
+// Row pass: (A x_tr)_j, the s and r blocks of the primal trial, the dual trial
+// and the averages of the previous acceptance (the arithmetic of rows_phase).
+template <typename T, bool LR, bool LONG>
+__device__ __forceinline__ void rows_phase_tiles(const Dev<T> &d, const DevState *st, Slot<T> *buf, double (&v)[4]) {
+  constexpr int TR = LONG ? 8 : 32;
   const int cur = st->cur, nx = 1 - cur, a0 = st->acur, acc = st->accepted;
-  const double t = (double)st->t;
-  const T alpha = T(2.0 / (t + 2.0)), oma = T(1) - alpha;
-  const T beta = T(t / (t + 1.0));
-  const T sct = T(st->kappa / st->omega), sce = T(st->kappa * st->omega);
-  const T ap = T(st->alpha_acc), omap = T(1) - ap;
+  const Scal<T> k0(st);
+  const T *xt = d.x[nx];
+  if (LR) long_rows_partial<T>(d, xt);
+  const WarpTiles wt;
+  const long long nt = ((long long)d.m + TR - 1) / TR;
   T Lt = T(0), Le = T(0), RH = T(0), RB = T(0);
-  struct Raw {
-    T y, r, rb, yb, tr, qr, bw, eta, hp, itr, ie, s, sb, ts, qs, ls, us, its;
-    double sig;
+  const int *ci = d.As.ci;
+  const T *val = d.As.val;
+  const MulLd<T> f{xt};
+  int nb = 0, ne = 0;  // entry range of this lane's row, a tile ahead
+  auto range = [&](long long tile) {
+    const long long j = tile * TR + wt.lane;
+    const bool ok = tile < nt && wt.lane < TR && j < d.m;
+    nb = ok ? __ldg(d.As.rp + j) : 0;
+    ne = ok ? __ldg(d.As.rp + j + 1) : 0;
   };
-  if (LR) long_rows_partial<T>(d, d.x[nx]);
-  const Mat<T> M[1] = {d.As};
-  const T *gx[1] = {d.x[nx]};
-  const bool ok = stream_panels<T, 1, 8>(
-      ctl, buf, ph, fault, M, gx, d.m,
-      [&](long long j, bool valid) {
-        Raw c;
-        memset(&c, 0, sizeof(c));
-        if (valid) {
-          c.y = d.y[cur][j];
-          c.r = d.r[cur][j];
-          c.rb = d.rbar[a0][j];
-          if (acc) c.yb = d.ybar[a0][j];
-          c.sig = d.sig[j];
-          c.tr = d.taur[j];
-          c.qr = d.qr[j];
-          c.bw = d.Bw[cur][j];
-          c.eta = d.eta[j];
-          c.hp = d.hp[j];
-          c.itr = d.itaur[j];
-          c.ie = d.ieta[j];
-          if (j >= d.mE) {
-            c.s = d.s[cur][j];
-            if (acc) c.sb = d.sbar[a0][j];
-            c.ts = d.taus[j];
-            c.qs = d.qs[j];
-            c.ls = d.ls[j];
-            c.us = d.us[j];
-            c.its = d.itaus[j];
-          }
-        }
-        return c;
-      },
-      [&](long long j, bool valid, const Raw &c, const T *sum) {
-        if (!valid || (LR && d.lr_flag[j])) return;
-        const bool ineq = j >= d.mE;
-        T rb = c.rb;
-        if (acc) {  // running averages of the previous acceptance
-          rb = omap * rb + ap * c.r;
-          d.rbar[a0 ^ 1][j] = rb;
-          d.ybar[a0 ^ 1][j] = omap * c.yb + ap * c.y;
-          if (ineq) d.sbar[a0 ^ 1][j] = omap * c.sb + ap * c.s;
-        }
-        const T sig = T(c.sig);
-        const T rt = c.r - (sct * c.tr) * (c.qr + sig * (oma * rb + alpha * c.r) + c.y);
-        d.r[nx][j] = rt;
-        T bwt = sum[0] - rt, ds = T(0);
-        if (ineq) {
-          const T stv = clampv<T>(c.s - (sct * c.ts) * (c.qs + c.y), c.ls, c.us);
-          d.s[nx][j] = stv;
-          ds = stv - c.s;
-          Lt += ds * ds * c.its;
-          bwt -= stv;
-        }
-        const T yt = c.y + (sce * c.eta) * (c.hp - bwt - beta * (bwt - c.bw));
-        d.Bw[nx][j] = bwt;
-        d.y[nx][j] = yt;
-        const T dr = rt - c.r, dyv = yt - c.y;
-        Lt += dr * dr * c.itr;
-        Le += dyv * dyv * c.ie;
-        RH += fabs(dr * sig * dr);
-        RB += fabs(ds * dyv) + fabs(dr * dyv);
-      });
-  double v[4] = {double(Lt), double(Le), double(RH), double(RB)};
-  block_reduce_store<4>(v, 0u, d.part + P_TR_R * kMaxBlocks);
-  return ok;
+  range(wt.first);
+  for (long long tile = wt.first; tile < nt; tile += wt.step) {
+    const int rb = nb, re = ne;
+    range(tile + wt.step);
+    const long long j = tile * TR + wt.lane;
+    const bool valid = wt.lane < TR && j < d.m && !(LR && d.lr_flag[j]), ineq = valid && j >= d.mE;
+    T y = T(0), r = T(0), rbar = T(0), yb = T(0), tr = T(0), qr = T(0), bw = T(0), eta = T(0), hp = T(0), itr = T(0),
+      ie = T(0), sig = T(0), s = T(0), sb = T(0), ts = T(0), qs = T(0), ls = T(0), us = T(0), its = T(0);
+    if (valid) {
+      y = d.y[cur][j];
+      r = d.r[cur][j];
+      rbar = d.rbar[a0][j];
+      if (acc) yb = d.ybar[a0][j];
+      sig = d.sg[j];
+      tr = d.taur[j];
+      qr = d.qr[j];
+      bw = d.Bw[cur][j];
+      eta = d.eta[j];
+      hp = d.hp[j];
+      itr = d.itaur[j];
+      ie = d.ieta[j];
+    }
+    if (ineq) {
+      s = d.s[cur][j];
+      if (acc) sb = d.sbar[a0][j];
+      ts = d.taus[j];
+      qs = d.qs[j];
+      ls = d.ls[j];
+      us = d.us[j];
+      its = d.itaus[j];
+    }
+    const T ax = LONG ? tile_long_rows<false, T>(ci, val, rb, re, f) : tile_rows1<false, T>(ci, val, rb, re, f, buf);
+    if (valid) {
+      if (acc) {  // running averages of the previous acceptance
+        rbar = k0.omap * rbar + k0.ap * r;
+        d.rbar[a0 ^ 1][j] = rbar;
+        d.ybar[a0 ^ 1][j] = k0.omap * yb + k0.ap * y;
+        if (ineq) d.sbar[a0 ^ 1][j] = k0.omap * sb + k0.ap * s;
+      }
+      const T rt = r - (k0.sct * tr) * (qr + sig * (k0.oma * rbar + k0.alpha * r) + y);
+      d.r[nx][j] = rt;
+      T bwt = ax - rt, ds = T(0);
+      if (ineq) {
+        const T stv = clampv<T>(s - (k0.sct * ts) * (qs + y), ls, us);
+        d.s[nx][j] = stv;
+        ds = stv - s;
+        Lt += ds * ds * its;
+        bwt -= stv;
+      }
+      const T yt = y + (k0.sce * eta) * (hp - bwt - k0.beta * (bwt - bw));
+      d.Bw[nx][j] = bwt;
+      d.y[nx][j] = yt;
+      const T dr = rt - r, dyv = yt - y;
+      Lt += dr * dr * itr;
+      Le += dyv * dyv * ie;
+      RH += fabs(dr * sig * dr);
+      RB += fabs(ds * dyv) + fabs(dr * dyv);
+    }
+  }
+  v[0] = widen(Lt);
+  v[1] = widen(Le);
+  v[2] = widen(RH);
+  v[3] = widen(RB);
 }
 
-// Column pass of the persistent loop: H x_tr and A' y_tr from the panel
-// stream (both matrices in the same panel), then the per-variable terms.
-template <typename T>
-__device__ __forceinline__ bool cols_phase_stream(const Dev<T> &d, const DevState *st, StreamCtl &ctl,
-                                                  unsigned char *buf, unsigned &ph, unsigned *fault) {
+// Column pass: H x_tr and A' y_tr (both matrices of a tile together), then the
+// per-variable terms of the acceptance sums.
+template <typename T, bool LONG>
+__device__ __forceinline__ void cols_phase_tiles(const Dev<T> &d, const DevState *st, Slot<T> *buf, double (&v)[4]) {
+  constexpr int TR = LONG ? 8 : 32;
   const int cur = st->cur, nx = 1 - cur;
+  const WarpTiles wt;
+  const long long nt = ((long long)d.n + TR - 1) / TR;
   T Lt = T(0), RH = T(0), RB = T(0);
-  struct Raw {
-    T xti, xci, hxc, atc, itx;
+  const int *const ci[2] = {d.H.ci, d.At.ci};
+  const T *const val[2] = {d.H.val, d.At.val};
+  const MulLd<T> f[2] = {{d.x[nx]}, {d.y[nx]}};
+  int nb[2], ne[2];  // entry ranges of this lane's row, a tile ahead
+  auto range = [&](long long tile) {
+    const long long i = tile * TR + wt.lane;
+    const bool ok = tile < nt && wt.lane < TR && i < d.n;
+    nb[0] = ok ? __ldg(d.H.rp + i) : 0;
+    ne[0] = ok ? __ldg(d.H.rp + i + 1) : 0;
+    nb[1] = ok ? __ldg(d.At.rp + i) : 0;
+    ne[1] = ok ? __ldg(d.At.rp + i + 1) : 0;
   };
-  const Mat<T> M[2] = {d.H, d.At};
-  const T *gx[2] = {d.x[nx], d.y[nx]};
-  const bool ok = stream_panels<T, 2, 6>(
-      ctl, buf, ph, fault, M, gx, d.n,
-      [&](long long i, bool valid) {
-        Raw c = {T(0), T(0), T(0), T(0), T(0)};
-        if (valid) {
-          c.xti = d.x[nx][i];
-          c.xci = d.x[cur][i];
-          c.hxc = d.Hx[cur][i];
-          c.atc = d.Aty[cur][i];
-          c.itx = d.itaux[i];
-        }
-        return c;
-      },
-      [&](long long i, bool valid, const Raw &c, const T *sum) {
-        if (!valid) return;
-        d.Hx[nx][i] = sum[0];
-        d.Aty[nx][i] = sum[1];
-        const T dx = c.xti - c.xci;
-        const T dh = sum[0] - c.hxc;
-        const T da = sum[1] - c.atc;
-        Lt += dx * dx * c.itx;
-        RH += fabs(dx * dh);
-        RB += fabs(dx * da);
-      });
-  double v[4] = {double(Lt), 0.0, double(RH), double(RB)};
-  block_reduce_store<4>(v, 0u, d.part + P_TR_C * kMaxBlocks);
-  return ok;
+  range(wt.first);
+  for (long long tile = wt.first; tile < nt; tile += wt.step) {
+    const int rb[2] = {nb[0], nb[1]}, re[2] = {ne[0], ne[1]};
+    range(tile + wt.step);
+    const long long i = tile * TR + wt.lane;
+    const bool valid = wt.lane < TR && i < d.n;
+    T xti = T(0), xci = T(0), hxc = T(0), atc = T(0), itx = T(0), sum[2];
+    if (valid) {
+      xti = d.x[nx][i];
+      xci = d.x[cur][i];
+      hxc = d.Hx[cur][i];
+      atc = d.Aty[cur][i];
+      itx = d.itaux[i];
+    }
+    if (LONG) {
+      sum[0] = tile_long_rows<false, T>(ci[0], val[0], rb[0], re[0], f[0]);
+      sum[1] = tile_long_rows<false, T>(ci[1], val[1], rb[1], re[1], f[1]);
+    } else {
+      tile_rows<2, false, T>(ci, val, rb, re, f, buf, sum);
+    }
+    if (valid) {
+      d.Hx[nx][i] = sum[0];
+      d.Aty[nx][i] = sum[1];
+      const T dx = xti - xci, dh = sum[0] - hxc, da = sum[1] - atc;
+      Lt += dx * dx * itx;
+      RH += fabs(dx * dh);
+      RB += fabs(dx * da);
+    }
+  }
+  v[0] = widen(Lt);
+  v[1] = 0.0;
+  v[2] = widen(RH);
+  v[3] = widen(RB);
+}
+
+// Acceptance decision of the persistent loop, by the whole last block: the
+// blocks' sums (8 quantities, block-major, so a group of 8 lanes reads one
+// block's) over 8 warps, then lane by lane in a fixed order; thread 0 decides
+// on the block's own copy of the state, lanes 0 and 1 form the two divisions
+// of the next trial's scalars side by side, and the state goes back to global
+// memory for the other blocks.
+template <typename T>
+__device__ __forceinline__ void decide_tiles(const Dev<T> &d, DevState &S, int nb, bool lr) {
+  __shared__ double red[8][8];
+  const double *part = d.part + P_TRP * kMaxBlocks;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (w < 8) {
+    const int q = lane & 7;
+    double a = 0.0;
+#pragma unroll 5
+    for (int b = w * 4 + (lane >> 3); b < nb; b += 32) a += __ldcg(part + 8 * b + q);
+    a += __shfl_xor_sync(0xffffffffu, a, 8);
+    a += __shfl_xor_sync(0xffffffffu, a, 16);
+    if (lane < 8) red[w][q] = a;
+  }
+  __syncthreads();
+  if (w == 0) {
+    const int q = lane & 7, g = lane >> 3;
+    double s = red[g][q] + red[g + 4][q];
+    s += __shfl_xor_sync(0xffffffffu, s, 8);
+    s += __shfl_xor_sync(0xffffffffu, s, 16);
+    double a[4], b[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      a[k] = __shfl_sync(0xffffffffu, s, k);
+      b[k] = __shfl_sync(0xffffffffu, s, 4 + k);
+      if (lr) a[k] += __ldcg(d.lr_acc + k);
+    }
+    if (lane == 0) decide_logic(&S, a, b);
+    __syncwarp();
+    const double t = (double)S.t;
+    const double num = lane == 0 ? 2.0 : lane == 1 ? t : S.kappa, den = lane == 0 ? t + 2.0 : lane == 1 ? t + 1.0 : S.omega;
+    double v = num / den;
+    if (lane == 3) v = S.kappa * S.omega;
+    if (lane == 4) v = S.alpha_acc;
+    if (lane < 5) {
+      const int k = lane == 0 ? 0 : lane + 1;  // alpha, beta, kappa / omega, kappa omega, alpha_acc
+      S.sd[k] = v;
+      S.sf[k] = (float)v;
+      if (lane == 0 || lane == 4) {
+        S.sd[k + 1] = 1.0 - v;
+        S.sf[k + 1] = 1.0f - (float)v;
+      }
+    }
+  }
+  state_store(d.st, S);
 }
 
 // Persistent trial loop (one cooperative launch): primal, rows and columns of
 // each trial are separated by grid barriers, and the last block to reach the
-// third barrier takes the acceptance decision (decide_body) before releasing
-// the others, which then reload the scalar state.  The loop leaves when the
-// solve stops, a periodic check is due (the check kernels follow this launch)
-// or the launch's trial allowance (slot_left) is used up; it does not start
-// while a check is pending (the check kernels clear check_due).  All blocks
-// take the same branches (the state is block-uniform), so every barrier is
-// reached by every block.  Partial sums use this grid's size for both passes.
-// LR: the instance has dense coupling rows (d.nlr > 0); a separate
-// instantiation keeps their branches out of the common case.
-template <typename T, bool LR>
-__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 3 : 2) k_trials(Dev<T> d) {
+// third barrier takes the acceptance decision before releasing the others,
+// which then reload the scalar state.  The loop leaves when the solve stops, a
+// periodic check is due (the check kernels follow this launch) or the launch's
+// trial allowance (slot_left) is used up; it does not start while a check is
+// pending (the check kernels clear check_due).  All blocks take the same
+// branches (the state is block-uniform), so every barrier is reached by every
+// block.  LR: the instance has dense coupling rows (d.nlr > 0); RL / CL: long
+// rows of A / of H and A' (tiles of 8).
+template <typename T, bool LR, bool RL, bool CL>
+__global__ void __launch_bounds__(kTrialThreads<T>, 1) k_trials(Dev<T> d) {
   __shared__ DevState S;
-  __shared__ StreamCtl ctl;
-  extern __shared__ __align__(128) unsigned char stage_buf[];
+  extern __shared__ __align__(16) unsigned char slots[];
+  Slot<T> *buf = reinterpret_cast<Slot<T> *>(slots) + (threadIdx.x >> 5) * 2 * kTileSlots;
   unsigned *bar = d.ctr + kCtrBar;
-  unsigned *fault = bar + kBarFault;
-  unsigned ph = 0u;  // parity of the next wait on each stage
-  stream_init(ctl);
   state_load(S, d.st);
   const int nb = gridDim.x;
+  double *part = d.part + P_TRP * kMaxBlocks + 8 * blockIdx.x;
   // Block 0 times each pass: its own work, then its wait at the barrier
   // (imbalance across blocks plus the barrier itself; the last one includes
   // the acceptance decision).
@@ -960,17 +844,23 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 3 : 2) k_trials(Dev<T
     lap(0);
     if (!grid_sync(bar)) return;
     lap(1);
-    if (!rows_phase_stream<T, LR>(d, &S, ctl, stage_buf, ph, fault)) return;
+    double v[4];
+    rows_phase_tiles<T, LR, RL>(d, &S, buf, v);
     lap(2);
-    if (!grid_sync(bar, [&] {
+    if (!sums_and_sync(v, part, bar, [&] {
           if (LR) long_rows_finish<T>(d, &S, nb);
         }))
       return;
     lap(3);
-    if (!cols_phase_stream<T>(d, &S, ctl, stage_buf, ph, fault)) return;
+    cols_phase_tiles<T, CL>(d, &S, buf, v);
     lap(4);
-    if (!grid_sync(bar, [&] { decide_body<false>(d.st, d.part, LR ? d.lr_acc : nullptr, nb, nb, 0, 0); })) return;
-    state_load(S, d.st);
+    bool led = false;
+    if (!sums_and_sync(v, part + 4, bar, [&] {
+          decide_tiles<T>(d, S, nb, LR);
+          led = true;
+        }))
+      return;
+    if (!led) state_load(S, d.st);
     lap(5);
   }
   if (timer && d.ptime)
@@ -1042,6 +932,7 @@ __device__ void decide_body(DevState *stg, const double *part, const double *lac
     for (int k = 0; k < 4; ++k) a[k] += __ldcg(lacc + k);
   if (threadIdx.x == 0) {
     decide_logic(&S, a, b);
+    refresh_scalars(&S);
     if (COND) {
       const bool run = S.status == ST_RUNNING;
       if (hw) cudaGraphSetConditional(hw, (run && S.slot_left > 0) ? 1u : 0u);
@@ -1333,6 +1224,7 @@ __device__ void check_final_body(DevState *stg, const double *part, int nb_r, in
       }
       if (st->t_total == st->pause_at) st->status = ST_PAUSED;
     }
+    refresh_scalars(st);
     if (COND && hw) cudaGraphSetConditional(hw, (st->status == ST_RUNNING && st->slot_left > 0) ? 1u : 0u);
   }
   state_store(stg, S);
@@ -1431,6 +1323,7 @@ __global__ void __launch_bounds__(kBlock) k_base_rows(Dev<T> d, Mat<double> Ad, 
     d.Bwb[j] = T(bw);
     d.hp[j] = T(h - bw);
     d.qr[j] = T(lam + sig * r + yb);
+    d.sg[j] = T(sig);
     d.r[cur][j] = T(0);
     d.y[cur][j] = T(0);
     d.Bw[cur][j] = T(0);

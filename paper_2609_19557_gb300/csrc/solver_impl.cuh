@@ -527,7 +527,7 @@ class Solver : public SolverBase {
     T **nv[] = {&d.qx, &d.qx0, &d.Hxb, &d.Atyb, &d.lx, &d.ux, &d.taux, &d.itaux, &d.ex, &d.xst, &d.Atybar};
     for (T **p : nv) PDNQP_TRY(dalloc(p, n_));
     T **mv[] = {&d.qs, &d.qr, &d.hp, &d.h, &d.Bwb, &d.ls, &d.us, &d.eta, &d.taus, &d.taur, &d.ieta, &d.itaus,
-                &d.itaur, &d.es, &d.er, &d.dy, &d.yst, &d.sst, &d.rst, &d.Bwbar};
+                &d.itaur, &d.es, &d.er, &d.dy, &d.yst, &d.sst, &d.rst, &d.Bwbar, &d.sg};
     for (T **p : mv) {
       PDNQP_TRY(dalloc(p, m_));
       PDNQP_CK(cudaMemsetAsync(*p, 0, sizeof(T) * std::max(m_, 1), s_));
@@ -662,11 +662,22 @@ class Solver : public SolverBase {
     launch_trial();
     launch_check_group();
   }
-  // The persistent loop with or without the dense-coupling-row split.
-  void (*trials_fn() const)(Dev<T>) { return d_.nlr ? k_trials<T, true> : k_trials<T, false>; }
-  // Persistent trial loop: one cooperative launch per slot, grid = the
-  // co-resident block count (capped by the work), each launch bracketed by a
-  // pair of events so the loop's device time is measured on its own stream.
+  // The persistent loop's variant: with the dense-coupling-row split or not,
+  // and rows or columns in tiles of 8 where their mean length is above 24
+  // entries (there a warp's lanes are better spent along a row: at 100 entries
+  // a row, 8 rows a warp keep 8 x 32 entries in flight as 32 short rows do).
+  void (*trials_fn() const)(Dev<T>) {
+    const bool lr = d_.nlr > 0, rl = nnzA_ - d_.lr_nnz > 24LL * m_, cl = std::max(nnzH_, nnzA_) > 24LL * n_;
+    if (lr) return rl ? (cl ? k_trials<T, true, true, true> : k_trials<T, true, true, false>)
+                      : (cl ? k_trials<T, true, false, true> : k_trials<T, true, false, false>);
+    return rl ? (cl ? k_trials<T, false, true, true> : k_trials<T, false, true, false>)
+              : (cl ? k_trials<T, false, false, true> : k_trials<T, false, false, false>);
+  }
+  // Blocks of the persistent loop (one per SM at most): a warp has a tile at a
+  // time, so the grid is the tiles over 8 warps a block up to one block per SM
+  // (spread over all SMs rather than packed), and a single block, whose
+  // barriers cost next to nothing, as long as that gives a warp two tiles at
+  // most.
   int coop_grid(int bps) {
     if (coop_key_ == bps) return coop_nb_;
     coop_key_ = bps;
@@ -675,19 +686,22 @@ class Solver : public SolverBase {
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&can, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !can) return 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    const int smem = (int)stream_smem_bytes<T>();
+    const int smem = (int)trials_smem_bytes<T>();
     if (cudaFuncSetAttribute(trials_fn(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
       cudaGetLastError();
       return 0;
     }
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, trials_fn(), kBlock, smem) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, trials_fn(), kTrialThreads<T>, smem) != cudaSuccess) {
       cudaGetLastError();
       return 0;
     }
     if (bps > 0) per_sm = std::min(per_sm, bps);
-    const int work = std::max(nb_rows(), nb_cols());
-    coop_nb_ = std::max(0, std::min(std::min(per_sm * sms, kMaxBlocks), work));
+    constexpr int W = kTrialThreads<T> / 32;
+    const long long tr = nnzA_ - d_.lr_nnz > 24LL * m_ ? 8 : 32, tc = std::max(nnzH_, nnzA_) > 24LL * n_ ? 8 : 32;
+    const long long tiles = std::max((m_ + tr - 1) / tr, (n_ + tc - 1) / tc);
+    const long long work = tiles <= 2 * W && d_.nlr == 0 ? 1 : (tiles + 7) / 8;
+    coop_nb_ = (int)std::max(0LL, std::min<long long>(std::min(per_sm * sms, kMaxBlocks), work));
     return coop_nb_;
   }
   int launch_trials_persistent(int nb, int slot) {
@@ -697,8 +711,8 @@ class Solver : public SolverBase {
     }
     PDNQP_CK(cudaEventRecord(loop_ev_[2 * slot], s_));
     void *args[] = {(void *)&d_};
-    PDNQP_CK(cudaLaunchCooperativeKernel((const void *)trials_fn(), dim3(nb), dim3(kBlock), args,
-                                         stream_smem_bytes<T>(), s_));
+    PDNQP_CK(cudaLaunchCooperativeKernel((const void *)trials_fn(), dim3(nb), dim3(kTrialThreads<T>), args,
+                                         trials_smem_bytes<T>(), s_));
     PDNQP_CK(cudaEventRecord(loop_ev_[2 * slot + 1], s_));
     return 0;
   }
@@ -946,6 +960,7 @@ class Solver : public SolverBase {
     S.beta_suff = prm.beta_suff;
     S.beta_nec = prm.beta_nec;
     S.beta_art = prm.beta_art;
+    refresh_scalars(&S);
     PDNQP_CK(cudaMemcpyAsync(st_, &S, sizeof(S), cudaMemcpyHostToDevice, s_));
     launch_check(1);  // its last block sets the restart metric of the start and the running status
     launches_ += 9 + 3LL * prm.ruiz_inner;
