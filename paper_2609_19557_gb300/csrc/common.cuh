@@ -36,6 +36,8 @@ struct DevState {
   int ret_avg;         // converged candidate is the average
   int ignore_conv;     // debug: never stop on the inner termination test
   int start_status;    // status the inner-solve setup ends in: ST_RUNNING, or ST_READY in the batched form
+  int xcur, xtr, xsp;  // indices (0..2) of the current, trial and spare x buffers
+  int spec;            // persistent loop: the next x_tr (in x[xtr]) and the averages of x are formed already
   long long t;         // accepted steps in the current epoch (N_p = N_d, Eq. pdqp-trial)
   long long t_total;   // accepted steps in this inner solve
   long long trials;    // all trials, all solves
@@ -57,49 +59,61 @@ struct DevState {
   double beta_suff, beta_nec, beta_art;
   double chk[16];      // reductions of the last check (diagnostics)
   // Scalars of the next trial, formed once where t, kappa, omega or alpha_acc
-  // change (refresh_scalars): alpha, 1 - alpha, beta, kappa / omega, kappa
-  // omega, alpha_acc, 1 - alpha_acc, in both storage types.  Formed by every
-  // thread of every pass they took 4 FP64 divisions a thread (5 us a pass with
-  // 24 warps on an SM's FP64 pipe).
-  double sd[8];
-  float sf[8];
+  // change, in both storage types (kAlpha ..).  Formed by every thread of every
+  // pass they took 4 FP64 divisions a thread (5 us a pass with 24 warps on an
+  // SM's FP64 pipe).
+  double sd[12];
+  float sf[12];
 };
+
+// Slots of DevState::sd / sf: alpha, 1 - alpha, beta, kappa / omega, kappa
+// omega, alpha_acc, 1 - alpha_acc; alpha and 1 - alpha of the trial after an
+// acceptance; omega / kappa and 1 / (kappa omega) (acceptance test, FP64 only).
+enum : int { kAlpha, kOma, kBeta, kSct, kSce, kAp, kOmap, kAlpha1, kOma1, kOka, kIko };
 
 // Scalars of one trial in the storage type T.
 template <typename T>
 struct Scal {
-  T alpha, oma, beta, sct, sce, ap, omap;
-  __device__ __forceinline__ explicit Scal(const DevState *st) {
-    const T *v = pick(st, T(0));
-    alpha = v[0];
-    oma = v[1];
-    beta = v[2];
-    sct = v[3];
-    sce = v[4];
-    ap = v[5];
-    omap = v[6];
-  }
+  const T *v;
+  __device__ __forceinline__ explicit Scal(const DevState *st) : v(pick(st, T(0))) {}
+  __device__ __forceinline__ T operator[](int k) const { return v[k]; }
   static __device__ __forceinline__ const double *pick(const DevState *st, double) { return st->sd; }
   static __device__ __forceinline__ const float *pick(const DevState *st, float) { return st->sf; }
 };
 
+__host__ __device__ inline void set_scalar(DevState *S, int k, double v) {
+  S->sd[k] = v;
+  S->sf[k] = (float)v;
+}
+// A weight and its complement (formed in the storage type).
+__host__ __device__ inline void set_weight(DevState *S, int k, double v) {
+  set_scalar(S, k, v);
+  S->sd[k + 1] = 1.0 - v;
+  S->sf[k + 1] = 1.0f - (float)v;
+}
 __host__ __device__ inline void refresh_scalars(DevState *S) {
   const double t = (double)S->t;
-  const double v[5] = {2.0 / (t + 2.0), t / (t + 1.0), S->kappa / S->omega, S->kappa * S->omega, S->alpha_acc};
-  S->sd[0] = v[0];
-  S->sd[2] = v[1];
-  S->sd[3] = v[2];
-  S->sd[4] = v[3];
-  S->sd[5] = v[4];
-  S->sf[0] = (float)v[0];
-  S->sf[2] = (float)v[1];
-  S->sf[3] = (float)v[2];
-  S->sf[4] = (float)v[3];
-  S->sf[5] = (float)v[4];
-  S->sd[1] = 1.0 - S->sd[0];
-  S->sd[6] = 1.0 - S->sd[5];
-  S->sf[1] = 1.0f - S->sf[0];
-  S->sf[6] = 1.0f - S->sf[5];
+  set_weight(S, kAlpha, 2.0 / (t + 2.0));
+  set_scalar(S, kBeta, t / (t + 1.0));
+  set_scalar(S, kSct, S->kappa / S->omega);
+  set_scalar(S, kSce, S->kappa * S->omega);
+  set_weight(S, kAp, S->alpha_acc);
+  set_weight(S, kAlpha1, 2.0 / (t + 3.0));
+  S->sd[kOka] = S->omega / S->kappa;
+  S->sd[kIko] = 1.0 / (S->kappa * S->omega);
+}
+// After an acceptance (t has advanced by one; kappa and omega have not
+// changed): the weights move on, and only alpha of the trial after the next and
+// beta are new (alpha1, beta: their values for the new t).
+__host__ __device__ inline void advance_scalars(DevState *S, double alpha1, double beta) {
+  for (int k = 0; k < 2; ++k) {
+    S->sd[kAp + k] = S->sd[kAlpha + k];
+    S->sf[kAp + k] = S->sf[kAlpha + k];
+    S->sd[kAlpha + k] = S->sd[kAlpha1 + k];
+    S->sf[kAlpha + k] = S->sf[kAlpha1 + k];
+  }
+  set_weight(S, kAlpha1, alpha1);
+  set_scalar(S, kBeta, beta);
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -645,8 +659,9 @@ __device__ __forceinline__ Acc warp_row(const int *__restrict__ ci, const T *__r
 // cheap, and the buffer would cost 16 shared-memory accesses a round.
 // Rows of more than kLongRowEntries entries are left out of the rounds and
 // summed by warp_row, so that one of them does not hold up its tile.  buf: NM
-// x kTileSlots slots of this warp (FP32: unused).
-template <int NM, bool IsMax, typename Acc, typename T, typename F>
+// x kTileSlots slots of this warp (FP32: unused).  LongRows = false: the caller
+// has taken the long rows out.
+template <int NM, bool IsMax, typename Acc, bool LongRows = true, typename T, typename F>
 __device__ __forceinline__ void tile_rows(const int *const (&ci)[NM], const T *const (&val)[NM], const int (&rb)[NM],
                                           const int (&re)[NM], const F (&f)[NM], Slot<Acc> *buf, Acc (&out)[NM]) {
   const int lane = threadIdx.x & 31, sub = lane >> 2, lg = lane & 3;
@@ -654,7 +669,7 @@ __device__ __forceinline__ void tile_rows(const int *const (&ci)[NM], const T *c
   bool lng = false;
 #pragma unroll
   for (int m = 0; m < NM; ++m) {
-    const bool l = re[m] - rb[m] > kLongRowEntries;
+    const bool l = LongRows && re[m] - rb[m] > kLongRowEntries;
     lng |= l;
     se[m] = l ? rb[m] : re[m];
     most = max(most, se[m] - rb[m]);
@@ -737,7 +752,7 @@ __device__ __forceinline__ void tile_rows(const int *const (&ci)[NM], const T *c
       out[m] = __shfl_sync(0xffffffffu, r, (lane & 7) * 4 + (lane >> 3));  // row 8 lg + sub
     }
   }
-  unsigned todo = __ballot_sync(0xffffffffu, lng);
+  unsigned todo = LongRows ? __ballot_sync(0xffffffffu, lng) : 0u;
   while (todo) {
     const int l = __ffs(todo) - 1;
     todo &= todo - 1;
@@ -754,14 +769,14 @@ __device__ __forceinline__ void tile_rows(const int *const (&ci)[NM], const T *c
 }
 
 // One matrix.
-template <bool IsMax, typename Acc, typename T, typename F>
+template <bool IsMax, typename Acc, bool LongRows = true, typename T, typename F>
 __device__ __forceinline__ Acc tile_rows1(const int *ci, const T *val, int rb, int re, const F &f, Slot<Acc> *buf) {
   const int *const ca[1] = {ci};
   const T *const va[1] = {val};
   const int ba[1] = {rb}, ea[1] = {re};
   const F fa[1] = {f};
   Acc out[1];
-  tile_rows<1, IsMax, Acc, T, F>(ca, va, ba, ea, fa, buf, out);
+  tile_rows<1, IsMax, Acc, LongRows>(ca, va, ba, ea, fa, buf, out);
   return out[0];
 }
 

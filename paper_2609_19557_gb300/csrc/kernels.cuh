@@ -35,7 +35,7 @@ constexpr int P_TR_R = 0;    // trial, row kernel: lhs_tau, lhs_eta, rhs_h, rhs_
 constexpr int P_TR_C = 4;    // trial, column kernel (same 4)
 constexpr int P_CK_R = 8;    // check, row kernel: 16 quantities
 constexpr int P_CK_C = 24;   // check, column kernel: 16 quantities
-constexpr int P_TRP = 40;    // persistent loop: 8 sums (4 of the row pass, 4 of the column pass) per block, block-major
+constexpr int P_TRP = 40;    // persistent loop: 4 sums per block, block-major
 constexpr unsigned CK_MAXMASK = 0x0F0Fu;  // quantities 0-3 and 8-11 of a check are maxima
 // Counter words (d.ctr): [0] column last-block counter, [1] check last-block
 // counter, [2] row last-block counter (long rows), [kCtrBar, kCtrBar + kBarWords) the grid barrier of the persistent loop.
@@ -59,7 +59,7 @@ struct Dev {
   int n, m, mE;
   Mat<T> H, A, At;  // H = Qbar + gamma^-1 I (x block of H_k), A (rows E then I), A^T
   // n-vectors: corrections dx and their cached products H dx, A' dy, averages
-  T *x[2], *Hx[2], *Aty[2], *xbar[2], *Hxbar[2];
+  T *x[3], *Hx[2], *Aty[2], *xbar[2], *Hxbar[2];  // x: current, trial and spare (DevState::xcur ..)
   T *qx;          // q'_x = c - z / gamma + H x_b - A' y_b
   T *qx0;         // q_x = c - z / gamma (scale s_d)
   T *Hxb, *Atyb;  // H x_b, A' y_b (scales)
@@ -90,6 +90,10 @@ struct Dev {
   const int *lr_ci;
   const T *lr_val;
   const unsigned char *lr_flag;  // [m] 1 for a long row
+  // Rows of As, and variables, with more than kLongRowEntries entries (variables: in H or A'): the persistent loop
+  // gives each a warp of its own, so that they do not hold up their tiles.
+  int nlong_r, nlong_c;
+  const int *long_r, *long_c;
   double *lr_part;     // [kMaxLong][kMaxBlocks] block partial products
   double *lr_acc;      // [4] acceptance-sum terms of the long rows (added to the row sums)
   DevState *st;
@@ -179,7 +183,9 @@ template <bool COND>
 __device__ void check_final_body(DevState *stg, const double *part, int nb_r, int nb_c,
                                  cudaGraphConditionalHandle hw);
 __device__ void inner_begin_body(DevState *st, const double *part, int nb_r, int nb_c);
-__device__ __forceinline__ void decide_logic(DevState *st, const double (&a)[4], const double (&b)[4]);
+__device__ __forceinline__ bool decide_logic(DevState *st, const double (&a)[4]);
+__device__ __forceinline__ void trial_begin(DevState *st);
+__device__ __forceinline__ void trial_accept(DevState *st);
 
 // ===========================================================================
 // Trial step (Eq. pdqp-trial) and acceptance test (Eq. adaptive-condition).
@@ -220,11 +226,11 @@ template <typename T>
 __device__ __forceinline__ void primal_phase(const Dev<T> &d, const DevState *st, GridCtx g = hw_grid()) {
   const int cur = st->cur, a0 = st->acur, acc = st->accepted;
   const Scal<T> k0(st);
-  const T alpha = k0.alpha, oma = k0.oma, sc = k0.sct, ap = k0.ap, omap = k0.omap;
-  const T *x = d.x[cur];
+  const T alpha = k0[kAlpha], oma = k0[kOma], sc = k0[kSct], ap = k0[kAp], omap = k0[kOmap];
+  const T *x = d.x[st->xcur];
   const T *Hx = d.Hx[cur];
   const T *Aty = d.Aty[cur];
-  T *xt = d.x[1 - cur];
+  T *xt = d.x[st->xtr];
   constexpr int W = Pack<T>::W;
   const long long nv = d.n / W;
   // W elements per thread and trip with 16-byte loads and stores; the same
@@ -331,7 +337,8 @@ __device__ __forceinline__ void row_update_one(const Dev<T> &d, const DevState *
                                                T &RH, T &RB) {
   const int cur = st->cur, nx = 1 - cur, a0 = st->acur, acc = st->accepted;
   const Scal<T> k0(st);
-  const T alpha = k0.alpha, oma = k0.oma, beta = k0.beta, sct = k0.sct, sce = k0.sce, ap = k0.ap, omap = k0.omap;
+  const T alpha = k0[kAlpha], oma = k0[kOma], beta = k0[kBeta], sct = k0[kSct], sce = k0[kSce], ap = k0[kAp],
+          omap = k0[kOmap];
   const bool ineq = j >= d.mE;
   const T y = d.y[cur][j], r = d.r[cur][j];
   T rb;
@@ -409,8 +416,9 @@ template <typename T, int G>
 __device__ __forceinline__ void rows_phase(const Dev<T> &d, const DevState *st, GridCtx g = hw_grid()) {
   const int cur = st->cur, nx = 1 - cur, a0 = st->acur, acc = st->accepted;
   const Scal<T> k0(st);
-  const T alpha = k0.alpha, oma = k0.oma, beta = k0.beta, sct = k0.sct, sce = k0.sce, ap = k0.ap, omap = k0.omap;
-  const T *xt = d.x[nx];
+  const T alpha = k0[kAlpha], oma = k0[kOma], beta = k0[kBeta], sct = k0[kSct], sce = k0[kSce], ap = k0[kAp],
+          omap = k0[kOmap];
+  const T *xt = d.x[st->xtr];
   T Lt = T(0), Le = T(0), RH = T(0), RB = T(0);
   TileIter ti(g);
   for (long long tile = ti.first; tile < d.m; tile += ti.step) {
@@ -468,7 +476,7 @@ __device__ __forceinline__ void rows_phase(const Dev<T> &d, const DevState *st, 
 template <typename T, int G>
 __device__ __forceinline__ void rows_trial_body(const Dev<T> &d, GridCtx g) {
   if (d.st->status != ST_RUNNING) return;
-  if (d.nlr) long_rows_partial<T>(d, d.x[1 - d.st->cur], g);
+  if (d.nlr) long_rows_partial<T>(d, d.x[d.st->xtr], g);
   rows_phase<T, G>(d, d.st, g);
   if (d.nlr && arrive_last(d.ctr + 2, g.nb)) {
     long_rows_finish<T>(d, d.st, g.nb);
@@ -486,7 +494,7 @@ __global__ void __launch_bounds__(kBlock) k_rows(Dev<T> d) {
 template <typename T, int GH, int GT>
 __device__ __forceinline__ void cols_phase(const Dev<T> &d, const DevState *st, GridCtx g = hw_grid()) {
   const int cur = st->cur, nx = 1 - cur;
-  const T *xt = d.x[nx];
+  const T *xt = d.x[st->xtr], *xc = d.x[st->xcur];
   const T *yt = d.y[nx];
   T Lt = T(0), RH = T(0), RB = T(0);
   TileIter ti(g);
@@ -496,7 +504,7 @@ __device__ __forceinline__ void cols_phase(const Dev<T> &d, const DevState *st, 
     T xti = T(0), xci = T(0), hxc = T(0), atc = T(0), itx = T(0);
     if (i < d.n) {
       xti = xt[i];
-      xci = d.x[cur][i];
+      xci = xc[i];
       hxc = d.Hx[cur][i];
       atc = d.Aty[cur][i];
       itx = d.itaux[i];
@@ -544,26 +552,26 @@ __global__ void __launch_bounds__(kBlock) k_cols(Dev<T> d, int nb_r) {
 // Persistent trial loop.  One block per SM (fewer for small problems), whose
 // warps take tiles of consecutive rows (columns) and work independently: per
 // tile the row-local operands, the entries and the gathers are all in flight
-// before the first is used, and the arithmetic and the stores follow.  Block
-// barriers only at the end of a pass.
+// before the first is used, and the arithmetic and the stores follow.
 // ===========================================================================
-// Threads of a block: as many as the registers of the two passes allow (FP32
-// 80 a thread, FP64 128); few blocks make the grid barrier and the final
-// reduction of the acceptance sums cheap.
-template <typename T>
-constexpr int kTrialThreads = sizeof(T) == 4 ? 768 : 512;
+// Threads of a block: 16 warps with 128 registers a thread hold the 16 gathers
+// and 11 row-local operands of a column tile without spills, and saturate the
+// gathers (an SM takes about one 32-byte sector a cycle at random addresses,
+// measured with 16 to 64 warps); one block per SM makes the grid barrier and
+// the final reduction of the acceptance sums cheap.
+constexpr int kTrialThreads = 512;
 // Slots of tile_rows (FP64: two matrices a warp).
 template <typename T>
 constexpr unsigned trials_smem_bytes() {
-  return sizeof(T) == 4 ? 0u : kTrialThreads<T> / 32 * 2 * kTileSlots * (unsigned)sizeof(Slot<T>);
+  return sizeof(T) == 4 ? 0u : kTrialThreads / 32 * 2 * kTileSlots * (unsigned)sizeof(Slot<T>);
 }
 
-// The tiles of this warp: tile w gridDim + b first, so that the last, partial
-// round of a pass is spread over all SMs.
-struct WarpTiles {
+// The work items of this warp: item w gridDim + b first, so that the last,
+// partial round of a pass is spread over all SMs.
+struct WarpItems {
   long long first, step;
   int lane;
-  __device__ __forceinline__ WarpTiles() {
+  __device__ __forceinline__ WarpItems() {
     lane = threadIdx.x & 31;
     first = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     step = (long long)(blockDim.x >> 5) * gridDim.x;
@@ -579,68 +587,61 @@ __device__ __forceinline__ double widen(float v) {
   return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
 }
 
-// End of a pass: this block's four sums to part[0..3] (fixed order), then the
-// grid barrier; the last block to arrive runs lead() before it releases the
-// others.  Per warp the four quantities are reduced together by halving (6 FP64
-// additions), then warp 0 adds the warps' sums.
-template <typename F>
-__device__ __forceinline__ bool sums_and_sync(double (&v)[4], double *part, unsigned *bar, F lead) {
-  __shared__ double ws[4][32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  {
-    const bool hi = (lane & 16) != 0;
-    double a0 = hi ? v[2] : v[0], a1 = hi ? v[3] : v[1];
-    a0 += __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[2], 16);
-    a1 += __shfl_xor_sync(0xffffffffu, hi ? v[1] : v[3], 16);
-    const bool lo = (lane & 8) != 0;
-    double b = lo ? a1 : a0;
-    b += __shfl_xor_sync(0xffffffffu, lo ? a0 : a1, 8);
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
-    if ((lane & 7) == 0) ws[lane >> 3][w] = b;  // quantity lane / 8
-  }
-  __syncthreads();
-  if (w == 0) {
-    const int q = lane >> 3;
-    double b = 0.0;
-    for (int k = lane & 7; k < nw; k += 8) b += ws[q][k];
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
-    if ((lane & 7) == 0) part[q] = b;
-  }
-  return grid_sync(bar, lead);
-}
+// This thread's terms of the acceptance sums of a trial, over its rows and
+// columns: dw^2 / tau0, dy^2 / eta0, |dw'H dw|, |dw'B'dy|.
+template <typename T>
+struct TrialSums {
+  T Lt, Le, RH, RB;
+};
 
 // Row pass: (A x_tr)_j, the s and r blocks of the primal trial, the dual trial
 // and the averages of the previous acceptance (the arithmetic of rows_phase).
+// Items: the rows of more than kLongRowEntries entries, one a warp, then the
+// tiles of 32 rows without them (LONG: tiles of 8 rows, whatever their length).
 template <typename T, bool LR, bool LONG>
-__device__ __forceinline__ void rows_phase_tiles(const Dev<T> &d, const DevState *st, Slot<T> *buf, double (&v)[4]) {
+__device__ __forceinline__ void rows_phase_tiles(const Dev<T> &d, const DevState *st, Slot<T> *buf, TrialSums<T> &ts) {
   constexpr int TR = LONG ? 8 : 32;
   const int cur = st->cur, nx = 1 - cur, a0 = st->acur, acc = st->accepted;
   const Scal<T> k0(st);
-  const T *xt = d.x[nx];
+  const T *xt = d.x[st->xtr];
   if (LR) long_rows_partial<T>(d, xt);
-  const WarpTiles wt;
-  const long long nt = ((long long)d.m + TR - 1) / TR;
-  T Lt = T(0), Le = T(0), RH = T(0), RB = T(0);
+  const WarpItems it;
+  const long long nlong = LONG ? 0 : d.nlong_r, items = nlong + ((long long)d.m + TR - 1) / TR;
   const int *ci = d.As.ci;
   const T *val = d.As.val;
   const MulLd<T> f{xt};
-  int nb = 0, ne = 0;  // entry range of this lane's row, a tile ahead
-  auto range = [&](long long tile) {
-    const long long j = tile * TR + wt.lane;
-    const bool ok = tile < nt && wt.lane < TR && j < d.m;
-    nb = ok ? __ldg(d.As.rp + j) : 0;
-    ne = ok ? __ldg(d.As.rp + j + 1) : 0;
+  // Row of this lane in an item and its entry range, an item ahead.
+  long long nj = 0;
+  int nb = 0, ne = 0;
+  bool nv = false;
+  auto fetch = [&](long long i) {
+    nv = false;
+    nb = ne = 0;
+    if (i >= items) return;
+    if (!LONG && i < nlong) {
+      nj = __ldg(d.long_r + i);
+      nv = it.lane == 0;
+      nb = __ldg(d.As.rp + nj);
+      ne = __ldg(d.As.rp + nj + 1);
+      return;
+    }
+    nj = (i - nlong) * TR + it.lane;
+    if (it.lane >= TR || nj >= d.m) return;
+    nb = __ldg(d.As.rp + nj);
+    ne = __ldg(d.As.rp + nj + 1);
+    nv = !(LR && d.lr_flag[nj]);
+    if (!LONG && ne - nb > kLongRowEntries) {
+      nv = false;
+      ne = nb;
+    }
   };
-  range(wt.first);
-  for (long long tile = wt.first; tile < nt; tile += wt.step) {
+  fetch(it.first);
+  for (long long i = it.first; i < items; i += it.step) {
+    const long long j = nj;
     const int rb = nb, re = ne;
-    range(tile + wt.step);
-    const long long j = tile * TR + wt.lane;
-    const bool valid = wt.lane < TR && j < d.m && !(LR && d.lr_flag[j]), ineq = valid && j >= d.mE;
+    const bool valid = nv, ineq = valid && j >= d.mE;
     T y = T(0), r = T(0), rbar = T(0), yb = T(0), tr = T(0), qr = T(0), bw = T(0), eta = T(0), hp = T(0), itr = T(0),
-      ie = T(0), sig = T(0), s = T(0), sb = T(0), ts = T(0), qs = T(0), ls = T(0), us = T(0), its = T(0);
+      ie = T(0), sig = T(0), s = T(0), sb = T(0), tus = T(0), qs = T(0), ls = T(0), us = T(0), its = T(0);
     if (valid) {
       y = d.y[cur][j];
       r = d.r[cur][j];
@@ -658,174 +659,294 @@ __device__ __forceinline__ void rows_phase_tiles(const Dev<T> &d, const DevState
     if (ineq) {
       s = d.s[cur][j];
       if (acc) sb = d.sbar[a0][j];
-      ts = d.taus[j];
+      tus = d.taus[j];
       qs = d.qs[j];
       ls = d.ls[j];
       us = d.us[j];
       its = d.itaus[j];
     }
-    const T ax = LONG ? tile_long_rows<false, T>(ci, val, rb, re, f) : tile_rows1<false, T>(ci, val, rb, re, f, buf);
+    fetch(i + it.step);
+    T ax;
+    if (LONG)
+      ax = tile_long_rows<false, T>(ci, val, rb, re, f);
+    else if (i < nlong)
+      ax = warp_row<false, T>(ci, val, rb, re, f);
+    else
+      ax = tile_rows1<false, T, false>(ci, val, rb, re, f, buf);
     if (valid) {
       if (acc) {  // running averages of the previous acceptance
-        rbar = k0.omap * rbar + k0.ap * r;
+        rbar = k0[kOmap] * rbar + k0[kAp] * r;
         d.rbar[a0 ^ 1][j] = rbar;
-        d.ybar[a0 ^ 1][j] = k0.omap * yb + k0.ap * y;
-        if (ineq) d.sbar[a0 ^ 1][j] = k0.omap * sb + k0.ap * s;
+        d.ybar[a0 ^ 1][j] = k0[kOmap] * yb + k0[kAp] * y;
+        if (ineq) d.sbar[a0 ^ 1][j] = k0[kOmap] * sb + k0[kAp] * s;
       }
-      const T rt = r - (k0.sct * tr) * (qr + sig * (k0.oma * rbar + k0.alpha * r) + y);
+      const T rt = r - (k0[kSct] * tr) * (qr + sig * (k0[kOma] * rbar + k0[kAlpha] * r) + y);
       d.r[nx][j] = rt;
       T bwt = ax - rt, ds = T(0);
       if (ineq) {
-        const T stv = clampv<T>(s - (k0.sct * ts) * (qs + y), ls, us);
+        const T stv = clampv<T>(s - (k0[kSct] * tus) * (qs + y), ls, us);
         d.s[nx][j] = stv;
         ds = stv - s;
-        Lt += ds * ds * its;
+        ts.Lt += ds * ds * its;
         bwt -= stv;
       }
-      const T yt = y + (k0.sce * eta) * (hp - bwt - k0.beta * (bwt - bw));
+      const T yt = y + (k0[kSce] * eta) * (hp - bwt - k0[kBeta] * (bwt - bw));
       d.Bw[nx][j] = bwt;
       d.y[nx][j] = yt;
       const T dr = rt - r, dyv = yt - y;
-      Lt += dr * dr * itr;
-      Le += dyv * dyv * ie;
-      RH += fabs(dr * sig * dr);
-      RB += fabs(ds * dyv) + fabs(dr * dyv);
+      ts.Lt += dr * dr * itr;
+      ts.Le += dyv * dyv * ie;
+      ts.RH += fabs(dr * sig * dr);
+      ts.RB += fabs(ds * dyv) + fabs(dr * dyv);
     }
   }
-  v[0] = widen(Lt);
-  v[1] = widen(Le);
-  v[2] = widen(RH);
-  v[3] = widen(RB);
 }
 
-// Column pass: H x_tr and A' y_tr (both matrices of a tile together), then the
-// per-variable terms of the acceptance sums.
+// Column pass: H x_tr and A' y_tr (both matrices of a tile together), the
+// per-variable terms of the acceptance sums, and, as if the trial were
+// accepted, the averages of x and H x and the primal step of the next trial
+// (primal_phase with t advanced by one) into the other average buffers and the
+// spare x buffer: an acceptance, nearly every trial, then goes on with the row
+// pass, without the primal pass (which would read 9 vectors again), its barrier
+// and its latency.  A rejection finds the buffers it goes on from untouched.
 template <typename T, bool LONG>
-__device__ __forceinline__ void cols_phase_tiles(const Dev<T> &d, const DevState *st, Slot<T> *buf, double (&v)[4]) {
+__device__ __forceinline__ void cols_phase_tiles(const Dev<T> &d, const DevState *st, Slot<T> *buf, TrialSums<T> &ts) {
   constexpr int TR = LONG ? 8 : 32;
-  const int cur = st->cur, nx = 1 - cur;
-  const WarpTiles wt;
-  const long long nt = ((long long)d.n + TR - 1) / TR;
-  T Lt = T(0), RH = T(0), RB = T(0);
+  const int cur = st->cur, nx = 1 - cur, a1 = st->acur ^ st->accepted;  // committed by this trial's passes
+  const Scal<T> k0(st);
+  const WarpItems it;
+  const long long nlong = LONG ? 0 : d.nlong_c, items = nlong + ((long long)d.n + TR - 1) / TR;
   const int *const ci[2] = {d.H.ci, d.At.ci};
   const T *const val[2] = {d.H.val, d.At.val};
-  const MulLd<T> f[2] = {{d.x[nx]}, {d.y[nx]}};
-  int nb[2], ne[2];  // entry ranges of this lane's row, a tile ahead
-  auto range = [&](long long tile) {
-    const long long i = tile * TR + wt.lane;
-    const bool ok = tile < nt && wt.lane < TR && i < d.n;
-    nb[0] = ok ? __ldg(d.H.rp + i) : 0;
-    ne[0] = ok ? __ldg(d.H.rp + i + 1) : 0;
-    nb[1] = ok ? __ldg(d.At.rp + i) : 0;
-    ne[1] = ok ? __ldg(d.At.rp + i + 1) : 0;
-  };
-  range(wt.first);
-  for (long long tile = wt.first; tile < nt; tile += wt.step) {
-    const int rb[2] = {nb[0], nb[1]}, re[2] = {ne[0], ne[1]};
-    range(tile + wt.step);
-    const long long i = tile * TR + wt.lane;
-    const bool valid = wt.lane < TR && i < d.n;
-    T xti = T(0), xci = T(0), hxc = T(0), atc = T(0), itx = T(0), sum[2];
-    if (valid) {
-      xti = d.x[nx][i];
-      xci = d.x[cur][i];
-      hxc = d.Hx[cur][i];
-      atc = d.Aty[cur][i];
-      itx = d.itaux[i];
+  const T *xt = d.x[st->xtr], *xc = d.x[st->xcur];
+  T *xs = d.x[st->xsp];
+  const MulLd<T> f[2] = {{xt}, {d.y[nx]}};
+  long long nj = 0;
+  int nb[2] = {0, 0}, ne[2] = {0, 0};
+  bool nv = false;
+  auto fetch = [&](long long i) {
+    nv = false;
+    nb[0] = ne[0] = nb[1] = ne[1] = 0;
+    if (i >= items) return;
+    const bool one = !LONG && i < nlong;
+    nj = one ? __ldg(d.long_c + i) : (i - nlong) * TR + it.lane;
+    if (!one && (it.lane >= TR || nj >= d.n)) return;
+    nv = !one || it.lane == 0;
+    nb[0] = __ldg(d.H.rp + nj);
+    ne[0] = __ldg(d.H.rp + nj + 1);
+    nb[1] = __ldg(d.At.rp + nj);
+    ne[1] = __ldg(d.At.rp + nj + 1);
+    if (!LONG && !one && (ne[0] - nb[0] > kLongRowEntries || ne[1] - nb[1] > kLongRowEntries)) {
+      nv = false;
+      ne[0] = nb[0];
+      ne[1] = nb[1];
     }
+  };
+  fetch(it.first);
+  for (long long i = it.first; i < items; i += it.step) {
+    const long long j = nj;
+    const int rb[2] = {nb[0], nb[1]}, re[2] = {ne[0], ne[1]};
+    const bool valid = nv;
+    T xti = T(0), xci = T(0), hxc = T(0), atc = T(0), itx = T(0), xb = T(0), hb = T(0), qx = T(0), tau = T(0),
+      lo = T(0), hi = T(0), sum[2];
+    if (valid) {
+      xti = xt[j];
+      xci = xc[j];
+      hxc = d.Hx[cur][j];
+      atc = d.Aty[cur][j];
+      itx = d.itaux[j];
+      xb = d.xbar[a1][j];
+      hb = d.Hxbar[a1][j];
+      qx = d.qx[j];
+      tau = d.taux[j];
+      lo = d.lx[j];
+      hi = d.ux[j];
+    }
+    fetch(i + it.step);
     if (LONG) {
       sum[0] = tile_long_rows<false, T>(ci[0], val[0], rb[0], re[0], f[0]);
       sum[1] = tile_long_rows<false, T>(ci[1], val[1], rb[1], re[1], f[1]);
+    } else if (i < nlong) {
+      sum[0] = warp_row<false, T>(ci[0], val[0], rb[0], re[0], f[0]);
+      sum[1] = warp_row<false, T>(ci[1], val[1], rb[1], re[1], f[1]);
     } else {
-      tile_rows<2, false, T>(ci, val, rb, re, f, buf, sum);
+      tile_rows<2, false, T, false>(ci, val, rb, re, f, buf, sum);
     }
     if (valid) {
-      d.Hx[nx][i] = sum[0];
-      d.Aty[nx][i] = sum[1];
+      d.Hx[nx][j] = sum[0];
+      d.Aty[nx][j] = sum[1];
       const T dx = xti - xci, dh = sum[0] - hxc, da = sum[1] - atc;
-      Lt += dx * dx * itx;
-      RH += fabs(dx * dh);
-      RB += fabs(dx * da);
+      ts.Lt += dx * dx * itx;
+      ts.RH += fabs(dx * dh);
+      ts.RB += fabs(dx * da);
+      // The next trial's averages (weight alpha of this trial) and x_tr.
+      hb = k0[kOma] * hb + k0[kAlpha] * sum[0];
+      xb = k0[kOma] * xb + k0[kAlpha] * xti;
+      d.Hxbar[a1 ^ 1][j] = hb;
+      d.xbar[a1 ^ 1][j] = xb;
+      const T g = qx + k0[kOma1] * hb + k0[kAlpha1] * sum[0] - sum[1];
+      xs[j] = clampv<T>(xti - (k0[kSct] * tau) * g, lo, hi);
     }
   }
-  v[0] = widen(Lt);
-  v[1] = 0.0;
-  v[2] = widen(RH);
-  v[3] = widen(RB);
 }
 
-// Acceptance decision of the persistent loop, by the whole last block: the
-// blocks' sums (8 quantities, block-major, so a group of 8 lanes reads one
-// block's) over 8 warps, then lane by lane in a fixed order; thread 0 decides
-// on the block's own copy of the state, lanes 0 and 1 form the two divisions
-// of the next trial's scalars side by side, and the state goes back to global
-// memory for the other blocks.
-template <typename T>
-__device__ __forceinline__ void decide_tiles(const Dev<T> &d, DevState &S, int nb, bool lr) {
-  __shared__ double red[8][8];
-  const double *part = d.part + P_TRP * kMaxBlocks;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (w < 8) {
-    const int q = lane & 7;
-    double a = 0.0;
-#pragma unroll 5
-    for (int b = w * 4 + (lane >> 3); b < nb; b += 32) a += __ldcg(part + 8 * b + q);
-    a += __shfl_xor_sync(0xffffffffu, a, 8);
-    a += __shfl_xor_sync(0xffffffffu, a, 16);
-    if (lane < 8) red[w][q] = a;
-  }
+// Grid barrier of the loop with a message: bar as in grid_sync, but the
+// generation word carries, in its low bit, what the last block's lead()
+// returned; every block gets it (-1: a wait ran out).  The arrivals are reset
+// before lead() runs, and `gen` is the caller's copy of the generation (thread
+// 0), so a waiting block polls one word and nothing else.
+template <typename F>
+__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, F lead) {
+  __shared__ int role;  // message, -1 fault, 2 leader
   __syncthreads();
-  if (w == 0) {
-    const int q = lane & 7, g = lane >> 3;
-    double s = red[g][q] + red[g + 4][q];
-    s += __shfl_xor_sync(0xffffffffu, s, 8);
-    s += __shfl_xor_sync(0xffffffffu, s, 16);
-    double a[4], b[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      a[k] = __shfl_sync(0xffffffffu, s, k);
-      b[k] = __shfl_sync(0xffffffffu, s, 4 + k);
-      if (lr) a[k] += __ldcg(d.lr_acc + k);
-    }
-    if (lane == 0) decide_logic(&S, a, b);
-    __syncwarp();
-    const double t = (double)S.t;
-    const double num = lane == 0 ? 2.0 : lane == 1 ? t : S.kappa, den = lane == 0 ? t + 2.0 : lane == 1 ? t + 1.0 : S.omega;
-    double v = num / den;
-    if (lane == 3) v = S.kappa * S.omega;
-    if (lane == 4) v = S.alpha_acc;
-    if (lane < 5) {
-      const int k = lane == 0 ? 0 : lane + 1;  // alpha, beta, kappa / omega, kappa omega, alpha_acc
-      S.sd[k] = v;
-      S.sf[k] = (float)v;
-      if (lane == 0 || lane == 4) {
-        S.sd[k + 1] = 1.0 - v;
-        S.sf[k + 1] = 1.0f - (float)v;
+  if (gridDim.x == 1) {
+    const int msg = lead();
+    __syncthreads();
+    return msg;
+  }
+  if (threadIdx.x == 0) {
+    __threadfence();
+    role = -2;
+    if (atomicAdd(bar, 1u) == gridDim.x - 1) {
+      atomicExch(bar, 0u);
+      __threadfence();
+      role = 2;
+    } else {
+      unsigned it = 0, v;
+      while ((v = ld_acquire_gpu(bar + kBarGen)) == gen) {
+        if (++it > kSpinLimit || ((it & 63u) == 0u && ld_acquire_gpu(bar + kBarFault) != 0u)) {
+          atomicExch(bar + kBarFault, 1u);
+          role = -1;
+          break;
+        }
+      }
+      if (role != -1) {
+        gen = v;
+        role = (int)(v & 1u);
       }
     }
   }
-  state_store(d.st, S);
+  __syncthreads();
+  if (role != 2) return role;
+  const int msg = lead();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    gen = ((gen >> 1) + 1u) << 1 | (unsigned)msg;
+    __threadfence();
+    st_release_gpu(bar + kBarGen, gen);
+  }
+  return msg;
 }
 
-// Persistent trial loop (one cooperative launch): primal, rows and columns of
-// each trial are separated by grid barriers, and the last block to reach the
-// third barrier takes the acceptance decision before releasing the others,
-// which then reload the scalar state.  The loop leaves when the solve stops, a
-// periodic check is due (the check kernels follow this launch) or the launch's
-// trial allowance (slot_left) is used up; it does not start while a check is
-// pending (the check kernels clear check_due).  All blocks take the same
-// branches (the state is block-uniform), so every barrier is reached by every
-// block.  LR: the instance has dense coupling rows (d.nlr > 0); RL / CL: long
-// rows of A / of H and A' (tiles of 8).
+// This block's four sums to part[0..3] (fixed order): per warp the quantities
+// are reduced together by halving (6 FP64 additions), then warp 0 adds the
+// warps' sums.  Visible to the block after its next barrier.
+__device__ __forceinline__ void block_sums(double (&v)[4], double *part) {
+  __shared__ double ws[4][kTrialThreads / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const bool hi = (lane & 16) != 0, lo = (lane & 8) != 0;
+  double a0 = hi ? v[2] : v[0], a1 = hi ? v[3] : v[1];
+  a0 += __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[2], 16);
+  a1 += __shfl_xor_sync(0xffffffffu, hi ? v[1] : v[3], 16);
+  double b = lo ? a1 : a0;
+  b += __shfl_xor_sync(0xffffffffu, lo ? a0 : a1, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+  if ((lane & 7) == 0) ws[lane >> 3][w] = b;  // quantity lane / 8
+  __syncthreads();
+  if (w == 0) {
+    const int q = lane >> 3, i = lane & 7;
+    b = i < nw ? ws[q][i] : 0.0;
+    if (i + 8 < nw) b += ws[q][i + 8];
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+    if (i == 0) part[q] = b;
+  }
+}
+
+// Acceptance decision of the persistent loop, by the whole last block, on the
+// block's own copy of the state: the blocks' sums (4 quantities, block-major)
+// over 4 warps, then across lanes and warps in a fixed order.  Returns 1 when
+// the loop goes on after an acceptance and nothing else: every block then
+// makes the same change to its own copy (advance_trial); else 0, with the state
+// in global memory for the others to load.  next: alpha of the trial after the
+// next and beta after an acceptance.
+__device__ __forceinline__ void advance_x(DevState *S) {
+  const int x = S->xcur;
+  S->xcur = S->xtr;
+  S->xtr = S->xsp;
+  S->xsp = x;
+  S->spec = 1;
+}
+__device__ __forceinline__ void advance_trial(DevState *S, const double *next) {
+  trial_begin(S);
+  trial_accept(S);
+  advance_x(S);
+  advance_scalars(S, next[0], next[1]);
+}
+template <typename T>
+__device__ __forceinline__ int decide_tiles(const Dev<T> &d, DevState &S, int nb, bool lr, const double *next) {
+  __shared__ double red[4][4];
+  __shared__ int go;
+  const double *part = d.part + P_TRP * kMaxBlocks;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (w < 4) {
+    double a = 0.0;
+    if (nb == 1) {
+      if (w == 0 && lane < 4) a = part[lane];
+    } else {
+#pragma unroll 5
+      for (int b = w * 8 + (lane >> 2); b < nb; b += 32) a += __ldcg(part + 4 * b + (lane & 3));
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    }
+    if (lane < 4) red[w][lane] = a;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double a[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      a[k] = (red[0][k] + red[1][k]) + (red[2][k] + red[3][k]);
+      if (lr) a[k] += __ldcg(d.lr_acc + k);
+    }
+    const bool accepted = decide_logic(&S, a);
+    if (accepted) {
+      advance_x(&S);
+      advance_scalars(&S, next[0], next[1]);
+    } else {
+      S.spec = 0;
+      refresh_scalars(&S);
+    }
+    go = accepted && S.status == ST_RUNNING && S.slot_left > 0 && !S.check_due;
+  }
+  __syncthreads();
+  if (!go) state_store(d.st, S);
+  return go;
+}
+
+// Persistent trial loop (one cooperative launch).  A trial is the row pass, a
+// grid barrier, the column pass (with the next trial's primal step) and a grid
+// barrier whose last block takes the acceptance decision; a trial whose primal
+// step is not there yet (the first one, after a rejection, after a restart)
+// starts with the primal pass and a barrier.  The loop leaves when the solve
+// stops, a periodic check is due (the check kernels follow this launch) or the
+// launch's trial allowance (slot_left) is used up; it does not start while a
+// check is pending (the check kernels clear check_due).  All blocks take the
+// same branches (the state is block-uniform), so every barrier is reached by
+// every block.  LR: the instance has dense coupling rows (d.nlr > 0); RL / CL:
+// long rows of A / of H and A' (tiles of 8).
 template <typename T, bool LR, bool RL, bool CL>
-__global__ void __launch_bounds__(kTrialThreads<T>, 1) k_trials(Dev<T> d) {
+__global__ void __launch_bounds__(kTrialThreads, 1) k_trials(Dev<T> d) {
   __shared__ DevState S;
+  __shared__ double next[2];
   extern __shared__ __align__(16) unsigned char slots[];
   Slot<T> *buf = reinterpret_cast<Slot<T> *>(slots) + (threadIdx.x >> 5) * 2 * kTileSlots;
   unsigned *bar = d.ctr + kCtrBar;
+  unsigned gen = threadIdx.x == 0 ? ld_acquire_gpu(bar + kBarGen) : 0u;
   state_load(S, d.st);
   const int nb = gridDim.x;
-  double *part = d.part + P_TRP * kMaxBlocks + 8 * blockIdx.x;
+  double *part = d.part + P_TRP * kMaxBlocks + 4 * blockIdx.x;
   // Block 0 times each pass: its own work, then its wait at the barrier
   // (imbalance across blocks plus the barrier itself; the last one includes
   // the acceptance decision).
@@ -840,27 +961,46 @@ __global__ void __launch_bounds__(kTrialThreads<T>, 1) k_trials(Dev<T> d) {
     }
   };
   while (S.status == ST_RUNNING && S.slot_left > 0 && !S.check_due) {
-    primal_phase<T>(d, &S);
-    lap(0);
-    if (!grid_sync(bar)) return;
-    lap(1);
-    double v[4];
-    rows_phase_tiles<T, LR, RL>(d, &S, buf, v);
+    if (!S.spec) {
+      primal_phase<T>(d, &S);
+      lap(0);
+      if (loop_sync(bar, gen, [] { return 0; }) < 0) return;
+      lap(1);
+    }
+    if (threadIdx.x >= kTrialThreads - 2) {  // a spare lane each, before the last warp's first item
+      const double t = (double)(S.t + 1);
+      if (threadIdx.x == kTrialThreads - 2)
+        next[0] = 2.0 / (t + 3.0);
+      else
+        next[1] = t / (t + 1.0);
+    }
+    TrialSums<T> ts = {T(0), T(0), T(0), T(0)};
+    rows_phase_tiles<T, LR, RL>(d, &S, buf, ts);
     lap(2);
-    if (!sums_and_sync(v, part, bar, [&] {
+    if (loop_sync(bar, gen, [&] {
           if (LR) long_rows_finish<T>(d, &S, nb);
-        }))
+          return 0;
+        }) < 0)
       return;
     lap(3);
-    cols_phase_tiles<T, CL>(d, &S, buf, v);
+    cols_phase_tiles<T, CL>(d, &S, buf, ts);
     lap(4);
+    double v[4] = {widen(ts.Lt), widen(ts.Le), widen(ts.RH), widen(ts.RB)};
+    block_sums(v, part);
     bool led = false;
-    if (!sums_and_sync(v, part + 4, bar, [&] {
-          decide_tiles<T>(d, S, nb, LR);
-          led = true;
-        }))
-      return;
-    if (!led) state_load(S, d.st);
+    const int go = loop_sync(bar, gen, [&] {
+      led = true;
+      return decide_tiles<T>(d, S, nb, LR, next);
+    });
+    if (go < 0) return;
+    if (!led) {
+      if (go) {
+        if (threadIdx.x == 0) advance_trial(&S, next);
+        __syncthreads();
+      } else {
+        state_load(S, d.st);
+      }
+    }
     lap(5);
   }
   if (timer && d.ptime)
@@ -877,37 +1017,55 @@ __global__ void __launch_bounds__(kTrialThreads<T>, 1) k_trials(Dev<T> d) {
 // rejection both step vectors shrink through kappa.  Sets the device-loop
 // handles: hw (continue while running and the launch has trials left) and hc
 // (a periodic check follows).
-// The scalar part of the acceptance decision (one thread), from the row (a)
-// and column (b) sums of the trial.
-__device__ __forceinline__ void decide_logic(DevState *st, const double (&a)[4], const double (&b)[4]) {
+// The scalar part of the acceptance decision (one thread), from the sums of the
+// trial over rows and columns: dw^2 / tau0, dy^2 / eta0, |dw'H dw| and |dw'B'dy|.
+__device__ __forceinline__ bool accepts(const DevState *st, const double (&a)[4], bool &finite) {
+  const double lhs = st->sd[kOka] * a[0] + st->sd[kIko] * a[1];
+  finite = !nonfinite(lhs) && !nonfinite(a[2]) && !nonfinite(a[3]);
+  return 0.5 * lhs >= 0.5 * a[2] + a[3];
+}
+// What every trial does to the state, and what an acceptance does (the x
+// buffers are turned by the caller).
+__device__ __forceinline__ void trial_begin(DevState *st) {
   // Commit the averages materialised by this trial's primal / row passes.
   st->acur ^= st->accepted;
   st->accepted = 0;
   st->restart_flag = 0;
   st->check_due = 0;
   st->trials += 1;
-  const double om = st->omega, ka = st->kappa;
-  const double lhs = (om / ka) * (a[0] + b[0]) + (a[1] + b[1]) / (ka * om);
-  const double rh = a[2] + b[2], rb = a[3] + b[3];
-  if (!isfinite(lhs) || !isfinite(rh) || !isfinite(rb)) {
+  st->slot_left -= 1;
+}
+__device__ __forceinline__ void trial_accept(DevState *st) {
+  st->alpha_acc = st->sd[kAlpha];
+  st->cur ^= 1;
+  st->accepted = 1;
+  st->t += 1;
+  st->t_total += 1;
+  st->accepted_all += 1;
+  st->rej = 0;
+}
+__device__ __forceinline__ bool decide_logic(DevState *st, const double (&a)[4]) {
+  bool finite;
+  const bool ok = accepts(st, a, finite);
+  trial_begin(st);
+  if (!finite) {
     st->status = ST_NUMERICAL_ERROR;
-  } else if (0.5 * lhs >= 0.5 * rh + rb) {
-    st->alpha_acc = 2.0 / ((double)st->t + 2.0);
-    st->cur ^= 1;
-    st->accepted = 1;
-    st->t += 1;
-    st->t_total += 1;
-    st->accepted_all += 1;
-    st->rej = 0;
-    const bool due = (st->k_chk > 0 && st->t_total % st->k_chk == 0) || st->t_total == st->k_in;
+    return false;
+  }
+  if (ok) {
+    trial_accept(st);
+    bool due = st->t_total == st->k_in;
+    if (st->k_chk > 0)
+      due |= ((st->t_total | st->k_chk) >> 32) == 0 ? (unsigned)st->t_total % (unsigned)st->k_chk == 0
+                                                     : st->t_total % st->k_chk == 0;
     st->check_due = due ? 1 : 0;
     if (!due && st->t_total == st->pause_at) st->status = ST_PAUSED;
-  } else {
-    st->kappa *= st->shrink;
-    st->rej += 1;
-    if (st->rej >= st->rej_limit) st->status = ST_NUMERICAL_ERROR;
+    return true;
   }
-  st->slot_left -= 1;
+  st->kappa *= st->shrink;
+  st->rej += 1;
+  if (st->rej >= st->rej_limit) st->status = ST_NUMERICAL_ERROR;
+  return false;
 }
 
 template <bool COND>
@@ -931,7 +1089,12 @@ __device__ void decide_body(DevState *stg, const double *part, const double *lac
   if (lacc)
     for (int k = 0; k < 4; ++k) a[k] += __ldcg(lacc + k);
   if (threadIdx.x == 0) {
-    decide_logic(&S, a, b);
+    for (int k = 0; k < 4; ++k) a[k] += b[k];
+    if (decide_logic(&S, a)) {
+      const int x = S.xcur;
+      S.xcur = S.xtr;
+      S.xtr = x;
+    }
     refresh_scalars(&S);
     if (COND) {
       const bool run = S.status == ST_RUNNING;
@@ -954,7 +1117,7 @@ __global__ void __launch_bounds__(kBlock) k_average(Dev<T> d) {
   const int cur = st->cur, a0 = st->acur, a1 = st->acur ^ 1;
   const T alpha = T(st->alpha_acc), oma = T(1) - alpha;
   PDNQP_GRID_STRIDE(i, d.n) {
-    d.xbar[a1][i] = oma * d.xbar[a0][i] + alpha * d.x[cur][i];
+    d.xbar[a1][i] = oma * d.xbar[a0][i] + alpha * d.x[st->xcur][i];
     d.Hxbar[a1][i] = oma * d.Hxbar[a0][i] + alpha * d.Hx[cur][i];
   }
   PDNQP_GRID_STRIDE(j, d.m) {
@@ -1026,7 +1189,7 @@ __device__ __forceinline__ void check_rows_body(const Dev<T> &d, int mode, GridC
   const int cur = st->cur, a0 = st->acur, acc = st->accepted, ab = a0 ^ acc;
   const T ap = T(st->alpha_acc), omap = T(1) - ap;
   const T *__restrict__ xb0 = d.xbar[a0];
-  const T *__restrict__ xc = d.x[cur];
+  const T *__restrict__ xc = d.x[st->xcur];
   double q[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) q[k] = 0.0;
@@ -1121,6 +1284,7 @@ __device__ __forceinline__ void check_cols_body(const Dev<T> &d, int mode, int n
   const int cur = st->cur, a0 = st->acur, acc = st->accepted, ab = a0 ^ acc;
   const T ap = T(st->alpha_acc), omap = T(1) - ap;
   const T *__restrict__ yb = d.ybar[ab];
+  const T *__restrict__ xc = d.x[st->xcur];
   double q[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) q[k] = 0.0;
@@ -1134,13 +1298,13 @@ __device__ __forceinline__ void check_cols_body(const Dev<T> &d, int mode, int n
       const double qx = double(d.qx[i]), qx0 = double(d.qx0[i]), hxb = double(d.Hxb[i]);
       const double atyb0 = double(d.Atyb[i]), lx = double(d.lx[i]), ux = double(d.ux[i]);
       const double ex = double(d.ex[i]), xst = double(d.xst[i]);
-      col_cand(q, double(d.x[cur][i]), double(d.Hx[cur][i]), double(d.Aty[cur][i]), qx, qx0, hxb, atyb0, lx, ux, ex,
+      col_cand(q, double(xc[i]), double(d.Hx[cur][i]), double(d.Aty[cur][i]), qx, qx0, hxb, atyb0, lx, ux, ex,
                xst);
       if (mode == 0) {
         d.Atybar[i] = atyb;
         T xa = d.xbar[a0][i], ha = d.Hxbar[a0][i];
         if (acc) {
-          xa = omap * xa + ap * d.x[cur][i];
+          xa = omap * xa + ap * xc[i];
           ha = omap * ha + ap * d.Hx[cur][i];
           d.xbar[ab][i] = xa;
           d.Hxbar[ab][i] = ha;
@@ -1220,6 +1384,7 @@ __device__ void check_final_body(DevState *stg, const double *part, int nb_r, in
         st->k_last = INFINITY;
         st->restarts += 1;
         st->restart_flag = 1;
+        st->spec = 0;
         st->restart_use_avg = use_avg ? 1 : 0;
       }
       if (st->t_total == st->pause_at) st->status = ST_PAUSED;
@@ -1239,12 +1404,13 @@ __device__ __forceinline__ void check_apply_body(const Dev<T> &d, GridCtx g) {
   if (!st->restart_flag) return;
   const int cur = st->cur, ab = st->acur;
   const bool ua = st->restart_use_avg;
+  T *xc = d.x[st->xcur];
   PDNQP_VGRID_STRIDE(i, d.n, g) {
-    T x = d.x[cur][i], hx = d.Hx[cur][i];
+    T x = xc[i], hx = d.Hx[cur][i];
     if (ua) {
       x = d.xbar[ab][i];
       hx = d.Hxbar[ab][i];
-      d.x[cur][i] = x;
+      xc[i] = x;
       d.Hx[cur][i] = hx;
       d.Aty[cur][i] = d.Atybar[i];
     }
@@ -1352,7 +1518,7 @@ __global__ void __launch_bounds__(kBlock) k_base_cols(Dev<T> d, Mat<double> Hd, 
       d.Atyb[i] = T(aty);
       d.lx[i] = T(lxd[i] - x[i]);
       d.ux[i] = T(uxd[i] - x[i]);
-      d.x[cur][i] = T(0);
+      d.x[d.st->xcur][i] = T(0);
       d.Hx[cur][i] = T(0);
       d.Aty[cur][i] = T(0);
     }
@@ -1492,8 +1658,8 @@ template <typename T>
 __global__ void k_inner_init(Dev<T> d) {
   const int cur = d.st->cur;
   PDNQP_GRID_STRIDE(i, d.n) {
-    d.xst[i] = d.x[cur][i];
-    d.xbar[0][i] = d.x[cur][i];
+    d.xst[i] = d.x[d.st->xcur][i];
+    d.xbar[0][i] = d.x[d.st->xcur][i];
     d.Hxbar[0][i] = d.Hx[cur][i];
   }
   PDNQP_GRID_STRIDE(j, d.m) {
@@ -1513,7 +1679,7 @@ __global__ void k_inner_init(Dev<T> d) {
 template <typename T>
 __global__ void k_finish(Dev<T> d, double *x64, double *y64, int use_avg) {
   const int cur = d.st->cur, ab = d.st->acur ^ d.st->accepted;
-  const T *__restrict__ dx = use_avg ? d.xbar[ab] : d.x[cur];
+  const T *__restrict__ dx = use_avg ? d.xbar[ab] : d.x[d.st->xcur];
   const T *__restrict__ dy = use_avg ? d.ybar[ab] : d.y[cur];
   PDNQP_GRID_STRIDE(i, d.n) x64[i] += double(dx[i]);
   PDNQP_GRID_STRIDE(j, d.m) y64[j] += double(dy[j]);
@@ -1526,7 +1692,7 @@ __global__ void k_totals(Dev<T> d, double *out) {
   const int cur = d.st->cur, ab = d.st->acur ^ d.st->accepted;
   const long long n = d.n, m = d.m, mI = m - d.mE, dw = n + mI + m;
   for (int a = 0; a < 2; ++a) {
-    const T *x = a ? d.xbar[ab] : d.x[cur];
+    const T *x = a ? d.xbar[ab] : d.x[d.st->xcur];
     const T *s = a ? d.sbar[ab] : d.s[cur];
     const T *r = a ? d.rbar[ab] : d.r[cur];
     const T *y = a ? d.ybar[ab] : d.y[cur];

@@ -397,7 +397,7 @@ class Solver : public SolverBase {
     k_add_diag<<<grid_n(), kBlock, 0, s_>>>(n_, qdiag_, qv_, 1.0 / gamma_);
     PDNQP_CK(cudaGetLastError());
     // ---- T-typed copies and inner vectors
-    PDNQP_TRY(alloc_T(P.a_rp));
+    PDNQP_TRY(alloc_T(P));
     PDNQP_CK(cudaStreamSynchronize(s_));
     ready_ = true;
     return 0;
@@ -484,7 +484,7 @@ class Solver : public SolverBase {
     return reduce_to_host(1, nb, 0u, out);
   }
 
-  int alloc_T(const std::vector<int> &arp) {
+  int alloc_T(const HostProblem &P) {
     Dev<T> &d = d_;
     d.n = n_;
     d.m = m_;
@@ -507,7 +507,9 @@ class Solver : public SolverBase {
       d.A = {Ad_.nrows, Ad_.rp, Ad_.ci, av};
       d.At = {Atd_.nrows, Atd_.rp, Atd_.ci, atv};
     }
-    PDNQP_TRY(split_long_rows(arp));
+    PDNQP_TRY(split_long_rows(P.a_rp));
+    PDNQP_TRY(list_long_rows(P));
+    PDNQP_TRY(dalloc(&d.x[2], n_));
     for (int b = 0; b < 2; ++b) {
       PDNQP_TRY(dalloc(&d.x[b], n_));
       PDNQP_TRY(dalloc(&d.Hx[b], n_));
@@ -557,6 +559,25 @@ class Solver : public SolverBase {
     return 0;
   }
 
+  // Rows and variables that the persistent loop takes out of their tiles.
+  int list_long_rows(const HostProblem &P) {
+    Dev<T> &d = d_;
+    auto len = [](const std::vector<int> &rp, int i) { return rp[i + 1] - rp[i]; };
+    std::vector<int> r, c;
+    for (int j = 0; j < m_; ++j)
+      if (len(P.a_rp, j) > kLongRowEntries && !(d.nlr && long_flag_[j])) r.push_back(j);
+    for (int i = 0; i < n_; ++i)
+      if (len(P.q_rp, i) > kLongRowEntries || len(P.at_rp, i) > kLongRowEntries) c.push_back(i);
+    d.nlong_r = (int)r.size();
+    d.nlong_c = (int)c.size();
+    int *lr, *lc;
+    PDNQP_TRY(upload(&lr, r));
+    PDNQP_TRY(upload(&lc, c));
+    d.long_r = lr;
+    d.long_c = lc;
+    return 0;
+  }
+
   // Dense coupling rows of A (more than kLongRowMin entries; the kMaxLong
   // longest when there are more): copies of their entries in row order for
   // the split products, and As = A with those rows emptied for the row-wise
@@ -583,7 +604,8 @@ class Solver : public SolverBase {
     }
     const int nl = (int)lr.size();
     std::vector<int> lptr(nl + 1, 0), srp(m_ + 1, 0);
-    std::vector<unsigned char> flag(m_, 0);
+    std::vector<unsigned char> &flag = long_flag_;
+    flag.assign(m_, 0);
     for (int k = 0; k < nl; ++k) {
       lptr[k + 1] = lptr[k] + len(lr[k]);
       flag[lr[k]] = 1;
@@ -692,15 +714,16 @@ class Solver : public SolverBase {
       return 0;
     }
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, trials_fn(), kTrialThreads<T>, smem) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, trials_fn(), kTrialThreads, smem) != cudaSuccess) {
       cudaGetLastError();
       return 0;
     }
     if (bps > 0) per_sm = std::min(per_sm, bps);
-    constexpr int W = kTrialThreads<T> / 32;
+    constexpr int W = kTrialThreads / 32;
     const long long tr = nnzA_ - d_.lr_nnz > 24LL * m_ ? 8 : 32, tc = std::max(nnzH_, nnzA_) > 24LL * n_ ? 8 : 32;
-    const long long tiles = std::max((m_ + tr - 1) / tr, (n_ + tc - 1) / tc);
-    const long long work = tiles <= 2 * W && d_.nlr == 0 ? 1 : (tiles + 7) / 8;
+    const long long tiles = std::max((m_ + tr - 1) / tr + (tr == 32 ? d_.nlong_r : 0),
+                                     (n_ + tc - 1) / tc + (tc == 32 ? d_.nlong_c : 0));
+    const long long work = tiles <= 3 * W && d_.nlr == 0 ? 1 : (tiles + 7) / 8;
     coop_nb_ = (int)std::max(0LL, std::min<long long>(std::min(per_sm * sms, kMaxBlocks), work));
     return coop_nb_;
   }
@@ -711,7 +734,7 @@ class Solver : public SolverBase {
     }
     PDNQP_CK(cudaEventRecord(loop_ev_[2 * slot], s_));
     void *args[] = {(void *)&d_};
-    PDNQP_CK(cudaLaunchCooperativeKernel((const void *)trials_fn(), dim3(nb), dim3(kTrialThreads<T>), args,
+    PDNQP_CK(cudaLaunchCooperativeKernel((const void *)trials_fn(), dim3(nb), dim3(kTrialThreads), args,
                                          trials_smem_bytes<T>(), s_));
     PDNQP_CK(cudaEventRecord(loop_ev_[2 * slot + 1], s_));
     return 0;
@@ -867,7 +890,7 @@ class Solver : public SolverBase {
     DevState S;
     memset(&S, 0, sizeof(S));
     S.status = ST_IDLE;
-    S.cur = 0;
+    reset_buffers(&S);
     PDNQP_CK(cudaMemcpyAsync(st_, &S, sizeof(S), cudaMemcpyHostToDevice, s_));
     if (has_x0_) PDNQP_CK(cudaMemcpyAsync(dx0_, h_x0_.data(), sizeof(double) * n_, cudaMemcpyHostToDevice, s_));
     if (has_l0_) PDNQP_CK(cudaMemcpyAsync(dl0_, h_l0_.data(), sizeof(double) * m_, cudaMemcpyHostToDevice, s_));
@@ -906,6 +929,15 @@ class Solver : public SolverBase {
     return 0;
   }
 
+  // Between inner solves the iterates sit in buffer 0.
+  static void reset_buffers(DevState *S) {
+    S->cur = 0;
+    S->xcur = 0;
+    S->xtr = 1;
+    S->xsp = 2;
+    S->spec = 0;
+  }
+
   // a0: setup of one inner solve (Algorithm 4 lines "warm start" and "inner scaling").
   int inner_setup(const Params &prm, double dta, double dtr, long long k_in, long long pause_at, int ignore) {
     const double ginv = 1.0 / gamma_;
@@ -932,7 +964,7 @@ class Solver : public SolverBase {
     // iterates sit in buffer 0 between inner solves).
     DevState &S = *hst_;
     memset(&S, 0, sizeof(S));
-    S.cur = 0;
+    reset_buffers(&S);
     S.status = ST_IDLE;
     S.accepted = 0;
     S.acur = 0;
@@ -1060,7 +1092,7 @@ class Solver : public SolverBase {
     k_finish<T><<<grid_nm(), kBlock, 0, s_>>>(d_, x64_, y64_, (S.status == ST_CONVERGED && S.ret_avg) ? 1 : 0);
     PDNQP_CK(cudaGetLastError());
     DevState Z = S;
-    Z.cur = 0;
+    reset_buffers(&Z);
     Z.status = ST_IDLE;
     PDNQP_CK(cudaMemcpyAsync(st_, &Z, sizeof(Z), cudaMemcpyHostToDevice, s_));
     return 0;
@@ -1599,6 +1631,7 @@ class Solver : public SolverBase {
   bool ready_ = false, solved_once_ = false, has_x0_ = false, has_l0_ = false, own_stream_ = false;
   bool tuned_ = false;
   std::vector<double> h_x0_, h_l0_;
+  std::vector<unsigned char> long_flag_;  // dense coupling rows (empty when there are none)
   Result res_;
 };
 
