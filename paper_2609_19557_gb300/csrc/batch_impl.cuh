@@ -73,7 +73,7 @@ class BatchRunner : public BatchBase, public BatchHook {
       devs[i] = sv_[i]->d_;
       devs[i].hw = 0;
       devs[i].hc = 0;
-      nbr[i] = sv_[i]->nb_rows();
+      nbr[i] = sv_[i]->nb_rows(lanes(g_rows_[i]));
     }
     BTRY(upload(&devs_, devs));
     BTRY(upload(&nbr_, nbr));
@@ -91,8 +91,8 @@ class BatchRunner : public BatchBase, public BatchHook {
     for (int g : {4, 8, 16}) {
       Launch r, c;
       r.g = c.g = g;
-      BTRY(add_map(&r, map_of([&](int i) { return sv_[i]->nb_rows(); }, [&](int i) { return g_rows_[i] == g; })));
-      BTRY(add_map(&c, map_of([&](int i) { return sv_[i]->nb_cols(); }, [&](int i) { return g_cols_[i] == g; })));
+      BTRY(add_map(&r, map_of([&](int i) { return sv_[i]->nb_rows(g); }, [&](int i) { return lanes(g_rows_[i]) == g; })));
+      BTRY(add_map(&c, map_of([&](int i) { return sv_[i]->nb_cols(g); }, [&](int i) { return lanes(g_cols_[i]) == g; })));
       if (r.nblk) rows_.push_back(r);
       if (c.nblk) cols_.push_back(c);
     }
@@ -202,6 +202,8 @@ class BatchRunner : public BatchBase, public BatchHook {
     BatchBlk *map = nullptr;
   };
 
+  // The setting that with_G makes of a lane parameter.
+  static int lanes(int g) { return g == 4 || g == 8 ? g : 16; }
   int fail(const std::string &m) {
     err_ = m;
     return PDNQP_ERR_CUDA;

@@ -126,19 +126,6 @@ __device__ __forceinline__ double warp_max(double v) {
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
-template <int G, typename A>
-__device__ __forceinline__ A group_sum(A v) {
-#pragma unroll
-  for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-template <int G, typename A>
-__device__ __forceinline__ A group_max(A v) {
-#pragma unroll
-  for (int o = G / 2; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-
 // The blocks a kernel's work is spread over: the hardware grid, or, in the
 // batched form, the contiguous run of blocks of one launch that one problem
 // of the batch owns (block b of nb).  Reductions and grid-stride loops use
@@ -149,52 +136,146 @@ struct GridCtx {
 };
 __device__ __forceinline__ GridCtx hw_grid() { return GridCtx{(int)blockIdx.x, (int)gridDim.x}; }
 
-// Block reduction of NQ doubles; bit q of kind_mask: 0 sum, 1 max (all maxima
-// are of non-negative values).  Thread 0... of the block writes
-// part[q * kMaxBlocks + blockIdx.x].  Must be called by every thread of the
-// block (kBlock threads).  On this GPU the FP64 pipe is narrow and its cost is
-// per active lane, so the reduction avoids FP64 shuffle trees: values go to
-// shared memory and 8 threads per quantity sum 32 values each serially, then
-// one thread sums the 8.  Fixed order: deterministic for a fixed grid.
-template <int NQ>
-__device__ __forceinline__ void block_reduce_store(double (&v)[NQ], const unsigned kind_mask, double *part,
-                                                   int blk = -1) {
-  if (blk < 0) blk = blockIdx.x;
-  constexpr int NW = kBlock / 32;
-  constexpr int WIN = 4;  // quantities staged at a time (8 KB of shared memory)
-  __shared__ double sm[WIN][kBlock];
-  __shared__ double s2[WIN][NW];
-  const int t = threadIdx.x;
+// Tests and comparisons of doubles on the integer pipes, a few instructions
+// each, instead of 16 cycles of the SM's FP64 pipe.  They work on the two words
+// (from the intrinsics: on the 64-bit pattern the compiler recognises the
+// floating-point test and emits it again).
+typedef unsigned long long u64;
+constexpr u64 kInfBits = 0x7ff0000000000000ull;
+__device__ __forceinline__ u64 abs_bits(double v) {
+  return ((u64)(unsigned)(__double2hiint(v) & 0x7fffffff) << 32) | (unsigned)__double2loint(v);
+}
+__device__ __forceinline__ bool nonfinite(double v) { return (__double2hiint(v) & 0x7fffffff) >= 0x7ff00000; }
+__device__ __forceinline__ bool is_nan_bits(double v) {
+  const int h = __double2hiint(v) & 0x7fffffff;
+  return h > 0x7ff00000 || (h == 0x7ff00000 && __double2loint(v) != 0);
+}
+// Order-preserving key (-0 before +0; NaN beyond the infinity of its sign).
+__device__ __forceinline__ long long order_key(double v) {
+  const int h = __double2hiint(v), s = h >> 31;
+  return ((long long)(h ^ (s & 0x7fffffff)) << 32) | (unsigned)(__double2loint(v) ^ s);
+}
+// a < b; false when either is NaN.
+__device__ __forceinline__ bool less_bits(double a, double b) {
+  return order_key(a) < order_key(b) && !is_nan_bits(a) && !is_nan_bits(b);
+}
+// Maximum of a non-negative `a` and |v|; a NaN v is left out (as fmax does).
+__device__ __forceinline__ double max_abs(double a, double v) {
+  const u64 b = abs_bits(v);
+  return b > abs_bits(a) && !is_nan_bits(v) ? __hiloint2double((int)(b >> 32), (int)(unsigned)b) : a;
+}
+__device__ __forceinline__ float max_abs(float a, float v) { return fmaxf(a, fabsf(v)); }
+
+// FP32 value as a double without the conversion instruction (which runs on the
+// FP64 pipe): exact; denormals, infinities and NaN take the instruction.
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v) {
+  const unsigned u = __float_as_uint(v), m = u & 0x7fffffffu;
+  if (m - 0x00800000u >= 0x7f000000u && m != 0u) return double(v);
+  return __hiloint2double((int)((u & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), (int)(u << 29));
+}
+
+// Reciprocal of a positive double by two Newton steps from the FP32 reciprocal
+// (4 FP64 instructions; a division is several times that), within a few units
+// in the last place; outside FP32's range the division.
+__device__ __forceinline__ double recip(double v) {
+  const float f = (float)v;
+  if (!(f > 1e-30f && f < 1e30f)) return 1.0 / v;
+  double r = widen(1.0f / f);
+  r = fma(r, fma(-v, r, 1.0), r);
+  return fma(r, fma(-v, r, 1.0), r);
+}
+__device__ __forceinline__ double recip(float v) {
+  if (!(v > 1e-30f && v < 1e30f)) return 1.0 / double(v);
+  const double d = widen(v);
+  double r = widen(1.0f / v);
+  r = fma(r, fma(-d, r, 1.0), r);
+  return fma(r, fma(-d, r, 1.0), r);
+}
+
+__host__ __device__ constexpr int count_bits(unsigned m) { return m == 0u ? 0 : (int)(m & 1u) + count_bits(m >> 1); }
+__host__ __device__ constexpr int next_pow2(int v) {
+  int p = 1;
+  while (p < v) p *= 2;
+  return p;
+}
+
+// Reduction of P values (a power of two up to 32) of every lane over the warp
+// by halving: at each level a lane hands over half of its values and joins the
+// other half, so P - 1 + log2(32 / P) additions instead of 5 P.  Lane l ends
+// with value l / (32 / P).
+template <int P, bool IsMax>
+__device__ __forceinline__ double warp_halve(double (&v)[P]) {
+  const int lane = threadIdx.x & 31;
+  int w = 16;
 #pragma unroll
-  for (int q0 = 0; q0 < NQ; q0 += WIN) {
+  for (int h = P / 2; h > 0; h >>= 1, w >>= 1) {
+    const bool up = (lane & w) != 0;
 #pragma unroll
-    for (int k = 0; k < WIN; ++k)
-      if (q0 + k < NQ) sm[k][t] = v[q0 + k];
-    __syncthreads();
-    if (t < WIN * NW) {
-      const int k = t / NW, c = t % NW, q = q0 + k;
-      if (q < NQ) {
-        const bool mx = (kind_mask >> q) & 1u;
-        const double *src = &sm[k][c * 32];
-        double a = src[0];
-        if (mx) {
-          for (int i = 1; i < 32; ++i) a = fmax(a, src[i]);
-        } else {
-          for (int i = 1; i < 32; ++i) a += src[i];
-        }
-        s2[k][c] = a;
-      }
+    for (int t = 0; t < h; ++t) {
+      const double keep = up ? v[t + h] : v[t], give = up ? v[t] : v[t + h];
+      const double o = __shfl_xor_sync(0xffffffffu, give, w);
+      v[t] = IsMax ? max_abs(keep, o) : keep + o;
     }
-    __syncthreads();
-    if (t < WIN && q0 + t < NQ) {
-      const int q = q0 + t;
-      const bool mx = (kind_mask >> q) & 1u;
-      double a = s2[t][0];
-      for (int c = 1; c < NW; ++c) a = mx ? fmax(a, s2[t][c]) : a + s2[t][c];
-      part[q * kMaxBlocks + blk] = a;
-    }
-    __syncthreads();
   }
+  double r = v[0];
+#pragma unroll
+  for (; w > 0; w >>= 1) {
+    const double o = __shfl_xor_sync(0xffffffffu, r, w);
+    r = IsMax ? max_abs(r, o) : r + o;
+  }
+  return r;
+}
+
+// Block reduction of NQ doubles; bit q of MASK: 0 sum, 1 maximum (of
+// non-negative values).  The block writes part[q * kMaxBlocks + blk].  Must be
+// called by every thread of the block (kBlock threads).  Sums and maxima are
+// reduced over the warp by halving, then one thread per quantity joins the
+// warps' values in order.  Fixed order: deterministic for a fixed grid.
+template <int NQ, unsigned MASK>
+__device__ __forceinline__ void block_reduce_store(double (&v)[NQ], double *part, int blk = -1) {
+  if (blk < 0) blk = blockIdx.x;
+  constexpr int NW = kBlock / 32, NM = count_bits(MASK), NS = NQ - NM;
+  constexpr int PS = next_pow2(NS > 0 ? NS : 1), PM = next_pow2(NM > 0 ? NM : 1);
+  static_assert(PS <= 32 && PM <= 32, "at most 32 quantities of a kind");
+  __shared__ double sm[NQ][NW];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  double s[PS], m[PM];
+#pragma unroll
+  for (int k = 0; k < PS; ++k) s[k] = 0.0;
+#pragma unroll
+  for (int k = 0; k < PM; ++k) m[k] = 0.0;
+  // idx: quantity of each slot (compile time after unrolling).
+  int is = 0, im = 0;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    if ((MASK >> q) & 1u)
+      m[im++] = v[q];
+    else
+      s[is++] = v[q];
+  }
+  __syncthreads();  // sm of an earlier call has been read
+  const double rs = NS > 0 ? warp_halve<PS, false>(s) : 0.0, rm = NM > 0 ? warp_halve<PM, true>(m) : 0.0;
+  is = 0;
+  im = 0;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    if ((MASK >> q) & 1u) {
+      if (lane == im * (32 / PM)) sm[q][w] = rm;
+      ++im;
+    } else {
+      if (lane == is * (32 / PS)) sm[q][w] = rs;
+      ++is;
+    }
+  }
+  __syncthreads();
+  if (t < NQ) {
+    const bool mx = (MASK >> t) & 1u;
+    double a = sm[t][0];
+    for (int k = 1; k < NW; ++k) a = mx ? max_abs(a, sm[t][k]) : a + sm[t][k];
+    part[t * kMaxBlocks + blk] = a;
+  }
+  __syncthreads();
 }
 
 // Grid barrier of a cooperative (co-resident) launch.  bar[0] counts the
@@ -384,212 +465,31 @@ __device__ __forceinline__ void final_reduce(const double *part, int nb, const u
   __syncthreads();
 }
 
-// Rows of a CSR matrix are processed by groups of G lanes (G divides 32).
-// Iteration is warp-uniform: every lane of a warp runs the same trips
-// (base is the same for the whole warp), with row >= nrows marking idle
-// groups, so group shuffles are always executed by the full warp.
-template <int G>
-struct GroupIter {
-  int lane_g, sub;
-  long long first, step;
-  __device__ __forceinline__ GroupIter() {
-    lane_g = threadIdx.x & (G - 1);
-    sub = (threadIdx.x & 31) / G;
-    const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    first = gw * (32 / G);
-    step = nw * (32 / G);
-  }
-};
-
-// Sum over the entries of one row of f(col, val), reduced over the group; every
-// lane of the group gets the result.
-template <int G, typename Acc, typename T, typename F>
-__device__ __forceinline__ Acc row_sum(const int *__restrict__ rp, const int *__restrict__ ci,
-                                       const T *__restrict__ val, long long row, bool valid, int lane_g, F f) {
-  Acc a = Acc(0);
-  if (valid) {
-    const int b = rp[row], e = rp[row + 1];
-    for (int k = b + lane_g; k < e; k += G) a += f(ci[k], val[k]);
-  }
-  return group_sum<G, Acc>(a);
-}
-template <int G, typename Acc, typename T, typename F>
-__device__ __forceinline__ Acc row_max(const int *__restrict__ rp, const int *__restrict__ ci,
-                                       const T *__restrict__ val, long long row, bool valid, int lane_g, F f) {
-  Acc a = Acc(0);
-  if (valid) {
-    const int b = rp[row], e = rp[row + 1];
-    for (int k = b + lane_g; k < e; k += G) a = fmax(a, f(ci[k], val[k]));
-  }
-  return group_max<G, Acc>(a);
-}
-
-
-// Warp tiles of 32 consecutive rows: lane l owns row tile + l for the
-// epilogue (all lanes active, coalesced per-row loads and stores), while the
-// row dot products are computed by groups of G lanes in G passes of 32/G rows
-// each, and the result of each row is shuffled to the lane that owns it.
+// Warp tiles of consecutive rows: lane l < TR owns row tile + l (coalesced
+// per-row loads and stores).  K: lane setting of the matrix the kernel works
+// through (tile_reduce): 32 rows a warp, 8 with K = 16, where a row keeps the
+// whole warp busy (on rows of 100 entries, 8 x 32 entries are in flight either
+// way, and a small matrix spreads over four times as many warps).
+template <int K>
 struct TileIter {
+  static constexpr int TR = K == 16 ? 8 : 32;
   int lane;
   long long first, step;
   __device__ __forceinline__ TileIter(GridCtx g = hw_grid()) {
     lane = threadIdx.x & 31;
     const long long gw = ((long long)g.b * blockDim.x + threadIdx.x) >> 5;
     const long long nw = ((long long)g.nb * blockDim.x) >> 5;
-    first = gw * 32;
-    step = nw * 32;
+    first = gw * TR;
+    step = nw * TR;
+  }
+  // Row of this lane in a tile; false past the tile or the matrix.
+  __device__ __forceinline__ bool row(long long tile, long long nrows, long long &i) const {
+    i = tile + lane;
+    return (TR == 32 || lane < TR) && i < nrows;
   }
 };
-
-template <typename Acc>
-__device__ __forceinline__ Acc shfl_any(Acc v, int src) {
-  return __shfl_sync(0xffffffffu, v, src);
-}
-
-// Per-warp staging buffer of one CSR-stream chunk: 32 * K entries.
-template <int K, typename Acc>
-__device__ __forceinline__ Acc *warp_stage_buffer() {
-  __shared__ Acc buf[kBlock / 32][32 * K];
-  return buf[threadIdx.x >> 5];
-}
-
-// CSR-stream row reduction over a warp tile of 32 consecutive rows: the
-// tile's contiguous nonzero range is streamed in chunks of 32 * K entries;
-// each lane loads K entries with coalesced, independent loads, evaluates
-// f(col, val) (including its gather) and stores it in the warp's staging
-// buffer; then lane l reduces the slice of the chunk that belongs to row
-// tile + l.  Rows of any length are handled (a long row spans several
-// chunks).  Lane l returns the result of row tile + l (0 past nrows).
-template <int K, bool IsMax, typename Acc, typename T, typename F>
-__device__ __forceinline__ Acc tile_stream(const int *__restrict__ rp, const int *__restrict__ ci,
-                                           const T *__restrict__ val, long long tile, long long nrows, F f) {
-  const int lane = threadIdx.x & 31;
-  Acc *sb = warp_stage_buffer<K, Acc>();
-  const long long my = tile + lane;
-  const long long last = (nrows - 1 - tile) < 31 ? (nrows - 1 - tile) : 31;  // last valid lane (>= 0)
-  int rb = 0, re = 0;
-  if (my < nrows) {
-    rb = rp[my];
-    re = rp[my + 1];
-  }
-  const int base = __shfl_sync(0xffffffffu, rb, 0);
-  const int end = __shfl_sync(0xffffffffu, re, (int)last);
-  if (my >= nrows) rb = re = end;
-  Acc acc = Acc(0);
-  for (int c0 = base; c0 < end; c0 += 32 * K) {
-    Acc p[K];
-#pragma unroll
-    for (int j = 0; j < K; ++j) {
-      const int k = c0 + j * 32 + lane;
-      p[j] = k < end ? f(ci[k], val[k]) : Acc(0);
-    }
-#pragma unroll
-    for (int j = 0; j < K; ++j) sb[j * 32 + lane] = p[j];
-    __syncwarp();
-    const int lo = rb > c0 ? rb : c0;
-    const int hi = re < c0 + 32 * K ? re : c0 + 32 * K;
-    for (int k = lo; k < hi; ++k) acc = IsMax ? fmax(acc, sb[k - c0]) : acc + sb[k - c0];
-    __syncwarp();
-  }
-  return acc;
-}
-
-// Two CSR matrices with the same rows streamed together over one warp tile
-// (the column pass: Q and A^T): both row-pointer pairs, then in every trip
-// one chunk of each matrix, so the two dependent load chains (row pointers ->
-// entries -> gathers) overlap instead of running one after the other.  Lane l
-// gets the sums of row tile + l of both matrices in o1, o2.
-template <int K1, int K2, typename Acc, typename T, typename F1, typename F2>
-__device__ __forceinline__ void tile_pair_sum(const int *__restrict__ rp1, const int *__restrict__ ci1,
-                                              const T *__restrict__ v1, const int *__restrict__ rp2,
-                                              const int *__restrict__ ci2, const T *__restrict__ v2, long long tile,
-                                              long long nrows, F1 f1, F2 f2, Acc &o1, Acc &o2) {
-  const int lane = threadIdx.x & 31;
-  Acc *sb1 = warp_stage_buffer<K1, Acc>();
-  __shared__ Acc buf2[kBlock / 32][32 * K2];
-  Acc *sb2 = buf2[threadIdx.x >> 5];
-  const long long my = tile + lane;
-  const long long last = (nrows - 1 - tile) < 31 ? (nrows - 1 - tile) : 31;
-  int rb1 = 0, re1 = 0, rb2 = 0, re2 = 0;
-  if (my < nrows) {
-    rb1 = rp1[my];
-    re1 = rp1[my + 1];
-    rb2 = rp2[my];
-    re2 = rp2[my + 1];
-  }
-  const int base1 = __shfl_sync(0xffffffffu, rb1, 0), end1 = __shfl_sync(0xffffffffu, re1, (int)last);
-  const int base2 = __shfl_sync(0xffffffffu, rb2, 0), end2 = __shfl_sync(0xffffffffu, re2, (int)last);
-  if (my >= nrows) {
-    rb1 = re1 = end1;
-    rb2 = re2 = end2;
-  }
-  Acc a1 = Acc(0), a2 = Acc(0);
-  for (int c1 = base1, c2 = base2; c1 < end1 || c2 < end2; c1 += 32 * K1, c2 += 32 * K2) {
-    Acc p1[K1], p2[K2];
-#pragma unroll
-    for (int j = 0; j < K1; ++j) {
-      const int k = c1 + j * 32 + lane;
-      p1[j] = k < end1 ? f1(ci1[k], v1[k]) : Acc(0);
-    }
-#pragma unroll
-    for (int j = 0; j < K2; ++j) {
-      const int k = c2 + j * 32 + lane;
-      p2[j] = k < end2 ? f2(ci2[k], v2[k]) : Acc(0);
-    }
-#pragma unroll
-    for (int j = 0; j < K1; ++j) sb1[j * 32 + lane] = p1[j];
-#pragma unroll
-    for (int j = 0; j < K2; ++j) sb2[j * 32 + lane] = p2[j];
-    __syncwarp();
-    {
-      const int lo = rb1 > c1 ? rb1 : c1, hi = re1 < c1 + 32 * K1 ? re1 : c1 + 32 * K1;
-      for (int k = lo; k < hi; ++k) a1 += sb1[k - c1];
-    }
-    {
-      const int lo = rb2 > c2 ? rb2 : c2, hi = re2 < c2 + 32 * K2 ? re2 : c2 + 32 * K2;
-      for (int k = lo; k < hi; ++k) a2 += sb2[k - c2];
-    }
-    __syncwarp();
-  }
-  o1 = a1;
-  o2 = a2;
-}
-
-template <int K, typename Acc, typename T, typename F>
-__device__ __forceinline__ Acc tile_row_sum(const int *__restrict__ rp, const int *__restrict__ ci,
-                                            const T *__restrict__ val, long long tile, long long nrows, F f) {
-  return tile_stream<K, false, Acc>(rp, ci, val, tile, nrows, f);
-}
-template <int K, typename Acc, typename T, typename F>
-__device__ __forceinline__ Acc tile_row_max(const int *__restrict__ rp, const int *__restrict__ ci,
-                                            const T *__restrict__ val, long long tile, long long nrows, F f) {
-  return tile_stream<K, true, Acc>(rp, ci, val, tile, nrows, f);
-}
-
-// Tests and comparisons of doubles on the integer pipes, a few instructions
-// each, instead of 16 cycles of the SM's FP64 pipe.  They work on the two words
-// (from the intrinsics: on the 64-bit pattern the compiler recognises the
-// floating-point test and emits it again).
-typedef unsigned long long u64;
-constexpr u64 kInfBits = 0x7ff0000000000000ull;
-__device__ __forceinline__ u64 abs_bits(double v) {
-  return ((u64)(unsigned)(__double2hiint(v) & 0x7fffffff) << 32) | (unsigned)__double2loint(v);
-}
-__device__ __forceinline__ bool nonfinite(double v) { return (__double2hiint(v) & 0x7fffffff) >= 0x7ff00000; }
-__device__ __forceinline__ bool is_nan_bits(double v) {
-  const int h = __double2hiint(v) & 0x7fffffff;
-  return h > 0x7ff00000 || (h == 0x7ff00000 && __double2loint(v) != 0);
-}
-// Order-preserving key (-0 before +0; NaN beyond the infinity of its sign).
-__device__ __forceinline__ long long order_key(double v) {
-  const int h = __double2hiint(v), s = h >> 31;
-  return ((long long)(h ^ (s & 0x7fffffff)) << 32) | (unsigned)(__double2loint(v) ^ s);
-}
-// a < b; false when either is NaN.
-__device__ __forceinline__ bool less_bits(double a, double b) {
-  return order_key(a) < order_key(b) && !is_nan_bits(a) && !is_nan_bits(b);
-}
+// Rows one block of a tile kernel takes in a trip.
+inline int tile_rows_per_block(int k) { return kBlock / 32 * (k == 16 ? 8 : 32); }
 
 // ---------------------------------------------------------------------------
 // Row reductions of CSR matrices, one warp per tile of consecutive rows.  Lane
@@ -611,10 +511,11 @@ struct __align__(2 * sizeof(Acc)) Slot {
 constexpr int kSlotLd = 9;                     // slots of a row in a round's buffer (8 and one of padding)
 constexpr int kTileSlots = 32 * kSlotLd;       // slots of one warp and matrix
 constexpr int kLongRowEntries = 32;            // longer rows are summed by the whole warp
+constexpr int kRowAlone = 512;                 // rows this long get a warp's 256 entries a round (tile_long_rows gives a row 32)
 
 template <bool IsMax, typename A>
-__device__ __forceinline__ A acc_join(A a, A b) {
-  return IsMax ? (a < b ? b : a) : a + b;
+__device__ __forceinline__ A acc_join(A a, A b) {  // maxima: of non-negative values
+  return IsMax ? max_abs(a, b) : a + b;
 }
 
 // One row of any length by the whole warp, 256 entries a round; every lane
@@ -780,7 +681,7 @@ __device__ __forceinline__ Acc tile_rows1(const int *ci, const T *val, int rb, i
   return out[0];
 }
 
-// Long rows (8 of them, lanes 0..7): all 32 lanes on each row, the 8 rows
+// Long rows (8 of them, brought by lanes 0..7; lane l gets row l mod 8): all 32 lanes on each row, the 8 rows
 // together (a round takes 32 entries of each).  The lanes' partial sums are
 // reduced by halving: at every level a lane hands over half of its rows and
 // adds the other half, 9 additions for the 8 rows instead of 40.
@@ -788,13 +689,15 @@ template <bool IsMax, typename Acc, typename T, typename F>
 __device__ __forceinline__ Acc tile_long_rows(const int *__restrict__ ci, const T *__restrict__ val, int rb, int re,
                                               const F &f) {
   const int lane = threadIdx.x & 31;
-  const int longest = (int)__reduce_max_sync(0xffffffffu, (unsigned)(re - rb));
+  const bool alone = re - rb > kRowAlone;
+  const int se = alone ? rb : re;
+  const int longest = (int)__reduce_max_sync(0xffffffffu, (unsigned)(se - rb));
   int pos[8], end[8];
   Acc acc[8];
 #pragma unroll
   for (int t = 0; t < 8; ++t) {
     pos[t] = __shfl_sync(0xffffffffu, rb, t) + lane;
-    end[t] = __shfl_sync(0xffffffffu, re, t);
+    end[t] = __shfl_sync(0xffffffffu, se, t);
     acc[t] = Acc(0);
   }
   for (int s = 0; s < longest; s += 32) {
@@ -827,7 +730,75 @@ __device__ __forceinline__ Acc tile_long_rows(const int *__restrict__ ci, const 
   }
 #pragma unroll
   for (int v = 2; v > 0; v >>= 1) acc[0] = acc_join<IsMax>(acc[0], __shfl_xor_sync(0xffffffffu, acc[0], v));
-  return __shfl_sync(0xffffffffu, acc[0], (lane & 7) * 4);  // row l ended in lanes 4 l .. 4 l + 3
+  Acc out = __shfl_sync(0xffffffffu, acc[0], (lane & 7) * 4);  // row l ended in lanes 4 l .. 4 l + 3
+  unsigned todo = __ballot_sync(0xffffffffu, alone);
+  while (todo) {
+    const int l = __ffs(todo) - 1;
+    todo &= todo - 1;
+    const Acc v = warp_row<IsMax, Acc>(ci, val, __shfl_sync(0xffffffffu, rb, l), __shfl_sync(0xffffffffu, re, l), f);
+    if ((lane & 7) == l) out = v;
+  }
+  return out;
+}
+
+// What an entry multiplies (gather) and how it is added (add), as two lambdas.
+template <typename G, typename A>
+struct Entry {
+  G g;
+  A a;
+  template <typename I>
+  __device__ __forceinline__ auto gather(I k) const { return g(k); }
+  template <typename Acc>
+  __device__ __forceinline__ void add(Acc &acc, Acc v, Acc x) const { a(acc, v, x); }
+};
+template <typename G, typename A>
+__device__ __forceinline__ Entry<G, A> entry(G g, A a) {
+  return Entry<G, A>{g, a};
+}
+// The usual ways to add an entry.
+struct AddProduct {
+  template <typename Acc>
+  __device__ __forceinline__ void operator()(Acc &acc, Acc v, Acc x) const { acc += v * x; }
+};
+struct AddAbs {
+  template <typename Acc>
+  __device__ __forceinline__ void operator()(Acc &acc, Acc v, Acc x) const { acc += fabs(v * x); }
+};
+struct MaxAbs {
+  template <typename Acc>
+  __device__ __forceinline__ void operator()(Acc &acc, Acc v, Acc x) const { acc = max_abs(acc, v * x); }
+};
+
+// The buffer of tile_rows for one warp and one matrix (kernels of kBlock
+// threads; FP32 needs none).
+template <typename Acc>
+__device__ __forceinline__ Slot<Acc> *warp_slots() {
+  if (sizeof(Acc) == 4) return nullptr;
+  __shared__ Slot<double> buf[kBlock / 32][kTileSlots];
+  return reinterpret_cast<Slot<Acc> *>(buf[threadIdx.x >> 5]);
+}
+
+// Row reduction of a warp tile (TileIter<K>); lane l gets row tile + l.  K: the
+// matrix's lane setting, 16 = long rows (8 rows, all 32 lanes on each), 4 or 8
+// = short rows (32 rows).
+template <int K, bool IsMax, typename Acc, typename T, typename F>
+__device__ __forceinline__ Acc tile_reduce(const int *rp, const int *ci, const T *val, long long tile, long long nrows,
+                                           const F &f) {
+  const long long my = tile + (threadIdx.x & 31);
+  const bool ok = (threadIdx.x & 31) < TileIter<K>::TR && my < nrows;
+  const int rb = ok ? rp[my] : 0, re = ok ? rp[my + 1] : 0;
+  return K == 16 ? tile_long_rows<IsMax, Acc>(ci, val, rb, re, f)
+                 : tile_rows1<IsMax, Acc>(ci, val, rb, re, f, warp_slots<Acc>());
+}
+template <int K, typename Acc, typename T, typename F>
+__device__ __forceinline__ Acc tile_row_sum(const int *rp, const int *ci, const T *val, long long tile, long long nrows,
+                                            const F &f) {
+  return tile_reduce<K, false, Acc>(rp, ci, val, tile, nrows, f);
+}
+template <int K, typename Acc, typename T, typename F>
+__device__ __forceinline__ Acc tile_row_max(const int *rp, const int *ci, const T *val, long long tile, long long nrows,
+                                            const F &f) {
+  return tile_reduce<K, true, Acc>(rp, ci, val, tile, nrows, f);
 }
 
 // Product with a vector that other blocks wrote before the last grid barrier of

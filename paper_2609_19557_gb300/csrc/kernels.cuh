@@ -420,10 +420,11 @@ __device__ __forceinline__ void rows_phase(const Dev<T> &d, const DevState *st, 
           omap = k0[kOmap];
   const T *xt = d.x[st->xtr];
   T Lt = T(0), Le = T(0), RH = T(0), RB = T(0);
-  TileIter ti(g);
+  TileIter<G> ti(g);
   for (long long tile = ti.first; tile < d.m; tile += ti.step) {
-    const long long j = tile + ti.lane;
-    const bool valid = j < d.m && !(d.nlr && d.lr_flag[j]), ineq = j >= d.mE;
+    long long j;
+    const bool own = ti.row(tile, d.m, j);
+    const bool valid = own && !(d.nlr && d.lr_flag[j]), ineq = j >= d.mE;
     // Everything that does not need (A x_tr)_j first (the r and s blocks of
     // the trial and the operands of the dual step), so that these loads
     // overlap the SpMV chain.
@@ -454,7 +455,7 @@ __device__ __forceinline__ void rows_phase(const Dev<T> &d, const DevState *st, 
       etj = d.eta[j];
       hpj = d.hp[j];
     }
-    const T ax = tile_row_sum<G, T>(d.As.rp, d.As.ci, d.As.val, tile, d.m, [&](int k, T a) { return a * __ldcg(xt + k); });
+    const T ax = tile_row_sum<G, T>(d.As.rp, d.As.ci, d.As.val, tile, d.m, MulLd<T>{xt});
     if (valid) {
       T bwt = ax - rt;
       if (ineq) bwt -= stv;
@@ -469,7 +470,7 @@ __device__ __forceinline__ void rows_phase(const Dev<T> &d, const DevState *st, 
     }
   }
   double v[4] = {double(Lt), double(Le), double(RH), double(RB)};
-  block_reduce_store<4>(v, 0u, d.part + P_TR_R * kMaxBlocks, g.b);
+  block_reduce_store<4, 0u>(v, d.part + P_TR_R * kMaxBlocks, g.b);
 }
 
 // Row pass of one trial over the blocks of g (graph and batched forms).
@@ -491,29 +492,28 @@ __global__ void __launch_bounds__(kBlock) k_rows(Dev<T> d) {
 
 // Variable rows: (H x_tr)_i and (A' y_tr)_i (the products with Q and A^T),
 // plus the x terms of the acceptance sums.
-template <typename T, int GH, int GT>
+template <typename T, int G>
 __device__ __forceinline__ void cols_phase(const Dev<T> &d, const DevState *st, GridCtx g = hw_grid()) {
   const int cur = st->cur, nx = 1 - cur;
   const T *xt = d.x[st->xtr], *xc = d.x[st->xcur];
   const T *yt = d.y[nx];
   T Lt = T(0), RH = T(0), RB = T(0);
-  TileIter ti(g);
+  TileIter<G> ti(g);
   for (long long tile = ti.first; tile < d.n; tile += ti.step) {
-    const long long i = tile + ti.lane;
+    long long i;
+    const bool own = ti.row(tile, d.n, i);
     // Row-local operands first: their loads overlap the SpMV chains.
     T xti = T(0), xci = T(0), hxc = T(0), atc = T(0), itx = T(0);
-    if (i < d.n) {
+    if (own) {
       xti = xt[i];
       xci = xc[i];
       hxc = d.Hx[cur][i];
       atc = d.Aty[cur][i];
       itx = d.itaux[i];
     }
-    T hx, aty;
-    tile_pair_sum<GH, GT, T>(
-        d.H.rp, d.H.ci, d.H.val, d.At.rp, d.At.ci, d.At.val, tile, d.n,
-        [&](int k, T a) { return a * __ldcg(xt + k); }, [&](int k, T a) { return a * __ldcg(yt + k); }, hx, aty);
-    if (i < d.n) {
+    const T hx = tile_row_sum<G, T>(d.H.rp, d.H.ci, d.H.val, tile, d.n, MulLd<T>{xt});
+    const T aty = tile_row_sum<G, T>(d.At.rp, d.At.ci, d.At.val, tile, d.n, MulLd<T>{yt});
+    if (own) {
       d.Hx[nx][i] = hx;
       d.Aty[nx][i] = aty;
       const T dx = xti - xci;
@@ -525,7 +525,7 @@ __device__ __forceinline__ void cols_phase(const Dev<T> &d, const DevState *st, 
     }
   }
   double v[4] = {double(Lt), 0.0, double(RH), double(RB)};
-  block_reduce_store<4>(v, 0u, d.part + P_TR_C * kMaxBlocks, g.b);
+  block_reduce_store<4, 0u>(v, d.part + P_TR_C * kMaxBlocks, g.b);
 }
 
 // Column pass of one trial over the blocks of g, with the acceptance decision
@@ -536,7 +536,7 @@ __device__ __forceinline__ void cols_trial_body(const Dev<T> &d, int nb_r, GridC
     stop_loop<COND>(d.hw, d.hc);
     return;
   }
-  cols_phase<T, G, G>(d, d.st, g);
+  cols_phase<T, G>(d, d.st, g);
   if (arrive_last(d.ctr, g.nb)) {
     decide_body<COND>(d.st, d.part, d.nlr ? d.lr_acc : nullptr, nb_r, g.nb, d.hw, d.hc);
     if (threadIdx.x == 0) d.ctr[0] = 0u;
@@ -577,15 +577,6 @@ struct WarpItems {
     step = (long long)(blockDim.x >> 5) * gridDim.x;
   }
 };
-
-// A FP32 sum as a double without the conversion instruction (which runs on the
-// FP64 pipe): exact; zeros, denormals, infinities and NaN take the instruction.
-__device__ __forceinline__ double widen(double v) { return v; }
-__device__ __forceinline__ double widen(float v) {
-  const unsigned u = __float_as_uint(v), e = u & 0x7f800000u;
-  if (e == 0u || e == 0x7f800000u) return double(v);
-  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
-}
 
 // This thread's terms of the acceptance sums of a trial, over its rows and
 // columns: dw^2 / tau0, dy^2 / eta0, |dw'H dw|, |dw'B'dy|.
@@ -1148,34 +1139,30 @@ struct RowIn {
   double rb, yb;                 // base r and y
   double ls, us;                 // shifted slack bounds
   double es, er, dsc;            // column scales of s, r and the row scale
+  double ies, ier, idsc;         // their reciprocals
   double sst, rst, yst;          // epoch-start corrections
 };
 
 __device__ __forceinline__ void row_cand(double *q, const RowIn &a) {
   const double e_bh = a.bwd - a.hp;  // (B w - h)_j
-  q[0] = fmax(q[0], fabs(e_bh));
-  q[1] = fmax(q[1], fmax(fabs(a.bwb + a.bwd), fabs(a.h)));
+  q[0] = max_abs(q[0], e_bh);
+  q[1] = max_abs(max_abs(q[1], a.bwb + a.bwd), a.h);
   const double gr = a.qr + a.sig * a.dr + a.dyv;  // sigma r + lambda + y at the point
-  q[2] = fmax(q[2], fabs(gr));
-  q[3] = fmax(q[3], fmax(fabs(a.sig * (a.rb + a.dr)), fmax(fabs(a.lam), fabs(a.yb + a.dyv))));
-  q[4] += (a.dsc * e_bh) * (a.dsc * e_bh);
-  q[5] += (a.er * gr) * (a.er * gr);
-  const double wr = (a.dr - a.rst) / a.er;
+  q[2] = max_abs(q[2], gr);
+  q[3] = max_abs(max_abs(max_abs(q[3], a.sig * (a.rb + a.dr)), a.lam), a.yb + a.dyv);
+  const double eb = a.dsc * e_bh, eg = a.er * gr;
+  q[4] += eb * eb;
+  q[5] += eg * eg;
+  const double wr = (a.dr - a.rst) * a.ier;
   q[6] += wr * wr;
-  const double wy = (a.dyv - a.yst) / a.dsc;
+  const double wy = (a.dyv - a.yst) * a.idsc;
   q[7] += wy * wy;
   if (a.ineq) {
     const double gs = a.qs + a.dyv;  // y at the point
-    double p = a.ds - gs;
-    p = p < a.ls ? a.ls : p;
-    p = p > a.us ? a.us : p;
-    q[2] = fmax(q[2], fabs(a.ds - p));
-    double p2 = a.ds - a.es * a.es * gs;
-    p2 = p2 < a.ls ? a.ls : p2;
-    p2 = p2 > a.us ? a.us : p2;
-    const double ks = (a.ds - p2) / a.es;
+    q[2] = max_abs(q[2], a.ds - clampv<double>(a.ds - gs, a.ls, a.us));
+    const double ks = (a.ds - clampv<double>(a.ds - a.es * a.es * gs, a.ls, a.us)) * a.ies;
     q[5] += ks * ks;
-    const double ws = (a.ds - a.sst) / a.es;
+    const double ws = (a.ds - a.sst) * a.ies;
     q[6] += ws * ws;
   }
 }
@@ -1193,39 +1180,42 @@ __device__ __forceinline__ void check_rows_body(const Dev<T> &d, int mode, GridC
   double q[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) q[k] = 0.0;
-  TileIter ti(g);
+  TileIter<G> ti(g);
   for (long long tile = ti.first; tile < d.m; tile += ti.step) {
     T axb = T(0);
     if (mode == 0)
-      axb = tile_row_sum<G, T>(d.A.rp, d.A.ci, d.A.val, tile, d.m, [&](int k, T a) {
-        return a * (acc ? omap * xb0[k] + ap * xc[k] : xb0[k]);
-      });
-    const long long j = tile + ti.lane;
-    if (j < d.m) {
+      axb = tile_row_sum<G, T>(d.A.rp, d.A.ci, d.A.val, tile, d.m,
+                               entry([&](int k) { return acc ? omap * xb0[k] + ap * xc[k] : xb0[k]; }, AddProduct()));
+    long long j;
+    const bool own = ti.row(tile, d.m, j);
+    if (own) {
       const bool ineq = j >= d.mE;
       RowIn a;
       a.ineq = ineq;
-      a.hp = double(d.hp[j]);
-      a.bwb = double(d.Bwb[j]);
-      a.h = double(d.h[j]);
-      a.qs = ineq ? double(d.qs[j]) : 0.0;
-      a.qr = double(d.qr[j]);
+      a.hp = widen(d.hp[j]);
+      a.bwb = widen(d.Bwb[j]);
+      a.h = widen(d.h[j]);
+      a.qs = ineq ? widen(d.qs[j]) : 0.0;
+      a.qr = widen(d.qr[j]);
       a.sig = d.sig[j];
       a.lam = d.lam[j];
       a.rb = d.rb[j];
       a.yb = d.yb[j];
-      a.ls = ineq ? double(d.ls[j]) : 0.0;
-      a.us = ineq ? double(d.us[j]) : 0.0;
-      a.es = ineq ? double(d.es[j]) : 1.0;
-      a.er = double(d.er[j]);
-      a.dsc = double(d.dy[j]);
-      a.sst = ineq ? double(d.sst[j]) : 0.0;
-      a.rst = double(d.rst[j]);
-      a.yst = double(d.yst[j]);
-      a.bwd = double(d.Bw[cur][j]);
-      a.ds = ineq ? double(d.s[cur][j]) : 0.0;
-      a.dr = double(d.r[cur][j]);
-      a.dyv = double(d.y[cur][j]);
+      a.ls = ineq ? widen(d.ls[j]) : 0.0;
+      a.us = ineq ? widen(d.us[j]) : 0.0;
+      a.es = ineq ? widen(d.es[j]) : 1.0;
+      a.er = widen(d.er[j]);
+      a.dsc = widen(d.dy[j]);
+      a.ies = ineq ? recip(d.es[j]) : 1.0;
+      a.ier = recip(d.er[j]);
+      a.idsc = recip(d.dy[j]);
+      a.sst = ineq ? widen(d.sst[j]) : 0.0;
+      a.rst = widen(d.rst[j]);
+      a.yst = widen(d.yst[j]);
+      a.bwd = widen(d.Bw[cur][j]);
+      a.ds = ineq ? widen(d.s[cur][j]) : 0.0;
+      a.dr = widen(d.r[cur][j]);
+      a.dyv = widen(d.y[cur][j]);
       row_cand(q, a);
       if (mode == 0) {
         T sa = ineq ? d.sbar[a0][j] : T(0), ra = d.rbar[a0][j], ya = d.ybar[a0][j];
@@ -1241,15 +1231,15 @@ __device__ __forceinline__ void check_rows_body(const Dev<T> &d, int mode, GridC
         }
         const T bwa = axb - sa - ra;
         d.Bwbar[j] = bwa;
-        a.bwd = double(bwa);
-        a.ds = double(sa);
-        a.dr = double(ra);
-        a.dyv = double(ya);
+        a.bwd = widen(bwa);
+        a.ds = widen(sa);
+        a.dr = widen(ra);
+        a.dyv = widen(ya);
         row_cand(q + 8, a);
       }
     }
   }
-  block_reduce_store<16>(q, CK_MAXMASK, d.part + P_CK_R * kMaxBlocks, g.b);
+  block_reduce_store<16, CK_MAXMASK>(q, d.part + P_CK_R * kMaxBlocks, g.b);
 }
 
 template <typename T, int G>
@@ -1260,19 +1250,14 @@ __global__ void __launch_bounds__(kBlock) k_check_rows(Dev<T> d, int mode) {
 // Contributions of one variable (x block) to the 8 quantities of a candidate:
 // dx, H dx, A' dy corrections plus the base data of the variable.
 __device__ __forceinline__ void col_cand(double *q, double dx, double hdx, double atdy, double qx, double qx0,
-                                         double hxb, double atyb, double lx, double ux, double ex, double xst) {
+                                         double hxb, double atyb, double lx, double ux, double ex2, double iex,
+                                         double xst) {
   const double g = hdx + qx - atdy;  // gradient of the inner Lagrangian at the point
-  double p = dx - g;
-  p = p < lx ? lx : p;
-  p = p > ux ? ux : p;
-  q[2] = fmax(q[2], fabs(dx - p));
-  q[3] = fmax(q[3], fmax(fabs(hxb + hdx), fmax(fabs(qx0), fabs(atyb + atdy))));
-  double p2 = dx - ex * ex * g;
-  p2 = p2 < lx ? lx : p2;
-  p2 = p2 > ux ? ux : p2;
-  const double k = (dx - p2) / ex;
+  q[2] = max_abs(q[2], dx - clampv<double>(dx - g, lx, ux));
+  q[3] = max_abs(max_abs(max_abs(q[3], hxb + hdx), qx0), atyb + atdy);
+  const double k = (dx - clampv<double>(dx - ex2 * g, lx, ux)) * iex;
   q[5] += k * k;
-  const double w = (dx - xst) / ex;
+  const double w = (dx - xst) * iex;
   q[6] += w * w;
 }
 
@@ -1288,18 +1273,18 @@ __device__ __forceinline__ void check_cols_body(const Dev<T> &d, int mode, int n
   double q[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) q[k] = 0.0;
-  TileIter ti(g);
+  TileIter<G> ti(g);
   for (long long tile = ti.first; tile < d.n; tile += ti.step) {
     T atyb = T(0);
     if (mode == 0)
-      atyb = tile_row_sum<G, T>(d.At.rp, d.At.ci, d.At.val, tile, d.n, [&](int k, T a) { return a * yb[k]; });
-    const long long i = tile + ti.lane;
-    if (i < d.n) {
-      const double qx = double(d.qx[i]), qx0 = double(d.qx0[i]), hxb = double(d.Hxb[i]);
-      const double atyb0 = double(d.Atyb[i]), lx = double(d.lx[i]), ux = double(d.ux[i]);
-      const double ex = double(d.ex[i]), xst = double(d.xst[i]);
-      col_cand(q, double(xc[i]), double(d.Hx[cur][i]), double(d.Aty[cur][i]), qx, qx0, hxb, atyb0, lx, ux, ex,
-               xst);
+      atyb = tile_row_sum<G, T>(d.At.rp, d.At.ci, d.At.val, tile, d.n, MulLdg<T>{yb});
+    long long i;
+    const bool own = ti.row(tile, d.n, i);
+    if (own) {
+      const double qx = widen(d.qx[i]), qx0 = widen(d.qx0[i]), hxb = widen(d.Hxb[i]);
+      const double atyb0 = widen(d.Atyb[i]), lx = widen(d.lx[i]), ux = widen(d.ux[i]);
+      const double ex = widen(d.ex[i]), xst = widen(d.xst[i]), iex = recip(d.ex[i]), ex2 = ex * ex;
+      col_cand(q, widen(xc[i]), widen(d.Hx[cur][i]), widen(d.Aty[cur][i]), qx, qx0, hxb, atyb0, lx, ux, ex2, iex, xst);
       if (mode == 0) {
         d.Atybar[i] = atyb;
         T xa = d.xbar[a0][i], ha = d.Hxbar[a0][i];
@@ -1309,11 +1294,11 @@ __device__ __forceinline__ void check_cols_body(const Dev<T> &d, int mode, int n
           d.xbar[ab][i] = xa;
           d.Hxbar[ab][i] = ha;
         }
-        col_cand(q + 8, double(xa), double(ha), double(atyb), qx, qx0, hxb, atyb0, lx, ux, ex, xst);
+        col_cand(q + 8, widen(xa), widen(ha), widen(atyb), qx, qx0, hxb, atyb0, lx, ux, ex2, iex, xst);
       }
     }
   }
-  block_reduce_store<16>(q, CK_MAXMASK, d.part + P_CK_C * kMaxBlocks, g.b);
+  block_reduce_store<16, CK_MAXMASK>(q, d.part + P_CK_C * kMaxBlocks, g.b);
   if (arrive_last(d.ctr + 1, g.nb)) {
     if (mode == 0)
       check_final_body<COND>(d.st, d.part, nb_r, g.nb, d.hw);
@@ -1458,14 +1443,16 @@ __global__ void __launch_bounds__(kBlock) k_check_apply(Dev<T> d) {
 // r_b = v - b_E on equality rows; then B w_b, h' = h - B w_b, the base
 // gradients of the s and r blocks, the shifted slack bounds, and zero
 // corrections.
-template <typename T>
+template <typename T, int G>
 __global__ void __launch_bounds__(kBlock) k_base_rows(Dev<T> d, Mat<double> Ad, const double *lc, const double *uc,
                                                       double *sb, double *rb) {
   const int cur = d.st->cur;
   const double *__restrict__ x = d.xb;
-  PDNQP_GRID_STRIDE(j, d.m) {
-    double v = 0.0;
-    for (int k = Ad.rp[j]; k < Ad.rp[j + 1]; ++k) v += Ad.val[k] * x[Ad.ci[k]];
+  TileIter<G> ti;
+  for (long long tile = ti.first; tile < d.m; tile += ti.step) {
+    const double v = tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double>{x});
+    long long j;
+    if (!ti.row(tile, d.m, j)) continue;
     const double lam = d.lam[j], sig = d.sig[j], yb = d.yb[j];
     double s = 0.0, r, bw;
     if (j >= d.mE) {
@@ -1505,12 +1492,13 @@ __global__ void __launch_bounds__(kBlock) k_base_cols(Dev<T> d, Mat<double> Hd, 
   const int cur = d.st->cur;
   const double *__restrict__ x = d.xb;
   const double *__restrict__ y = d.yb;
-  TileIter ti;
+  TileIter<G> ti;
   for (long long tile = ti.first; tile < d.n; tile += ti.step) {
-    const double hx = tile_row_sum<G, double>(Hd.rp, Hd.ci, Hd.val, tile, d.n, [&](int k, double a) { return a * x[k]; });
-    const double aty = tile_row_sum<G, double>(Atd.rp, Atd.ci, Atd.val, tile, d.n, [&](int k, double a) { return a * y[k]; });
-    const long long i = tile + ti.lane;
-    if (i < d.n) {
+    const double hx = tile_row_sum<G, double>(Hd.rp, Hd.ci, Hd.val, tile, d.n, MulLdg<double>{x});
+    const double aty = tile_row_sum<G, double>(Atd.rp, Atd.ci, Atd.val, tile, d.n, MulLdg<double>{y});
+    long long i;
+    const bool own = ti.row(tile, d.n, i);
+    if (own) {
       const double q0 = c[i] - z[i] * ginv;
       d.qx0[i] = T(q0);
       d.qx[i] = T(q0 + hx - aty);
@@ -1544,13 +1532,14 @@ __device__ __forceinline__ double rsqrt_t(double v) { return rsqrt(v); }
 // max(max_k |e_k H_ki e_i|, max_j |d_j A_ji e_i|), in the storage precision T.
 template <typename T, int G>
 __global__ void __launch_bounds__(kBlock) k_iruiz_cols(Dev<T> d, double *cnx) {
-  TileIter ti;
+  TileIter<G> ti;
   for (long long tile = ti.first; tile < d.n; tile += ti.step) {
-    const long long i = tile + ti.lane;
+    long long i;
+    const bool own = ti.row(tile, d.n, i);
     // e_i is applied after the reduction (max over k of |e_k H_ki| times e_i).
-    const T a = tile_row_max<G, T>(d.H.rp, d.H.ci, d.H.val, tile, d.n, [&](int k, T v) { return fabs(d.ex[k] * v); });
-    const T b = tile_row_max<G, T>(d.At.rp, d.At.ci, d.At.val, tile, d.n, [&](int k, T v) { return fabs(d.dy[k] * v); });
-    if (i < d.n) cnx[i] = double(fmax(a, b) * d.ex[i]);
+    const T a = tile_row_max<G, T>(d.H.rp, d.H.ci, d.H.val, tile, d.n, entry([&](int k) { return d.ex[k]; }, MaxAbs()));
+    const T b = tile_row_max<G, T>(d.At.rp, d.At.ci, d.At.val, tile, d.n, entry([&](int k) { return d.dy[k]; }, MaxAbs()));
+    if (own) cnx[i] = double(fmax(a, b) * d.ex[i]);
   }
 }
 
@@ -1558,11 +1547,12 @@ __global__ void __launch_bounds__(kBlock) k_iruiz_cols(Dev<T> d, double *cnx) {
 // d_j e_s (I rows), d_j e_r); s column: d_j e_s; r column: max(e_r^2 sigma_j, d_j e_r).
 template <typename T, int G>
 __global__ void __launch_bounds__(kBlock) k_iruiz_rows(Dev<T> d, double *rn, double *cns, double *cnr) {
-  TileIter ti;
+  TileIter<G> ti;
   for (long long tile = ti.first; tile < d.m; tile += ti.step) {
-    const T a = tile_row_max<G, T>(d.A.rp, d.A.ci, d.A.val, tile, d.m, [&](int k, T v) { return fabs(v * d.ex[k]); });
-    const long long j = tile + ti.lane;
-    if (j < d.m) {
+    const T a = tile_row_max<G, T>(d.A.rp, d.A.ci, d.A.val, tile, d.m, entry([&](int k) { return d.ex[k]; }, MaxAbs()));
+    long long j;
+    const bool own = ti.row(tile, d.m, j);
+    if (own) {
       const T dj = d.dy[j];
       const T er = d.er[j];
       T rowv = fmax(a * dj, dj * er);
@@ -1600,16 +1590,14 @@ __global__ void k_iruiz_update(Dev<T> d, const double *cnx, const double *rn, co
 // storage precision; imwx = 1 / m_w is kept for m_y.
 template <typename T, int G>
 __global__ void __launch_bounds__(kBlock) k_mw_cols(Dev<T> d, double *imwx) {
-  TileIter ti;
+  TileIter<G> ti;
   for (long long tile = ti.first; tile < d.n; tile += ti.step) {
-    const T h1 = tile_row_sum<G, T>(d.H.rp, d.H.ci, d.H.val, tile, d.n, [&](int k, T v) { return fabs(d.ex[k] * v); });
-    const T b1 = tile_row_sum<G, T>(d.At.rp, d.At.ci, d.At.val, tile, d.n, [&](int k, T v) { return fabs(d.dy[k] * v); });
-    const T b2 = tile_row_sum<G, T>(d.At.rp, d.At.ci, d.At.val, tile, d.n, [&](int k, T v) {
-      const T bb = d.dy[k] * v;
-      return T(d.sig[k]) * bb * bb;
-    });
-    const long long i = tile + ti.lane;
-    if (i < d.n) {
+    const T h1 = tile_row_sum<G, T>(d.H.rp, d.H.ci, d.H.val, tile, d.n, entry([&](int k) { return d.ex[k]; }, AddAbs()));
+    const T b1 = tile_row_sum<G, T>(d.At.rp, d.At.ci, d.At.val, tile, d.n, entry([&](int k) { return d.dy[k]; }, AddAbs()));
+    const T b2 = tile_row_sum<G, T>(d.At.rp, d.At.ci, d.At.val, tile, d.n, entry([&](int k) { return d.sg[k] * d.dy[k] * d.dy[k]; }, [](T &acc, T v, T x) { acc += x * v * v; }));
+    long long i;
+    const bool own = ti.row(tile, d.n, i);
+    if (own) {
       const T ei = d.ex[i];
       const T mw = h1 * ei + fmax(b1 * ei, sqrt(b2) * ei);
       imwx[i] = double(T(1) / mw);
@@ -1623,14 +1611,12 @@ __global__ void __launch_bounds__(kBlock) k_mw_cols(Dev<T> d, double *imwx) {
 // eta_eff / (kappa omega) = d^2 * 0.99 / m_y.
 template <typename T, int G>
 __global__ void __launch_bounds__(kBlock) k_my_rows(Dev<T> d, const double *imwx) {
-  TileIter ti;
+  TileIter<G> ti;
   for (long long tile = ti.first; tile < d.m; tile += ti.step) {
-    const T a = tile_row_sum<G, T>(d.A.rp, d.A.ci, d.A.val, tile, d.m, [&](int k, T v) {
-      const T bb = v * d.ex[k];
-      return bb * bb * T(imwx[k]);
-    });
-    const long long j = tile + ti.lane;
-    if (j < d.m) {
+    const T a = tile_row_sum<G, T>(d.A.rp, d.A.ci, d.A.val, tile, d.m, entry([&](int k) { return d.ex[k] * d.ex[k] * T(imwx[k]); }, [](T &acc, T v, T x) { acc += x * v * v; }));
+    long long j;
+    const bool own = ti.row(tile, d.m, j);
+    if (own) {
       const T dj = d.dy[j];
       const T sg = T(d.sig[j]);
       const T er = d.er[j];

@@ -17,30 +17,25 @@ namespace {  // internal linkage: each solver TU owns its kernels
 // ---------------------------------------------------------------------------
 template <int G>
 __global__ void __launch_bounds__(kBlock) k_oruiz_rows(Mat<double> A, const double *Dc, const double *Dx, double *rn) {
-  GroupIter<G> it;
-  for (long long base = it.first; base < A.nrows; base += it.step) {
-    const long long j = base + it.sub;
-    const bool valid = j < A.nrows;
-    const double dj = valid ? Dc[j] : 0.0;
-    const double a = row_max<G, double>(A.rp, A.ci, A.val, j, valid, it.lane_g,
-                                        [&](int k, double v) { return fabs(dj * v * Dx[k]); });
-    if (valid && it.lane_g == 0) rn[j] = a;
+  TileIter<G> ti;
+  for (long long tile = ti.first; tile < A.nrows; tile += ti.step) {
+    long long j;
+    const bool own = ti.row(tile, A.nrows, j);
+    const double a = tile_row_max<G, double>(A.rp, A.ci, A.val, tile, A.nrows, entry([&](int k) { return Dx[k]; }, MaxAbs()));
+    if (own) rn[j] = a * Dc[j];
   }
 }
 
 template <int G>
 __global__ void __launch_bounds__(kBlock) k_oruiz_cols(Mat<double> At, Mat<double> Q, const double *Dc,
                                                        const double *Dx, double *cn) {
-  GroupIter<G> it;
-  for (long long base = it.first; base < Q.nrows; base += it.step) {
-    const long long i = base + it.sub;
-    const bool valid = i < Q.nrows;
-    const double di = valid ? Dx[i] : 0.0;
-    const double a = row_max<G, double>(At.rp, At.ci, At.val, i, valid, it.lane_g,
-                                        [&](int k, double v) { return fabs(Dc[k] * v * di); });
-    const double b = row_max<G, double>(Q.rp, Q.ci, Q.val, i, valid, it.lane_g,
-                                        [&](int k, double v) { return fabs(di * v * Dx[k]); });
-    if (valid && it.lane_g == 0) cn[i] = fmax(a, b);
+  TileIter<G> ti;
+  for (long long tile = ti.first; tile < Q.nrows; tile += ti.step) {
+    long long i;
+    const bool own = ti.row(tile, Q.nrows, i);
+    const double a = tile_row_max<G, double>(At.rp, At.ci, At.val, tile, Q.nrows, entry([&](int k) { return Dc[k]; }, MaxAbs()));
+    const double b = tile_row_max<G, double>(Q.rp, Q.ci, Q.val, tile, Q.nrows, entry([&](int k) { return Dx[k]; }, MaxAbs()));
+    if (own) cn[i] = max_abs(a, b) * Dx[i];
   }
 }
 
@@ -51,12 +46,14 @@ __global__ void k_ruiz_apply(double *D, const double *nrm, long long len) {
   }
 }
 
-// val_k *= mult * rs[row] * cs[col]
+// val_k *= mult * rs[row] * cs[col] (a warp per row)
 __global__ void k_scale_csr(int nrows, const int *rp, const int *ci, double *val, const double *rs, const double *cs,
                             double mult) {
-  PDNQP_GRID_STRIDE(i, nrows) {
+  const int lane = threadIdx.x & 31;
+  for (long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < nrows;
+       i += ((long long)gridDim.x * blockDim.x) >> 5) {
     const double ri = rs[i] * mult;
-    for (int k = rp[i]; k < rp[i + 1]; ++k) val[k] = ri * val[k] * cs[ci[k]];
+    for (int k = rp[i] + lane; k < rp[i + 1]; k += 32) val[k] = ri * val[k] * cs[ci[k]];
   }
 }
 
@@ -64,22 +61,18 @@ __global__ void k_scale_csr(int nrows, const int *rp, const int *ci, double *val
 template <int G>
 __global__ void __launch_bounds__(kBlock) k_rowabs_max(Mat<double> M, double *part) {
   double best = 0.0;
-  GroupIter<G> it;
-  for (long long base = it.first; base < M.nrows; base += it.step) {
-    const long long i = base + it.sub;
-    const bool valid = i < M.nrows;
-    const double s = row_sum<G, double>(M.rp, M.ci, M.val, i, valid, it.lane_g, [&](int, double v) { return fabs(v); });
-    if (valid && it.lane_g == 0) best = fmax(best, s);
-  }
+  TileIter<G> ti;
+  for (long long tile = ti.first; tile < M.nrows; tile += ti.step)
+    best = max_abs(best, tile_row_sum<G, double>(M.rp, M.ci, M.val, tile, M.nrows, entry([](int) { return 1.0; }, AddAbs())));
   double v[1] = {best};
-  block_reduce_store<1>(v, 1u, part);
+  block_reduce_store<1, 1u>(v, part);
 }
 
 __global__ void k_absmax(const double *v, long long n, double *part) {
   double best = 0.0;
   PDNQP_GRID_STRIDE(i, n) best = fmax(best, fabs(v[i]));
   double q[1] = {best};
-  block_reduce_store<1>(q, 1u, part);
+  block_reduce_store<1, 1u>(q, part);
 }
 
 // Reduction of nq quantities (row q of part, nb partials each) -> out[q]:
@@ -132,7 +125,7 @@ __global__ void __launch_bounds__(kBlock) k_dot(const double *a, const double *b
   double s = 0.0;
   PDNQP_GRID_STRIDE(i, n) s += a[i] * b[i];
   double q[1] = {s};
-  block_reduce_store<1>(q, 0u, part);
+  block_reduce_store<1, 0u>(q, part);
 }
 // h = (b_E, 0) (Eq. inner-qp), b_E = l_c on the equality rows.
 template <typename T>
@@ -158,12 +151,11 @@ __global__ void k_start_vector(double *v, long long n, uint64_t seed) {
 
 template <int G>
 __global__ void __launch_bounds__(kBlock) k_spmv(Mat<double> M, const double *x, double *y) {
-  GroupIter<G> it;
-  for (long long base = it.first; base < M.nrows; base += it.step) {
-    const long long i = base + it.sub;
-    const bool valid = i < M.nrows;
-    const double s = row_sum<G, double>(M.rp, M.ci, M.val, i, valid, it.lane_g, [&](int k, double v) { return v * x[k]; });
-    if (valid && it.lane_g == 0) y[i] = s;
+  TileIter<G> ti;
+  for (long long tile = ti.first; tile < M.nrows; tile += ti.step) {
+    const double s = tile_row_sum<G, double>(M.rp, M.ci, M.val, tile, M.nrows, MulLdg<double>{x});
+    long long i;
+    if (ti.row(tile, M.nrows, i)) y[i] = s;
   }
 }
 
@@ -174,7 +166,7 @@ __global__ void __launch_bounds__(kBlock) k_multidot(const double *V, long long 
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     s += vp[i] * w[i];
   double q[1] = {s};
-  block_reduce_store<1>(q, 0u, part + (long long)blockIdx.y * kMaxBlocks);
+  block_reduce_store<1, 0u>(q, part + (long long)blockIdx.y * kMaxBlocks);
 }
 
 // w -= sum_{p < np} h[p] V[p]
@@ -230,13 +222,12 @@ __global__ void __launch_bounds__(kBlock) k_init_rows(Dev<T> d, Mat<double> Ad, 
                                                       double *lam, const double *sig, double *rprev, int pass) {
   const double *__restrict__ x = d.xb;
   double acc = 0.0;
-  GroupIter<G> it;
-  for (long long base = it.first; base < d.m; base += it.step) {
-    const long long j = base + it.sub;
-    const bool valid = j < d.m;
-    const double ax = row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, j, valid, it.lane_g,
-                                         [&](int k, double a) { return a * double(x[k]); });
-    if (valid && it.lane_g == 0) {
+  TileIter<G> ti;
+  for (long long tile = ti.first; tile < d.m; tile += ti.step) {
+    long long j;
+    const bool own = ti.row(tile, d.m, j);
+    const double ax = tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double>{x});
+    if (own) {
       const double lo = lc[j], hi = uc[j];
       if (pass == 0) {
         double p = ax;
@@ -257,7 +248,7 @@ __global__ void __launch_bounds__(kBlock) k_init_rows(Dev<T> d, Mat<double> Ad, 
     }
   }
   double v[1] = {acc};
-  block_reduce_store<1>(v, 0u, d.part);
+  block_reduce_store<1, 0u>(v, d.part);
 }
 
 // Partials of x'Qx (from H x - gamma^-1 x) and c'x.
@@ -265,20 +256,19 @@ template <typename T, int G>
 __global__ void __launch_bounds__(kBlock) k_objective(Dev<T> d, Mat<double> Hd, const double *c, double ginv) {
   const double *__restrict__ x = d.xb;
   double xqx = 0.0, cx = 0.0;
-  GroupIter<G> it;
-  for (long long base = it.first; base < d.n; base += it.step) {
-    const long long i = base + it.sub;
-    const bool valid = i < d.n;
-    const double hx = row_sum<G, double>(Hd.rp, Hd.ci, Hd.val, i, valid, it.lane_g,
-                                         [&](int k, double a) { return a * double(x[k]); });
-    if (valid && it.lane_g == 0) {
+  TileIter<G> ti;
+  for (long long tile = ti.first; tile < d.n; tile += ti.step) {
+    long long i;
+    const bool own = ti.row(tile, d.n, i);
+    const double hx = tile_row_sum<G, double>(Hd.rp, Hd.ci, Hd.val, tile, d.n, MulLdg<double>{x});
+    if (own) {
       const double xi = double(x[i]);
       xqx += xi * (hx - ginv * xi);
       cx += c[i] * xi;
     }
   }
   double v[2] = {xqx, cx};
-  block_reduce_store<2>(v, 0u, d.part);
+  block_reduce_store<2, 0u>(v, d.part);
 }
 
 // ---------------------------------------------------------------------------
@@ -299,12 +289,12 @@ __global__ void __launch_bounds__(kBlock) k_outer_rows(Dev<T> d, Mat<double> Ad,
   double q[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) q[k] = 0.0;
-  TileIter ti;
+  TileIter<G> ti;
   for (long long tile = ti.first; tile < d.m; tile += ti.step) {
-    const double ax = tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m,
-                                              [&](int k, double a) { return a * double(x[k]); });
-    const long long j = tile + ti.lane;
-    if (j < d.m) {
+    const double ax = tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double>{x});
+    long long j;
+    const bool own = ti.row(tile, d.m, j);
+    if (own) {
       const double lo = lc[j], hi = uc[j];
       if (update) {
         double s;
@@ -331,7 +321,7 @@ __global__ void __launch_bounds__(kBlock) k_outer_rows(Dev<T> d, Mat<double> Ad,
       q[3] = fmax(q[3], spv / dc);
     }
   }
-  block_reduce_store<12>(q, OUT_MAXMASK, d.part);
+  block_reduce_store<12, OUT_MAXMASK>(q, d.part);
 }
 
 // Column terms: Qx = H x - gamma^-1 x, A' lambda, projected stationarity in the
@@ -344,14 +334,13 @@ __global__ void __launch_bounds__(kBlock) k_outer_cols(Dev<T> d, Mat<double> Hd,
   double q[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) q[k] = 0.0;
-  TileIter ti;
+  TileIter<G> ti;
   for (long long tile = ti.first; tile < d.n; tile += ti.step) {
-    const double hx = tile_row_sum<G, double>(Hd.rp, Hd.ci, Hd.val, tile, d.n,
-                                              [&](int k, double a) { return a * double(x[k]); });
-    const double atl = tile_row_sum<G, double>(Atd.rp, Atd.ci, Atd.val, tile, d.n,
-                                               [&](int k, double a) { return a * lam[k]; });
-    const long long i = tile + ti.lane;
-    if (i < d.n) {
+    const double hx = tile_row_sum<G, double>(Hd.rp, Hd.ci, Hd.val, tile, d.n, MulLdg<double>{x});
+    const double atl = tile_row_sum<G, double>(Atd.rp, Atd.ci, Atd.val, tile, d.n, MulLdg<double>{lam});
+    long long i;
+    const bool own = ti.row(tile, d.n, i);
+    if (own) {
       const double xi = double(x[i]);
       const double qx = hx - ginv * xi;
       const double g = qx + c[i] + atl;
@@ -374,7 +363,7 @@ __global__ void __launch_bounds__(kBlock) k_outer_cols(Dev<T> d, Mat<double> Hd,
       q[11] += c[i] * xi;
     }
   }
-  block_reduce_store<12>(q, OUT_MAXMASK, d.part + 12 * kMaxBlocks);
+  block_reduce_store<12, OUT_MAXMASK>(q, d.part + 12 * kMaxBlocks);
 }
 
 // Infeasibility tests (Sec. "Infeasibility detection") on the scaled problem,
@@ -389,11 +378,12 @@ template <typename T, int G>
 __global__ void __launch_bounds__(kBlock) k_inf_rows(Dev<T> d, Mat<double> Ad, const double *lc, const double *uc,
                                                      const double *lam, const double *lam0, const double *dx) {
   double q[4] = {0.0, 0.0, 0.0, 0.0};
-  TileIter ti;
+  TileIter<G> ti;
   for (long long tile = ti.first; tile < d.m; tile += ti.step) {
-    const double ad = tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, [&](int k, double a) { return a * dx[k]; });
-    const long long j = tile + ti.lane;
-    if (j < d.m) {
+    const double ad = tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double>{dx});
+    long long j;
+    const bool own = ti.row(tile, d.m, j);
+    if (own) {
       const double y = lam[j] - lam0[j], lo = lc[j], hi = uc[j];
       if (y > 0.0) {
         if (isinf(hi)) q[0] = fmax(q[0], y); else q[1] += hi * y;
@@ -405,7 +395,7 @@ __global__ void __launch_bounds__(kBlock) k_inf_rows(Dev<T> d, Mat<double> Ad, c
       q[3] = fmax(q[3], fabs(y));
     }
   }
-  block_reduce_store<4>(q, INF_R_MAXMASK, d.part);
+  block_reduce_store<4, INF_R_MAXMASK>(q, d.part);
 }
 
 // Columns (7): 0 largest |v_i|, v = -A' dlam, that would need an infinite
@@ -418,13 +408,14 @@ __global__ void __launch_bounds__(kBlock) k_inf_cols(Dev<T> d, Mat<double> Hd, M
                                                      const double *lx, const double *ux, const double *lam,
                                                      const double *lam0, const double *dx, double ginv) {
   double q[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  TileIter ti;
+  TileIter<G> ti;
   for (long long tile = ti.first; tile < d.n; tile += ti.step) {
     const double atl = tile_row_sum<G, double>(Atd.rp, Atd.ci, Atd.val, tile, d.n,
-                                               [&](int k, double a) { return a * (lam[k] - lam0[k]); });
-    const double hd = tile_row_sum<G, double>(Hd.rp, Hd.ci, Hd.val, tile, d.n, [&](int k, double a) { return a * dx[k]; });
-    const long long i = tile + ti.lane;
-    if (i < d.n) {
+                                               entry([&](int k) { return lam[k] - lam0[k]; }, AddProduct()));
+    const double hd = tile_row_sum<G, double>(Hd.rp, Hd.ci, Hd.val, tile, d.n, MulLdg<double>{dx});
+    long long i;
+    const bool own = ti.row(tile, d.n, i);
+    if (own) {
       const double v = -atl, di = dx[i], qd = hd - ginv * di, lo = lx[i], hi = ux[i];
       if (v > 0.0) {
         if (isinf(hi)) q[0] = fmax(q[0], v); else q[1] += hi * v;
@@ -439,7 +430,7 @@ __global__ void __launch_bounds__(kBlock) k_inf_cols(Dev<T> d, Mat<double> Hd, M
       q[6] = fmax(q[6], fabs(di));
     }
   }
-  block_reduce_store<7>(q, INF_C_MAXMASK, d.part);
+  block_reduce_store<7, INF_C_MAXMASK>(q, d.part);
 }
 
 // Anderson acceleration (Sec. "Anderson acceleration"): sums of one Type-II
@@ -472,7 +463,7 @@ __global__ void __launch_bounds__(kBlock) k_aa_dots(const double *U, const doubl
     }
     q[NC * NC + NC] += f[NC] * f[NC];
   }
-  block_reduce_store<NQ>(q, 0u, part);
+  block_reduce_store<NQ, 0u>(q, part);
 }
 
 // The extrapolated point out = G_{L-1} - sum_a gam_a (G_{a+1} - G_a) and the
@@ -491,7 +482,7 @@ __global__ void __launch_bounds__(kBlock) k_aa_apply(const double *G, int head, 
     out[i] = G[(long long)((head + nc) % cap) * D + i] - v;
     sn[0] += v * v;
   }
-  block_reduce_store<1>(sn, 0u, part);
+  block_reduce_store<1, 0u>(sn, part);
 }
 
 __global__ void k_sub(long long n, const double *a, const double *b, double *out) {

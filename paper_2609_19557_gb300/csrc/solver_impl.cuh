@@ -25,9 +25,8 @@ namespace pdq {
     if (_r < 0) return _r;    \
   } while (0)
 
-// K = entries per lane per CSR-stream chunk (chunk = 32 K nonzeros per warp).
-// Kernels are instantiated for K in {4, 8, 16}; GroupIter kernels read it as
-// lanes per row.
+// The lane setting of a matrix (tile_reduce): 16 spreads a warp along each row,
+// 4 and 8 take tiles of 32 short rows.
 template <typename F>
 static void with_G(int g, F f) {
   switch (g) {
@@ -37,13 +36,9 @@ static void with_G(int g, F f) {
   }
 }
 
-// K from the mean row length: the smallest power of two >= mean, in [4, 16].
-static int pick_g(long long nnz, long long rows) {
-  const double mean = rows > 0 ? (double)nnz / (double)rows : 1.0;
-  int g = 4;
-  while (g < 16 && g < mean) g *= 2;
-  return g;
-}
+// From the mean row length: rounds of 8 entries a row pay until a row fills most
+// of a warp.
+static int pick_g(long long nnz, long long rows) { return rows > 0 && nnz > 24 * rows ? 16 : 8; }
 
 // Where a solver in the batched form hands its inner solves (BatchRunner).
 struct BatchHook {
@@ -271,7 +266,6 @@ class Solver : public SolverBase {
   int grid_n() const { return grid_for(n_, kBlock); }
   int grid_m() const { return grid_for(m_, kBlock); }
   int grid_nm() const { return grid_for(std::max(n_, m_), kBlock); }
-  int grid_rows_g(long long rows, int g) const { return grid_for(rows, kBlock / g); }
 
   int reduce_to_host(int nq, int nb, unsigned mask, double *out) {
     k_reduce_rows<<<nq, 32, 0, s_>>>(part_, nq, nb, mask, dred_);
@@ -345,25 +339,25 @@ class Solver : public SolverBase {
     for (int sw = 0; sw < prm.ruiz_outer; ++sw) {
       if (m_)
         with_G(gA_, [&](auto GG) {
-          k_oruiz_rows<decltype(GG)::value><<<grid_rows_g(m_, gA_), kBlock, 0, s_>>>(Ad_, Dc_, Dx_, scm_[0]);
+          k_oruiz_rows<decltype(GG)::value><<<nb_rows(), kBlock, 0, s_>>>(Ad_, Dc_, Dx_, scm_[0]);
         });
       with_G(gN_, [&](auto GG) {
-        k_oruiz_cols<decltype(GG)::value><<<grid_rows_g(n_, gN_), kBlock, 0, s_>>>(Atd_, Hd_, Dc_, Dx_, scn_[0]);
+        k_oruiz_cols<decltype(GG)::value><<<nb_cols(), kBlock, 0, s_>>>(Atd_, Hd_, Dc_, Dx_, scn_[0]);
       });
       if (m_) k_ruiz_apply<<<grid_m(), kBlock, 0, s_>>>(Dc_, scm_[0], m_);
       k_ruiz_apply<<<grid_n(), kBlock, 0, s_>>>(Dx_, scn_[0], n_);
     }
     PDNQP_CK(cudaGetLastError());
     if (m_) {
-      k_scale_csr<<<grid_m(), kBlock, 0, s_>>>(m_, arp, aci, av_, Dc_, Dx_, 1.0);
-      k_scale_csr<<<grid_n(), kBlock, 0, s_>>>(n_, atrp, atci, atv_, Dx_, Dc_, 1.0);
+      k_scale_csr<<<grid_for(m_, kBlock / 32), kBlock, 0, s_>>>(m_, arp, aci, av_, Dc_, Dx_, 1.0);
+      k_scale_csr<<<grid_for(n_, kBlock / 32), kBlock, 0, s_>>>(n_, atrp, atci, atv_, Dx_, Dc_, 1.0);
     }
-    k_scale_csr<<<grid_n(), kBlock, 0, s_>>>(n_, qrp, qci, qv_, Dx_, Dx_, 1.0);
+    k_scale_csr<<<grid_for(n_, kBlock / 32), kBlock, 0, s_>>>(n_, qrp, qci, qv_, Dx_, Dx_, 1.0);
     k_scale_vec<<<grid_n(), kBlock, 0, s_>>>(c_, Dx_, n_, 0, 1.0);
     // objective scalar c_s = 1 / max(1, ||Dx Q Dx||_inf, ||Dx c||_inf)
     double qn, cn;
     {
-      int nb = grid_rows_g(n_, gN_);
+      int nb = nb_cols();
       with_G(gN_, [&](auto GG) { k_rowabs_max<decltype(GG)::value><<<nb, kBlock, 0, s_>>>(Hd_, part_); });
       PDNQP_TRY(reduce_to_host(1, nb, 1u, &qn));
       nb = grid_n();
@@ -374,7 +368,7 @@ class Solver : public SolverBase {
     k_mul_scalar<<<grid_for(nnzH_, kBlock), kBlock, 0, s_>>>(qv_, nnzH_, cs_);
     k_mul_scalar<<<grid_n(), kBlock, 0, s_>>>(c_, n_, cs_);
     {
-      int nb = grid_rows_g(n_, gN_);
+      int nb = nb_cols();
       with_G(gN_, [&](auto GG) { k_rowabs_max<decltype(GG)::value><<<nb, kBlock, 0, s_>>>(Hd_, part_); });
       PDNQP_TRY(reduce_to_host(1, nb, 1u, &qnorm_));
     }
@@ -424,7 +418,7 @@ class Solver : public SolverBase {
     for (int j = 0; j < k; ++j) {
       double *vj = V_ + (long long)j * n;
       with_G(gN_, [&](auto GG) {
-        k_spmv<decltype(GG)::value><<<grid_rows_g(n, gN_), kBlock, 0, s_>>>(Hd_, vj, w);
+        k_spmv<decltype(GG)::value><<<nb_cols(), kBlock, 0, s_>>>(Hd_, vj, w);
       });
       PDNQP_TRY(dot(w, vj, &al[j]));
       used = j + 1;
@@ -652,9 +646,11 @@ class Solver : public SolverBase {
   }
 
   // ------------------------------------------------------- launchers
-  // Tile kernels: one warp per 32 rows and trip, kBlock / 32 warps per block.
-  int nb_rows() const { return grid_for(std::max(m_, 1), kBlock); }
-  int nb_cols() const { return grid_for(n_, kBlock); }
+  // Tile kernels: a tile per warp and trip, kBlock / 32 warps per block.
+  int nb_rows(int g) const { return grid_for(std::max(m_, 1), tile_rows_per_block(g)); }
+  int nb_cols(int g) const { return grid_for(n_, tile_rows_per_block(g)); }
+  int nb_rows() const { return nb_rows(gA_); }
+  int nb_cols() const { return nb_cols(gN_); }
   void launch_primal() { k_primal<T><<<grid_n(), kBlock, 0, s_>>>(d_); }
   void launch_rows() {
     with_G(gA_, [&](auto GG) { k_rows<T, decltype(GG)::value><<<nb_rows(), kBlock, 0, s_>>>(d_); });
@@ -942,7 +938,10 @@ class Solver : public SolverBase {
   int inner_setup(const Params &prm, double dta, double dtr, long long k_in, long long pause_at, int ignore) {
     const double ginv = 1.0 / gamma_;
     // Base point of this solve (FP64) and zero corrections.
-    if (m_) k_base_rows<T><<<grid_m(), kBlock, 0, s_>>>(d_, Ad_, lcd_, ucd_, sb64_, rb64_);
+    if (m_)
+      with_G(gA_, [&](auto GG) {
+        k_base_rows<T, decltype(GG)::value><<<nb_rows(), kBlock, 0, s_>>>(d_, Ad_, lcd_, ucd_, sb64_, rb64_);
+      });
     with_G(gN_, [&](auto GG) {
       k_base_cols<T, decltype(GG)::value><<<nb_cols(), kBlock, 0, s_>>>(d_, Hd_, Atd_, c_, z_, lxd_, uxd_, ginv);
     });
