@@ -511,6 +511,7 @@ struct __align__(2 * sizeof(Acc)) Slot {
 constexpr int kSlotLd = 9;                     // slots of a row in a round's buffer (8 and one of padding)
 constexpr int kTileSlots = 32 * kSlotLd;       // slots of one warp and matrix
 constexpr int kLongRowEntries = 32;            // longer rows are summed by the whole warp
+constexpr int kDenseRow = 1024;                // see one_row
 constexpr int kRowAlone = 512;                 // rows this long get a warp's 256 entries a round (tile_long_rows gives a row 32)
 
 template <bool IsMax, typename A>
@@ -545,6 +546,66 @@ __device__ __forceinline__ Acc warp_row(const int *__restrict__ ci, const T *__r
 #pragma unroll
   for (int w = 16; w > 0; w >>= 1) acc = acc_join<IsMax>(acc, __shfl_xor_sync(0xffffffffu, acc, w));
   return acc;
+}
+
+// The buffer of tile_rows for one warp and one matrix (kernels of kBlock
+// threads; FP32 needs none).
+template <typename Acc>
+__device__ __forceinline__ Slot<Acc> *warp_slots() {
+  if (sizeof(Acc) == 4) return nullptr;
+  __shared__ Slot<double> buf[kBlock / 32][kTileSlots];
+  return reinterpret_cast<Slot<Acc> *>(buf[threadIdx.x >> 5]);
+}
+
+// A row by one warp, in the order F asks for.  kOrder = 1 or 2: a dense row (more
+// than kDenseRow entries) is added entry by entry from the first, each with a
+// multiply-add (1) or its product rounded first (2).  The residual of a dense
+// equality row (the simplex row of a Motzkin-Straus problem) is a difference of
+// nearly equal numbers, and its multiplier follows the rounding of that sum: in
+// another order it moves by some 1e-9 of itself at 10,000 entries, so the two
+// kernels that take it (base point, multiplier update: once an outer iteration)
+// keep the order they always had.  Operands are loaded and gathered 256 at a
+// time; what is left is the chain of additions, 64 cycles each (0.3 ms at
+// 10,000 entries).
+template <bool IsMax, typename Acc, typename T, typename F>
+__device__ __forceinline__ Acc one_row(const int *__restrict__ ci, const T *__restrict__ val, int b, int e, const F &f) {
+  if constexpr (F::kOrder == 0) {
+    return warp_row<IsMax, Acc>(ci, val, b, e, f);
+  } else {
+    if (e - b <= kDenseRow) return warp_row<IsMax, Acc>(ci, val, b, e, f);
+    Slot<Acc> *buf = warp_slots<Acc>();
+    const int lane = threadIdx.x & 31;
+    Acc acc = Acc(0);
+    for (int k0 = b; k0 < e; k0 += 256) {
+      Slot<Acc> r[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int k = k0 + 32 * u + lane;
+        r[u] = k < e ? Slot<Acc>{Acc(__ldg(val + k)), f.gather(__ldg(ci + k))} : Slot<Acc>{Acc(0), Acc(0)};
+        if (F::kOrder == 2) r[u].x = __dmul_rn(r[u].a, r[u].x);
+      }
+      __syncwarp();
+      int cnt = 0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {  // entries that multiply zero change nothing: left out
+        const unsigned nz = __ballot_sync(0xffffffffu, r[u].x != Acc(0));
+        if (r[u].x != Acc(0)) buf[cnt + __popc(nz & ((1u << lane) - 1u))] = r[u];
+        cnt += __popc(nz);
+      }
+      __syncwarp();
+      int k = 0;
+      for (; k + 8 <= cnt; k += 8) {
+        Slot<Acc> v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = buf[k + u];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc = F::kOrder == 1 ? fma(v[u].a, v[u].x, acc) : acc + v[u].x;
+      }
+      for (; k < cnt; ++k) acc = F::kOrder == 1 ? fma(buf[k].a, buf[k].x, acc) : acc + buf[k].x;
+    }
+    __syncwarp();
+    return acc;
+  }
 }
 
 // Short rows (32 of them, NM matrices with the same rows).  A round takes 8
@@ -661,7 +722,7 @@ __device__ __forceinline__ void tile_rows(const int *const (&ci)[NM], const T *c
     for (int m = 0; m < NM; ++m) {
       const int b = __shfl_sync(0xffffffffu, rb[m], l), e = __shfl_sync(0xffffffffu, re[m], l);
       if (e - b > kLongRowEntries) {
-        const Acc v = warp_row<IsMax, Acc>(ci[m], val[m], b, e, f[m]);
+        const Acc v = one_row<IsMax, Acc>(ci[m], val[m], b, e, f[m]);
         if (lane == l) out[m] = v;
       }
     }
@@ -735,7 +796,7 @@ __device__ __forceinline__ Acc tile_long_rows(const int *__restrict__ ci, const 
   while (todo) {
     const int l = __ffs(todo) - 1;
     todo &= todo - 1;
-    const Acc v = warp_row<IsMax, Acc>(ci, val, __shfl_sync(0xffffffffu, rb, l), __shfl_sync(0xffffffffu, re, l), f);
+    const Acc v = one_row<IsMax, Acc>(ci, val, __shfl_sync(0xffffffffu, rb, l), __shfl_sync(0xffffffffu, re, l), f);
     if ((lane & 7) == l) out = v;
   }
   return out;
@@ -744,6 +805,7 @@ __device__ __forceinline__ Acc tile_long_rows(const int *__restrict__ ci, const 
 // What an entry multiplies (gather) and how it is added (add), as two lambdas.
 template <typename G, typename A>
 struct Entry {
+  static constexpr int kOrder = 0;
   G g;
   A a;
   template <typename I>
@@ -768,15 +830,6 @@ struct MaxAbs {
   template <typename Acc>
   __device__ __forceinline__ void operator()(Acc &acc, Acc v, Acc x) const { acc = max_abs(acc, v * x); }
 };
-
-// The buffer of tile_rows for one warp and one matrix (kernels of kBlock
-// threads; FP32 needs none).
-template <typename Acc>
-__device__ __forceinline__ Slot<Acc> *warp_slots() {
-  if (sizeof(Acc) == 4) return nullptr;
-  __shared__ Slot<double> buf[kBlock / 32][kTileSlots];
-  return reinterpret_cast<Slot<Acc> *>(buf[threadIdx.x >> 5]);
-}
 
 // Row reduction of a warp tile (TileIter<K>); lane l gets row tile + l.  K: the
 // matrix's lane setting, 16 = long rows (8 rows, all 32 lanes on each), 4 or 8
@@ -805,14 +858,16 @@ __device__ __forceinline__ Acc tile_row_max(const int *rp, const int *ci, const 
 // the same launch (not through the read-only path).
 template <typename T>
 struct MulLd {
+  static constexpr int kOrder = 0;
   const T *x;
   __device__ __forceinline__ T gather(int k) const { return x[k]; }
   __device__ __forceinline__ void add(T &acc, T a, T v) const { acc += a * v; }
 };
 
 // Product with a vector that no block writes meanwhile.
-template <typename T>
+template <typename T, int Order = 0>
 struct MulLdg {
+  static constexpr int kOrder = Order;  // see one_row
   const T *x;
   __device__ __forceinline__ T gather(int k) const { return __ldg(x + k); }
   __device__ __forceinline__ void add(T &acc, T a, T v) const { acc += a * v; }

@@ -42,7 +42,7 @@ constexpr unsigned CK_MAXMASK = 0x0F0Fu;  // quantities 0-3 and 8-11 of a check 
 constexpr int kCtrBar = 128, kCtrWords = kCtrBar + kBarWords;
 // Rows of A with more entries than this are treated as dense coupling rows
 // (at most kMaxLong of them, the longest first; the rest stay row-wise).
-constexpr int kLongRowMin = 1024;
+constexpr int kLongRowMin = kDenseRow;
 constexpr int kMaxLong = 64;
 
 template <typename T>
@@ -84,6 +84,7 @@ struct Dev {
   // those rows.  As is A with these rows emptied (As == A when nlr == 0).
   int nlr;
   int lr_nnz;
+  int lr_nb;       // parts of the split in the persistent loop
   Mat<T> As;
   const int *lr_row;   // [nlr] row index of each long row (ascending)
   const int *lr_ptr;   // [nlr + 1] offsets into lr_ci / lr_val
@@ -324,7 +325,8 @@ __device__ __forceinline__ void long_rows_partial(const Dev<T> &d, const T *xt, 
     const long long a0 = e0 > d.lr_ptr[s] ? e0 : d.lr_ptr[s];
     const long long a1 = e1 < d.lr_ptr[s + 1] ? e1 : d.lr_ptr[s + 1];
     T acc = T(0);
-    for (long long k = a0 + threadIdx.x; k < a1; k += blockDim.x) acc += d.lr_val[k] * __ldcg(xt + d.lr_ci[k]);
+    if (threadIdx.x < kBlock)
+      for (long long k = a0 + threadIdx.x; k < a1; k += kBlock) acc += d.lr_val[k] * __ldcg(xt + d.lr_ci[k]);
     const double v = block_sum_fixed(double(acc));
     if (threadIdx.x == 0) d.lr_part[(long long)s * kMaxBlocks + b] = v;
   }
@@ -595,7 +597,9 @@ __device__ __forceinline__ void rows_phase_tiles(const Dev<T> &d, const DevState
   const int cur = st->cur, nx = 1 - cur, a0 = st->acur, acc = st->accepted;
   const Scal<T> k0(st);
   const T *xt = d.x[st->xtr];
-  if (LR) long_rows_partial<T>(d, xt);
+  // The split of the dense rows is the instance's own (lr_nb parts), whatever the grid.
+  if (LR)
+    for (int b = blockIdx.x; b < d.lr_nb; b += gridDim.x) long_rows_partial<T>(d, xt, GridCtx{b, d.lr_nb});
   const WarpItems it;
   const long long nlong = LONG ? 0 : d.nlong_r, items = nlong + ((long long)d.m + TR - 1) / TR;
   const int *ci = d.As.ci;
@@ -969,7 +973,7 @@ __global__ void __launch_bounds__(kTrialThreads, 1) k_trials(Dev<T> d) {
     rows_phase_tiles<T, LR, RL>(d, &S, buf, ts);
     lap(2);
     if (loop_sync(bar, gen, [&] {
-          if (LR) long_rows_finish<T>(d, &S, nb);
+          if (LR) long_rows_finish<T>(d, &S, d.lr_nb);
           return 0;
         }) < 0)
       return;
@@ -1450,7 +1454,7 @@ __global__ void __launch_bounds__(kBlock) k_base_rows(Dev<T> d, Mat<double> Ad, 
   const double *__restrict__ x = d.xb;
   TileIter<G> ti;
   for (long long tile = ti.first; tile < d.m; tile += ti.step) {
-    const double v = tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double>{x});
+    const double v = tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double, 1>{x});
     long long j;
     if (!ti.row(tile, d.m, j)) continue;
     const double lam = d.lam[j], sig = d.sig[j], yb = d.yb[j];

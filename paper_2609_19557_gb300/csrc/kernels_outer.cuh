@@ -291,7 +291,8 @@ __global__ void __launch_bounds__(kBlock) k_outer_rows(Dev<T> d, Mat<double> Ad,
   for (int k = 0; k < 12; ++k) q[k] = 0.0;
   TileIter<G> ti;
   for (long long tile = ti.first; tile < d.m; tile += ti.step) {
-    const double ax = tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double>{x});
+    const double ax = update ? tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double, 2>{x})
+                             : tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double>{x});
     long long j;
     const bool own = ti.row(tile, d.m, j);
     if (own) {

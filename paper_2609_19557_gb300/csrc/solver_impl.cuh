@@ -581,6 +581,7 @@ class Solver : public SolverBase {
     Dev<T> &d = d_;
     d.nlr = 0;
     d.lr_nnz = 0;
+    d.lr_nb = 0;
     d.As = d.A;
     d.lr_row = d.lr_ptr = d.lr_ci = nullptr;
     d.lr_val = nullptr;
@@ -636,6 +637,8 @@ class Solver : public SolverBase {
     PDNQP_CK(cudaMemsetAsync(d.lr_acc, 0, 4 * sizeof(double), s_));
     d.nlr = nl;
     d.lr_nnz = lptr[nl];
+    // 256 threads a part: up to 3 (FP32) or 2 (FP64) parts an SM on 152 SMs, no more than the vectors have blocks.
+    d.lr_nb = std::min((sizeof(T) == 4 ? 3 : 2) * 152, grid_nm());
     d.lr_row = lrow;
     d.lr_ptr = lp;
     d.lr_ci = lci;
