@@ -121,12 +121,6 @@ __global__ void k_fill_d(double *p, long long n, double v) {
 __global__ void k_mul_scalar(double *p, long long n, double a) {
   PDNQP_GRID_STRIDE(i, n) p[i] *= a;
 }
-__global__ void __launch_bounds__(kBlock) k_dot(const double *a, const double *b, long long n, double *part) {
-  double s = 0.0;
-  PDNQP_GRID_STRIDE(i, n) s += a[i] * b[i];
-  double q[1] = {s};
-  block_reduce_store<1, 0u>(q, part);
-}
 // h = (b_E, 0) (Eq. inner-qp), b_E = l_c on the equality rows.
 template <typename T>
 __global__ void k_form_h(T *h, const double *lc, long long m, int mE) {
@@ -134,8 +128,7 @@ __global__ void k_form_h(T *h, const double *lc, long long m, int mE) {
 }
 
 // ---------------------------------------------------------------------------
-// Lanczos (Eq. R-choice): SpMV, dot products, full reorthogonalisation by
-// classical Gram-Schmidt applied twice.
+// Lanczos (Eq. R-choice): both starts in one cooperative launch.
 // ---------------------------------------------------------------------------
 // i-th output of the splitmix64 generator seeded with `seed`, mapped to [-0.5, 0.5).
 __device__ __forceinline__ double splitmix_uniform(uint64_t seed, uint64_t i) {
@@ -145,49 +138,238 @@ __device__ __forceinline__ double splitmix_uniform(uint64_t seed, uint64_t i) {
   z = z ^ (z >> 31);
   return (double)(z >> 11) * (1.0 / 9007199254740992.0) - 0.5;
 }
-__global__ void k_start_vector(double *v, long long n, uint64_t seed) {
-  PDNQP_GRID_STRIDE(i, n) v[i] = splitmix_uniform(seed, (uint64_t)i);
-}
+constexpr int kLzMax = 80;       // steps of a run, at most (and one)
+constexpr int kLzThreads = 512;  // as the trial loop: one block per SM
+constexpr int kLzFull = 1024;    // up to this size every step is orthogonalised in full
+// Loss of orthogonality at which a step is orthogonalised (the tridiagonal
+// matrix differs from that of exact arithmetic by its square).
+constexpr double kLzOmega = 1e-10;
 
-template <int G>
-__global__ void __launch_bounds__(kBlock) k_spmv(Mat<double> M, const double *x, double *y) {
-  TileIter<G> ti;
-  for (long long tile = ti.first; tile < M.nrows; tile += ti.step) {
-    const double s = tile_row_sum<G, double>(M.rp, M.ci, M.val, tile, M.nrows, MulLdg<double>{x});
-    long long i;
-    if (ti.row(tile, M.nrows, i)) y[i] = s;
+// Runs of `steps` Lanczos steps on the symmetric matrix Q from two start
+// vectors (seeds 1 and 2) side by side: out[s][0] = steps taken, then the
+// diagonal and the off-diagonal entries (kLzMax each).  V: [2][steps + 1][n]
+// basis vectors, w: [2][n].
+//
+// The basis is kept semi-orthogonal by partial reorthogonalisation (H. D.
+// Simon, Math. Comp. 42, 1984): the recurrence for the loss of orthogonality
+// runs along with the coefficients, and a step and the next one are
+// orthogonalised against the whole basis only when it passes kLzOmega.  Twice
+// orthogonalising every step reads the basis 4 times a step and needs 4 n j
+// FP64 multiply-adds, 8 ms at n = 300,000 for the pipe alone.  One launch
+// instead of 128 x 12 with 256 host synchronisations: the sums that a step
+// needs are formed by every block from the block partials (fixed order, the
+// same in all blocks), so a step is 3 grid barriers.  Measured (n = 300,001, 64
+// steps): see Solver::lanczos.
+template <int K>
+__global__ void __launch_bounds__(kLzThreads, 1) k_lanczos(Mat<double> Q, int steps, double *V, double *w, double *part,
+                                                           unsigned *bar, double *out) {
+  constexpr int NW = kLzThreads / 32;
+  __shared__ double al[2][kLzMax], be[2][kLzMax], om[2][3][kLzMax + 2];  // om: rows j - 1, j, j + 1 by j mod 3
+  __shared__ double red[NW][32], tot[2][kLzMax];
+  __shared__ int used[2], active[2], force[2], doit[2];
+  extern __shared__ __align__(16) unsigned char slots[];
+  const long long n = Q.nrows;
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5, nb = gridDim.x;
+  Slot<double> *buf = reinterpret_cast<Slot<double> *>(slots) + wid * kTileSlots;
+  unsigned gen = t == 0 ? ld_acquire_gpu(bar + kBarGen) : 0u;
+  const long long e0 = (long long)blockIdx.x * kLzThreads + t, es = (long long)nb * kLzThreads;
+  const WarpItems it;
+  constexpr int TR = TileIter<K>::TR;
+  const long long tiles = (n + TR - 1) / TR;
+  auto sync = [&] { return loop_sync(bar, gen, [] { return 0; }) >= 0; };
+  // One sum per start: block partials to part, then after a barrier totals in tot[s][0].
+  auto put2 = [&](double a, double b, double *dst) {
+    double v[2] = {a, b};
+    const double r = warp_halve<2, false>(v);
+    if ((lane & 15) == 0) red[wid][lane >> 4] = r;
+    __syncthreads();
+    if (t < 2) {
+      double x = red[0][t];
+      for (int k = 1; k < NW; ++k) x += red[k][t];
+      dst[2 * blockIdx.x + t] = x;
+    }
+  };
+  auto get2 = [&](const double *src) {
+    if (wid < 2) {
+      double x = 0.0;
+#pragma unroll 5
+      for (int b = lane; b < nb; b += 32) x += __ldcg(src + 2 * b + wid);
+      x = warp_sum(x);
+      if (lane == 0) tot[wid][0] = x;
+    }
+    __syncthreads();
+  };
+  double *pa = part, *pb = part + 2 * kMaxBlocks, *ph = part + 4 * kMaxBlocks;  // ph: [block][2][kLzMax]
+  if (t < 2) {
+    used[t] = 0;
+    active[t] = 1;
+    force[t] = 0;
   }
-}
-
-// Partials of V[p] . w for p = blockIdx.y (rows p of part).
-__global__ void __launch_bounds__(kBlock) k_multidot(const double *V, long long n, const double *w, double *part) {
-  const double *vp = V + (long long)blockIdx.y * n;
-  double s = 0.0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    s += vp[i] * w[i];
-  double q[1] = {s};
-  block_reduce_store<1, 0u>(q, part + (long long)blockIdx.y * kMaxBlocks);
-}
-
-// w -= sum_{p < np} h[p] V[p]
-__global__ void k_multiaxpy(const double *V, long long n, const double *h, int np, double *w) {
-  PDNQP_GRID_STRIDE(i, n) {
-    double s = w[i];
-    for (int p = 0; p < np; ++p) s -= h[p] * V[(long long)p * n + i];
-    w[i] = s;
+  // Normalised start vectors.
+  double s0 = 0.0, s1 = 0.0;
+  for (long long i = e0; i < n; i += es) {
+    const double a = splitmix_uniform(1ull, (uint64_t)i), b = splitmix_uniform(2ull, (uint64_t)i);
+    w[i] = a;
+    w[n + i] = b;
+    s0 += a * a;
+    s1 += b * b;
   }
-}
-
-// w = w - a v - b u   (u may be null)
-__global__ void k_lanczos_axpy(double *w, const double *v, const double *u, double a, double b, long long n) {
-  PDNQP_GRID_STRIDE(i, n) {
-    double s = w[i] - a * v[i];
-    if (u) s -= b * u[i];
-    w[i] = s;
+  put2(s0, s1, pb);
+  if (!sync()) return;
+  get2(pb);
+  for (int s = 0; s < 2; ++s) {
+    const double f = 1.0 / sqrt(tot[s][0]);
+    for (long long i = e0; i < n; i += es) V[(size_t)s * (steps + 1) * n + i] = w[s * n + i] * f;
   }
-}
-__global__ void k_scale_into(double *dst, const double *src, double a, long long n) {
-  PDNQP_GRID_STRIDE(i, n) dst[i] = src[i] * a;
+  if (!sync()) return;
+  for (int j = 0; j < steps; ++j) {
+    // w = Q v_j and alpha_j = w . v_j.
+    double a[2] = {0.0, 0.0};
+    for (long long tile = it.first; tile < tiles; tile += it.step) {
+      const long long i = tile * TR + lane;
+      const bool ok = lane < TR && i < n;
+      const int rb = ok ? __ldg(Q.rp + i) : 0, re = ok ? __ldg(Q.rp + i + 1) : 0;
+#pragma unroll
+      for (int s = 0; s < 2; ++s)
+        if (active[s]) {
+          const double *v = V + ((size_t)s * (steps + 1) + j) * n;
+          const MulLd<double> f{v};
+          const double q = K == 16 ? tile_long_rows<false, double>(Q.ci, Q.val, rb, re, f)
+                                   : tile_rows1<false, double>(Q.ci, Q.val, rb, re, f, buf);
+          if (ok) {
+            w[s * n + i] = q;
+            a[s] += q * v[i];
+          }
+        }
+    }
+    put2(a[0], a[1], pa);
+    if (!sync()) return;
+    get2(pa);
+    if (t < 2 && active[t]) {
+      al[t][j] = tot[t][0];
+      used[t] = j + 1;
+    }
+    __syncthreads();
+    // w -= alpha_j v_j + beta_{j-1} v_{j-1}.
+    a[0] = a[1] = 0.0;
+    for (int s = 0; s < 2; ++s)
+      if (active[s]) {
+        const double *v = V + ((size_t)s * (steps + 1) + j) * n;
+        const double aj = al[s][j], bj = j > 0 ? be[s][j - 1] : 0.0;
+        for (long long i = e0; i < n; i += es) {
+          double x = w[s * n + i] - aj * v[i];
+          if (j > 0) x -= bj * v[i - n];
+          w[s * n + i] = x;
+          a[s] += x * x;
+        }
+      }
+    put2(a[0], a[1], pb);
+    if (!sync()) return;
+    get2(pb);
+    // Loss of orthogonality of the new vector against v_0 .. v_{j-1}, a lane each.
+    if (wid < 2 && active[wid]) {
+      const int s = wid;
+      const double b = sqrt(tot[s][0]), eps = 1.1102230246251565e-16;
+      const double *oj = om[s][j % 3], *om1 = om[s][(j + 2) % 3];
+      double *on = om[s][(j + 1) % 3];
+      double worst = 0.0;
+      for (int k = lane; k < j; k += 32) {
+        double x = be[s][k] * (k + 1 == j ? 1.0 : oj[k + 1]) + (al[s][k] - al[s][j]) * oj[k];
+        if (k > 0) x += be[s][k - 1] * oj[k - 1];
+        x -= be[s][j - 1] * (k + 1 == j ? 1.0 : om1[k]);
+        x = (x + copysign(eps * (be[s][k] + b), x)) / b;
+        on[k] = x;
+        worst = fmax(worst, fabs(x));
+      }
+      worst = warp_max(worst);
+      if (lane == 0) {
+        on[j] = eps * sqrt((double)n);
+        doit[s] = n <= kLzFull || force[s] || !(worst < kLzOmega);
+        force[s] = doit[s] && !force[s];
+        be[s][j] = b;
+      }
+    } else if (wid < 2 && lane == 0) {
+      doit[wid] = 0;
+    }
+    __syncthreads();
+    if (doit[0] | doit[1]) {
+      // h = V' w over 32 basis vectors at a time (a lane's 32 sums are joined by
+      // halving), then w -= V h.
+      for (int s = 0; s < 2; ++s)
+        if (doit[s])
+          for (int p0 = 0; p0 <= j; p0 += 32) {
+            double acc[32];
+#pragma unroll
+            for (int p = 0; p < 32; ++p) acc[p] = 0.0;
+            const double *v = V + ((size_t)s * (steps + 1) + p0) * n;
+            for (long long i = e0; i < n; i += es) {
+              const double x = w[s * n + i];
+#pragma unroll
+              for (int p = 0; p < 32; ++p)
+                if (p0 + p <= j) acc[p] += v[(size_t)p * n + i] * x;
+            }
+            const double r = warp_halve<32, false>(acc);
+            red[wid][lane] = r;
+            __syncthreads();
+            if (t < 32) {
+              double x = red[0][t];
+              for (int k = 1; k < NW; ++k) x += red[k][t];
+              if (p0 + t < kLzMax) ph[((size_t)blockIdx.x * 2 + s) * kLzMax + p0 + t] = x;
+            }
+            __syncthreads();
+          }
+      if (!sync()) return;
+      for (int s = 0; s < 2; ++s)
+        if (doit[s])
+          for (int p = t; p <= j; p += kLzThreads) {
+            double x = 0.0;
+            for (int b = 0; b < nb; ++b) x += __ldcg(ph + ((size_t)b * 2 + s) * kLzMax + p);
+            tot[s][p] = x;
+          }
+      __syncthreads();
+      a[0] = a[1] = 0.0;
+      for (int s = 0; s < 2; ++s)
+        if (doit[s]) {
+          const double *v = V + (size_t)s * (steps + 1) * n;
+          for (long long i = e0; i < n; i += es) {
+            double x = w[s * n + i];
+            for (int p = 0; p <= j; ++p) x -= tot[s][p] * v[(size_t)p * n + i];
+            w[s * n + i] = x;
+            a[s] += x * x;
+          }
+        }
+      __syncthreads();
+      put2(a[0], a[1], pa);
+      if (!sync()) return;
+      get2(pa);
+      if (t < 2 && doit[t]) be[t][j] = sqrt(tot[t][0]);
+      for (int s = 0; s < 2; ++s)
+        if (doit[s])
+          for (int k = t; k < j; k += kLzThreads) om[s][(j + 1) % 3][k] = 1.1102230246251565e-16;
+      __syncthreads();
+    }
+    if (t < 2 && active[t]) {
+      const double b = be[t][j];
+      if (b <= 1e-12 * (fabs(al[t][j]) + (j > 0 ? be[t][j - 1] : 0.0) + 1e-300)) active[t] = 0;
+    }
+    __syncthreads();
+    if (j == steps - 1 || !(active[0] | active[1])) break;
+    for (int s = 0; s < 2; ++s)
+      if (active[s]) {
+        const double f = 1.0 / be[s][j];
+        double *v = V + ((size_t)s * (steps + 1) + j + 1) * n;
+        for (long long i = e0; i < n; i += es) v[i] = w[s * n + i] * f;
+      }
+    if (!sync()) return;
+  }
+  if (blockIdx.x == 0 && t < 2) {
+    double *o = out + t * (2 * kLzMax + 1);
+    o[0] = used[t];
+    for (int k = 0; k < used[t]; ++k) {
+      o[1 + k] = al[t][k];
+      o[1 + kLzMax + k] = be[t][k];
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------

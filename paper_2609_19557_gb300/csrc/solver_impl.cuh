@@ -327,7 +327,6 @@ class Solver : public SolverBase {
     PDNQP_TRY(dalloc(&xo_, n_));
     PDNQP_TRY(dalloc(&lo_, m_));
     PDNQP_TRY(dalloc(&scn_[0], n_));
-    PDNQP_TRY(dalloc(&scn_[1], n_));
     PDNQP_TRY(dalloc(&scm_[0], m_));
     PDNQP_TRY(dalloc(&scm_[1], m_));
     PDNQP_TRY(dalloc(&scm_[2], m_));
@@ -381,10 +380,7 @@ class Solver : public SolverBase {
     }
     PDNQP_CK(cudaGetLastError());
     // ---- gamma (Eq. R-choice): two Lanczos starts, the smaller estimate.
-    double l1, l2;
-    PDNQP_TRY(lanczos(prm.lanczos_steps, 1ULL, &l1));
-    PDNQP_TRY(lanczos(prm.lanczos_steps, 2ULL, &l2));
-    lam_min_ = std::min(l1, l2);
+    PDNQP_TRY(lanczos(prm.lanczos_steps, &lam_min_));
     gamma_ = prm.gamma_override > 0 ? prm.gamma_override
                                      : 1.0 / (std::max(0.0, -lam_min_) + prm.delta_gamma * std::max(1.0, qnorm_));
     // H = Qbar + gamma^-1 I
@@ -397,54 +393,70 @@ class Solver : public SolverBase {
     return 0;
   }
 
-  int lanczos(int steps, unsigned long long seed, double *out) {
+  // The smaller of the smallest Ritz values of two Lanczos runs on the scaled Q
+  // (k_lanczos; gamma is not yet added to Hd_).
+  int lanczos(int steps, double *out) {
     const long long n = n_;
     if (n == 0) {
       *out = 0.0;
       return 0;
     }
-    const int k = (int)std::min<long long>(std::min(steps, 79), n);  // part_lz() holds 80 rows
-    if (!V_) PDNQP_TRY(dalloc(&V_, (size_t)(k + 1) * n));
-    if (!hdev_) PDNQP_TRY(dalloc(&hdev_, 256));
-    double *w = scn_[1];
-    std::vector<double> al(k + 1, 0.0), be(k + 1, 0.0);
-    // Hd currently holds the scaled Q (gamma not yet added).
-    k_start_vector<<<grid_n(), kBlock, 0, s_>>>(V_, n, seed);
-    double nrm;
-    PDNQP_TRY(dot(V_, V_, &nrm));
-    k_scale_into<<<grid_n(), kBlock, 0, s_>>>(V_, V_, 1.0 / std::sqrt(nrm), n);
-    int used = 0;
-    const int nbd = grid_n();
-    for (int j = 0; j < k; ++j) {
-      double *vj = V_ + (long long)j * n;
-      with_G(gN_, [&](auto GG) {
-        k_spmv<decltype(GG)::value><<<nb_cols(), kBlock, 0, s_>>>(Hd_, vj, w);
-      });
-      PDNQP_TRY(dot(w, vj, &al[j]));
-      used = j + 1;
-      k_lanczos_axpy<<<grid_n(), kBlock, 0, s_>>>(w, vj, j > 0 ? V_ + (long long)(j - 1) * n : nullptr, al[j],
-                                                   j > 0 ? be[j - 1] : 0.0, n);
-      for (int pass = 0; pass < 2; ++pass) {  // classical Gram-Schmidt, twice
-        dim3 grid(nbd, j + 1);
-        k_multidot<<<grid, kBlock, 0, s_>>>(V_, n, w, part_lz());
-        k_reduce_rows<<<j + 1, 32, 0, s_>>>(part_lz(), j + 1, nbd, 0u, hdev_);
-        k_multiaxpy<<<grid_n(), kBlock, 0, s_>>>(V_, n, hdev_, j + 1, w);
-      }
-      double b2;
-      PDNQP_TRY(dot(w, w, &b2));
-      const double b = std::sqrt(b2);
-      be[j] = b;
-      if (j == k - 1) break;
-      if (b <= 1e-12 * (std::fabs(al[j]) + (j > 0 ? be[j - 1] : 0.0) + 1e-300)) break;
-      k_scale_into<<<grid_n(), kBlock, 0, s_>>>(V_ + (long long)(j + 1) * n, w, 1.0 / b, n);
+    const int k = (int)std::min<long long>(std::min(steps, kLzMax - 1), n);
+    int dev = 0, sms = 0;
+    PDNQP_CK(cudaGetDevice(&dev));
+    PDNQP_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int nb = (int)std::min<long long>(std::min(sms, kMaxBlocks), (n + 255) / 256);
+    // Basis and sums of this call only.
+    double *V = nullptr;
+    const size_t nV = 2 * (size_t)(k + 1) * n, nw = 2 * (size_t)n, np = 4 * (size_t)kMaxBlocks + (size_t)nb * 2 * kLzMax,
+                 no = 2 * (2 * kLzMax + 1);
+    if (cudaMalloc(&V, (nV + nw + np + no) * sizeof(double) + kBarWords * sizeof(unsigned)) != cudaSuccess) {
+      last_err_ = "cudaMalloc: Lanczos basis";
+      cudaGetLastError();
+      return PDNQP_ERR_OOM;
     }
-    PDNQP_CK(cudaGetLastError());
-    *out = tridiag_min(al, be, used);
+    double *w = V + nV, *part = w + nw, *res = part + np;
+    unsigned *bar = (unsigned *)(res + no);
+    const int rc = lanczos_run(k, nb, V, w, part, bar, res, no, out);
+    cudaFree(V);
+    return rc;
+  }
+  int lanczos_run(int k, int nb, double *V, double *w, double *part, unsigned *bar, double *res, size_t no, double *out) {
+    PDNQP_CK(cudaMemsetAsync(bar, 0, kBarWords * sizeof(unsigned), s_));
+    int rc = 0;
+    with_G(gN_, [&](auto GG) {
+      auto fn = k_lanczos<decltype(GG)::value>;
+      const int smem = kLzThreads / 32 * kTileSlots * (int)sizeof(Slot<double>);
+      cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      void *args[] = {(void *)&Hd_, (void *)&k, (void *)&V, (void *)&w, (void *)&part, (void *)&bar, (void *)&res};
+      if (e == cudaSuccess)
+        e = cudaLaunchCooperativeKernel((const void *)fn, dim3(nb), dim3(kLzThreads), args, smem, s_);
+      if (e != cudaSuccess) {
+        last_err_ = std::string("k_lanczos: ") + cudaGetErrorString(e);
+        rc = PDNQP_ERR_CUDA;
+      }
+    });
+    if (rc) return rc;
+    std::vector<double> h(no);
+    unsigned fault = 0;
+    PDNQP_CK(cudaMemcpyAsync(h.data(), res, no * sizeof(double), cudaMemcpyDeviceToHost, s_));
+    PDNQP_CK(cudaMemcpyAsync(&fault, bar + kBarFault, sizeof(fault), cudaMemcpyDeviceToHost, s_));
+    PDNQP_CK(cudaStreamSynchronize(s_));
+    if (fault) {
+      last_err_ = "k_lanczos: grid barrier timed out";
+      return PDNQP_ERR_CUDA;
+    }
+    double best = INFINITY;
+    for (int s = 0; s < 2; ++s) {
+      const double *o = h.data() + s * (2 * kLzMax + 1);
+      best = std::min(best, tridiag_min(o + 1, o + 1 + kLzMax, (int)o[0]));
+    }
+    *out = best;
     return 0;
   }
 
   // Smallest eigenvalue of the Lanczos tridiagonal by Sturm-count bisection.
-  static double tridiag_min(const std::vector<double> &a, const std::vector<double> &b, int k) {
+  static double tridiag_min(const double *a, const double *b, int k) {
     double lo = INFINITY, hi = -INFINITY;
     for (int i = 0; i < k; ++i) {
       const double r = (i > 0 ? std::fabs(b[i - 1]) : 0.0) + (i < k - 1 ? std::fabs(b[i]) : 0.0);
@@ -468,14 +480,6 @@ class Solver : public SolverBase {
       else lo = mid;
     }
     return 0.5 * (lo + hi);
-  }
-
-  double *part_lz() { return lzpart_ ? lzpart_ : (dalloc(&lzpart_, (size_t)80 * kMaxBlocks), lzpart_); }
-
-  int dot(const double *a, const double *b, double *out) {
-    const int nb = grid_n();
-    k_dot<<<nb, kBlock, 0, s_>>>(a, b, n_, part_);
-    return reduce_to_host(1, nb, 0u, out);
   }
 
   int alloc_T(const HostProblem &P) {
@@ -1583,8 +1587,7 @@ class Solver : public SolverBase {
   double *Dc_ = nullptr, *Dx_ = nullptr, *lam_ = nullptr, *sig_ = nullptr, *rprev_ = nullptr, *rcur_ = nullptr;
   double *z_ = nullptr, *xo_ = nullptr, *lo_ = nullptr, *dx0_ = nullptr, *dl0_ = nullptr;
   double *x64_ = nullptr, *y64_ = nullptr, *sb64_ = nullptr, *rb64_ = nullptr, *snapbuf_ = nullptr;
-  double *scn_[2] = {nullptr, nullptr}, *scm_[3] = {nullptr, nullptr, nullptr};
-  double *V_ = nullptr, *hdev_ = nullptr, *lzpart_ = nullptr;
+  double *scn_[1] = {nullptr}, *scm_[3] = {nullptr, nullptr, nullptr};
   double *part_ = nullptr, *dred_ = nullptr;
   std::vector<double> hred_;
   DevState *st_ = nullptr, *hst_ = nullptr;
