@@ -229,17 +229,17 @@ __device__ __forceinline__ double warp_halve(double (&v)[P]) {
 
 // Block reduction of NQ doubles; bit q of MASK: 0 sum, 1 maximum (of
 // non-negative values).  The block writes part[q * kMaxBlocks + blk].  Must be
-// called by every thread of the block (kBlock threads).  Sums and maxima are
+// called by every thread of the block (up to 512).  Sums and maxima are
 // reduced over the warp by halving, then one thread per quantity joins the
 // warps' values in order.  Fixed order: deterministic for a fixed grid.
 template <int NQ, unsigned MASK>
 __device__ __forceinline__ void block_reduce_store(double (&v)[NQ], double *part, int blk = -1) {
   if (blk < 0) blk = blockIdx.x;
-  constexpr int NW = kBlock / 32, NM = count_bits(MASK), NS = NQ - NM;
+  constexpr int NM = count_bits(MASK), NS = NQ - NM;
   constexpr int PS = next_pow2(NS > 0 ? NS : 1), PM = next_pow2(NM > 0 ? NM : 1);
   static_assert(PS <= 32 && PM <= 32, "at most 32 quantities of a kind");
-  __shared__ double sm[NQ][NW];
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  __shared__ double sm[NQ][16];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5, nw = blockDim.x >> 5;
   double s[PS], m[PM];
 #pragma unroll
   for (int k = 0; k < PS; ++k) s[k] = 0.0;
@@ -272,7 +272,7 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[NQ], double *part
   if (t < NQ) {
     const bool mx = (MASK >> t) & 1u;
     double a = sm[t][0];
-    for (int k = 1; k < NW; ++k) a = mx ? max_abs(a, sm[t][k]) : a + sm[t][k];
+    for (int k = 1; k < nw; ++k) a = mx ? max_abs(a, sm[t][k]) : a + sm[t][k];
     part[t * kMaxBlocks + blk] = a;
   }
   __syncthreads();
@@ -477,10 +477,8 @@ struct TileIter {
   long long first, step;
   __device__ __forceinline__ TileIter(GridCtx g = hw_grid()) {
     lane = threadIdx.x & 31;
-    const long long gw = ((long long)g.b * blockDim.x + threadIdx.x) >> 5;
-    const long long nw = ((long long)g.nb * blockDim.x) >> 5;
-    first = gw * TR;
-    step = nw * TR;
+    first = ((long long)(threadIdx.x >> 5) * g.nb + g.b) * TR;  // a few tiles spread over all blocks
+    step = (((long long)g.nb * blockDim.x) >> 5) * TR;
   }
   // Row of this lane in a tile; false past the tile or the matrix.
   __device__ __forceinline__ bool row(long long tile, long long nrows, long long &i) const {
@@ -836,22 +834,22 @@ struct MaxAbs {
 // = short rows (32 rows).
 template <int K, bool IsMax, typename Acc, typename T, typename F>
 __device__ __forceinline__ Acc tile_reduce(const int *rp, const int *ci, const T *val, long long tile, long long nrows,
-                                           const F &f) {
+                                           const F &f, Slot<Acc> *buf) {
   const long long my = tile + (threadIdx.x & 31);
   const bool ok = (threadIdx.x & 31) < TileIter<K>::TR && my < nrows;
   const int rb = ok ? rp[my] : 0, re = ok ? rp[my + 1] : 0;
   return K == 16 ? tile_long_rows<IsMax, Acc>(ci, val, rb, re, f)
-                 : tile_rows1<IsMax, Acc>(ci, val, rb, re, f, warp_slots<Acc>());
+                 : tile_rows1<IsMax, Acc>(ci, val, rb, re, f, buf);
 }
 template <int K, typename Acc, typename T, typename F>
 __device__ __forceinline__ Acc tile_row_sum(const int *rp, const int *ci, const T *val, long long tile, long long nrows,
-                                            const F &f) {
-  return tile_reduce<K, false, Acc>(rp, ci, val, tile, nrows, f);
+                                            const F &f, Slot<Acc> *buf = warp_slots<Acc>()) {
+  return tile_reduce<K, false, Acc>(rp, ci, val, tile, nrows, f, buf);
 }
 template <int K, typename Acc, typename T, typename F>
 __device__ __forceinline__ Acc tile_row_max(const int *rp, const int *ci, const T *val, long long tile, long long nrows,
-                                            const F &f) {
-  return tile_reduce<K, true, Acc>(rp, ci, val, tile, nrows, f);
+                                            const F &f, Slot<Acc> *buf = warp_slots<Acc>()) {
+  return tile_reduce<K, true, Acc>(rp, ci, val, tile, nrows, f, buf);
 }
 
 // Product with a vector that other blocks wrote before the last grid barrier of

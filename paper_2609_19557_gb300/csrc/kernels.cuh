@@ -38,7 +38,7 @@ constexpr int P_CK_C = 24;   // check, column kernel: 16 quantities
 constexpr int P_TRP = 40;    // persistent loop: 4 sums per block, block-major
 constexpr unsigned CK_MAXMASK = 0x0F0Fu;  // quantities 0-3 and 8-11 of a check are maxima
 // Counter words (d.ctr): [0] column last-block counter, [1] check last-block
-// counter, [2] row last-block counter (long rows), [kCtrBar, kCtrBar + kBarWords) the grid barrier of the persistent loop.
+// counter, [2] row last-block counter (long rows), [3] outer column last-block counter, [kCtrBar, kCtrBar + kBarWords) the grid barrier of the persistent loop.
 constexpr int kCtrBar = 128, kCtrWords = kCtrBar + kBarWords;
 // Rows of A with more entries than this are treated as dense coupling rows
 // (at most kMaxLong of them, the longest first; the rest stay row-wise).
@@ -920,88 +920,6 @@ __device__ __forceinline__ int decide_tiles(const Dev<T> &d, DevState &S, int nb
   return go;
 }
 
-// Persistent trial loop (one cooperative launch).  A trial is the row pass, a
-// grid barrier, the column pass (with the next trial's primal step) and a grid
-// barrier whose last block takes the acceptance decision; a trial whose primal
-// step is not there yet (the first one, after a rejection, after a restart)
-// starts with the primal pass and a barrier.  The loop leaves when the solve
-// stops, a periodic check is due (the check kernels follow this launch) or the
-// launch's trial allowance (slot_left) is used up; it does not start while a
-// check is pending (the check kernels clear check_due).  All blocks take the
-// same branches (the state is block-uniform), so every barrier is reached by
-// every block.  LR: the instance has dense coupling rows (d.nlr > 0); RL / CL:
-// long rows of A / of H and A' (tiles of 8).
-template <typename T, bool LR, bool RL, bool CL>
-__global__ void __launch_bounds__(kTrialThreads, 1) k_trials(Dev<T> d) {
-  __shared__ DevState S;
-  __shared__ double next[2];
-  extern __shared__ __align__(16) unsigned char slots[];
-  Slot<T> *buf = reinterpret_cast<Slot<T> *>(slots) + (threadIdx.x >> 5) * 2 * kTileSlots;
-  unsigned *bar = d.ctr + kCtrBar;
-  unsigned gen = threadIdx.x == 0 ? ld_acquire_gpu(bar + kBarGen) : 0u;
-  state_load(S, d.st);
-  const int nb = gridDim.x;
-  double *part = d.part + P_TRP * kMaxBlocks + 4 * blockIdx.x;
-  // Block 0 times each pass: its own work, then its wait at the barrier
-  // (imbalance across blocks plus the barrier itself; the last one includes
-  // the acceptance decision).
-  const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
-  unsigned long long tp[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
-  unsigned long long tk = timer ? global_ns() : 0ull;
-  auto lap = [&](int k) {
-    if (timer) {
-      const unsigned long long t = global_ns();
-      tp[k] += t - tk;
-      tk = t;
-    }
-  };
-  while (S.status == ST_RUNNING && S.slot_left > 0 && !S.check_due) {
-    if (!S.spec) {
-      primal_phase<T>(d, &S);
-      lap(0);
-      if (loop_sync(bar, gen, [] { return 0; }) < 0) return;
-      lap(1);
-    }
-    if (threadIdx.x >= kTrialThreads - 2) {  // a spare lane each, before the last warp's first item
-      const double t = (double)(S.t + 1);
-      if (threadIdx.x == kTrialThreads - 2)
-        next[0] = 2.0 / (t + 3.0);
-      else
-        next[1] = t / (t + 1.0);
-    }
-    TrialSums<T> ts = {T(0), T(0), T(0), T(0)};
-    rows_phase_tiles<T, LR, RL>(d, &S, buf, ts);
-    lap(2);
-    if (loop_sync(bar, gen, [&] {
-          if (LR) long_rows_finish<T>(d, &S, d.lr_nb);
-          return 0;
-        }) < 0)
-      return;
-    lap(3);
-    cols_phase_tiles<T, CL>(d, &S, buf, ts);
-    lap(4);
-    double v[4] = {widen(ts.Lt), widen(ts.Le), widen(ts.RH), widen(ts.RB)};
-    block_sums(v, part);
-    bool led = false;
-    const int go = loop_sync(bar, gen, [&] {
-      led = true;
-      return decide_tiles<T>(d, S, nb, LR, next);
-    });
-    if (go < 0) return;
-    if (!led) {
-      if (go) {
-        if (threadIdx.x == 0) advance_trial(&S, next);
-        __syncthreads();
-      } else {
-        state_load(S, d.st);
-      }
-    }
-    lap(5);
-  }
-  if (timer && d.ptime)
-    for (int k = 0; k < 6; ++k) d.ptime[k] += tp[k];
-}
-
 // Acceptance decision (single block, deterministic order).  On acceptance the
 // trial buffers become current (index flip); on rejection both step vectors
 // are shrunk through kappa.
@@ -1172,15 +1090,14 @@ __device__ __forceinline__ void row_cand(double *q, const RowIn &a) {
 }
 
 template <typename T, int G>
-__device__ __forceinline__ void check_rows_body(const Dev<T> &d, int mode, GridCtx g) {
-  const DevState *st = d.st;
-  if (mode == 0 && !(st->status == ST_RUNNING && st->check_due)) return;
+__device__ __forceinline__ void check_rows_body(const Dev<T> &d, const DevState *st, int mode, GridCtx g,
+                                                Slot<T> *buf) {
   // Averages of a pending acceptance are formed on the fly (and written for the
   // row blocks); x bar is gathered as (1 - alpha) xbar + alpha x.
   const int cur = st->cur, a0 = st->acur, acc = st->accepted, ab = a0 ^ acc;
   const T ap = T(st->alpha_acc), omap = T(1) - ap;
-  const T *__restrict__ xb0 = d.xbar[a0];
-  const T *__restrict__ xc = d.x[st->xcur];
+  const T *xb0 = d.xbar[a0];
+  const T *xc = d.x[st->xcur];
   double q[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) q[k] = 0.0;
@@ -1189,7 +1106,7 @@ __device__ __forceinline__ void check_rows_body(const Dev<T> &d, int mode, GridC
     T axb = T(0);
     if (mode == 0)
       axb = tile_row_sum<G, T>(d.A.rp, d.A.ci, d.A.val, tile, d.m,
-                               entry([&](int k) { return acc ? omap * xb0[k] + ap * xc[k] : xb0[k]; }, AddProduct()));
+                               entry([&](int k) { return acc ? omap * xb0[k] + ap * xc[k] : xb0[k]; }, AddProduct()), buf);
     long long j;
     const bool own = ti.row(tile, d.m, j);
     if (own) {
@@ -1246,9 +1163,15 @@ __device__ __forceinline__ void check_rows_body(const Dev<T> &d, int mode, GridC
   block_reduce_store<16, CK_MAXMASK>(q, d.part + P_CK_R * kMaxBlocks, g.b);
 }
 
+template <typename T>
+__device__ __forceinline__ bool check_pending(const Dev<T> &d) {
+  return d.st->status == ST_RUNNING && d.st->check_due;
+}
+
 template <typename T, int G>
 __global__ void __launch_bounds__(kBlock) k_check_rows(Dev<T> d, int mode) {
-  check_rows_body<T, G>(d, mode, hw_grid());
+  if (mode == 0 && !check_pending(d)) return;
+  check_rows_body<T, G>(d, d.st, mode, hw_grid(), warp_slots<T>());
 }
 
 // Contributions of one variable (x block) to the 8 quantities of a candidate:
@@ -1265,15 +1188,14 @@ __device__ __forceinline__ void col_cand(double *q, double dx, double hdx, doubl
   q[6] += w * w;
 }
 
-template <typename T, int G, bool COND>
-__device__ __forceinline__ void check_cols_body(const Dev<T> &d, int mode, int nb_r, GridCtx g) {
-  const DevState *st = d.st;
-  if (mode == 0 && !(st->status == ST_RUNNING && st->check_due)) return;
+template <typename T, int G>
+__device__ __forceinline__ void check_cols_terms(const Dev<T> &d, const DevState *st, int mode, GridCtx g,
+                                                 Slot<T> *buf) {
   // y bar of a pending acceptance was materialised by k_check_rows.
   const int cur = st->cur, a0 = st->acur, acc = st->accepted, ab = a0 ^ acc;
   const T ap = T(st->alpha_acc), omap = T(1) - ap;
-  const T *__restrict__ yb = d.ybar[ab];
-  const T *__restrict__ xc = d.x[st->xcur];
+  const T *yb = d.ybar[ab];
+  const T *xc = d.x[st->xcur];
   double q[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) q[k] = 0.0;
@@ -1281,7 +1203,7 @@ __device__ __forceinline__ void check_cols_body(const Dev<T> &d, int mode, int n
   for (long long tile = ti.first; tile < d.n; tile += ti.step) {
     T atyb = T(0);
     if (mode == 0)
-      atyb = tile_row_sum<G, T>(d.At.rp, d.At.ci, d.At.val, tile, d.n, MulLdg<T>{yb});
+      atyb = tile_row_sum<G, T>(d.At.rp, d.At.ci, d.At.val, tile, d.n, MulLd<T>{yb}, buf);
     long long i;
     const bool own = ti.row(tile, d.n, i);
     if (own) {
@@ -1303,6 +1225,12 @@ __device__ __forceinline__ void check_cols_body(const Dev<T> &d, int mode, int n
     }
   }
   block_reduce_store<16, CK_MAXMASK>(q, d.part + P_CK_C * kMaxBlocks, g.b);
+}
+
+template <typename T, int G, bool COND>
+__device__ __forceinline__ void check_cols_body(const Dev<T> &d, int mode, int nb_r, GridCtx g) {
+  if (mode == 0 && !check_pending(d)) return;
+  check_cols_terms<T, G>(d, d.st, mode, g, warp_slots<T>());
   if (arrive_last(d.ctr + 1, g.nb)) {
     if (mode == 0)
       check_final_body<COND>(d.st, d.part, nb_r, g.nb, d.hw);
@@ -1317,69 +1245,77 @@ __global__ void __launch_bounds__(kBlock) k_check_cols(Dev<T> d, int mode, int n
   check_cols_body<T, G, COND>(d, mode, nb_r, hw_grid());
 }
 
-// Decisions of the check (single block): inner termination of both candidates
-// (Eq. inner-termination), iteration limit, restart criteria and primal weight.
+// Decisions of the check (one thread), from its 16 quantities: inner termination
+// of both candidates (Eq. inner-termination), iteration limit, restart criteria
+// and primal weight.
+__device__ __forceinline__ void check_logic(DevState *st, const double (&q)[16]) {
+  for (int k = 0; k < 16; ++k) st->chk[k] = q[k];
+  // The averages of this trial's acceptance were materialised by the check's
+  // passes.  The check is consumed here; the restart itself is applied by
+  // check_apply_body on restart_flag.
+  st->acur ^= st->accepted;
+  st->accepted = 0;
+  st->restart_flag = 0;
+  st->check_due = 0;
+  const double dta = st->dta, dtr = st->dtr;
+  const double spc = fmax(1.0, q[1]), sdc = fmax(1.0, q[3]);
+  const double spa = fmax(1.0, q[9]), sda = fmax(1.0, q[11]);
+  const bool okc = q[0] <= dta + dtr * spc && q[2] <= dta + dtr * sdc;
+  const bool oka = q[8] <= dta + dtr * spa && q[10] <= dta + dtr * sda;
+  if (!st->ignore_conv && okc) {
+    st->status = ST_CONVERGED;
+    st->ret_avg = 0;
+  } else if (!st->ignore_conv && oka) {
+    st->status = ST_CONVERGED;
+    st->ret_avg = 1;
+  } else if (st->t_total == st->k_in) {
+    st->status = ST_ITER_LIMIT;
+  } else {
+    const double om = st->omega;
+    const double kc = sqrt(om * q[4] + q[5] / om);
+    const double ka = sqrt(om * q[12] + q[13] / om);
+    const bool use_avg = ka < kc;
+    const double kcand = use_avg ? ka : kc;
+    const bool restart = kcand <= st->beta_suff * st->k_restart ||
+                         (kcand <= st->beta_nec * st->k_restart && kcand > st->k_last) ||
+                         (double)st->t >= st->beta_art * (double)st->t_total;
+    st->k_last = kcand;
+    if (restart) {
+      const double dW = sqrt(use_avg ? q[14] : q[6]);
+      const double dY = sqrt(use_avg ? q[15] : q[7]);
+      if (dW > 0.0 && dY > 0.0) st->omega = exp(0.25 * log(dY / dW) + 0.75 * log(om));
+      st->kappa = 1.0;
+      st->t = 0;
+      st->k_restart = kcand;
+      st->k_last = INFINITY;
+      st->restarts += 1;
+      st->restart_flag = 1;
+      st->spec = 0;
+      st->restart_use_avg = use_avg ? 1 : 0;
+    }
+    if (st->t_total == st->pause_at) st->status = ST_PAUSED;
+  }
+  refresh_scalars(st);
+}
+// The quantities of a check from the row and column partials (whole block).
+__device__ __forceinline__ void check_sums(const double *part, int nb_r, int nb_c, double (&q)[16]) {
+  double b[16];
+  final_reduce<16>(part + P_CK_R * kMaxBlocks, nb_r, CK_MAXMASK, q);
+  final_reduce<16>(part + P_CK_C * kMaxBlocks, nb_c, CK_MAXMASK, b);
+#pragma unroll
+  for (int k = 0; k < 16; ++k) q[k] = ((CK_MAXMASK >> k) & 1u) ? fmax(q[k], b[k]) : q[k] + b[k];
+}
+
 template <bool COND>
 __device__ void check_final_body(DevState *stg, const double *part, int nb_r, int nb_c,
                                  cudaGraphConditionalHandle hw) {
   __shared__ DevState S;
   state_load(S, stg);
-  double a[16], b[16];
-  final_reduce<16>(part + P_CK_R * kMaxBlocks, nb_r, CK_MAXMASK, a);
-  final_reduce<16>(part + P_CK_C * kMaxBlocks, nb_c, CK_MAXMASK, b);
+  double q[16];
+  check_sums(part, nb_r, nb_c, q);
   if (threadIdx.x == 0) {
-    DevState *st = &S;
-    double q[16];
-    for (int k = 0; k < 16; ++k) q[k] = ((CK_MAXMASK >> k) & 1u) ? fmax(a[k], b[k]) : a[k] + b[k];
-    for (int k = 0; k < 16; ++k) st->chk[k] = q[k];
-    // The averages of this trial's acceptance were materialised by the check
-    // kernels.  The check is consumed here (a repeated launch of the check
-    // kernels without a trial in between does nothing); the restart itself is
-    // applied by k_check_apply on restart_flag.
-    st->acur ^= st->accepted;
-    st->accepted = 0;
-    st->restart_flag = 0;
-    st->check_due = 0;
-    const double dta = st->dta, dtr = st->dtr;
-    const double spc = fmax(1.0, q[1]), sdc = fmax(1.0, q[3]);
-    const double spa = fmax(1.0, q[9]), sda = fmax(1.0, q[11]);
-    const bool okc = q[0] <= dta + dtr * spc && q[2] <= dta + dtr * sdc;
-    const bool oka = q[8] <= dta + dtr * spa && q[10] <= dta + dtr * sda;
-    if (!st->ignore_conv && okc) {
-      st->status = ST_CONVERGED;
-      st->ret_avg = 0;
-    } else if (!st->ignore_conv && oka) {
-      st->status = ST_CONVERGED;
-      st->ret_avg = 1;
-    } else if (st->t_total == st->k_in) {
-      st->status = ST_ITER_LIMIT;
-    } else {
-      const double om = st->omega;
-      const double kc = sqrt(om * q[4] + q[5] / om);
-      const double ka = sqrt(om * q[12] + q[13] / om);
-      const bool use_avg = ka < kc;
-      const double kcand = use_avg ? ka : kc;
-      const bool restart = kcand <= st->beta_suff * st->k_restart ||
-                           (kcand <= st->beta_nec * st->k_restart && kcand > st->k_last) ||
-                           (double)st->t >= st->beta_art * (double)st->t_total;
-      st->k_last = kcand;
-      if (restart) {
-        const double dW = sqrt(use_avg ? q[14] : q[6]);
-        const double dY = sqrt(use_avg ? q[15] : q[7]);
-        if (dW > 0.0 && dY > 0.0) st->omega = exp(0.25 * log(dY / dW) + 0.75 * log(om));
-        st->kappa = 1.0;
-        st->t = 0;
-        st->k_restart = kcand;
-        st->k_last = INFINITY;
-        st->restarts += 1;
-        st->restart_flag = 1;
-        st->spec = 0;
-        st->restart_use_avg = use_avg ? 1 : 0;
-      }
-      if (st->t_total == st->pause_at) st->status = ST_PAUSED;
-    }
-    refresh_scalars(st);
-    if (COND && hw) cudaGraphSetConditional(hw, (st->status == ST_RUNNING && st->slot_left > 0) ? 1u : 0u);
+    check_logic(&S, q);
+    if (COND && hw) cudaGraphSetConditional(hw, (S.status == ST_RUNNING && S.slot_left > 0) ? 1u : 0u);
   }
   state_store(stg, S);
 }
@@ -1388,8 +1324,7 @@ __device__ void check_final_body(DevState *stg, const double *part, int nb_r, in
 // (with its cached products), then make it the epoch start and clear the
 // averages.  Idempotent, so a repeated launch is harmless.
 template <typename T>
-__device__ __forceinline__ void check_apply_body(const Dev<T> &d, GridCtx g) {
-  const DevState *st = d.st;
+__device__ __forceinline__ void check_apply_body(const Dev<T> &d, const DevState *st, GridCtx g) {
   if (!st->restart_flag) return;
   const int cur = st->cur, ab = st->acur;
   const bool ua = st->restart_use_avg;
@@ -1434,7 +1369,126 @@ __device__ __forceinline__ void check_apply_body(const Dev<T> &d, GridCtx g) {
 
 template <typename T>
 __global__ void __launch_bounds__(kBlock) k_check_apply(Dev<T> d) {
-  check_apply_body<T>(d, hw_grid());
+  check_apply_body<T>(d, d.st, hw_grid());
+}
+
+// ===========================================================================
+// The persistent loop.
+// ===========================================================================
+// Persistent trial loop (one cooperative launch).  A trial is the row pass, a
+// grid barrier, the column pass (with the next trial's primal step) and a grid
+// barrier whose last block takes the acceptance decision; a trial whose primal
+// step is not there yet (the first one, after a rejection, after a restart)
+// starts with the primal pass and a barrier.  The loop leaves when the solve
+// stops, a periodic check is due (k_check follows this launch; in this kernel
+// its FP64 terms would take registers from the passes, 62.7 instead of 54 us for
+// the FP64 row pass at n = 1e6) or the trial allowance is used up (chunk >= 0
+// sets it); it does not start while a check is pending.  All blocks take the same
+// branches (the state is block-uniform), so every barrier is reached by every
+// block.  LR: the instance has dense coupling rows (d.nlr > 0); RL / CL:
+// long rows of A / of H and A' (tiles of 8).
+template <typename T, bool LR, bool RL, bool CL>
+__global__ void __launch_bounds__(kTrialThreads, 1) k_trials(Dev<T> d, long long chunk) {
+  __shared__ DevState S;
+  __shared__ double next[2];
+  extern __shared__ __align__(16) unsigned char slots[];
+  Slot<T> *buf = reinterpret_cast<Slot<T> *>(slots) + (threadIdx.x >> 5) * 2 * kTileSlots;
+  unsigned *bar = d.ctr + kCtrBar;
+  unsigned gen = threadIdx.x == 0 ? ld_acquire_gpu(bar + kBarGen) : 0u;
+  state_load(S, d.st);
+  if (threadIdx.x == 0 && chunk >= 0) S.slot_left = chunk;
+  __syncthreads();
+  const int nb = gridDim.x;
+  double *part = d.part + P_TRP * kMaxBlocks + 4 * blockIdx.x;
+  // Block 0 times each pass: its own work, then its wait at the barrier
+  // (imbalance across blocks plus the barrier itself; the last one includes
+  // the acceptance decision).
+  const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
+  unsigned long long tp[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
+  unsigned long long tk = timer ? global_ns() : 0ull;
+  auto lap = [&](int k) {
+    if (timer) {
+      const unsigned long long t = global_ns();
+      tp[k] += t - tk;
+      tk = t;
+    }
+  };
+  while (S.status == ST_RUNNING && S.slot_left > 0 && !S.check_due) {
+    if (!S.spec) {
+      primal_phase<T>(d, &S);
+      lap(0);
+      if (loop_sync(bar, gen, [] { return 0; }) < 0) return;
+      lap(1);
+    }
+    if (threadIdx.x >= kTrialThreads - 2) {  // a spare lane each, before the last warp's first item
+      const double t = (double)(S.t + 1);
+      if (threadIdx.x == kTrialThreads - 2)
+        next[0] = 2.0 / (t + 3.0);
+      else
+        next[1] = t / (t + 1.0);
+    }
+    TrialSums<T> ts = {T(0), T(0), T(0), T(0)};
+    rows_phase_tiles<T, LR, RL>(d, &S, buf, ts);
+    lap(2);
+    if (loop_sync(bar, gen, [&] {
+          if (LR) long_rows_finish<T>(d, &S, d.lr_nb);
+          return 0;
+        }) < 0)
+      return;
+    lap(3);
+    cols_phase_tiles<T, CL>(d, &S, buf, ts);
+    lap(4);
+    double v[4] = {widen(ts.Lt), widen(ts.Le), widen(ts.RH), widen(ts.RB)};
+    block_sums(v, part);
+    bool led = false;
+    const int go = loop_sync(bar, gen, [&] {
+      led = true;
+      return decide_tiles<T>(d, S, nb, LR, next);
+    });
+    if (go < 0) return;
+    if (!led) {
+      if (go) {
+        if (threadIdx.x == 0) advance_trial(&S, next);
+        __syncthreads();
+      } else {
+        state_load(S, d.st);
+      }
+    }
+    lap(5);
+  }
+  if (timer && d.ptime)
+    for (int k = 0; k < 6; ++k) d.ptime[k] += tp[k];
+}
+
+// Periodic check of the persistent form, with its restart, in one cooperative
+// launch on the loop's grid: the two passes, the decision in the last block of
+// the second barrier, and the restart.  Does nothing when no check is pending.
+template <typename T, bool RL, bool CL>
+__global__ void __launch_bounds__(kTrialThreads, 1) k_check(Dev<T> d) {
+  __shared__ DevState S;
+  extern __shared__ __align__(16) unsigned char slots[];
+  Slot<T> *buf = reinterpret_cast<Slot<T> *>(slots) + (threadIdx.x >> 5) * kTileSlots;
+  unsigned *bar = d.ctr + kCtrBar;
+  unsigned gen = threadIdx.x == 0 ? ld_acquire_gpu(bar + kBarGen) : 0u;
+  state_load(S, d.st);
+  if (S.status != ST_RUNNING || !S.check_due) return;
+  const int nb = gridDim.x;
+  const GridCtx g{(int)blockIdx.x, nb};
+  check_rows_body<T, RL ? 16 : 8>(d, &S, 0, g, buf);
+  if (loop_sync(bar, gen, [] { return 0; }) < 0) return;
+  check_cols_terms<T, CL ? 16 : 8>(d, &S, 0, g, buf);
+  bool led = false;
+  if (loop_sync(bar, gen, [&] {
+        led = true;
+        double q[16];
+        check_sums(d.part, nb, nb, q);
+        if (threadIdx.x == 0) check_logic(&S, q);
+        state_store(d.st, S);
+        return 0;
+      }) < 0)
+    return;
+  if (!led) state_load(S, d.st);
+  check_apply_body<T>(d, &S, g);
 }
 
 // ===========================================================================
@@ -1665,13 +1719,18 @@ __global__ void k_inner_init(Dev<T> d) {
 }
 
 // End of an inner solve: the outer x and inner y become base + correction
-// (the current point, or the average when it is the converged candidate).
+// (the current point, or the average when it is the converged candidate), and
+// dx = x - x_prev over the outer iteration (infeasibility tests).
 template <typename T>
-__global__ void k_finish(Dev<T> d, double *x64, double *y64, int use_avg) {
+__global__ void k_finish(Dev<T> d, double *x64, double *y64, const double *xprev, double *dxv, int use_avg) {
   const int cur = d.st->cur, ab = d.st->acur ^ d.st->accepted;
   const T *__restrict__ dx = use_avg ? d.xbar[ab] : d.x[d.st->xcur];
   const T *__restrict__ dy = use_avg ? d.ybar[ab] : d.y[cur];
-  PDNQP_GRID_STRIDE(i, d.n) x64[i] += double(dx[i]);
+  PDNQP_GRID_STRIDE(i, d.n) {
+    const double x = x64[i] + double(dx[i]);
+    x64[i] = x;
+    dxv[i] = x - xprev[i];
+  }
   PDNQP_GRID_STRIDE(j, d.m) y64[j] += double(dy[j]);
 }
 
@@ -1758,7 +1817,9 @@ __global__ void __launch_bounds__(kBlock) kb_cols(const Dev<T> *devs, const Batc
 template <typename T, int G>
 __global__ void __launch_bounds__(kBlock) kb_check_rows(const Dev<T> *devs, const BatchBlk *map) {
   const BatchBlk e = map[blockIdx.x];
-  check_rows_body<T, G>(batch_dev(devs, e.p), 0, GridCtx{e.b, e.nb});
+  const Dev<T> &d = batch_dev(devs, e.p);
+  if (!check_pending(d)) return;
+  check_rows_body<T, G>(d, d.st, 0, GridCtx{e.b, e.nb}, warp_slots<T>());
 }
 
 template <typename T, int G>
@@ -1771,7 +1832,8 @@ __global__ void __launch_bounds__(kBlock) kb_check_cols(const Dev<T> *devs, cons
 template <typename T>
 __global__ void __launch_bounds__(kBlock) kb_check_apply(const Dev<T> *devs, const BatchBlk *map) {
   const BatchBlk e = map[blockIdx.x];
-  check_apply_body<T>(batch_dev(devs, e.p), GridCtx{e.b, e.nb});
+  const Dev<T> &d = batch_dev(devs, e.p);
+  check_apply_body<T>(d, d.st, GridCtx{e.b, e.nb});
 }
 
 // Scheduler edits between graph launches: problems in `go` that are set up

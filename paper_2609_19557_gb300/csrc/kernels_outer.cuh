@@ -456,164 +456,161 @@ __global__ void __launch_bounds__(kBlock) k_objective(Dev<T> d, Mat<double> Hd, 
 // ---------------------------------------------------------------------------
 // Outer glue (Algorithm 3).
 // ---------------------------------------------------------------------------
-// Quantities of the outer residual reduction (rows of part):
+// Quantities of the outer residual reduction:
 //   0 r_p scaled, 1 s_p scaled, 2 r_p unscaled, 3 s_p unscaled, 4 ||r||_inf (rows)
 //   5 r_d scaled, 6 s_d scaled, 7 r_d unscaled, 8 s_d unscaled, 9 ||x - z||_inf,
 //   10 x'Qx, 11 c'x                         (10, 11 sums; the rest maxima)
-constexpr unsigned OUT_MAXMASK = 0x3FFu;
+// and of the infeasibility tests (Sec. "Infeasibility detection") on the scaled
+// problem, from the changes over one outer iteration dlam = lambda^{k+1} -
+// lambda^k and dx = x^{k+1} - x^k (unnormalised; the host divides by the norms).
+// Rows (4): 0 largest |dlam_j| that would need an infinite row bound (sign
+// condition), 1 sum of the finite-bound terms of sigma_C(dlam), 2 largest
+// departure of (A dx)_j from the recession cone of [l_c, u_c], 3 ||dlam||_inf.
+// Columns (7): 0 largest |v_i|, v = -A' dlam, that would need an infinite
+// variable bound, 1 sum of the finite-bound terms of sigma_X(v), 2 largest
+// departure of dx_i from the recession cone of [l_x, u_x], 3 dx'Q dx, 4 c'dx,
+// 5 ||Q dx||_inf, 6 ||dx||_inf (Q dx = H dx - dx / gamma).
+// Both in one pass over each matrix: the second product of a tile finds its
+// entries in the caches (separate passes, each with its own reduction, read and
+// synchronisation, took 0.55 ms at n = 1e6 and 0.1 ms of launches and waits at
+// any size).
+constexpr int OUT_Q = 12, INF_R = 4, INF_C = 7, INF_Q = INF_R + INF_C;
+constexpr unsigned OUT_MAXMASK = 0x3FFu, INF_R_MAXMASK = 0xDu, INF_C_MAXMASK = 0x65u;
+constexpr int kOutRows = OUT_Q + INF_R, kOutCols = OUT_Q + INF_C;  // rows of part: rows first, then columns
+constexpr unsigned kOutRowsMask = OUT_MAXMASK | INF_R_MAXMASK << OUT_Q, kOutColsMask = OUT_MAXMASK | INF_C_MAXMASK << OUT_Q;
+static_assert(kOutRows + kOutCols <= kMaxPartials, "partials of the outer pass");
 
-// Eq. practical-multiplier-update (two-sided rows) + row terms of the residuals.
+// Residual and scale terms (res_term / scale_term) of the maxima.
+__device__ __forceinline__ double res_of(double v) { return nonfinite(v) ? INFINITY : fabs(v); }
+__device__ __forceinline__ double scale_of(double v) { return nonfinite(v) ? 0.0 : fabs(v); }
+
+// Eq. practical-multiplier-update (two-sided rows) + row terms of the residuals;
+// with update also lam0 = the previous multipliers and the infeasibility terms.
 template <typename T, int G>
 __global__ void __launch_bounds__(kBlock) k_outer_rows(Dev<T> d, Mat<double> Ad, const double *lc, const double *uc,
-                                                       const double *Dc, double *lam, const double *sig, double *rcur,
-                                                       int update) {
+                                                       const double *Dc, double *lam, double *lam0, const double *sig,
+                                                       double *rcur, const double *dx, int update) {
   const double *__restrict__ x = d.xb;  // outer x (FP64)
-  double q[12];
+  double q[kOutRows];
 #pragma unroll
-  for (int k = 0; k < 12; ++k) q[k] = 0.0;
+  for (int k = 0; k < kOutRows; ++k) q[k] = 0.0;
   TileIter<G> ti;
   for (long long tile = ti.first; tile < d.m; tile += ti.step) {
     const double ax = update ? tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double, 2>{x})
                              : tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double>{x});
+    const double ad =
+        update ? tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double>{dx}) : 0.0;
     long long j;
     const bool own = ti.row(tile, d.m, j);
     if (own) {
       const double lo = lc[j], hi = uc[j];
       if (update) {
+        const double l0 = lam[j];
         double s;
         if (j < d.mE) {
           s = lo;
         } else {
-          s = ax + lam[j] / sig[j];
-          s = s < lo ? lo : s;
-          s = s > hi ? hi : s;
+          s = clampv<double>(ax + l0 / sig[j], lo, hi);
         }
-        const double r = ax - s;
-        lam[j] = lam[j] + sig[j] * r;
+        const double r = ax - s, l1 = l0 + sig[j] * r;
+        lam0[j] = l0;
+        lam[j] = l1;
         rcur[j] = r;
-        q[4] = fmax(q[4], fabs(r));
+        q[4] = max_abs(q[4], r);
+        const double y = l1 - l0;
+        if (y > 0.0) {
+          if (isinf(hi)) q[OUT_Q] = max_abs(q[OUT_Q], y); else q[OUT_Q + 1] += hi * y;
+        } else if (y < 0.0) {
+          if (isinf(lo)) q[OUT_Q] = max_abs(q[OUT_Q], y); else q[OUT_Q + 1] += lo * y;
+        }
+        if (!isinf(lo) && ad < 0.0) q[OUT_Q + 2] = max_abs(q[OUT_Q + 2], ad);
+        if (!isinf(hi) && ad > 0.0) q[OUT_Q + 2] = max_abs(q[OUT_Q + 2], ad);
+        q[OUT_Q + 3] = max_abs(q[OUT_Q + 3], y);
       }
-      const double viol = ax < lo ? lo - ax : (ax > hi ? ax - hi : 0.0);
-      double spv = scale_term(fabs(ax));
-      if (isfinite(lo)) spv = fmax(spv, fabs(lo));
-      if (isfinite(hi)) spv = fmax(spv, fabs(hi));
-      q[0] = fmax(q[0], res_term(viol));
-      q[1] = fmax(q[1], spv);
-      const double dc = Dc[j];
-      q[2] = fmax(q[2], res_term(viol / dc));
-      q[3] = fmax(q[3], spv / dc);
+      const double viol = less_bits(ax, lo) ? lo - ax : (less_bits(hi, ax) ? ax - hi : 0.0);
+      double spv = scale_of(ax);
+      spv = max_abs(spv, scale_of(lo));
+      spv = max_abs(spv, scale_of(hi));
+      q[0] = max_abs(q[0], res_of(viol));
+      q[1] = max_abs(q[1], spv);
+      const double idc = recip(Dc[j]);
+      q[2] = max_abs(q[2], res_of(viol * idc));
+      q[3] = max_abs(q[3], spv * idc);
     }
   }
-  block_reduce_store<12, OUT_MAXMASK>(q, d.part);
+  block_reduce_store<kOutRows, kOutRowsMask>(q, d.part);
 }
 
 // Column terms: Qx = H x - gamma^-1 x, A' lambda, projected stationarity in the
-// scaled and the original coordinates (x = Dx xbar, lambda = Dc lambdabar / c_s).
+// scaled and the original coordinates (x = Dx xbar, lambda = Dc lambdabar /
+// c_s).  The last block joins the row and column partials into out.
 template <typename T, int G>
 __global__ void __launch_bounds__(kBlock) k_outer_cols(Dev<T> d, Mat<double> Hd, Mat<double> Atd, const double *c,
                                                        const double *lx, const double *ux, const double *Dx,
-                                                       const double *lam, const double *z, double ginv, double cs) {
+                                                       const double *lam, const double *lam0, const double *dx,
+                                                       const double *z, double ginv, double cs, int update, int nb_r,
+                                                       double *out) {
   const double *__restrict__ x = d.xb;  // outer x (FP64)
-  double q[12];
+  double q[kOutCols];
 #pragma unroll
-  for (int k = 0; k < 12; ++k) q[k] = 0.0;
+  for (int k = 0; k < kOutCols; ++k) q[k] = 0.0;
+  const double ics = 1.0 / cs;
   TileIter<G> ti;
   for (long long tile = ti.first; tile < d.n; tile += ti.step) {
     const double hx = tile_row_sum<G, double>(Hd.rp, Hd.ci, Hd.val, tile, d.n, MulLdg<double>{x});
     const double atl = tile_row_sum<G, double>(Atd.rp, Atd.ci, Atd.val, tile, d.n, MulLdg<double>{lam});
+    double hd = 0.0, atd = 0.0;
+    if (update) {
+      hd = tile_row_sum<G, double>(Hd.rp, Hd.ci, Hd.val, tile, d.n, MulLdg<double>{dx});
+      atd = tile_row_sum<G, double>(Atd.rp, Atd.ci, Atd.val, tile, d.n,
+                                    entry([&](int k) { return lam[k] - lam0[k]; }, AddProduct()));
+    }
     long long i;
     const bool own = ti.row(tile, d.n, i);
     if (own) {
-      const double xi = double(x[i]);
+      const double xi = x[i], ci = c[i], lo = lx[i], hi = ux[i], dxi = Dx[i];
       const double qx = hx - ginv * xi;
-      const double g = qx + c[i] + atl;
-      const double lo = lx[i], hi = ux[i];
-      double p = xi - g;
-      p = p < lo ? lo : p;
-      p = p > hi ? hi : p;
-      q[5] = fmax(q[5], res_term(fabs(xi - p)));
-      q[6] = fmax(q[6], fmax(scale_term(fabs(qx)), fmax(fabs(c[i]), scale_term(fabs(atl)))));
-      const double f = 1.0 / (cs * Dx[i]);
-      const double xo = Dx[i] * xi, loo = lo * Dx[i], hio = hi * Dx[i], go = g * f;
-      double po = xo - go;
-      po = po < loo ? loo : po;
-      po = po > hio ? hio : po;
-      q[7] = fmax(q[7], res_term(fabs(xo - po)));
-      q[2] = fmax(q[2], res_term(xo < loo ? loo - xo : (xo > hio ? xo - hio : 0.0)));
-      q[8] = fmax(q[8], fmax(scale_term(fabs(qx * f)), fmax(fabs(c[i] * f), scale_term(fabs(atl * f)))));
-      q[9] = fmax(q[9], fabs(xi - z[i]));
+      const double g = qx + ci + atl;
+      q[5] = max_abs(q[5], res_of(xi - clampv<double>(xi - g, lo, hi)));
+      const double sc = max_abs(max_abs(scale_of(qx), ci), scale_of(atl));
+      q[6] = max_abs(q[6], sc);
+      const double f = ics * recip(dxi);
+      const double xo = dxi * xi, loo = lo * dxi, hio = hi * dxi, go = g * f;
+      q[7] = max_abs(q[7], res_of(xo - clampv<double>(xo - go, loo, hio)));
+      q[2] = max_abs(q[2], res_of(less_bits(xo, loo) ? loo - xo : (less_bits(hio, xo) ? xo - hio : 0.0)));
+      q[8] = max_abs(q[8], sc * f);
+      q[9] = max_abs(q[9], xi - z[i]);
       q[10] += xi * qx;
-      q[11] += c[i] * xi;
-    }
-  }
-  block_reduce_store<12, OUT_MAXMASK>(q, d.part + 12 * kMaxBlocks);
-}
-
-// Infeasibility tests (Sec. "Infeasibility detection") on the scaled problem,
-// from the changes over one outer iteration dlam = lambda^{k+1} - lambda^k and
-// dx = x^{k+1} - x^k.  Unnormalised quantities; the host divides by the
-// norms.  Rows (4): 0 largest |dlam_j| that would need an infinite row bound
-// (sign condition), 1 sum of the finite-bound terms of sigma_C(dlam), 2
-// largest departure of (A dx)_j from the recession cone of [l_c, u_c], 3
-// ||dlam||_inf.
-constexpr unsigned INF_R_MAXMASK = 0xDu;
-template <typename T, int G>
-__global__ void __launch_bounds__(kBlock) k_inf_rows(Dev<T> d, Mat<double> Ad, const double *lc, const double *uc,
-                                                     const double *lam, const double *lam0, const double *dx) {
-  double q[4] = {0.0, 0.0, 0.0, 0.0};
-  TileIter<G> ti;
-  for (long long tile = ti.first; tile < d.m; tile += ti.step) {
-    const double ad = tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double>{dx});
-    long long j;
-    const bool own = ti.row(tile, d.m, j);
-    if (own) {
-      const double y = lam[j] - lam0[j], lo = lc[j], hi = uc[j];
-      if (y > 0.0) {
-        if (isinf(hi)) q[0] = fmax(q[0], y); else q[1] += hi * y;
-      } else if (y < 0.0) {
-        if (isinf(lo)) q[0] = fmax(q[0], -y); else q[1] += lo * y;
+      q[11] += ci * xi;
+      if (update) {
+        const double v = -atd, di = dx[i], qd = hd - ginv * di;
+        double *p = q + OUT_Q;
+        if (v > 0.0) {
+          if (isinf(hi)) p[0] = max_abs(p[0], v); else p[1] += hi * v;
+        } else if (v < 0.0) {
+          if (isinf(lo)) p[0] = max_abs(p[0], v); else p[1] += lo * v;
+        }
+        if (!isinf(lo) && di < 0.0) p[2] = max_abs(p[2], di);
+        if (!isinf(hi) && di > 0.0) p[2] = max_abs(p[2], di);
+        p[3] += di * qd;
+        p[4] += ci * di;
+        p[5] = max_abs(p[5], qd);
+        p[6] = max_abs(p[6], di);
       }
-      if (!isinf(lo) && ad < 0.0) q[2] = fmax(q[2], -ad);
-      if (!isinf(hi) && ad > 0.0) q[2] = fmax(q[2], ad);
-      q[3] = fmax(q[3], fabs(y));
     }
   }
-  block_reduce_store<4, INF_R_MAXMASK>(q, d.part);
-}
-
-// Columns (7): 0 largest |v_i|, v = -A' dlam, that would need an infinite
-// variable bound, 1 sum of the finite-bound terms of sigma_X(v), 2 largest
-// departure of dx_i from the recession cone of [l_x, u_x], 3 dx'Q dx, 4 c'dx,
-// 5 ||Q dx||_inf, 6 ||dx||_inf (Q dx = H dx - dx / gamma).
-constexpr unsigned INF_C_MAXMASK = 0x65u;
-template <typename T, int G>
-__global__ void __launch_bounds__(kBlock) k_inf_cols(Dev<T> d, Mat<double> Hd, Mat<double> Atd, const double *c,
-                                                     const double *lx, const double *ux, const double *lam,
-                                                     const double *lam0, const double *dx, double ginv) {
-  double q[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  TileIter<G> ti;
-  for (long long tile = ti.first; tile < d.n; tile += ti.step) {
-    const double atl = tile_row_sum<G, double>(Atd.rp, Atd.ci, Atd.val, tile, d.n,
-                                               entry([&](int k) { return lam[k] - lam0[k]; }, AddProduct()));
-    const double hd = tile_row_sum<G, double>(Hd.rp, Hd.ci, Hd.val, tile, d.n, MulLdg<double>{dx});
-    long long i;
-    const bool own = ti.row(tile, d.n, i);
-    if (own) {
-      const double v = -atl, di = dx[i], qd = hd - ginv * di, lo = lx[i], hi = ux[i];
-      if (v > 0.0) {
-        if (isinf(hi)) q[0] = fmax(q[0], v); else q[1] += hi * v;
-      } else if (v < 0.0) {
-        if (isinf(lo)) q[0] = fmax(q[0], -v); else q[1] += lo * v;
-      }
-      if (!isinf(lo) && di < 0.0) q[2] = fmax(q[2], -di);
-      if (!isinf(hi) && di > 0.0) q[2] = fmax(q[2], di);
-      q[3] += di * qd;
-      q[4] += c[i] * di;
-      q[5] = fmax(q[5], fabs(qd));
-      q[6] = fmax(q[6], fabs(di));
+  block_reduce_store<kOutCols, kOutColsMask>(q, d.part + kOutRows * kMaxBlocks);
+  if (arrive_last(d.ctr + 3)) {
+    double a[kOutRows], b[kOutCols];
+    final_reduce<kOutRows>(d.part, nb_r, kOutRowsMask, a);
+    final_reduce<kOutCols>(d.part + kOutRows * kMaxBlocks, gridDim.x, kOutColsMask, b);
+    if (threadIdx.x == 0) {
+      for (int k = 0; k < OUT_Q; ++k) out[k] = ((OUT_MAXMASK >> k) & 1u) ? fmax(a[k], b[k]) : a[k] + b[k];
+      for (int k = 0; k < INF_R; ++k) out[OUT_Q + k] = a[OUT_Q + k];
+      for (int k = 0; k < INF_C; ++k) out[OUT_Q + INF_R + k] = b[OUT_Q + k];
+      d.ctr[3] = 0u;
     }
   }
-  block_reduce_store<7, INF_C_MAXMASK>(q, d.part);
 }
 
 // Anderson acceleration (Sec. "Anderson acceleration"): sums of one Type-II
@@ -666,10 +663,6 @@ __global__ void __launch_bounds__(kBlock) k_aa_apply(const double *G, int head, 
     sn[0] += v * v;
   }
   block_reduce_store<1, 0u>(sn, part);
-}
-
-__global__ void k_sub(long long n, const double *a, const double *b, double *out) {
-  PDNQP_GRID_STRIDE(i, n) out[i] = a[i] - b[i];
 }
 
 // Eq. penalty-trigger-eq with the growth rule (only when `grow`: the primal

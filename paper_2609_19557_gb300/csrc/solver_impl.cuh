@@ -691,12 +691,17 @@ class Solver : public SolverBase {
   // and rows or columns in tiles of 8 where their mean length is above 24
   // entries (there a warp's lanes are better spent along a row: at 100 entries
   // a row, 8 rows a warp keep 8 x 32 entries in flight as 32 short rows do).
-  void (*trials_fn() const)(Dev<T>) {
+  void (*trials_fn() const)(Dev<T>, long long) {
     const bool lr = d_.nlr > 0, rl = nnzA_ - d_.lr_nnz > 24LL * m_, cl = std::max(nnzH_, nnzA_) > 24LL * n_;
     if (lr) return rl ? (cl ? k_trials<T, true, true, true> : k_trials<T, true, true, false>)
                       : (cl ? k_trials<T, true, false, true> : k_trials<T, true, false, false>);
     return rl ? (cl ? k_trials<T, false, true, true> : k_trials<T, false, true, false>)
               : (cl ? k_trials<T, false, false, true> : k_trials<T, false, false, false>);
+  }
+  void (*check_fn() const)(Dev<T>) {
+    const bool rl = nnzA_ > 24LL * m_, cl = std::max(nnzH_, nnzA_) > 24LL * n_;
+    return rl ? (cl ? k_check<T, true, true> : k_check<T, true, false>)
+              : (cl ? k_check<T, false, true> : k_check<T, false, false>);
   }
   // Blocks of the persistent loop (one per SM at most): a warp has a tile at a
   // time, so the grid is the tiles over 8 warps a block up to one block per SM
@@ -712,7 +717,8 @@ class Solver : public SolverBase {
     if (cudaDeviceGetAttribute(&can, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !can) return 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
     const int smem = (int)trials_smem_bytes<T>();
-    if (cudaFuncSetAttribute(trials_fn(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+    if (cudaFuncSetAttribute(trials_fn(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        cudaFuncSetAttribute(check_fn(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem / 2) != cudaSuccess) {
       cudaGetLastError();
       return 0;
     }
@@ -730,16 +736,20 @@ class Solver : public SolverBase {
     coop_nb_ = (int)std::max(0LL, std::min<long long>(std::min(per_sm * sms, kMaxBlocks), work));
     return coop_nb_;
   }
-  int launch_trials_persistent(int nb, int slot) {
+  // One slot: the trial loop up to the next check (timed by events of its own),
+  // then the check.
+  int launch_loop_slot(int nb, int slot, long long chunk) {
     if (!loop_ev_[2 * slot]) {
       PDNQP_CK(cudaEventCreate(&loop_ev_[2 * slot]));
       PDNQP_CK(cudaEventCreate(&loop_ev_[2 * slot + 1]));
     }
     PDNQP_CK(cudaEventRecord(loop_ev_[2 * slot], s_));
-    void *args[] = {(void *)&d_};
+    void *args[] = {(void *)&d_, (void *)&chunk};
     PDNQP_CK(cudaLaunchCooperativeKernel((const void *)trials_fn(), dim3(nb), dim3(kTrialThreads), args,
                                          trials_smem_bytes<T>(), s_));
     PDNQP_CK(cudaEventRecord(loop_ev_[2 * slot + 1], s_));
+    PDNQP_CK(cudaLaunchCooperativeKernel((const void *)check_fn(), dim3(nb), dim3(kTrialThreads), args,
+                                         trials_smem_bytes<T>() / 2, s_));
     return 0;
   }
   void launch_check(int mode) {
@@ -1036,20 +1046,15 @@ class Solver : public SolverBase {
     }
     const int nbp = prm.persistent ? coop_grid(prm.loop_blocks_per_sm) : 0;
     if (nbp > 0) {
-      // Persistent loop: batches of slots [trial loop, check rows, check cols
-      // (+ decisions), check apply]; a batch runs at most `per` trials, after
-      // which the host reads the state once.
-      const long long kc = std::max<long long>(1, prm.k_chk);
-      const long long per = std::max<long long>(prm.chunk, 8 * kc);
-      const int R = (int)std::min<long long>(kMaxLoopSlots, per / kc + 1);
-      for (;;) {
-        k_loop_begin<<<1, 1, 0, s_>>>(st_, per);
-        for (int r = 0; r < R; ++r) {
-          PDNQP_TRY(launch_trials_persistent(nbp, r));
-          launch_check_group();
-        }
-        PDNQP_CK(cudaGetLastError());
-        launches_ += 1 + 4LL * R;
+      // Persistent loop: batches of slots [trial loop, check] of at most `per`
+      // trials, after which the host reads the state once.  Most inner solves
+      // stop at one of the first checks, and a slot that finds the solve stopped
+      // still costs two launches (5 us): the first batch has 2 slots, each
+      // further one twice as many.
+      const long long per = std::max<long long>(prm.chunk, 8 * std::max<long long>(1, prm.k_chk));
+      for (int R = 2;; R = std::min(2 * R, kMaxLoopSlots)) {
+        for (int r = 0; r < R; ++r) PDNQP_TRY(launch_loop_slot(nbp, r, r == 0 ? per : -1));
+        launches_ += 2LL * R;
         loop_launches_ += R;
         const long long tr_before = hst_->trials;
         PDNQP_TRY(read_state(S));
@@ -1095,7 +1100,7 @@ class Solver : public SolverBase {
     restarts_ = S.restarts;
     omega_ = S.omega;
     // Outer x and inner y = base + correction (current point or converged average).
-    k_finish<T><<<grid_nm(), kBlock, 0, s_>>>(d_, x64_, y64_, (S.status == ST_CONVERGED && S.ret_avg) ? 1 : 0);
+    k_finish<T><<<grid_nm(), kBlock, 0, s_>>>(d_, x64_, y64_, xprev_, dxv_, (S.status == ST_CONVERGED && S.ret_avg) ? 1 : 0);
     PDNQP_CK(cudaGetLastError());
     DevState Z = S;
     reset_buffers(&Z);
@@ -1104,32 +1109,29 @@ class Solver : public SolverBase {
     return 0;
   }
 
-  // Outer residuals; update = 1 also applies the multiplier update first.
-  int outer_residuals(int update, double *q) {
+  // Outer residuals; update = 1 also applies the multiplier update first and
+  // forms the sums of the infeasibility tests (inf[0..10]).
+  int outer_residuals(int update, double *q, double *inf) {
     const double ginv = 1.0 / gamma_;
-    launches_ += 4;
-    double a[12] = {0}, b[12] = {0};
-    const int nbr = nb_rows(), nbc = nb_cols();
-    if (m_) {
+    const int nbr = m_ ? nb_rows() : 0, nbc = nb_cols();
+    if (m_)
       with_G(gA_, [&](auto GG) {
-        k_outer_rows<T, decltype(GG)::value><<<nbr, kBlock, 0, s_>>>(d_, Ad_, lcd_, ucd_, Dc_, lam_, sig_, rcur_,
-                                                                      update);
+        k_outer_rows<T, decltype(GG)::value><<<nbr, kBlock, 0, s_>>>(d_, Ad_, lcd_, ucd_, Dc_, lam_, lamprev_, sig_, rcur_,
+                                                                      dxv_, update);
       });
-      k_reduce_rows<<<12, 32, 0, s_>>>(part_, 12, nbr, OUT_MAXMASK, dred_);
-    }
     // A' lambda uses the updated multipliers: launched after the row kernel.
     with_G(gN_, [&](auto GG) {
-      k_outer_cols<T, decltype(GG)::value><<<nbc, kBlock, 0, s_>>>(d_, Hd_, Atd_, c_, lxd_, uxd_, Dx_, lam_, z_,
-                                                                    ginv, cs_);
+      k_outer_cols<T, decltype(GG)::value><<<nbc, kBlock, 0, s_>>>(d_, Hd_, Atd_, c_, lxd_, uxd_, Dx_, lam_,
+                                                                    m_ ? lamprev_ : lam_, dxv_, z_, ginv, cs_, update, nbr,
+                                                                    dred_);
     });
-    k_reduce_rows<<<12, 32, 0, s_>>>(part_ + 12 * kMaxBlocks, 12, nbc, OUT_MAXMASK, dred_ + 12);
+    launches_ += m_ ? 2 : 1;
     PDNQP_CK(cudaGetLastError());
-    PDNQP_CK(cudaMemcpyAsync(hred_.data(), dred_, sizeof(double) * 24, cudaMemcpyDeviceToHost, s_));
+    PDNQP_CK(cudaMemcpyAsync(hred_.data(), dred_, sizeof(double) * (OUT_Q + INF_Q), cudaMemcpyDeviceToHost, s_));
     PDNQP_CK(cudaStreamSynchronize(s_));
-    if (m_)
-      for (int k = 0; k < 12; ++k) a[k] = hred_[k];
-    for (int k = 0; k < 12; ++k) b[k] = hred_[12 + k];
-    for (int k = 0; k < 12; ++k) q[k] = ((OUT_MAXMASK >> k) & 1u) ? std::max(a[k], b[k]) : a[k] + b[k];
+    for (int k = 0; k < OUT_Q; ++k) q[k] = hred_[k];
+    if (inf)
+      for (int k = 0; k < INF_Q; ++k) inf[k] = hred_[OUT_Q + k];
     return 0;
   }
 
@@ -1224,8 +1226,8 @@ class Solver : public SolverBase {
       }
       if (S.status == ST_ITER_LIMIT) continue;
       // Multiplier update + outer residuals (Eqs. practical-multiplier-update, outer-residuals).
-      if (m_) PDNQP_CK(cudaMemcpyAsync(lamprev_, lam_, sizeof(double) * m_, cudaMemcpyDeviceToDevice, s_));
-      PDNQP_TRY(outer_residuals(1, q));
+      double infq[INF_Q];
+      PDNQP_TRY(outer_residuals(1, q, infq));
       const double rps = q[0], sps = std::max(1.0, q[1]), rpu = q[2], spu = std::max(1.0, q[3]), rn = q[4];
       const double rds = q[5], rdu = q[7], sdu = std::max(1.0, q[8]), dxz = q[9];
       if (rpu <= ea + er * spu && rdu <= ea + er * sdu) {
@@ -1234,8 +1236,7 @@ class Solver : public SolverBase {
         break;
       }
       {
-        int inf = 0;
-        PDNQP_TRY(inf = infeasibility(prm.eps_inf > 0.0 ? prm.eps_inf : 1e-5));
+        const int inf = infeasibility(infq, prm.eps_inf > 0.0 ? prm.eps_inf : 1e-5);
         if (inf) {
           status = inf;
           ++k;
@@ -1363,7 +1364,7 @@ class Solver : public SolverBase {
       PDNQP_CK(cudaGetLastError());
     }
     // Result in the original coordinates.
-    PDNQP_TRY(outer_residuals(0, q));
+    PDNQP_TRY(outer_residuals(0, q, nullptr));
     k_unscale<double><<<grid_nm(), kBlock, 0, s_>>>(x64_, Dx_, n_, lam_, Dc_, m_, cs_, xo_, lo_);
     PDNQP_CK(cudaGetLastError());
     PDNQP_CK(cudaStreamSynchronize(s_));
@@ -1478,30 +1479,12 @@ class Solver : public SolverBase {
     return 0;
   }
 
-  // Sec. "Infeasibility detection" on the scaled problem (see k_inf_rows /
-  // k_inf_cols): PDNQP_PRIMAL_INFEASIBLE when lambda^{k+1} - lambda^k is an
+  // Sec. "Infeasibility detection" on the scaled problem (see outer_rows_inf /
+  // outer_cols_inf): PDNQP_PRIMAL_INFEASIBLE when lambda^{k+1} - lambda^k is an
   // approximate Farkas certificate, PDNQP_DUAL_INFEASIBLE when x^{k+1} - x^k
   // is an approximate recession direction of descent, else 0.
-  int infeasibility(double eps) {
-    const double ginv = 1.0 / gamma_;
-    k_sub<<<grid_n(), kBlock, 0, s_>>>(n_, x64_, xprev_, dxv_);
-    double a[4] = {0.0, 0.0, 0.0, 0.0}, b[7];
-    if (m_) {
-      const int nb = nb_rows();
-      with_G(gA_, [&](auto GG) {
-        k_inf_rows<T, decltype(GG)::value><<<nb, kBlock, 0, s_>>>(d_, Ad_, lcd_, ucd_, lam_, lamprev_, dxv_);
-      });
-      PDNQP_TRY(reduce_to_host(4, nb, INF_R_MAXMASK, a));
-    }
-    {
-      const int nb = nb_cols();
-      with_G(gN_, [&](auto GG) {
-        k_inf_cols<T, decltype(GG)::value><<<nb, kBlock, 0, s_>>>(d_, Hd_, Atd_, c_, lxd_, uxd_, lam_,
-                                                                  m_ ? lamprev_ : lam_, dxv_, ginv);
-      });
-      PDNQP_TRY(reduce_to_host(7, nb, INF_C_MAXMASK, b));
-    }
-    launches_ += m_ ? 3 : 2;
+  static int infeasibility(const double *v, double eps) {
+    const double *a = v, *b = v + INF_R;
     const double nl = a[3], nx = b[6];
     if (nl > 0.0 && std::max(a[0], b[0]) <= eps * nl && a[1] + b[1] < -eps * nl) return PDNQP_PRIMAL_INFEASIBLE;
     if (nx > 0.0 && std::max(a[2], b[2]) <= eps * nx &&
@@ -1594,7 +1577,7 @@ class Solver : public SolverBase {
   Dev<T> d_{};
   cudaGraphExec_t gexec_ = nullptr;
   cudaEvent_t replay_ev_[2] = {nullptr, nullptr};
-  static constexpr int kMaxLoopSlots = 32;
+  static constexpr int kMaxLoopSlots = 8;
   cudaEvent_t loop_ev_[2 * kMaxLoopSlots] = {};
   double loop_seconds_ = 0.0;  // device time of the persistent trial-loop launches
   long long loop_launches_ = 0;
