@@ -562,16 +562,16 @@ __device__ __forceinline__ Slot<Acc> *warp_slots() {
 // nearly equal numbers, and its multiplier follows the rounding of that sum: in
 // another order it moves by some 1e-9 of itself at 10,000 entries, so the two
 // kernels that take it (base point, multiplier update: once an outer iteration)
-// keep the order they always had.  Operands are loaded and gathered 256 at a
+// keep the order they always had (buf: the warp's slots).  Operands are loaded and gathered 256 at a
 // time; what is left is the chain of additions, 64 cycles each (0.3 ms at
 // 10,000 entries).
 template <bool IsMax, typename Acc, typename T, typename F>
-__device__ __forceinline__ Acc one_row(const int *__restrict__ ci, const T *__restrict__ val, int b, int e, const F &f) {
+__device__ __forceinline__ Acc one_row(const int *__restrict__ ci, const T *__restrict__ val, int b, int e, const F &f,
+                                       Slot<Acc> *buf) {
   if constexpr (F::kOrder == 0) {
     return warp_row<IsMax, Acc>(ci, val, b, e, f);
   } else {
     if (e - b <= kDenseRow) return warp_row<IsMax, Acc>(ci, val, b, e, f);
-    Slot<Acc> *buf = warp_slots<Acc>();
     const int lane = threadIdx.x & 31;
     Acc acc = Acc(0);
     for (int k0 = b; k0 < e; k0 += 256) {
@@ -720,7 +720,7 @@ __device__ __forceinline__ void tile_rows(const int *const (&ci)[NM], const T *c
     for (int m = 0; m < NM; ++m) {
       const int b = __shfl_sync(0xffffffffu, rb[m], l), e = __shfl_sync(0xffffffffu, re[m], l);
       if (e - b > kLongRowEntries) {
-        const Acc v = one_row<IsMax, Acc>(ci[m], val[m], b, e, f[m]);
+        const Acc v = one_row<IsMax, Acc>(ci[m], val[m], b, e, f[m], buf);
         if (lane == l) out[m] = v;
       }
     }
@@ -746,7 +746,7 @@ __device__ __forceinline__ Acc tile_rows1(const int *ci, const T *val, int rb, i
 // adds the other half, 9 additions for the 8 rows instead of 40.
 template <bool IsMax, typename Acc, typename T, typename F>
 __device__ __forceinline__ Acc tile_long_rows(const int *__restrict__ ci, const T *__restrict__ val, int rb, int re,
-                                              const F &f) {
+                                              const F &f, Slot<Acc> *buf = nullptr) {
   const int lane = threadIdx.x & 31;
   const bool alone = re - rb > kRowAlone;
   const int se = alone ? rb : re;
@@ -794,7 +794,7 @@ __device__ __forceinline__ Acc tile_long_rows(const int *__restrict__ ci, const 
   while (todo) {
     const int l = __ffs(todo) - 1;
     todo &= todo - 1;
-    const Acc v = one_row<IsMax, Acc>(ci, val, __shfl_sync(0xffffffffu, rb, l), __shfl_sync(0xffffffffu, re, l), f);
+    const Acc v = one_row<IsMax, Acc>(ci, val, __shfl_sync(0xffffffffu, rb, l), __shfl_sync(0xffffffffu, re, l), f, buf);
     if ((lane & 7) == l) out = v;
   }
   return out;
@@ -838,7 +838,7 @@ __device__ __forceinline__ Acc tile_reduce(const int *rp, const int *ci, const T
   const long long my = tile + (threadIdx.x & 31);
   const bool ok = (threadIdx.x & 31) < TileIter<K>::TR && my < nrows;
   const int rb = ok ? rp[my] : 0, re = ok ? rp[my + 1] : 0;
-  return K == 16 ? tile_long_rows<IsMax, Acc>(ci, val, rb, re, f)
+  return K == 16 ? tile_long_rows<IsMax, Acc>(ci, val, rb, re, f, buf)
                  : tile_rows1<IsMax, Acc>(ci, val, rb, re, f, buf);
 }
 template <int K, typename Acc, typename T, typename F>

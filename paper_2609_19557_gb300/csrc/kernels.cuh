@@ -183,7 +183,6 @@ __device__ void decide_body(DevState *stg, const double *part, const double *lac
 template <bool COND>
 __device__ void check_final_body(DevState *stg, const double *part, int nb_r, int nb_c,
                                  cudaGraphConditionalHandle hw);
-__device__ void inner_begin_body(DevState *st, const double *part, int nb_r, int nb_c);
 __device__ __forceinline__ bool decide_logic(DevState *st, const double (&a)[4]);
 __device__ __forceinline__ void trial_begin(DevState *st);
 __device__ __forceinline__ void trial_accept(DevState *st);
@@ -1047,8 +1046,7 @@ __global__ void __launch_bounds__(kBlock) k_average(Dev<T> d) {
 //   0 r_p (max), 1 s_p (max), 2 r_d (max), 3 s_d (max),
 //   4 sum (d (Bw - h))^2, 5 sum ((w - P(w - e^2 g)) / e)^2,
 //   6 sum ((w - w_start) / e)^2, 7 sum ((y - y_start) / d)^2
-// stored as [c0..c7, a0..a7].  mode 1 = only the current point's 4 and 5
-// (restart metric of the inner start).
+// stored as [c0..c7, a0..a7].
 // ===========================================================================
 // Contributions of one row (its s and r components and its dual) to the 8
 // quantities of one candidate, in FP64.  Inputs are corrections (bwd = B dw,
@@ -1090,7 +1088,7 @@ __device__ __forceinline__ void row_cand(double *q, const RowIn &a) {
 }
 
 template <typename T, int G>
-__device__ __forceinline__ void check_rows_body(const Dev<T> &d, const DevState *st, int mode, GridCtx g,
+__device__ __forceinline__ void check_rows_body(const Dev<T> &d, const DevState *st, GridCtx g,
                                                 Slot<T> *buf) {
   // Averages of a pending acceptance are formed on the fly (and written for the
   // row blocks); x bar is gathered as (1 - alpha) xbar + alpha x.
@@ -1103,9 +1101,7 @@ __device__ __forceinline__ void check_rows_body(const Dev<T> &d, const DevState 
   for (int k = 0; k < 16; ++k) q[k] = 0.0;
   TileIter<G> ti(g);
   for (long long tile = ti.first; tile < d.m; tile += ti.step) {
-    T axb = T(0);
-    if (mode == 0)
-      axb = tile_row_sum<G, T>(d.A.rp, d.A.ci, d.A.val, tile, d.m,
+    const T axb = tile_row_sum<G, T>(d.A.rp, d.A.ci, d.A.val, tile, d.m,
                                entry([&](int k) { return acc ? omap * xb0[k] + ap * xc[k] : xb0[k]; }, AddProduct()), buf);
     long long j;
     const bool own = ti.row(tile, d.m, j);
@@ -1138,7 +1134,7 @@ __device__ __forceinline__ void check_rows_body(const Dev<T> &d, const DevState 
       a.dr = widen(d.r[cur][j]);
       a.dyv = widen(d.y[cur][j]);
       row_cand(q, a);
-      if (mode == 0) {
+      {
         T sa = ineq ? d.sbar[a0][j] : T(0), ra = d.rbar[a0][j], ya = d.ybar[a0][j];
         if (acc) {
           ra = omap * ra + ap * d.r[cur][j];
@@ -1169,9 +1165,9 @@ __device__ __forceinline__ bool check_pending(const Dev<T> &d) {
 }
 
 template <typename T, int G>
-__global__ void __launch_bounds__(kBlock) k_check_rows(Dev<T> d, int mode) {
-  if (mode == 0 && !check_pending(d)) return;
-  check_rows_body<T, G>(d, d.st, mode, hw_grid(), warp_slots<T>());
+__global__ void __launch_bounds__(kBlock) k_check_rows(Dev<T> d) {
+  if (!check_pending(d)) return;
+  check_rows_body<T, G>(d, d.st, hw_grid(), warp_slots<T>());
 }
 
 // Contributions of one variable (x block) to the 8 quantities of a candidate:
@@ -1189,7 +1185,7 @@ __device__ __forceinline__ void col_cand(double *q, double dx, double hdx, doubl
 }
 
 template <typename T, int G>
-__device__ __forceinline__ void check_cols_terms(const Dev<T> &d, const DevState *st, int mode, GridCtx g,
+__device__ __forceinline__ void check_cols_terms(const Dev<T> &d, const DevState *st, GridCtx g,
                                                  Slot<T> *buf) {
   // y bar of a pending acceptance was materialised by k_check_rows.
   const int cur = st->cur, a0 = st->acur, acc = st->accepted, ab = a0 ^ acc;
@@ -1201,9 +1197,7 @@ __device__ __forceinline__ void check_cols_terms(const Dev<T> &d, const DevState
   for (int k = 0; k < 16; ++k) q[k] = 0.0;
   TileIter<G> ti(g);
   for (long long tile = ti.first; tile < d.n; tile += ti.step) {
-    T atyb = T(0);
-    if (mode == 0)
-      atyb = tile_row_sum<G, T>(d.At.rp, d.At.ci, d.At.val, tile, d.n, MulLd<T>{yb}, buf);
+    const T atyb = tile_row_sum<G, T>(d.At.rp, d.At.ci, d.At.val, tile, d.n, MulLd<T>{yb}, buf);
     long long i;
     const bool own = ti.row(tile, d.n, i);
     if (own) {
@@ -1211,7 +1205,7 @@ __device__ __forceinline__ void check_cols_terms(const Dev<T> &d, const DevState
       const double atyb0 = widen(d.Atyb[i]), lx = widen(d.lx[i]), ux = widen(d.ux[i]);
       const double ex = widen(d.ex[i]), xst = widen(d.xst[i]), iex = recip(d.ex[i]), ex2 = ex * ex;
       col_cand(q, widen(xc[i]), widen(d.Hx[cur][i]), widen(d.Aty[cur][i]), qx, qx0, hxb, atyb0, lx, ux, ex2, iex, xst);
-      if (mode == 0) {
+      {
         d.Atybar[i] = atyb;
         T xa = d.xbar[a0][i], ha = d.Hxbar[a0][i];
         if (acc) {
@@ -1228,21 +1222,18 @@ __device__ __forceinline__ void check_cols_terms(const Dev<T> &d, const DevState
 }
 
 template <typename T, int G, bool COND>
-__device__ __forceinline__ void check_cols_body(const Dev<T> &d, int mode, int nb_r, GridCtx g) {
-  if (mode == 0 && !check_pending(d)) return;
-  check_cols_terms<T, G>(d, d.st, mode, g, warp_slots<T>());
+__device__ __forceinline__ void check_cols_body(const Dev<T> &d, int nb_r, GridCtx g) {
+  if (!check_pending(d)) return;
+  check_cols_terms<T, G>(d, d.st, g, warp_slots<T>());
   if (arrive_last(d.ctr + 1, g.nb)) {
-    if (mode == 0)
-      check_final_body<COND>(d.st, d.part, nb_r, g.nb, d.hw);
-    else
-      inner_begin_body(d.st, d.part, nb_r, g.nb);
+    check_final_body<COND>(d.st, d.part, nb_r, g.nb, d.hw);
     if (threadIdx.x == 0) d.ctr[1] = 0u;
   }
 }
 
 template <typename T, int G, bool COND>
-__global__ void __launch_bounds__(kBlock) k_check_cols(Dev<T> d, int mode, int nb_r) {
-  check_cols_body<T, G, COND>(d, mode, nb_r, hw_grid());
+__global__ void __launch_bounds__(kBlock) k_check_cols(Dev<T> d, int nb_r) {
+  check_cols_body<T, G, COND>(d, nb_r, hw_grid());
 }
 
 // Decisions of the check (one thread), from its 16 quantities: inner termination
@@ -1474,9 +1465,9 @@ __global__ void __launch_bounds__(kTrialThreads, 1) k_check(Dev<T> d) {
   if (S.status != ST_RUNNING || !S.check_due) return;
   const int nb = gridDim.x;
   const GridCtx g{(int)blockIdx.x, nb};
-  check_rows_body<T, RL ? 16 : 8>(d, &S, 0, g, buf);
+  check_rows_body<T, RL ? 16 : 8>(d, &S, g, buf);
   if (loop_sync(bar, gen, [] { return 0; }) < 0) return;
-  check_cols_terms<T, CL ? 16 : 8>(d, &S, 0, g, buf);
+  check_cols_terms<T, CL ? 16 : 8>(d, &S, g, buf);
   bool led = false;
   if (loop_sync(bar, gen, [&] {
         led = true;
@@ -1489,233 +1480,6 @@ __global__ void __launch_bounds__(kTrialThreads, 1) k_check(Dev<T> d) {
     return;
   if (!led) state_load(S, d.st);
   check_apply_body<T>(d, &S, g);
-}
-
-// ===========================================================================
-// Setup of one inner solve (a0): warm start, penalty + inner Ruiz scaling,
-// diagonal steps, cached products.
-// ===========================================================================
-
-// Base rows of one inner solve (Eq. inner-warm-start, in FP64): v = A x_b,
-// s_b = P_[l_c,u_c](v + lambda / sigma) and r_b = v - s_b on inequality rows,
-// r_b = v - b_E on equality rows; then B w_b, h' = h - B w_b, the base
-// gradients of the s and r blocks, the shifted slack bounds, and zero
-// corrections.
-template <typename T, int G>
-__global__ void __launch_bounds__(kBlock) k_base_rows(Dev<T> d, Mat<double> Ad, const double *lc, const double *uc,
-                                                      double *sb, double *rb) {
-  const int cur = d.st->cur;
-  const double *__restrict__ x = d.xb;
-  TileIter<G> ti;
-  for (long long tile = ti.first; tile < d.m; tile += ti.step) {
-    const double v = tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double, 1>{x});
-    long long j;
-    if (!ti.row(tile, d.m, j)) continue;
-    const double lam = d.lam[j], sig = d.sig[j], yb = d.yb[j];
-    double s = 0.0, r, bw;
-    if (j >= d.mE) {
-      s = v + lam / sig;
-      s = s < lc[j] ? lc[j] : s;
-      s = s > uc[j] ? uc[j] : s;
-      r = v - s;
-      bw = v - s - r;
-      d.ls[j] = T(lc[j] - s);
-      d.us[j] = T(uc[j] - s);
-      d.qs[j] = T(yb);
-      d.s[cur][j] = T(0);
-    } else {
-      r = v - lc[j];
-      bw = v - r;
-    }
-    const double h = j < d.mE ? lc[j] : 0.0;
-    sb[j] = s;
-    rb[j] = r;
-    d.h[j] = T(h);
-    d.Bwb[j] = T(bw);
-    d.hp[j] = T(h - bw);
-    d.qr[j] = T(lam + sig * r + yb);
-    d.sg[j] = T(sig);
-    d.r[cur][j] = T(0);
-    d.y[cur][j] = T(0);
-    d.Bw[cur][j] = T(0);
-  }
-}
-
-// Base columns: H x_b and A' y_b in FP64, q'_x = c - z / gamma + H x_b - A' y_b,
-// q_x, the shifted bounds, and zero corrections with zero cached products.
-template <typename T, int G>
-__global__ void __launch_bounds__(kBlock) k_base_cols(Dev<T> d, Mat<double> Hd, Mat<double> Atd, const double *c,
-                                                      const double *z, const double *lxd, const double *uxd,
-                                                      double ginv) {
-  const int cur = d.st->cur;
-  const double *__restrict__ x = d.xb;
-  const double *__restrict__ y = d.yb;
-  TileIter<G> ti;
-  for (long long tile = ti.first; tile < d.n; tile += ti.step) {
-    const double hx = tile_row_sum<G, double>(Hd.rp, Hd.ci, Hd.val, tile, d.n, MulLdg<double>{x});
-    const double aty = tile_row_sum<G, double>(Atd.rp, Atd.ci, Atd.val, tile, d.n, MulLdg<double>{y});
-    long long i;
-    const bool own = ti.row(tile, d.n, i);
-    if (own) {
-      const double q0 = c[i] - z[i] * ginv;
-      d.qx0[i] = T(q0);
-      d.qx[i] = T(q0 + hx - aty);
-      d.Hxb[i] = T(hx);
-      d.Atyb[i] = T(aty);
-      d.lx[i] = T(lxd[i] - x[i]);
-      d.ux[i] = T(uxd[i] - x[i]);
-      d.x[d.st->xcur][i] = T(0);
-      d.Hx[cur][i] = T(0);
-      d.Aty[cur][i] = T(0);
-    }
-  }
-}
-
-// Penalty scaling as the initial column scale of the r block: e_r = 1/sqrt(sigma).
-template <typename T>
-__global__ void k_iscale_init(Dev<T> d) {
-  PDNQP_GRID_STRIDE(i, d.n) d.ex[i] = T(1);
-  PDNQP_GRID_STRIDE(j, d.m) {
-    d.es[j] = T(1);
-    d.er[j] = T(1.0 / sqrt(d.sig[j]));
-    d.dy[j] = T(1);
-  }
-}
-
-// Reciprocal square root in the storage precision.
-__device__ __forceinline__ float rsqrt_t(float v) { return rsqrtf(v); }
-__device__ __forceinline__ double rsqrt_t(double v) { return rsqrt(v); }
-
-// Inner Ruiz, l_inf norms of the x columns of [[H~, B~^T], [B~, 0]]:
-// max(max_k |e_k H_ki e_i|, max_j |d_j A_ji e_i|), in the storage precision T.
-template <typename T, int G>
-__global__ void __launch_bounds__(kBlock) k_iruiz_cols(Dev<T> d, double *cnx) {
-  TileIter<G> ti;
-  for (long long tile = ti.first; tile < d.n; tile += ti.step) {
-    long long i;
-    const bool own = ti.row(tile, d.n, i);
-    // e_i is applied after the reduction (max over k of |e_k H_ki| times e_i).
-    const T a = tile_row_max<G, T>(d.H.rp, d.H.ci, d.H.val, tile, d.n, entry([&](int k) { return d.ex[k]; }, MaxAbs()));
-    const T b = tile_row_max<G, T>(d.At.rp, d.At.ci, d.At.val, tile, d.n, entry([&](int k) { return d.dy[k]; }, MaxAbs()));
-    if (own) cnx[i] = double(fmax(a, b) * d.ex[i]);
-  }
-}
-
-// Inner Ruiz, rows of B~ and the s / r columns: row j: max(max_k |d_j A_jk e_k|,
-// d_j e_s (I rows), d_j e_r); s column: d_j e_s; r column: max(e_r^2 sigma_j, d_j e_r).
-template <typename T, int G>
-__global__ void __launch_bounds__(kBlock) k_iruiz_rows(Dev<T> d, double *rn, double *cns, double *cnr) {
-  TileIter<G> ti;
-  for (long long tile = ti.first; tile < d.m; tile += ti.step) {
-    const T a = tile_row_max<G, T>(d.A.rp, d.A.ci, d.A.val, tile, d.m, entry([&](int k) { return d.ex[k]; }, MaxAbs()));
-    long long j;
-    const bool own = ti.row(tile, d.m, j);
-    if (own) {
-      const T dj = d.dy[j];
-      const T er = d.er[j];
-      T rowv = fmax(a * dj, dj * er);
-      if (j >= d.mE) {
-        const T es = d.es[j];
-        rowv = fmax(rowv, dj * es);
-        cns[j] = double(dj * es);
-      }
-      rn[j] = double(rowv);
-      cnr[j] = double(fmax(er * er * T(d.sig[j]), dj * er));
-    }
-  }
-}
-
-template <typename T>
-__global__ void k_iruiz_update(Dev<T> d, const double *cnx, const double *rn, const double *cns, const double *cnr) {
-  PDNQP_GRID_STRIDE(i, d.n) {
-    const T c = T(cnx[i]);
-    if (c > T(0)) d.ex[i] = d.ex[i] * rsqrt_t(c);
-  }
-  PDNQP_GRID_STRIDE(j, d.m) {
-    const T r = T(rn[j]);
-    if (r > T(0)) d.dy[j] = d.dy[j] * rsqrt_t(r);
-    const T cr = T(cnr[j]);
-    if (cr > T(0)) d.er[j] = d.er[j] * rsqrt_t(cr);
-    if (j >= d.mE) {
-      const T cs = T(cns[j]);
-      if (cs > T(0)) d.es[j] = d.es[j] * rsqrt_t(cs);
-    }
-  }
-}
-
-// Eq. diagonal-scales for the x columns (m_w) and the effective primal step
-// tau_eff / (kappa / omega) = e^2 * 0.99 / m_w (Eq. diagonal-steps), in the
-// storage precision; imwx = 1 / m_w is kept for m_y.
-template <typename T, int G>
-__global__ void __launch_bounds__(kBlock) k_mw_cols(Dev<T> d, double *imwx) {
-  TileIter<G> ti;
-  for (long long tile = ti.first; tile < d.n; tile += ti.step) {
-    const T h1 = tile_row_sum<G, T>(d.H.rp, d.H.ci, d.H.val, tile, d.n, entry([&](int k) { return d.ex[k]; }, AddAbs()));
-    const T b1 = tile_row_sum<G, T>(d.At.rp, d.At.ci, d.At.val, tile, d.n, entry([&](int k) { return d.dy[k]; }, AddAbs()));
-    const T b2 = tile_row_sum<G, T>(d.At.rp, d.At.ci, d.At.val, tile, d.n, entry([&](int k) { return d.sg[k] * d.dy[k] * d.dy[k]; }, [](T &acc, T v, T x) { acc += x * v * v; }));
-    long long i;
-    const bool own = ti.row(tile, d.n, i);
-    if (own) {
-      const T ei = d.ex[i];
-      const T mw = h1 * ei + fmax(b1 * ei, sqrt(b2) * ei);
-      imwx[i] = double(T(1) / mw);
-      d.taux[i] = ei * ei * (T(0.99) / mw);
-      d.itaux[i] = mw / (T(0.99) * ei * ei);
-    }
-  }
-}
-
-// m_w of the s and r columns, their steps, and m_y with the dual step
-// eta_eff / (kappa omega) = d^2 * 0.99 / m_y.
-template <typename T, int G>
-__global__ void __launch_bounds__(kBlock) k_my_rows(Dev<T> d, const double *imwx) {
-  TileIter<G> ti;
-  for (long long tile = ti.first; tile < d.m; tile += ti.step) {
-    const T a = tile_row_sum<G, T>(d.A.rp, d.A.ci, d.A.val, tile, d.m, entry([&](int k) { return d.ex[k] * d.ex[k] * T(imwx[k]); }, [](T &acc, T v, T x) { acc += x * v * v; }));
-    long long j;
-    const bool own = ti.row(tile, d.m, j);
-    if (own) {
-      const T dj = d.dy[j];
-      const T sg = T(d.sig[j]);
-      const T er = d.er[j];
-      const T br = dj * er;
-      const T mwr = er * er * sg + br;
-      d.taur[j] = er * er * (T(0.99) / mwr);
-      d.itaur[j] = mwr / (T(0.99) * er * er);
-      T my = a * dj * dj + br * br / mwr;
-      if (j >= d.mE) {
-        const T es = d.es[j];
-        const T bs = dj * es;
-        const T mws = fmax(bs, sqrt(sg * bs * bs));
-        d.taus[j] = es * es * (T(0.99) / mws);
-        d.itaus[j] = mws / (T(0.99) * es * es);
-        my += bs * bs / mws;
-      }
-      d.eta[j] = dj * dj * (T(0.99) / my);
-      d.ieta[j] = my / (T(0.99) * dj * dj);
-    }
-  }
-}
-
-// Epoch start and averages of the inner start (buffer 0).
-template <typename T>
-__global__ void k_inner_init(Dev<T> d) {
-  const int cur = d.st->cur;
-  PDNQP_GRID_STRIDE(i, d.n) {
-    d.xst[i] = d.x[d.st->xcur][i];
-    d.xbar[0][i] = d.x[d.st->xcur][i];
-    d.Hxbar[0][i] = d.Hx[cur][i];
-  }
-  PDNQP_GRID_STRIDE(j, d.m) {
-    d.yst[j] = d.y[cur][j];
-    d.rst[j] = d.r[cur][j];
-    d.ybar[0][j] = d.y[cur][j];
-    d.rbar[0][j] = d.r[cur][j];
-    if (j >= d.mE) {
-      d.sst[j] = d.s[cur][j];
-      d.sbar[0][j] = d.s[cur][j];
-    }
-  }
 }
 
 // End of an inner solve: the outer x and inner y become base + correction
@@ -1754,19 +1518,6 @@ __global__ void k_totals(Dev<T> d, double *out) {
     }
   }
 }
-
-// Restart metric of the inner start (last block of the mode-1 check).
-__device__ void inner_begin_body(DevState *st, const double *part, int nb_r, int nb_c) {
-  double a[16], b[16];
-  final_reduce<16>(part + P_CK_R * kMaxBlocks, nb_r, CK_MAXMASK, a);
-  final_reduce<16>(part + P_CK_C * kMaxBlocks, nb_c, CK_MAXMASK, b);
-  if (threadIdx.x != 0) return;
-  const double om = st->omega;
-  st->k_restart = sqrt(om * (a[4] + b[4]) + (a[5] + b[5]) / om);
-  st->k_last = INFINITY;
-  st->status = st->start_status;
-}
-
 
 // ===========================================================================
 // Batched form: the inner iterations of many problems in one launch per
@@ -1819,14 +1570,14 @@ __global__ void __launch_bounds__(kBlock) kb_check_rows(const Dev<T> *devs, cons
   const BatchBlk e = map[blockIdx.x];
   const Dev<T> &d = batch_dev(devs, e.p);
   if (!check_pending(d)) return;
-  check_rows_body<T, G>(d, d.st, 0, GridCtx{e.b, e.nb}, warp_slots<T>());
+  check_rows_body<T, G>(d, d.st, GridCtx{e.b, e.nb}, warp_slots<T>());
 }
 
 template <typename T, int G>
 __global__ void __launch_bounds__(kBlock) kb_check_cols(const Dev<T> *devs, const BatchBlk *map,
                                                         const int *nb_rows) {
   const BatchBlk e = map[blockIdx.x];
-  check_cols_body<T, G, false>(batch_dev(devs, e.p), 0, nb_rows[e.p], GridCtx{e.b, e.nb});
+  check_cols_body<T, G, false>(batch_dev(devs, e.p), nb_rows[e.p], GridCtx{e.b, e.nb});
 }
 
 template <typename T>

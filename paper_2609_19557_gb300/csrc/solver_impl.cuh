@@ -6,6 +6,7 @@
 
 #include "kernels.cuh"
 #include "kernels_outer.cuh"
+#include "kernels_setup.cuh"
 #include "solver.cuh"
 
 namespace pdq {
@@ -328,8 +329,6 @@ class Solver : public SolverBase {
     PDNQP_TRY(dalloc(&lo_, m_));
     PDNQP_TRY(dalloc(&scn_[0], n_));
     PDNQP_TRY(dalloc(&scm_[0], m_));
-    PDNQP_TRY(dalloc(&scm_[1], m_));
-    PDNQP_TRY(dalloc(&scm_[2], m_));
     PDNQP_TRY(dalloc(&dx0_, n_));
     PDNQP_TRY(dalloc(&dl0_, m_));
     // ---- outer Ruiz on [[Q, A^T], [A, 0]] (Eq. scaled-problem)
@@ -532,6 +531,8 @@ class Solver : public SolverBase {
       PDNQP_TRY(dalloc(p, m_));
       PDNQP_CK(cudaMemsetAsync(*p, 0, sizeof(T) * std::max(m_, 1), s_));
     }
+    PDNQP_TRY(dalloc(&ex2_, n_));
+    PDNQP_TRY(dalloc(&dy2_, m_));
     PDNQP_TRY(dalloc(&x64_, n_));
     PDNQP_TRY(dalloc(&y64_, m_));
     PDNQP_TRY(dalloc(&sb64_, m_));
@@ -553,6 +554,11 @@ class Solver : public SolverBase {
     PDNQP_CK(cudaMemsetAsync(d.ptime, 0, 8 * sizeof(unsigned long long), s_));
     d.hw = 0;
     d.hc = 0;
+    int dev = 0;
+    PDNQP_CK(cudaGetDevice(&dev));
+    PDNQP_CK(cudaDeviceGetAttribute(&sms_, cudaDevAttrMultiProcessorCount, dev));
+    PDNQP_CK(cudaFuncSetAttribute(setup_fn<true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, setup_smem_bytes<T>()));
+    PDNQP_CK(cudaFuncSetAttribute(setup_fn<false>(), cudaFuncAttributeMaxDynamicSharedMemorySize, setup_smem_bytes<T>()));
     PDNQP_CK(cudaGetLastError());
     return 0;
   }
@@ -680,7 +686,7 @@ class Solver : public SolverBase {
     launch_cols();
   }
   void launch_check_group() {
-    launch_check(0);
+    launch_check();
     k_check_apply<T><<<grid_nm(), kBlock, 0, s_>>>(d_);
   }
   void launch_slot() {
@@ -752,13 +758,13 @@ class Solver : public SolverBase {
                                          trials_smem_bytes<T>() / 2, s_));
     return 0;
   }
-  void launch_check(int mode) {
-    with_G(gA_, [&](auto GG) { k_check_rows<T, decltype(GG)::value><<<nb_rows(), kBlock, 0, s_>>>(d_, mode); });
+  void launch_check() {
+    with_G(gA_, [&](auto GG) { k_check_rows<T, decltype(GG)::value><<<nb_rows(), kBlock, 0, s_>>>(d_); });
     with_G(gN_, [&](auto GG) {
       if (d_.hw)
-        k_check_cols<T, decltype(GG)::value, true><<<nb_cols(), kBlock, 0, s_>>>(d_, mode, nb_rows());
+        k_check_cols<T, decltype(GG)::value, true><<<nb_cols(), kBlock, 0, s_>>>(d_, nb_rows());
       else
-        k_check_cols<T, decltype(GG)::value, false><<<nb_cols(), kBlock, 0, s_>>>(d_, mode, nb_rows());
+        k_check_cols<T, decltype(GG)::value, false><<<nb_cols(), kBlock, 0, s_>>>(d_, nb_rows());
     });
   }
 
@@ -952,30 +958,25 @@ class Solver : public SolverBase {
   }
 
   // a0: setup of one inner solve (Algorithm 4 lines "warm start" and "inner scaling").
-  int inner_setup(const Params &prm, double dta, double dtr, long long k_in, long long pause_at, int ignore) {
-    const double ginv = 1.0 / gamma_;
-    // Base point of this solve (FP64) and zero corrections.
-    if (m_)
-      with_G(gA_, [&](auto GG) {
-        k_base_rows<T, decltype(GG)::value><<<nb_rows(), kBlock, 0, s_>>>(d_, Ad_, lcd_, ucd_, sb64_, rb64_);
-      });
-    with_G(gN_, [&](auto GG) {
-      k_base_cols<T, decltype(GG)::value><<<nb_cols(), kBlock, 0, s_>>>(d_, Hd_, Atd_, c_, z_, lxd_, uxd_, ginv);
-    });
-    k_iscale_init<T><<<grid_nm(), kBlock, 0, s_>>>(d_);
-    for (int sw = 0; sw < prm.ruiz_inner; ++sw) {
-      with_G(gN_, [&](auto GG) {
-        k_iruiz_cols<T, decltype(GG)::value><<<nb_cols(), kBlock, 0, s_>>>(d_, scn_[0]);
-      });
-      if (m_)
-        with_G(gA_, [&](auto GG) {
-          k_iruiz_rows<T, decltype(GG)::value><<<nb_rows(), kBlock, 0, s_>>>(d_, scm_[0], scm_[1], scm_[2]);
-        });
-      k_iruiz_update<T><<<grid_nm(), kBlock, 0, s_>>>(d_, scn_[0], scm_[0], scm_[1], scm_[2]);
-    }
-    with_G(gN_, [&](auto GG) { k_mw_cols<T, decltype(GG)::value><<<nb_cols(), kBlock, 0, s_>>>(d_, scn_[0]); });
-    if (m_) with_G(gA_, [&](auto GG) { k_my_rows<T, decltype(GG)::value><<<nb_rows(), kBlock, 0, s_>>>(d_, scn_[0]); });
-    k_inner_init<T><<<grid_nm(), kBlock, 0, s_>>>(d_);
+  template <bool COOP, bool LR, bool RL>
+  static auto setup_cl(bool cl) {
+    return cl ? k_setup<T, LR, RL, true, COOP> : k_setup<T, LR, RL, false, COOP>;
+  }
+  template <bool COOP>
+  void (*setup_fn() const)(Dev<T>, SetupArgs<T>, int, int) {
+    const bool rl = nnzA_ - d_.lr_nnz > 24LL * m_, cl = std::max(nnzH_, nnzA_) > 24LL * n_;
+    if (d_.nlr) return rl ? setup_cl<COOP, true, true>(cl) : setup_cl<COOP, true, false>(cl);
+    return rl ? setup_cl<COOP, false, true>(cl) : setup_cl<COOP, false, false>(cl);
+  }
+  // Blocks of the setup: a tile or two per warp (rows after columns in every
+  // phase), one block per SM at most.
+  int setup_grid() const {
+    const bool rl = nnzA_ - d_.lr_nnz > 24LL * m_, cl = std::max(nnzH_, nnzA_) > 24LL * n_;
+    const long long tiles = (m_ + (rl ? 7 : 31)) / (rl ? 8 : 32) + (n_ + (cl ? 7 : 31)) / (cl ? 8 : 32);
+    return (int)std::max(1LL, std::min<long long>(sms_, (tiles + 15) / 16));
+  }
+  int inner_setup(const Params &prm, double dta, double dtr, long long k_in, long long pause_at, int ignore,
+                  double *u = nullptr) {
     // Device state of this solve (the host holds every field it needs; the
     // iterates sit in buffer 0 between inner solves).
     DevState &S = *hst_;
@@ -1010,8 +1011,22 @@ class Solver : public SolverBase {
     S.beta_art = prm.beta_art;
     refresh_scalars(&S);
     PDNQP_CK(cudaMemcpyAsync(st_, &S, sizeof(S), cudaMemcpyHostToDevice, s_));
-    launch_check(1);  // its last block sets the restart metric of the start and the running status
-    launches_ += 9 + 3LL * prm.ruiz_inner;
+    // The phases; the last one sets the restart metric of the start and the running status.
+    SetupArgs<T> a{Hd_, Ad_, Atd_, c_, z_, lcd_, ucd_, lxd_, uxd_, sb64_, rb64_, xprev_, u, 1.0 / gamma_, prm.ruiz_inner,
+                   ex2_, dy2_, d_.Bwbar, d_.Atybar};
+    const int last = prm.ruiz_inner + 3;
+    int nb = setup_grid();
+    if (prm.persistent && coop_grid(prm.loop_blocks_per_sm) > 0) {
+      int from = 0, to = last;
+      void *args[] = {(void *)&d_, (void *)&a, (void *)&from, (void *)&to};
+      PDNQP_CK(cudaLaunchCooperativeKernel((const void *)setup_fn<true>(), dim3(nb), dim3(kTrialThreads), args,
+                                           setup_smem_bytes<T>(), s_));
+      launches_ += 1;
+    } else {
+      for (int ph = 0; ph < last; ++ph)
+        setup_fn<false>()<<<nb, kTrialThreads, setup_smem_bytes<T>(), s_>>>(d_, a, ph, ph + 1);
+      launches_ += last;
+    }
     PDNQP_CK(cudaGetLastError());
     return 0;
   }
@@ -1182,9 +1197,7 @@ class Solver : public SolverBase {
         break;
       }
       const double ts0 = now();
-      PDNQP_CK(cudaMemcpyAsync(xprev_, x64_, sizeof(double) * n_, cudaMemcpyDeviceToDevice, s_));
-      if (prm.anderson) PDNQP_TRY(aa_stage_u());
-      PDNQP_TRY(inner_setup(prm, dta, dtr, std::min(prm.k_in, left), -1, 0));
+      PDNQP_TRY(inner_setup(prm, dta, dtr, std::min(prm.k_in, left), -1, 0, prm.anderson ? aa_slot_u() : nullptr));
       if (prm.autotune && !tuned_ && (!prm.persistent || !coop_grid(prm.loop_blocks_per_sm))) {
         PDNQP_TRY(autotune_g());
         apply_g(prm);
@@ -1455,14 +1468,9 @@ class Solver : public SolverBase {
   }
   // Ring of kAaRing = 6 slots (logical pair a at (head + a) % 6, at most
   // aa_cap_ <= 5 pairs), so the slot after the last pair is always free: it
-  // receives u, the point this outer iteration starts from.
-  int aa_stage_u() {
-    const long long D = (long long)m_ + n_;
-    const int slot = (aa_head_ + aa_len_) % kAaRing;
-    double *u = aa_u_ + (size_t)slot * D;
-    if (m_) PDNQP_CK(cudaMemcpyAsync(u, lam_, sizeof(double) * m_, cudaMemcpyDeviceToDevice, s_));
-    PDNQP_CK(cudaMemcpyAsync(u + m_, z_, sizeof(double) * n_, cudaMemcpyDeviceToDevice, s_));
-    return 0;
+  // receives u, the point this outer iteration starts from (written by the setup).
+  double *aa_slot_u() {
+    return aa_u_ + (size_t)((aa_head_ + aa_len_) % kAaRing) * ((size_t)m_ + n_);
   }
   // Appends G(u) = (lambda, z) to the staged slot (dropping the oldest pair when full).
   int aa_push_g() {
@@ -1569,8 +1577,10 @@ class Solver : public SolverBase {
   double *c_ = nullptr, *lxd_ = nullptr, *uxd_ = nullptr, *lcd_ = nullptr, *ucd_ = nullptr;
   double *Dc_ = nullptr, *Dx_ = nullptr, *lam_ = nullptr, *sig_ = nullptr, *rprev_ = nullptr, *rcur_ = nullptr;
   double *z_ = nullptr, *xo_ = nullptr, *lo_ = nullptr, *dx0_ = nullptr, *dl0_ = nullptr;
+  T *ex2_ = nullptr, *dy2_ = nullptr;  // second scale buffers of the inner Ruiz sweeps
+  int sms_ = 1;
   double *x64_ = nullptr, *y64_ = nullptr, *sb64_ = nullptr, *rb64_ = nullptr, *snapbuf_ = nullptr;
-  double *scn_[1] = {nullptr}, *scm_[3] = {nullptr, nullptr, nullptr};
+  double *scn_[1] = {nullptr}, *scm_[1] = {nullptr};
   double *part_ = nullptr, *dred_ = nullptr;
   std::vector<double> hred_;
   DevState *st_ = nullptr, *hst_ = nullptr;
