@@ -511,11 +511,15 @@ static int solve_batch_fused(pdnqp_t *const *hs, int count, double eps_abs, doub
   for (int i = 0; i < count; ++i)
     if (hs[i]->device != dev) return PDNQP_ERR_STATE;
   cudaSetDevice(dev);
-  std::vector<int> keep(count), keep_tune(count);
+  // Problems that fit the cluster form (a few SMs each, no cooperative launch) run
+  // it on their own streams beside each other, at their own pace; the others
+  // share the graph.
+  std::vector<int> keep(count), keep_tune(count), own(count);
   for (int i = 0; i < count; ++i) {
     keep[i] = hs[i]->prm.persistent;
     keep_tune[i] = hs[i]->prm.autotune;
-    hs[i]->prm.persistent = 0;  // escalated FP64 solves run the graph form: no cooperative launch beside the batch
+    own[i] = keep[i] && hs[i]->solver->cluster_size() > 0;
+    if (!own[i]) hs[i]->prm.persistent = 0;  // escalated FP64 solves run the graph form: no cooperative launch beside the batch
     hs[i]->prm.autotune = 0;    // the per-handle tuner replays kernels on a running state: not beside the batch
   }
   struct Group {
@@ -523,7 +527,8 @@ static int solve_batch_fused(pdnqp_t *const *hs, int count, double eps_abs, doub
     std::unique_ptr<pdq::BatchBase> batch;
   };
   Group groups[2];  // FP64, FP32-bulk
-  for (int i = 0; i < count; ++i) groups[hs[i]->precision == PDNQP_FP32_BULK ? 1 : 0].idx.push_back(i);
+  for (int i = 0; i < count; ++i)
+    if (!own[i]) groups[hs[i]->precision == PDNQP_FP32_BULK ? 1 : 0].idx.push_back(i);
   std::string err;
   int rc = 0;
   for (int g = 0; g < 2 && rc == 0; ++g) {
@@ -561,6 +566,12 @@ static int solve_batch_fused(pdnqp_t *const *hs, int count, double eps_abs, doub
           groups[g].batch->finished(k);
         });
     }
+    for (int i = 0; i < count; ++i)
+      if (own[i])
+        workers.emplace_back([&, i] {
+          rcs[i] = pdnqp_solve(hs[i], eps_abs, eps_rel);
+          if (rcs[i] < 0) errs[i] = g_err;
+        });
     for (auto &t : workers) t.join();
     for (auto &t : schedulers) t.join();
     for (int g = 0; g < 2; ++g)

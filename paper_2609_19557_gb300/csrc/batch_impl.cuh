@@ -3,8 +3,8 @@
 // keeps its own solver, device state and host thread for the outer
 // iteration (Algorithm 3, on the CPU as in Sec. 3.4); when its inner solve
 // is set up, its thread hands it here and sleeps.  The scheduler launches one
-// captured CUDA graph of `chunk` trial slots over the whole batch, one launch
-// per phase (kernels.cuh, "Batched form"): every running problem takes its
+// captured CUDA graph of `chunk` trials and one check over the whole batch, one
+// launch per phase (kernels.cuh, "Batched form"): every running problem takes its
 // trial, its acceptance decision, its periodic check, restart and inner
 // termination on the device, and problems that are not running skip.  After
 // each graph launch one gather of all device states tells the scheduler
@@ -100,11 +100,12 @@ class BatchRunner : public BatchBase, public BatchHook {
     BTRY(dalloc(&dlist_, (size_t)2 * P));
     BK(cudaMallocHost(&hstates_, sizeof(DevState) * (size_t)P));
     BK(cudaMallocHost(&hlist_, sizeof(int) * (size_t)2 * P));
-    // The graph: chunk slots of [primal, rows, cols (+ decisions), check rows,
-    // check cols (+ check decisions), check apply] over the whole batch.
+    // The graph: chunk trials [primal, rows, cols (+ decisions)], then one check
+    // [rows, cols (+ decisions), apply] over the whole batch.
     cudaGraph_t g;
     BK(cudaStreamBeginCapture(bs_, cudaStreamCaptureModeThreadLocal));
-    for (int k = 0; k < chunk_; ++k) launch_slot();
+    for (int k = 0; k < chunk_; ++k) launch_trial();
+    launch_check();
     BK(cudaStreamEndCapture(bs_, &g));
     cudaError_t e = cudaGraphInstantiate(&gexec_, g, 0);
     cudaGraphDestroy(g);
@@ -228,13 +229,19 @@ class BatchRunner : public BatchBase, public BatchHook {
     return 0;
   }
 
-  // One trial slot over the batch (captured into the graph).
-  void launch_slot() {
+  // One trial over the batch, and one check (captured into the graph).  The check
+  // comes once a graph launch: an inner solve starts with a launch and its check
+  // period is a multiple of the default chunk, so that without rejections its
+  // checks fall due at the end of one; otherwise it waits for the end.  (Checks
+  // after every trial were 5 of 10 launches of a slot, nearly all idle.)
+  void launch_trial() {
     kb_primal<T><<<primal_.nblk, kBlock, 0, bs_>>>(devs_, primal_.map);
     for (const Launch &L : rows_)
       with_G(L.g, [&](auto GG) { kb_rows<T, decltype(GG)::value><<<L.nblk, kBlock, 0, bs_>>>(devs_, L.map); });
     for (const Launch &L : cols_)
       with_G(L.g, [&](auto GG) { kb_cols<T, decltype(GG)::value><<<L.nblk, kBlock, 0, bs_>>>(devs_, L.map, nbr_); });
+  }
+  void launch_check() {
     for (const Launch &L : rows_)
       with_G(L.g, [&](auto GG) {
         kb_check_rows<T, decltype(GG)::value><<<L.nblk, kBlock, 0, bs_>>>(devs_, L.map);
@@ -245,7 +252,10 @@ class BatchRunner : public BatchBase, public BatchHook {
       });
     kb_check_apply<T><<<apply_.nblk, kBlock, 0, bs_>>>(devs_, apply_.map);
   }
-  long long kernels_per_slot() const { return 2 + 2 * (long long)(rows_.size() + cols_.size()); }
+  long long kernels_per_launch() const {
+    const long long g = (long long)(rows_.size() + cols_.size());
+    return chunk_ * (1 + g) + g + 1;
+  }
 
   // Scheduler edits, one graph launch, one read-back of all states.
   int step(const std::vector<int> &go, const std::vector<int> &stop) {
@@ -262,7 +272,7 @@ class BatchRunner : public BatchBase, public BatchHook {
     BK(cudaGraphLaunch(gexec_, bs_));
     BK(cudaEventRecord(ev_[1], bs_));
     ++graph_launches_;
-    kernel_launches_ += chunk_ * kernels_per_slot();
+    kernel_launches_ += kernels_per_launch();
     kb_gather_states<T><<<(P * (int)(sizeof(DevState) / 4) + 255) / 256, 256, 0, bs_>>>(devs_, P, dstates_);
     ++kernel_launches_;
     BK(cudaGetLastError());

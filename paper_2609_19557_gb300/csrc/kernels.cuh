@@ -477,7 +477,7 @@ __device__ __forceinline__ void rows_phase(const Dev<T> &d, const DevState *st, 
 // Row pass of one trial over the blocks of g (graph and batched forms).
 template <typename T, int G>
 __device__ __forceinline__ void rows_trial_body(const Dev<T> &d, GridCtx g) {
-  if (d.st->status != ST_RUNNING) return;
+  if (d.st->status != ST_RUNNING || d.st->check_due) return;
   if (d.nlr) long_rows_partial<T>(d, d.x[d.st->xtr], g);
   rows_phase<T, G>(d, d.st, g);
   if (d.nlr && arrive_last(d.ctr + 2, g.nb)) {
@@ -533,7 +533,7 @@ __device__ __forceinline__ void cols_phase(const Dev<T> &d, const DevState *st, 
 // in the problem's last block (graph and batched forms).
 template <typename T, int G, bool COND>
 __device__ __forceinline__ void cols_trial_body(const Dev<T> &d, int nb_r, GridCtx g) {
-  if (d.st->status != ST_RUNNING) {
+  if (d.st->status != ST_RUNNING || d.st->check_due) {
     stop_loop<COND>(d.hw, d.hc);
     return;
   }
@@ -784,12 +784,24 @@ __device__ __forceinline__ void cols_phase_tiles(const Dev<T> &d, const DevState
   }
 }
 
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+// The barrier alone.
+template <bool CLU>
+__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen);
+
 // Grid barrier of the loop with a message: bar as in grid_sync, but the
 // generation word carries, in its low bit, what the last block's lead()
 // returned; every block gets it (-1: a wait ran out).  The arrivals are reset
 // before lead() runs, and `gen` is the caller's copy of the generation (thread
 // 0), so a waiting block polls one word and nothing else.
-template <typename F>
+//
+// CLU: the grid is one thread-block cluster (small problems), whose hardware
+// barrier orders the blocks' memory accesses like a block barrier (about 0.3 us
+// where the grid barrier takes 1.5 to 2.5); block 0 runs lead(), and no message
+// comes back.
+template <bool CLU, typename F>
 __device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, F lead) {
   __shared__ int role;  // message, -1 fault, 2 leader
   __syncthreads();
@@ -797,6 +809,12 @@ __device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, F lead) {
     const int msg = lead();
     __syncthreads();
     return msg;
+  }
+  if (CLU) {
+    cluster_sync();
+    if (blockIdx.x == 0) lead();
+    cluster_sync();
+    return 0;
   }
   if (threadIdx.x == 0) {
     __threadfence();
@@ -830,6 +848,15 @@ __device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, F lead) {
     st_release_gpu(bar + kBarGen, gen);
   }
   return msg;
+}
+
+template <bool CLU>
+__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen) {
+  if (CLU && gridDim.x > 1) {
+    cluster_sync();
+    return 0;
+  }
+  return loop_sync<CLU>(bar, gen, [] { return 0; });
 }
 
 // This block's four sums to part[0..3] (fixed order): per warp the quantities
@@ -879,7 +906,8 @@ __device__ __forceinline__ void advance_trial(DevState *S, const double *next) {
   advance_scalars(S, next[0], next[1]);
 }
 template <typename T>
-__device__ __forceinline__ int decide_tiles(const Dev<T> &d, DevState &S, int nb, bool lr, const double *next) {
+__device__ __forceinline__ int decide_tiles(const Dev<T> &d, DevState &S, int nb, bool lr, const double *next,
+                                            bool store = true) {
   __shared__ double red[4][4];
   __shared__ int go;
   const double *part = d.part + P_TRP * kMaxBlocks;
@@ -915,7 +943,7 @@ __device__ __forceinline__ int decide_tiles(const Dev<T> &d, DevState &S, int nb
     go = accepted && S.status == ST_RUNNING && S.slot_left > 0 && !S.check_due;
   }
   __syncthreads();
-  if (!go) state_store(d.st, S);
+  if (!go && store) state_store(d.st, S);
   return go;
 }
 
@@ -1378,7 +1406,7 @@ __global__ void __launch_bounds__(kBlock) k_check_apply(Dev<T> d) {
 // branches (the state is block-uniform), so every barrier is reached by every
 // block.  LR: the instance has dense coupling rows (d.nlr > 0); RL / CL:
 // long rows of A / of H and A' (tiles of 8).
-template <typename T, bool LR, bool RL, bool CL>
+template <typename T, bool LR, bool RL, bool CL, bool CLU>
 __global__ void __launch_bounds__(kTrialThreads, 1) k_trials(Dev<T> d, long long chunk) {
   __shared__ DevState S;
   __shared__ double next[2];
@@ -1408,7 +1436,7 @@ __global__ void __launch_bounds__(kTrialThreads, 1) k_trials(Dev<T> d, long long
     if (!S.spec) {
       primal_phase<T>(d, &S);
       lap(0);
-      if (loop_sync(bar, gen, [] { return 0; }) < 0) return;
+      if (loop_sync<CLU>(bar, gen) < 0) return;
       lap(1);
     }
     if (threadIdx.x >= kTrialThreads - 2) {  // a spare lane each, before the last warp's first item
@@ -1421,21 +1449,31 @@ __global__ void __launch_bounds__(kTrialThreads, 1) k_trials(Dev<T> d, long long
     TrialSums<T> ts = {T(0), T(0), T(0), T(0)};
     rows_phase_tiles<T, LR, RL>(d, &S, buf, ts);
     lap(2);
-    if (loop_sync(bar, gen, [&] {
-          if (LR) long_rows_finish<T>(d, &S, d.lr_nb);
-          return 0;
-        }) < 0)
+    if (LR) {
+      if (loop_sync<CLU>(bar, gen, [&] {
+            long_rows_finish<T>(d, &S, d.lr_nb);
+            return 0;
+          }) < 0)
+        return;
+    } else if (loop_sync<CLU>(bar, gen) < 0) {
       return;
+    }
     lap(3);
     cols_phase_tiles<T, CL>(d, &S, buf, ts);
     lap(4);
     double v[4] = {widen(ts.Lt), widen(ts.Le), widen(ts.RH), widen(ts.RB)};
     block_sums(v, part);
-    bool led = false;
-    const int go = loop_sync(bar, gen, [&] {
-      led = true;
-      return decide_tiles<T>(d, S, nb, LR, next);
-    });
+    bool led = CLU;
+    int go;
+    if (CLU) {  // every block of a cluster decides for itself, on the same sums
+      loop_sync<CLU>(bar, gen);
+      go = decide_tiles<T>(d, S, nb, LR, next, blockIdx.x == 0);
+    } else {
+      go = loop_sync<CLU>(bar, gen, [&] {
+        led = true;
+        return decide_tiles<T>(d, S, nb, LR, next);
+      });
+    }
     if (go < 0) return;
     if (!led) {
       if (go) {
@@ -1454,7 +1492,7 @@ __global__ void __launch_bounds__(kTrialThreads, 1) k_trials(Dev<T> d, long long
 // Periodic check of the persistent form, with its restart, in one cooperative
 // launch on the loop's grid: the two passes, the decision in the last block of
 // the second barrier, and the restart.  Does nothing when no check is pending.
-template <typename T, bool RL, bool CL>
+template <typename T, bool RL, bool CL, bool CLU>
 __global__ void __launch_bounds__(kTrialThreads, 1) k_check(Dev<T> d) {
   __shared__ DevState S;
   extern __shared__ __align__(16) unsigned char slots[];
@@ -1466,10 +1504,10 @@ __global__ void __launch_bounds__(kTrialThreads, 1) k_check(Dev<T> d) {
   const int nb = gridDim.x;
   const GridCtx g{(int)blockIdx.x, nb};
   check_rows_body<T, RL ? 16 : 8>(d, &S, g, buf);
-  if (loop_sync(bar, gen, [] { return 0; }) < 0) return;
+  if (loop_sync<CLU>(bar, gen) < 0) return;
   check_cols_terms<T, CL ? 16 : 8>(d, &S, g, buf);
   bool led = false;
-  if (loop_sync(bar, gen, [&] {
+  if (loop_sync<CLU>(bar, gen, [&] {
         led = true;
         double q[16];
         check_sums(d.part, nb, nb, q);
@@ -1526,7 +1564,8 @@ __global__ void k_totals(Dev<T> d, double *out) {
 // runs alone, so its reductions and its iterates are bitwise those of its
 // solo graph-form solve); the problem's device pointers come from devs[p].
 // Every phase skips a problem whose status is not ST_RUNNING, so problems
-// that wait for their host outer iteration cost one state read per block.
+// that wait for their host outer iteration cost one state read per block; the
+// trial phases also skip one whose periodic check is due.
 // ===========================================================================
 struct BatchBlk {
   int p, b, nb;
@@ -1548,7 +1587,7 @@ template <typename T>
 __global__ void __launch_bounds__(kBlock) kb_primal(const Dev<T> *devs, const BatchBlk *map) {
   const BatchBlk e = map[blockIdx.x];
   const Dev<T> &d = batch_dev(devs, e.p);
-  if (d.st->status != ST_RUNNING) return;
+  if (d.st->status != ST_RUNNING || d.st->check_due) return;
   primal_phase<T>(d, d.st, GridCtx{e.b, e.nb});
 }
 

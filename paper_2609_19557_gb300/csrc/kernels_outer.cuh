@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos(Mat<double> Q, int st
   const WarpItems it;
   constexpr int TR = TileIter<K>::TR;
   const long long tiles = (n + TR - 1) / TR;
-  auto sync = [&] { return loop_sync(bar, gen, [] { return 0; }) >= 0; };
+  auto sync = [&] { return loop_sync<false>(bar, gen) >= 0; };
   // One sum per start: block partials to part, then after a barrier totals in tot[s][0].
   auto put2 = [&](double a, double b, double *dst) {
     double v[2] = {a, b};
@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(kBlock) k_outer_rows(Dev<T> d, Mat<double> Ad,
   for (int k = 0; k < kOutRows; ++k) q[k] = 0.0;
   TileIter<G> ti;
   for (long long tile = ti.first; tile < d.m; tile += ti.step) {
-    const double ax = update ? tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double, 2>{x})
+    const double ax = update ? tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double, sizeof(T) == 8 ? 2 : 0>{x})
                              : tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double>{x});
     const double ad =
         update ? tile_row_sum<G, double>(Ad.rp, Ad.ci, Ad.val, tile, d.m, MulLdg<double>{dx}) : 0.0;

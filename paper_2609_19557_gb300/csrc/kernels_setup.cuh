@@ -206,6 +206,11 @@ __device__ __forceinline__ void base_row(const Dev<T> &d, const SetupArgs<T> &a,
   a.qa[j] = T(sig);
 }
 
+// Order of dense rows (one_row): the FP64 form's; the bulk form's multipliers hold
+// FP32 corrections, which do not see it.
+template <typename T>
+constexpr int kBaseOrder = sizeof(T) == 8 ? 1 : 0;
+
 // Base columns: H x_b and A' y_b in FP64, q'_x = c - z / gamma + H x_b - A' y_b,
 // q_x, the shifted bounds, zero corrections with zero cached products.
 template <typename T, bool LR, bool RL, bool CL>
@@ -239,7 +244,7 @@ __device__ __forceinline__ void setup_base(const Dev<T> &d, const SetupArgs<T> &
     for (int s = w; s < d.nlr; s += (blockDim.x >> 5) * g.nb) {
       const int j = d.lr_row[s];
       const double v = one_row<false, double>(a.Ad.ci, a.Ad.val, __ldg(a.Ad.rp + j), __ldg(a.Ad.rp + j + 1),
-                                              MulLdg<double, 1>{d.xb}, buf);
+                                              MulLdg<double, kBaseOrder<T>>{d.xb}, buf);
       if ((threadIdx.x & 31) == 0) base_row<T>(d, a, j, v);
     }
   }
@@ -248,7 +253,7 @@ __device__ __forceinline__ void setup_base(const Dev<T> &d, const SetupArgs<T> &
                    [&](long long j, bool valid, const int(&rb)[1], const int(&re)[1], bool one) {
                      double v;
                      if (RL || one) {  // rows above kDenseRow that the split left out keep the order too
-                       const MulLdg<double, 1> fo{d.xb};
+                       const MulLdg<double, kBaseOrder<T>> fo{d.xb};
                        v = RL ? tile_long_rows<false, double>(a.Ad.ci, a.Ad.val, rb[0], re[0], fo, buf)
                               : one_row<false, double>(a.Ad.ci, a.Ad.val, __shfl_sync(0xffffffffu, rb[0], 0),
                                                        __shfl_sync(0xffffffffu, re[0], 0), fo, buf);
@@ -416,13 +421,17 @@ constexpr unsigned setup_smem_bytes() {  // FP64 base products in both forms
   return kTrialThreads / 32 * kTileSlots * (unsigned)sizeof(Slot<double>);
 }
 
+// Forms of the launch: a kernel per phase, a cooperative grid, one cluster.
+enum : int { kByPhase = 0, kGrid = 1, kCluster = 2 };
+
 // Phases [from, to): 0 base, 1 .. sweeps the Ruiz sweeps, then m_w, then m_y (and
-// the end).  In one cooperative launch the grid barrier separates them; a launch
-// of a single phase (COOP = false) takes its last block for what the barrier's
+// the end).  In one launch the grid's (cluster's) barrier separates them; a launch
+// of a single phase (kByPhase) takes its last block for what the barrier's
 // leader does.  What bounds it: at small sizes the barriers (12 phases, about 3 us
 // each, where 33 launches took 0.25 ms), at n = 1e6 the gathers of the sweeps.
-template <typename T, bool LR, bool RL, bool CL, bool COOP>
+template <typename T, bool LR, bool RL, bool CL, int FORM>
 __global__ void __launch_bounds__(kTrialThreads, 1) k_setup(Dev<T> d, SetupArgs<T> a, int from, int to) {
+  constexpr bool COOP = FORM != kByPhase;
   extern __shared__ __align__(16) unsigned char slots[];
   Slot<double> *buf64 = reinterpret_cast<Slot<double> *>(slots) + (threadIdx.x >> 5) * kTileSlots;
   Slot<T> *buf = reinterpret_cast<Slot<T> *>(buf64);
@@ -456,7 +465,9 @@ __global__ void __launch_bounds__(kTrialThreads, 1) k_setup(Dev<T> d, SetupArgs<
       return 0;
     };
     if (COOP) {
-      if (loop_sync(bar, gen, lead) < 0) return;
+      if (((LR && ph >= 1 && ph <= S) || ph == S + 2 ? loop_sync<FORM == kCluster>(bar, gen, lead)
+                                                     : loop_sync<FORM == kCluster>(bar, gen)) < 0)
+        return;
     } else if ((LR && ph >= 1 && ph <= S) || ph == S + 2) {
       if (arrive_last(d.ctr + 1)) {
         lead();

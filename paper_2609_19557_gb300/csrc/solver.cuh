@@ -92,6 +92,7 @@ class SolverBase {
   virtual int debug_inner(Params &prm, int nck, const int64_t *ck, double *snap, std::string *err) = 0;
   virtual int replay(int which, int reps) = 0;
   virtual int tuned_g(int which) const = 0;
+  virtual int cluster_size() const = 0;  // blocks of the cluster form, 0: too large for it
   virtual double kernel_bytes(int which) const = 0;
   virtual double last_replay_ms() const = 0;
   virtual double gamma() const = 0;

@@ -557,8 +557,16 @@ class Solver : public SolverBase {
     int dev = 0;
     PDNQP_CK(cudaGetDevice(&dev));
     PDNQP_CK(cudaDeviceGetAttribute(&sms_, cudaDevAttrMultiProcessorCount, dev));
-    PDNQP_CK(cudaFuncSetAttribute(setup_fn<true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, setup_smem_bytes<T>()));
-    PDNQP_CK(cudaFuncSetAttribute(setup_fn<false>(), cudaFuncAttributeMaxDynamicSharedMemorySize, setup_smem_bytes<T>()));
+    auto smem = [](auto fn, unsigned bytes) {
+      return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    PDNQP_CK(smem(setup_fn<kGrid>(), setup_smem_bytes<T>()));
+    PDNQP_CK(smem(setup_fn<kByPhase>(), setup_smem_bytes<T>()));
+    if (cluster_size()) {
+      PDNQP_CK(smem(setup_clu_fn(), setup_smem_bytes<T>()));
+      PDNQP_CK(smem(trials_clu_fn(), trials_smem_bytes<T>()));
+      PDNQP_CK(smem(check_clu_fn(), trials_smem_bytes<T>() / 2));
+    }
     PDNQP_CK(cudaGetLastError());
     return 0;
   }
@@ -660,7 +668,13 @@ class Solver : public SolverBase {
 
   // ------------------------------------------------------- launchers
   // Tile kernels: a tile per warp and trip, kBlock / 32 warps per block.
-  int nb_rows(int g) const { return grid_for(std::max(m_, 1), tile_rows_per_block(g)); }
+  // Row kernels of an instance with dense rows: a block per 512 of their entries
+  // too (the split of long_rows_partial; with the blocks of the rows alone, one
+  // block walked through the simplex row of 20,404 entries, 56 of the 80 us of a
+  // batched trial).
+  int nb_rows(int g) const {
+    return std::max(grid_for(std::max(m_, 1), tile_rows_per_block(g)), std::min(152, (d_.lr_nnz + 511) / 512));
+  }
   int nb_cols(int g) const { return grid_for(n_, tile_rows_per_block(g)); }
   int nb_rows() const { return nb_rows(gA_); }
   int nb_cols() const { return nb_cols(gN_); }
@@ -697,17 +711,56 @@ class Solver : public SolverBase {
   // and rows or columns in tiles of 8 where their mean length is above 24
   // entries (there a warp's lanes are better spent along a row: at 100 entries
   // a row, 8 rows a warp keep 8 x 32 entries in flight as 32 short rows do).
+  bool long_tiles_r() const { return nnzA_ - d_.lr_nnz > 24LL * m_; }
+  bool long_tiles_c() const { return std::max(nnzH_, nnzA_) > 24LL * n_; }
+  template <bool CLU, bool LR, bool RL>
+  static auto trials_cl(bool cl) {
+    return cl ? k_trials<T, LR, RL, true, CLU> : k_trials<T, LR, RL, false, CLU>;
+  }
   void (*trials_fn() const)(Dev<T>, long long) {
-    const bool lr = d_.nlr > 0, rl = nnzA_ - d_.lr_nnz > 24LL * m_, cl = std::max(nnzH_, nnzA_) > 24LL * n_;
-    if (lr) return rl ? (cl ? k_trials<T, true, true, true> : k_trials<T, true, true, false>)
-                      : (cl ? k_trials<T, true, false, true> : k_trials<T, true, false, false>);
-    return rl ? (cl ? k_trials<T, false, true, true> : k_trials<T, false, true, false>)
-              : (cl ? k_trials<T, false, false, true> : k_trials<T, false, false, false>);
+    const bool lr = d_.nlr > 0, rl = long_tiles_r(), cl = long_tiles_c();
+    if (lr) return rl ? trials_cl<false, true, true>(cl) : trials_cl<false, true, false>(cl);
+    return rl ? trials_cl<false, false, true>(cl) : trials_cl<false, false, false>(cl);
   }
   void (*check_fn() const)(Dev<T>) {
-    const bool rl = nnzA_ > 24LL * m_, cl = std::max(nnzH_, nnzA_) > 24LL * n_;
-    return rl ? (cl ? k_check<T, true, true> : k_check<T, true, false>)
-              : (cl ? k_check<T, false, true> : k_check<T, false, false>);
+    const bool rl = nnzA_ > 24LL * m_, cl = long_tiles_c();
+    return rl ? (cl ? k_check<T, true, true, false> : k_check<T, true, false, false>)
+              : (cl ? k_check<T, false, true, false> : k_check<T, false, false, false>);
+  }
+  // The cluster form (no tiles of 8 rows: rows of A that long are items of their own).
+  void (*trials_clu_fn() const)(Dev<T>, long long) {
+    return d_.nlr > 0 ? trials_cl<true, true, false>(long_tiles_c()) : trials_cl<true, false, false>(long_tiles_c());
+  }
+  void (*check_clu_fn() const)(Dev<T>) {
+    return long_tiles_c() ? k_check<T, false, true, true> : k_check<T, false, false, true>;
+  }
+  // Blocks of the cluster form (0: the problem is too large for it).  Up to 8
+  // blocks, a warp with a tile or a few; the limits are where a pass by 8 SMs
+  // costs what the grid form saves on its barriers: 4 tiles a warp (n = 16,000
+  // in tiles of 32), and 120,000 gathers a trial (8 us at one a cycle and SM).
+  int cluster_size() const override {
+    const long long tc = long_tiles_c() ? 8 : 32;
+    const long long tiles = std::max<long long>((m_ + 31) / 32 + d_.nlong_r, (n_ + tc - 1) / tc + (tc == 32 ? d_.nlong_c : 0));
+    if (tiles > 512 || nnzH_ + 2 * nnzA_ > 120000) return 0;
+    // One block as long as each of its 16 warps has a tile at most (at n = 200 a
+    // cluster of 4 takes 10.1 us a trial, a block 9.9).
+    return tiles <= 16 ? 1 : 8;
+  }
+  template <typename... P, typename... A>
+  int launch_cluster(void (*fn)(P...), int nb, unsigned smem, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nb);
+    cfg.blockDim = dim3(kTrialThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s_;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = nb;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    PDNQP_CK(cudaLaunchKernelEx(&cfg, fn, args...));
+    return 0;
   }
   // Blocks of the persistent loop (one per SM at most): a warp has a tile at a
   // time, so the grid is the tiles over 8 warps a block up to one block per SM
@@ -735,7 +788,7 @@ class Solver : public SolverBase {
     }
     if (bps > 0) per_sm = std::min(per_sm, bps);
     constexpr int W = kTrialThreads / 32;
-    const long long tr = nnzA_ - d_.lr_nnz > 24LL * m_ ? 8 : 32, tc = std::max(nnzH_, nnzA_) > 24LL * n_ ? 8 : 32;
+    const long long tr = long_tiles_r() ? 8 : 32, tc = long_tiles_c() ? 8 : 32;
     const long long tiles = std::max((m_ + tr - 1) / tr + (tr == 32 ? d_.nlong_r : 0),
                                      (n_ + tc - 1) / tc + (tc == 32 ? d_.nlong_c : 0));
     const long long work = tiles <= 3 * W && d_.nlr == 0 ? 1 : (tiles + 7) / 8;
@@ -744,12 +797,17 @@ class Solver : public SolverBase {
   }
   // One slot: the trial loop up to the next check (timed by events of its own),
   // then the check.
-  int launch_loop_slot(int nb, int slot, long long chunk) {
+  int launch_loop_slot(int nb, bool clu, int slot, long long chunk) {
     if (!loop_ev_[2 * slot]) {
       PDNQP_CK(cudaEventCreate(&loop_ev_[2 * slot]));
       PDNQP_CK(cudaEventCreate(&loop_ev_[2 * slot + 1]));
     }
     PDNQP_CK(cudaEventRecord(loop_ev_[2 * slot], s_));
+    if (clu) {
+      PDNQP_TRY(launch_cluster(trials_clu_fn(), nb, trials_smem_bytes<T>(), d_, chunk));
+      PDNQP_CK(cudaEventRecord(loop_ev_[2 * slot + 1], s_));
+      return launch_cluster(check_clu_fn(), nb, trials_smem_bytes<T>() / 2, d_);
+    }
     void *args[] = {(void *)&d_, (void *)&chunk};
     PDNQP_CK(cudaLaunchCooperativeKernel((const void *)trials_fn(), dim3(nb), dim3(kTrialThreads), args,
                                          trials_smem_bytes<T>(), s_));
@@ -958,20 +1016,23 @@ class Solver : public SolverBase {
   }
 
   // a0: setup of one inner solve (Algorithm 4 lines "warm start" and "inner scaling").
-  template <bool COOP, bool LR, bool RL>
+  template <int FORM, bool LR, bool RL>
   static auto setup_cl(bool cl) {
-    return cl ? k_setup<T, LR, RL, true, COOP> : k_setup<T, LR, RL, false, COOP>;
+    return cl ? k_setup<T, LR, RL, true, FORM> : k_setup<T, LR, RL, false, FORM>;
   }
-  template <bool COOP>
+  template <int FORM>
   void (*setup_fn() const)(Dev<T>, SetupArgs<T>, int, int) {
-    const bool rl = nnzA_ - d_.lr_nnz > 24LL * m_, cl = std::max(nnzH_, nnzA_) > 24LL * n_;
-    if (d_.nlr) return rl ? setup_cl<COOP, true, true>(cl) : setup_cl<COOP, true, false>(cl);
-    return rl ? setup_cl<COOP, false, true>(cl) : setup_cl<COOP, false, false>(cl);
+    const bool rl = long_tiles_r(), cl = long_tiles_c();
+    if (d_.nlr) return rl ? setup_cl<FORM, true, true>(cl) : setup_cl<FORM, true, false>(cl);
+    return rl ? setup_cl<FORM, false, true>(cl) : setup_cl<FORM, false, false>(cl);
+  }
+  void (*setup_clu_fn() const)(Dev<T>, SetupArgs<T>, int, int) {
+    return d_.nlr ? setup_cl<kCluster, true, false>(long_tiles_c()) : setup_cl<kCluster, false, false>(long_tiles_c());
   }
   // Blocks of the setup: a tile or two per warp (rows after columns in every
   // phase), one block per SM at most.
   int setup_grid() const {
-    const bool rl = nnzA_ - d_.lr_nnz > 24LL * m_, cl = std::max(nnzH_, nnzA_) > 24LL * n_;
+    const bool rl = long_tiles_r(), cl = long_tiles_c();
     const long long tiles = (m_ + (rl ? 7 : 31)) / (rl ? 8 : 32) + (n_ + (cl ? 7 : 31)) / (cl ? 8 : 32);
     return (int)std::max(1LL, std::min<long long>(sms_, (tiles + 15) / 16));
   }
@@ -1015,16 +1076,19 @@ class Solver : public SolverBase {
     SetupArgs<T> a{Hd_, Ad_, Atd_, c_, z_, lcd_, ucd_, lxd_, uxd_, sb64_, rb64_, xprev_, u, 1.0 / gamma_, prm.ruiz_inner,
                    ex2_, dy2_, d_.Bwbar, d_.Atybar};
     const int last = prm.ruiz_inner + 3;
-    int nb = setup_grid();
-    if (prm.persistent && coop_grid(prm.loop_blocks_per_sm) > 0) {
+    const int nb = setup_grid(), clu = prm.persistent ? cluster_size() : 0;
+    if (clu) {
+      PDNQP_TRY(launch_cluster(setup_clu_fn(), clu, setup_smem_bytes<T>(), d_, a, 0, last));
+      launches_ += 1;
+    } else if (prm.persistent && coop_grid(prm.loop_blocks_per_sm) > 0) {
       int from = 0, to = last;
       void *args[] = {(void *)&d_, (void *)&a, (void *)&from, (void *)&to};
-      PDNQP_CK(cudaLaunchCooperativeKernel((const void *)setup_fn<true>(), dim3(nb), dim3(kTrialThreads), args,
+      PDNQP_CK(cudaLaunchCooperativeKernel((const void *)setup_fn<kGrid>(), dim3(nb), dim3(kTrialThreads), args,
                                            setup_smem_bytes<T>(), s_));
       launches_ += 1;
     } else {
       for (int ph = 0; ph < last; ++ph)
-        setup_fn<false>()<<<nb, kTrialThreads, setup_smem_bytes<T>(), s_>>>(d_, a, ph, ph + 1);
+        setup_fn<kByPhase>()<<<nb, kTrialThreads, setup_smem_bytes<T>(), s_>>>(d_, a, ph, ph + 1);
       launches_ += last;
     }
     PDNQP_CK(cudaGetLastError());
@@ -1059,7 +1123,9 @@ class Solver : public SolverBase {
       *hst_ = *S;
       return r;
     }
-    const int nbp = prm.persistent ? coop_grid(prm.loop_blocks_per_sm) : 0;
+    const int clu = prm.persistent ? cluster_size() : 0;
+    const int nbp = clu ? clu : prm.persistent ? coop_grid(prm.loop_blocks_per_sm) : 0;
+    loop_nb_ = nbp;
     if (nbp > 0) {
       // Persistent loop: batches of slots [trial loop, check] of at most `per`
       // trials, after which the host reads the state once.  Most inner solves
@@ -1068,7 +1134,7 @@ class Solver : public SolverBase {
       // further one twice as many.
       const long long per = std::max<long long>(prm.chunk, 8 * std::max<long long>(1, prm.k_chk));
       for (int R = 2;; R = std::min(2 * R, kMaxLoopSlots)) {
-        for (int r = 0; r < R; ++r) PDNQP_TRY(launch_loop_slot(nbp, r, r == 0 ? per : -1));
+        for (int r = 0; r < R; ++r) PDNQP_TRY(launch_loop_slot(nbp, clu > 0, r, r == 0 ? per : -1));
         launches_ += 2LL * R;
         loop_launches_ += R;
         const long long tr_before = hst_->trials;
@@ -1400,7 +1466,7 @@ class Solver : public SolverBase {
     res_.setup_seconds = t_setup;
     res_.loop_seconds = loop_seconds_;
     res_.loop_trials = loop_trials_;
-    res_.loop_blocks = coop_nb_;
+    res_.loop_blocks = loop_nb_;
     res_.loop_launches = loop_launches_;
     res_.ctrl_used = ctrl_used_;
     res_.ctrl_fallbacks = ctrl_fallbacks_;
@@ -1592,7 +1658,7 @@ class Solver : public SolverBase {
   double loop_seconds_ = 0.0;  // device time of the persistent trial-loop launches
   long long loop_launches_ = 0;
   long long loop_trials_ = 0;  // trials they ran
-  int coop_key_ = -1, coop_nb_ = 0;
+  int coop_key_ = -1, coop_nb_ = 0, loop_nb_ = 0;
   unsigned *hfault_ = nullptr;
   // learned controller
   double *xprev_ = nullptr, *lamprev_ = nullptr, *dxv_ = nullptr;  // infeasibility tests
