@@ -507,7 +507,7 @@ struct __align__(2 * sizeof(Acc)) Slot {
   Acc a, x;
 };
 constexpr int kSlotLd = 9;                     // slots of a row in a round's buffer (8 and one of padding)
-constexpr int kTileSlots = 32 * kSlotLd;       // slots of one warp and matrix
+constexpr int kTileSlots = 32 * kSlotLd;       // slots of one warp
 constexpr int kLongRowEntries = 32;            // longer rows are summed by the whole warp
 constexpr int kDenseRow = 1024;                // see one_row
 constexpr int kRowAlone = 512;                 // rows this long get a warp's 256 entries a round (tile_long_rows gives a row 32)
@@ -618,9 +618,10 @@ __device__ __forceinline__ Acc one_row(const int *__restrict__ ci, const T *__re
 // joined by halving (3 additions and 4 shuffles for the 32 rows): arithmetic is
 // cheap, and the buffer would cost 16 shared-memory accesses a round.
 // Rows of more than kLongRowEntries entries are left out of the rounds and
-// summed by warp_row, so that one of them does not hold up its tile.  buf: NM
-// x kTileSlots slots of this warp (FP32: unused).  LongRows = false: the caller
-// has taken the long rows out.
+// summed by warp_row, so that one of them does not hold up its tile.  buf:
+// kTileSlots slots of this warp (FP32: unused).  LongRows = false: the caller
+// has taken the long rows out.  The matrices take turns in the slots: a set for
+// each would take 147 KB of a block of 16 warps' L1, one set 74 KB.
 template <int NM, bool IsMax, typename Acc, bool LongRows = true, typename T, typename F>
 __device__ __forceinline__ void tile_rows(const int *const (&ci)[NM], const T *const (&val)[NM], const int (&rb)[NM],
                                           const int (&re)[NM], const F (&f)[NM], Slot<Acc> *buf, Acc (&out)[NM]) {
@@ -675,20 +676,18 @@ __device__ __forceinline__ void tile_rows(const int *const (&ci)[NM], const T *c
             if (c[m][t][u] >= 0) f[m].add(part[m][t], Acc(a[m][t][u]), x[m][t][u]);
       continue;
     }
-    __syncwarp();  // the last round's slots have been read
 #pragma unroll
-    for (int m = 0; m < NM; ++m)
+    for (int m = 0; m < NM; ++m) {
+      __syncwarp();  // the slots written last have been read
 #pragma unroll
       for (int t = 0; t < 4; ++t)
 #pragma unroll
         for (int u = 0; u < 2; ++u)
           if (c[m][t][u] >= 0)
-            buf[m * kTileSlots + (t * 8 + sub) * kSlotLd + 4 * u + lg] = Slot<Acc>{Acc(a[m][t][u]), x[m][t][u]};
-    __syncwarp();
-#pragma unroll
-    for (int m = 0; m < NM; ++m) {
+            buf[(t * 8 + sub) * kSlotLd + 4 * u + lg] = Slot<Acc>{Acc(a[m][t][u]), x[m][t][u]};
+      __syncwarp();
       const int n = se[m] - rb[m] - s;
-      const Slot<Acc> *row = buf + m * kTileSlots + lane * kSlotLd;
+      const Slot<Acc> *row = buf + lane * kSlotLd;
 #pragma unroll
       for (int j = 0; j < 8; ++j)
         if (j < longest - s) {  // the same for the whole warp

@@ -561,10 +561,10 @@ __global__ void __launch_bounds__(kBlock) k_cols(Dev<T> d, int nb_r) {
 // measured with 16 to 64 warps); one block per SM makes the grid barrier and
 // the final reduction of the acceptance sums cheap.
 constexpr int kTrialThreads = 512;
-// Slots of tile_rows (FP64: two matrices a warp).
+// Slots of tile_rows (FP64).
 template <typename T>
 constexpr unsigned trials_smem_bytes() {
-  return sizeof(T) == 4 ? 0u : kTrialThreads / 32 * 2 * kTileSlots * (unsigned)sizeof(Slot<T>);
+  return sizeof(T) == 4 ? 0u : kTrialThreads / 32 * kTileSlots * (unsigned)sizeof(Slot<T>);
 }
 
 // The work items of this warp: item w gridDim + b first, so that the last,
@@ -687,16 +687,16 @@ __device__ __forceinline__ void rows_phase_tiles(const Dev<T> &d, const DevState
       const T yt = y + (k0[kSce] * eta) * (hp - bwt - k0[kBeta] * (bwt - bw));
       d.Bw[nx][j] = bwt;
       d.y[nx][j] = yt;
-      const T dr = rt - r, dyv = yt - y;
-      ts.Lt += dr * dr * itr;
+      const T dr = rt - r, dyv = yt - y, dr2 = dr * dr;
+      ts.Lt += dr2 * itr;
       ts.Le += dyv * dyv * ie;
-      ts.RH += fabs(dr * sig * dr);
-      ts.RB += fabs(ds * dyv) + fabs(dr * dyv);
+      ts.RH += dr2 * sig;
+      ts.RB += fabs(dyv) * (fabs(ds) + fabs(dr));
     }
   }
 }
 
-// Column pass: H x_tr and A' y_tr (both matrices of a tile together), the
+// Column pass: H x_tr and A' y_tr, the
 // per-variable terms of the acceptance sums, and, as if the trial were
 // accepted, the averages of x and H x and the primal step of the next trial
 // (primal_phase with t advanced by one) into the other average buffers and the
@@ -764,15 +764,24 @@ __device__ __forceinline__ void cols_phase_tiles(const Dev<T> &d, const DevState
       sum[0] = warp_row<false, T>(ci[0], val[0], rb[0], re[0], f[0]);
       sum[1] = warp_row<false, T>(ci[1], val[1], rb[1], re[1], f[1]);
     } else {
-      tile_rows<2, false, T, false>(ci, val, rb, re, f, buf, sum);
+      // FP32 gathers for both matrices together.  FP64, bound by its arithmetic,
+      // takes them in turn: together 180 bytes of registers spill, and a call at
+      // n = 200 takes 6.6 ms instead of 6.2, at n = 50,000 19.3 instead of 18.3, while
+      // n = 1,000,000 gains 3 % (53.4 instead of 55.1).
+      if (sizeof(T) == 4) {
+        tile_rows<2, false, T, false>(ci, val, rb, re, f, buf, sum);
+      } else {
+        sum[0] = tile_rows1<false, T, false>(ci[0], val[0], rb[0], re[0], f[0], buf);
+        sum[1] = tile_rows1<false, T, false>(ci[1], val[1], rb[1], re[1], f[1], buf);
+      }
     }
     if (valid) {
       d.Hx[nx][j] = sum[0];
       d.Aty[nx][j] = sum[1];
       const T dx = xti - xci, dh = sum[0] - hxc, da = sum[1] - atc;
       ts.Lt += dx * dx * itx;
-      ts.RH += fabs(dx * dh);
-      ts.RB += fabs(dx * da);
+      ts.RH += fabs(dx) * fabs(dh);
+      ts.RB += fabs(dx) * fabs(da);
       // The next trial's averages (weight alpha of this trial) and x_tr.
       hb = k0[kOma] * hb + k0[kAlpha] * sum[0];
       xb = k0[kOma] * xb + k0[kAlpha] * xti;
@@ -1411,7 +1420,7 @@ __global__ void __launch_bounds__(kTrialThreads, 1) k_trials(Dev<T> d, long long
   __shared__ DevState S;
   __shared__ double next[2];
   extern __shared__ __align__(16) unsigned char slots[];
-  Slot<T> *buf = reinterpret_cast<Slot<T> *>(slots) + (threadIdx.x >> 5) * 2 * kTileSlots;
+  Slot<T> *buf = reinterpret_cast<Slot<T> *>(slots) + (threadIdx.x >> 5) * kTileSlots;
   unsigned *bar = d.ctr + kCtrBar;
   unsigned gen = threadIdx.x == 0 ? ld_acquire_gpu(bar + kBarGen) : 0u;
   state_load(S, d.st);

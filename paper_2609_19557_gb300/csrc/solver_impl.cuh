@@ -565,7 +565,7 @@ class Solver : public SolverBase {
     if (cluster_size()) {
       PDNQP_CK(smem(setup_clu_fn(), setup_smem_bytes<T>()));
       PDNQP_CK(smem(trials_clu_fn(), trials_smem_bytes<T>()));
-      PDNQP_CK(smem(check_clu_fn(), trials_smem_bytes<T>() / 2));
+      PDNQP_CK(smem(check_clu_fn(), trials_smem_bytes<T>()));
     }
     PDNQP_CK(cudaGetLastError());
     return 0;
@@ -777,7 +777,7 @@ class Solver : public SolverBase {
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
     const int smem = (int)trials_smem_bytes<T>();
     if (cudaFuncSetAttribute(trials_fn(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-        cudaFuncSetAttribute(check_fn(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem / 2) != cudaSuccess) {
+        cudaFuncSetAttribute(check_fn(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
       cudaGetLastError();
       return 0;
     }
@@ -806,14 +806,14 @@ class Solver : public SolverBase {
     if (clu) {
       PDNQP_TRY(launch_cluster(trials_clu_fn(), nb, trials_smem_bytes<T>(), d_, chunk));
       PDNQP_CK(cudaEventRecord(loop_ev_[2 * slot + 1], s_));
-      return launch_cluster(check_clu_fn(), nb, trials_smem_bytes<T>() / 2, d_);
+      return launch_cluster(check_clu_fn(), nb, trials_smem_bytes<T>(), d_);
     }
     void *args[] = {(void *)&d_, (void *)&chunk};
     PDNQP_CK(cudaLaunchCooperativeKernel((const void *)trials_fn(), dim3(nb), dim3(kTrialThreads), args,
                                          trials_smem_bytes<T>(), s_));
     PDNQP_CK(cudaEventRecord(loop_ev_[2 * slot + 1], s_));
     PDNQP_CK(cudaLaunchCooperativeKernel((const void *)check_fn(), dim3(nb), dim3(kTrialThreads), args,
-                                         trials_smem_bytes<T>() / 2, s_));
+                                         trials_smem_bytes<T>(), s_));
     return 0;
   }
   void launch_check() {
