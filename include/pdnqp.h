@@ -100,8 +100,8 @@ typedef struct {
   int64_t loop_trials;       /* trials run inside those launches */
   int64_t loop_blocks;       /* blocks of the persistent launch (0: graph modes) */
   int64_t loop_launches;     /* persistent trial-loop launches (including ones that found nothing to do) */
-  double loop_phase_seconds[6]; /* device time of their passes as seen by block 0 (globaltimer): primal work,
-                                   primal barrier wait, row work, row barrier wait, column work, column barrier
+  double loop_phase_seconds[6]; /* device time of their passes as seen by block 0 (globaltimer): primal work
+                                   (0 where the column pass formed the step), its barrier wait, row work, row barrier wait, column work, column barrier
                                    wait + acceptance decision */
   int64_t ctrl_used;         /* outer iterations whose rho_in / primal weight came from the learned controller */
   int64_t ctrl_fallbacks;    /* outer iterations where the paper's rule overrode it (fallback) */
@@ -158,23 +158,25 @@ PDNQP_API int pdnqp_solve(pdnqp_t *h, double eps_abs, double eps_rel);
  * pdnqp_create does when no stream is given), with per-problem termination
  * (Eq. outer-termination with eps_abs / eps_rel), restarts and limits.
  * Fused form (parameter batch_fused = 1 on hs[0], the default; handles on one
- * device): the inner iterations (Algorithm 4) of all problems of one
- * precision run together in one captured CUDA graph of batch_chunk trial
- * slots, one kernel launch per phase for the whole batch (per lanes-per-row
+ * device): the inner iterations (Algorithm 4) of the problems of one precision
+ * run together in one captured CUDA graph of batch_chunk trials and one periodic
+ * check, one kernel launch per phase for the whole batch (per lanes-per-row
  * group), with every problem's acceptance test, periodic check, restart and
- * inner termination taken on the device; each problem's outer iteration
- * (Algorithm 3, Sec. 3.4's CPU side) runs on a host thread of its own (one
- * per problem; `threads` is not used), which sleeps while its inner solve is
- * in the graph.  A problem keeps its solo block partition, so its results
- * are bitwise those of its solo graph-form solve.  Thread-pool form
- * (batch_fused = 0): `threads` host threads (0: min(count, 16)) run
- * pdnqp_solve on the problems, largest first, so their graph-form inner
- * solves overlap on the GPU.  In both forms every solve runs the graph form
- * (the handles' "persistent" and "autotune" parameters are set to 0 for the
- * call and restored).  status[i] receives pdnqp_solve's return for hs[i];
- * the results are read with pdnqp_get per handle.  Returns 0, or the first
- * negative code of a failed solve (the others still run to the end).  Blocks
- * until all solves have finished. */
+ * inner termination taken on the device; problems small enough for the cluster
+ * form (see "persistent" below; handles with persistent = 1) run their inner
+ * loops in that form on their own streams beside the graph.  Each problem's
+ * outer iteration (Algorithm 3, Sec. 3.4's CPU side) runs on a host thread of
+ * its own (one per problem; `threads` is not used), which sleeps while its inner
+ * solve is in the graph.  A problem keeps its solo block partition, so its
+ * results are bitwise those of its solo solve in the same form.  Thread-pool
+ * form (batch_fused = 0): `threads` host threads (0: min(count, 16)) run
+ * pdnqp_solve on the problems, largest first, so their graph-form inner solves
+ * overlap on the GPU.  The "autotune" parameter of every handle, and
+ * "persistent" where the cluster form is not taken, are set to 0 for the call
+ * and restored.  status[i] receives pdnqp_solve's return for hs[i]; the results
+ * are read with pdnqp_get per handle.  Returns 0, or the first negative code of
+ * a failed solve (the others still run to the end).  Blocks until all solves
+ * have finished. */
 PDNQP_API int pdnqp_solve_batch(pdnqp_t *const *hs, int count, double eps_abs, double eps_rel, int threads,
                                 int *status);
 
@@ -208,12 +210,14 @@ PDNQP_API int pdnqp_set_start(pdnqp_t *h, const double *x0, const double *y0);
  * delta_sigma, sigma_max, tol_floor, gamma (override, > 0; setting it
  * replaces the Lanczos choice), chunk (trial slots per CUDA-graph launch),
  * iter_budget (cap on accepted inner iterations per pdnqp_solve, summed over
- * outer iterations; ITER_LIMIT when reached), g_rows / g_cols (nonzeros per
- * lane per CSR-stream chunk in the row / column SpMV kernels: 4, 8 or 16; 0 =
- * from the mean row length), persistent (1, the default: the trials of the
- * inner loop run inside one cooperative kernel launch per check period, with
- * bounded grid barriers between the primal, row and column passes; used when
- * the device supports cooperative launches, else the graph modes below),
+ * outer iterations; ITER_LIMIT when reached), g_rows / g_cols (row / column
+ * kernels of the graph form: 4 or 8 = a warp takes tiles of 32 rows, 16 = tiles
+ * of 8 rows; 0 = from the mean row length), persistent (1, the default: the trials of the
+ * inner loop run inside one kernel launch per check period: small problems in
+ * one thread block or one cluster of 8 (at most 512 tiles of rows or columns and
+ * 120,000 gathers a trial, without long-row tiles), larger ones in a cooperative
+ * launch with bounded grid barriers between the row and column passes; where the
+ * device has no cooperative launches, the graph modes below),
  * loop_blocks_per_sm (blocks per SM of that launch; 0 = as many as fit),
  * cond_graph (with persistent = 0; 1: inner loop as a device-driven CUDA
  * graph with conditional WHILE/IF nodes; 0: unrolled graph of `chunk` trial

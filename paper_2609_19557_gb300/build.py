@@ -1,7 +1,7 @@
 """Builds the CUDA library libpdnqp.so in-tree (paper_2609_19557_gb300/_build/).
 
-Four translation units (C ABI, FP64 solver, FP32-bulk solver, KKT test) are compiled
-in parallel with nvcc for sm_103a only, then linked into one shared library
+The translation units (C ABI, FP64 solver, FP32-bulk solver, KKT test, controller
+network, self-test) are compiled in parallel with nvcc for sm_103a only, then linked into one shared library
 with the CUDA runtime linked statically.
 """
 from __future__ import annotations

@@ -9,7 +9,6 @@ namespace pdq {
 
 constexpr int kBlock = 256;        // threads per block of every vector/SpMV kernel
 constexpr int kMaxBlocks = 152 * 8;  // grid cap: 8 resident 256-thread blocks on each of 152 SMs
-constexpr int kRedThreads = 1024;  // threads of the single-block final reductions
 constexpr int kMaxPartials = 48;   // quantities reduced per launch (rows of the partials array)
 
 // Inner-solver status kept on the device (Algorithm 4 return paths).
@@ -300,9 +299,8 @@ __device__ __forceinline__ void st_release_gpu(unsigned *p, unsigned v) {
 }
 
 // ---------------------------------------------------------------------------
-// Shared-memory mbarriers and bulk (TMA) copies global -> shared.  One thread
-// arms a barrier with the byte count it expects and issues the copies; the
-// barrier's phase completes when the bytes have landed.
+// Shared-memory mbarriers: one thread arms a barrier with the byte count that it
+// expects, and the barrier's phase completes when the bytes have landed.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -313,35 +311,9 @@ __device__ __forceinline__ void mbar_init(unsigned long long *bar, unsigned coun
 __device__ __forceinline__ void mbar_init_fence() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
-// Orders this thread's earlier shared-memory accesses before later bulk copies.
-__device__ __forceinline__ void fence_proxy_async_smem() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
 __device__ __forceinline__ void mbar_arrive_expect_tx(unsigned long long *bar, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                : "memory");
-}
-// Bulk copy of `bytes` (multiple of 16; both addresses 16-byte aligned).
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned bytes, unsigned long long *bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-// L2 policy for data read once per pass (the CSR streams): evict first, so
-// that it does not push the iterate vectors, re-read every pass, out of L2.
-__device__ __forceinline__ unsigned long long l2_evict_first_policy() {
-  unsigned long long p;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-__device__ __forceinline__ void bulk_g2s_hint(void *dst, const void *src, unsigned bytes, unsigned long long *bar,
-                                              unsigned long long policy) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
-          smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(policy)
-      : "memory");
 }
 __device__ __forceinline__ bool mbar_test(unsigned long long *bar, unsigned parity) {
   unsigned ok;
@@ -438,13 +410,6 @@ __device__ __forceinline__ bool grid_sync(unsigned *bar) {
 // warp w handles quantities w, w + nwarps, ...; lane l sums partials l, l + 32,
 // ... serially, then a fixed butterfly combines the 32 lane sums.  Every thread
 // of the block gets out[].  blockDim.x must be a multiple of 32.
-// Terms of the termination-test maxima (Eqs. outer-residuals / outer-scales).
-// fmax drops a NaN operand, so a residual term that is not finite counts as
-// +inf (a point with NaN or infinite entries never passes), and a scale term
-// that is not finite is left out (an infinite scale would excuse any residual).
-__device__ __forceinline__ double res_term(double v) { return isfinite(v) ? v : INFINITY; }
-__device__ __forceinline__ double scale_term(double v) { return isfinite(v) ? v : 0.0; }
-
 template <int NQ>
 __device__ __forceinline__ void final_reduce(const double *part, int nb, const unsigned kind_mask, double (&out)[NQ]) {
   __shared__ double res[NQ];

@@ -120,14 +120,6 @@ __device__ __forceinline__ double clampv<double>(double v, double lo, double hi)
   return is_nan_bits(v) ? v : p;
 }
 
-// Per-thread accumulator of the acceptance sums: FP64 in the FP64 form; in
-// the FP32-bulk form each thread sums its few rows in FP32 and the cross-
-// thread reduction is FP64 (block_reduce_store / final_reduce).
-template <typename T>
-struct SumT {
-  typedef T type;
-};
-
 #define PDNQP_GRID_STRIDE(i, N) \
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < (long long)(N); \
        i += (long long)gridDim.x * blockDim.x)

@@ -110,23 +110,12 @@ template <typename T>
 __global__ void k_to_T(T *dst, const double *src, long long n) {
   PDNQP_GRID_STRIDE(i, n) dst[i] = T(src[i]);
 }
-template <typename T>
-__global__ void k_from_T(double *dst, const T *src, long long n) {
-  PDNQP_GRID_STRIDE(i, n) dst[i] = double(src[i]);
-}
-
 __global__ void k_fill_d(double *p, long long n, double v) {
   PDNQP_GRID_STRIDE(i, n) p[i] = v;
 }
 __global__ void k_mul_scalar(double *p, long long n, double a) {
   PDNQP_GRID_STRIDE(i, n) p[i] *= a;
 }
-// h = (b_E, 0) (Eq. inner-qp), b_E = l_c on the equality rows.
-template <typename T>
-__global__ void k_form_h(T *h, const double *lc, long long m, int mE) {
-  PDNQP_GRID_STRIDE(j, m) h[j] = j < mE ? T(lc[j]) : T(0);
-}
-
 // ---------------------------------------------------------------------------
 // Lanczos (Eq. R-choice): both starts in one cooperative launch.
 // ---------------------------------------------------------------------------
@@ -480,7 +469,10 @@ constexpr int kOutRows = OUT_Q + INF_R, kOutCols = OUT_Q + INF_C;  // rows of pa
 constexpr unsigned kOutRowsMask = OUT_MAXMASK | INF_R_MAXMASK << OUT_Q, kOutColsMask = OUT_MAXMASK | INF_C_MAXMASK << OUT_Q;
 static_assert(kOutRows + kOutCols <= kMaxPartials, "partials of the outer pass");
 
-// Residual and scale terms (res_term / scale_term) of the maxima.
+// Terms of the termination-test maxima (Eqs. outer-residuals / outer-scales): a
+// residual term that is not finite counts as +inf (a point with NaN or infinite
+// entries never passes), and a scale term that is not finite is left out (an
+// infinite scale would excuse any residual).
 __device__ __forceinline__ double res_of(double v) { return nonfinite(v) ? INFINITY : fabs(v); }
 __device__ __forceinline__ double scale_of(double v) { return nonfinite(v) ? 0.0 : fabs(v); }
 
@@ -676,15 +668,6 @@ __global__ void k_sigma_update(int m, int mE, double *sig, const double *lam, co
       sig[j] = fmin(smax, sig[j] * fmax(1.0, dsig * fabs(r) / rn));
     rprev[j] = r;
   }
-}
-
-template <typename T>
-__global__ void k_copy_T(T *dst, const T *src, long long n) {
-  PDNQP_GRID_STRIDE(i, n) dst[i] = src[i];
-}
-template <typename T>
-__global__ void k_copy_to_double(double *dst, const T *src, long long n) {
-  PDNQP_GRID_STRIDE(i, n) dst[i] = double(src[i]);
 }
 
 // Unscaling for the result: x_orig = Dx x, lambda_orig = Dc lambda / c_s.

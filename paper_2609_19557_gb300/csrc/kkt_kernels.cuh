@@ -19,9 +19,9 @@ namespace pdq {
 namespace {
 
 __device__ __forceinline__ u64 umax64(u64 a, u64 b) { return a < b ? b : a; }
-// |v| as a residual term: +inf when it is not finite (res_term).
+// |v| as a residual term: +inf when it is not finite.
 __device__ __forceinline__ u64 res_bits(double v) { return nonfinite(v) ? kInfBits : abs_bits(v); }
-// |v| as a scale term: left out when it is not finite (scale_term).
+// |v| as a scale term: left out when it is not finite.
 __device__ __forceinline__ u64 scale_bits(double v) { return nonfinite(v) ? 0ull : abs_bits(v); }
 // |v| with NaN left out (what fmax does with a NaN operand).
 __device__ __forceinline__ u64 nonan_bits(double v) { return is_nan_bits(v) ? 0ull : abs_bits(v); }

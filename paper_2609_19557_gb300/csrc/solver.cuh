@@ -1,11 +1,11 @@
 // Host orchestration of the PDNQP solver on one GPU: setup (Sec. 3.1), the
 // outer proximal-ALM loop (Algorithm 3) on the host with its vector work in
 // kernels, and the inner rAPDHG solve (Algorithm 4) driven entirely by the
-// device: a CUDA graph of `chunk` trial slots is replayed, each slot being
-// [primal, rows, cols, decide, average, check-rows, check-cols, check-final,
-// check-apply]; every kernel reads the device-resident state and does nothing
-// once the inner solve has stopped, so the host only polls the status
-// between graph launches (Sec. 3.4, "GPU inner iterations").
+// device: launches of the persistent trial loop and of the periodic check follow
+// one another on the solve's stream (in the graph modes, captured trial slots);
+// every kernel reads the device-resident state and does nothing once the inner
+// solve has stopped, so the host only polls the status between batches of
+// launches (Sec. 3.4, "GPU inner iterations").
 #pragma once
 #include <cuda_runtime.h>
 

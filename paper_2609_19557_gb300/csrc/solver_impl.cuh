@@ -219,17 +219,15 @@ class Solver : public SolverBase {
     if (which == 5) {
       // One trial of the persistent loop (k_trials) after an accepted trial,
       // each array counted once per pass (gathers assumed served from L2):
-      // primal: reads x, Hx, Hxbar, xbar, qx, A'y, taux, lx, ux; writes x_tr,
-      //   Hxbar', xbar'.
-      const double p5 = 12 * v * n;
-      // rows: A; gathers x_tr; reads y, r, rbar, ybar, taur, qr, Bw, eta, hp,
-      //   itaur, ieta and sig (FP64) per row, s, sbar, taus, qs, ls, us,
-      //   itaus per inequality row; writes rbar', ybar', r, Bw, y (+ sbar', s).
-      const double r5 = mat_a + v * n + m * (16 * v + 8) + mI * 9 * v;
-      // cols: H, A^T; gathers x_tr (also read per row) and y_tr; reads x,
-      //   Hx, A'y, taux; writes Hx_tr, A'y_tr.
-      const double c5 = mat_h + mat_at + 7 * v * n + v * m;
-      return p5 + r5 + c5;
+      // rows: A; gathers x_tr; reads y, r, rbar, ybar, sig, taur, qr, Bw, eta,
+      //   hp, itaur, ieta per row, s, sbar, taus, qs, ls, us, itaus per
+      //   inequality row; writes rbar', ybar', r, Bw, y (+ sbar', s).
+      const double r5 = mat_a + v * n + 17 * v * m + mI * 9 * v;
+      // cols: H, A^T; gathers x_tr (also read per column) and y_tr; reads x, Hx,
+      //   A'y, itaux, xbar, Hxbar, qx, taux, lx, ux; writes Hx_tr, A'y_tr,
+      //   Hxbar', xbar' and the next x_tr.
+      const double c5 = mat_h + mat_at + 16 * v * n + v * m;
+      return r5 + c5;
     }
     if (which == 0) return cols;
     if (which == 1) return rows;
@@ -240,8 +238,8 @@ class Solver : public SolverBase {
 
  private:
   // ------------------------------------------------------------- helpers
-  // Every array carries kPad zeroed elements past its end: the bulk copies of
-  // the panel stream round their ranges up to 16 bytes and may read them.
+  // Every array carries kPad zeroed elements past its end, so that an access
+  // rounded up to 16 bytes stays inside it.
   static constexpr size_t kPad = 4;
   template <typename U>
   int dalloc(U **p, size_t count) {
