@@ -331,8 +331,7 @@ def run_native(args):
                                    "traffic": captured_traffic(64, lt64 / max(1, ll64)),
                                    "algorithmic_bytes_per_trial": b64, "us_per_trial": 1e6 * ls64 / lt64,
                                    "trials_per_launch": lt64 / max(1, ll64),
-                                   "fp64_pipe": "the FP64 pipe is 67 % busy in this kernel (ncu, "
-                                                "profiles/k_trials_n1e6_fp64.md): it binds before HBM"}
+                                   "fp64_pipe": "the FP64 pipe and the gathers bind this kernel before HBM"}
         h64.close()
 
     ttk = None

@@ -181,7 +181,7 @@ PDNQP_API int pdnqp_solve_batch(pdnqp_t *const *hs, int count, double eps_abs, d
                                 int *status);
 
 /* Failure-detection self-test (no counterpart in the paper).  Makes one kind
- * of bounded device wait of the persistent trial loop run out on purpose on
+ * of bounded device wait (the trial loop's, or a bulk copy's) run out on purpose on
  * the current device, without a fault: kind 0 = a grid barrier that one of
  * its 4 blocks never reaches (the others poll the release up to their limit),
  * kind 1 = a bulk-copy mbarrier that expects 16 bytes nothing sends.  On
