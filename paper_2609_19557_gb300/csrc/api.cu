@@ -514,11 +514,15 @@ static int solve_batch_fused(pdnqp_t *const *hs, int count, double eps_abs, doub
   // Problems that fit the cluster form (a few SMs each, no cooperative launch) run
   // it on their own streams beside each other, at their own pace; the others
   // share the graph.
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const bool roomy = 8LL * count <= sms;  // 8 blocks a cluster, one per SM
   std::vector<int> keep(count), keep_tune(count), own(count);
   for (int i = 0; i < count; ++i) {
     keep[i] = hs[i]->prm.persistent;
     keep_tune[i] = hs[i]->prm.autotune;
-    own[i] = keep[i] && hs[i]->solver->cluster_size() > 0;
+    own[i] = keep[i] && hs[i]->solver->cluster_size(roomy) > 0;
+    hs[i]->prm.roomy_batch = roomy;
     if (!own[i]) hs[i]->prm.persistent = 0;  // escalated FP64 solves run the graph form: no cooperative launch beside the batch
     hs[i]->prm.autotune = 0;    // the per-handle tuner replays kernels on a running state: not beside the batch
   }
@@ -592,6 +596,7 @@ static int solve_batch_fused(pdnqp_t *const *hs, int count, double eps_abs, doub
   for (int i = 0; i < count; ++i) {
     hs[i]->prm.persistent = keep[i];
     hs[i]->prm.autotune = keep_tune[i];
+    hs[i]->prm.roomy_batch = false;
   }
   if (rc < 0) return fail(nullptr, rc, "batch: " + err);
   int worst = 0;

@@ -63,6 +63,7 @@ struct Params {
   int autotune = 0;            // 1: time the lanes-per-row choices of the graph form once, keep the fastest
   int escalate = 1;            // FP32-bulk: continue in FP64 after a NUMERICAL_ERROR
   int batch_fused = 1;         // pdnqp_solve_batch: 1 = one batched graph for all inner loops, 0 = thread pool
+  bool roomy_batch = false;    // in a batch whose clusters all find room at once (set for the call)
   int batch_chunk = 16;        // trial slots per launch of the batched graph
 };
 
@@ -92,7 +93,7 @@ class SolverBase {
   virtual int debug_inner(Params &prm, int nck, const int64_t *ck, double *snap, std::string *err) = 0;
   virtual int replay(int which, int reps) = 0;
   virtual int tuned_g(int which) const = 0;
-  virtual int cluster_size() const = 0;  // blocks of the cluster form, 0: too large for it
+  virtual int cluster_size(bool roomy) const = 0;  // blocks of the cluster form, 0: too large for it
   virtual double kernel_bytes(int which) const = 0;
   virtual double last_replay_ms() const = 0;
   virtual double gamma() const = 0;

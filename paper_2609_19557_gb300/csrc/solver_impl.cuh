@@ -560,7 +560,7 @@ class Solver : public SolverBase {
     };
     PDNQP_CK(smem(setup_fn<kGrid>(), setup_smem_bytes<T>()));
     PDNQP_CK(smem(setup_fn<kByPhase>(), setup_smem_bytes<T>()));
-    if (cluster_size()) {
+    if (cluster_size(true)) {
       PDNQP_CK(smem(setup_clu_fn(), setup_smem_bytes<T>()));
       PDNQP_CK(smem(trials_clu_fn(), trials_smem_bytes<T>()));
       PDNQP_CK(smem(check_clu_fn(), trials_smem_bytes<T>()));
@@ -733,13 +733,19 @@ class Solver : public SolverBase {
     return long_tiles_c() ? k_check<T, false, true, true> : k_check<T, false, false, true>;
   }
   // Blocks of the cluster form (0: the problem is too large for it).  Up to 8
-  // blocks, a warp with a tile or a few; the limits are where a pass by 8 SMs
-  // costs what the grid form saves on its barriers: 4 tiles a warp (n = 16,000
-  // in tiles of 32), and 120,000 gathers a trial (8 us at one a cycle and SM).
-  int cluster_size() const override {
+  // blocks, a warp with a tile or a few.  Alone, the limits are where a pass by 8
+  // SMs costs what the grid form saves on its barriers: 4 tiles a warp (n =
+  // 16,000 in tiles of 32), and 120,000 gathers a trial (8 us at one a cycle and
+  // SM).  In a batch whose clusters all find room on the GPU at once (roomy) the
+  // alternative is the shared graph, whose trial takes 50 us and more: up to 1,024
+  // tiles and 700,000 gathers (12 problems of n = 10,000-20,000 to 1e-4, twice: 16.3
+  // against 18.8 s).  Clusters that have to wait for one another gain nothing (a
+  // batch of 24 with these limits: 28.4 against 26.9 ms).
+  int cluster_size(bool roomy) const override {
     const long long tc = long_tiles_c() ? 8 : 32;
-    const long long tiles = std::max<long long>((m_ + 31) / 32 + d_.nlong_r, (n_ + tc - 1) / tc + (tc == 32 ? d_.nlong_c : 0));
-    if (tiles > 512 || nnzH_ + 2 * nnzA_ > 120000) return 0;
+    const long long tiles =
+        std::max<long long>((m_ + 31) / 32 + d_.nlong_r, (n_ + tc - 1) / tc + (tc == 32 ? d_.nlong_c : 0));
+    if (tiles > (roomy ? 1024 : 512) || nnzH_ + 2 * nnzA_ > (roomy ? 700000 : 120000)) return 0;
     // One block as long as each of its 16 warps has a tile at most (at n = 200 a
     // cluster of 4 takes 10.1 us a trial, a block 9.9).
     return tiles <= 16 ? 1 : 8;
@@ -1074,7 +1080,7 @@ class Solver : public SolverBase {
     SetupArgs<T> a{Hd_, Ad_, Atd_, c_, z_, lcd_, ucd_, lxd_, uxd_, sb64_, rb64_, xprev_, u, 1.0 / gamma_, prm.ruiz_inner,
                    ex2_, dy2_, d_.Bwbar, d_.Atybar};
     const int last = prm.ruiz_inner + 3;
-    const int nb = setup_grid(), clu = prm.persistent ? cluster_size() : 0;
+    const int nb = setup_grid(), clu = prm.persistent ? cluster_size(prm.roomy_batch) : 0;
     if (clu) {
       PDNQP_TRY(launch_cluster(setup_clu_fn(), clu, setup_smem_bytes<T>(), d_, a, 0, last));
       launches_ += 1;
@@ -1121,7 +1127,7 @@ class Solver : public SolverBase {
       *hst_ = *S;
       return r;
     }
-    const int clu = prm.persistent ? cluster_size() : 0;
+    const int clu = prm.persistent ? cluster_size(prm.roomy_batch) : 0;
     const int nbp = clu ? clu : prm.persistent ? coop_grid(prm.loop_blocks_per_sm) : 0;
     loop_nb_ = nbp;
     if (nbp > 0) {

@@ -98,7 +98,8 @@ def test_forms_fp32(P, refs, name):
 def test_batch_of_both_forms(P, precision):
     """Problems in the cluster form and in the shared graph of one batch: each ends
     with the bits of its own solo solve in that form."""
-    insts = [sized(300, 100), sized(1500, 700), sized(17000, 8000), rows_qp(1, 2000, [3] * 400 + EDGES), sized(20000, 9000)]
+    insts = [sized(300, 100), sized(1500, 700), sized(33000, 8000), rows_qp(1, 2000, [3] * 400 + EDGES),
+             sized(36000, 9000)]
 
     def make(inst, persistent):
         h = P.create_from_instance(inst, precision=precision)
