@@ -163,7 +163,8 @@ PDNQP_API int pdnqp_solve(pdnqp_t *h, double eps_abs, double eps_rel);
  * check, one kernel launch per phase for the whole batch (per lanes-per-row
  * group), with every problem's acceptance test, periodic check, restart and
  * inner termination taken on the device; problems small enough for the cluster
- * form (see "persistent" below; handles with persistent = 1) run their inner
+ * form (see "persistent" below; up to 1,024 tiles and 700,000 gathers where the
+ * GPU has 8 SMs for every problem; handles with persistent = 1) run their inner
  * loops in that form on their own streams beside the graph.  Each problem's
  * outer iteration (Algorithm 3, Sec. 3.4's CPU side) runs on a host thread of
  * its own (one per problem; `threads` is not used), which sleeps while its inner
