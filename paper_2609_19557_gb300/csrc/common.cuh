@@ -459,7 +459,9 @@ inline int tile_rows_per_block(int k) { return kBlock / 32 * (k == 16 ? 8 : 32);
 // l brings the entry range [rb, re) of row tile + l (empty past the matrix)
 // and gets that row's sum (or maximum): F::gather(col) loads what an entry
 // multiplies, F::add(acc, val, x) adds the entry.  The order of every sum is
-// fixed.
+// fixed.  A round looks up to 512 entries past the end of its row, beyond 2^31 - 1
+// in the last rows of the largest matrices: positions are unsigned, and what is
+// compared is the entries left in the row (end - position, as a signed number).
 //
 // What the two forms are built around: gathers are bound by memory latency, so
 // a warp issues the 8 index and value loads of a round, then the 8 gathers (16
@@ -487,14 +489,17 @@ __device__ __forceinline__ A acc_join(A a, A b) {  // maxima: of non-negative va
 template <bool IsMax, typename Acc, typename T, typename F>
 __device__ __forceinline__ Acc warp_row(const int *__restrict__ ci, const T *__restrict__ val, int b, int e,
                                         const F &f) {
+  const int lane = threadIdx.x & 31;
   Acc acc = Acc(0);
-  for (int k0 = b + (int)(threadIdx.x & 31); k0 - (int)(threadIdx.x & 31) < e; k0 += 256) {
+  for (unsigned k0 = (unsigned)b + lane;; k0 += 256) {
+    const int left = (int)((unsigned)e - k0);
+    if (left + lane <= 0) break;  // the same for the whole warp
     int c[8];
     T a[8];
     Acc p[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const bool ok = k0 + 32 * u < e;
+      const bool ok = left > 32 * u;
       c[u] = ok ? __ldg(ci + k0 + 32 * u) : -1;
       a[u] = ok ? __ldg(val + k0 + 32 * u) : T(0);
     }
@@ -502,7 +507,7 @@ __device__ __forceinline__ Acc warp_row(const int *__restrict__ ci, const T *__r
     for (int u = 0; u < 8; ++u) p[u] = c[u] >= 0 ? f.gather(c[u]) : Acc(0);
 #pragma unroll
     for (int u = 0; u < 8; ++u)
-      if (k0 - (int)(threadIdx.x & 31) + 32 * u < e) {  // the same for the whole warp
+      if (left + lane > 32 * u) {  // the same for the whole warp
         if (c[u] >= 0) f.add(acc, Acc(a[u]), p[u]);
       }
   }
@@ -539,12 +544,12 @@ __device__ __forceinline__ Acc one_row(const int *__restrict__ ci, const T *__re
     if (e - b <= kDenseRow) return warp_row<IsMax, Acc>(ci, val, b, e, f);
     const int lane = threadIdx.x & 31;
     Acc acc = Acc(0);
-    for (int k0 = b; k0 < e; k0 += 256) {
+    for (unsigned k0 = b; k0 < (unsigned)e; k0 += 256) {
       Slot<Acc> r[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        const int k = k0 + 32 * u + lane;
-        r[u] = k < e ? Slot<Acc>{Acc(__ldg(val + k)), f.gather(__ldg(ci + k))} : Slot<Acc>{Acc(0), Acc(0)};
+        const unsigned k = k0 + 32 * u + lane;
+        r[u] = k < (unsigned)e ? Slot<Acc>{Acc(__ldg(val + k)), f.gather(__ldg(ci + k))} : Slot<Acc>{Acc(0), Acc(0)};
         if (F::kOrder == 2) r[u].x = __dmul_rn(r[u].a, r[u].x);
       }
       __syncwarp();
@@ -615,11 +620,11 @@ __device__ __forceinline__ void tile_rows(const int *const (&ci)[NM], const T *c
     for (int m = 0; m < NM; ++m)
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
-        const int p = __shfl_sync(0xffffffffu, rb[m], t * 8 + sub) + s + lg;
-        const int e = __shfl_sync(0xffffffffu, se[m], t * 8 + sub);
+        const unsigned p = (unsigned)__shfl_sync(0xffffffffu, rb[m], t * 8 + sub) + s + lg;
+        const int left = (int)((unsigned)__shfl_sync(0xffffffffu, se[m], t * 8 + sub) - p);
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          const bool ok = p + 4 * u < e;
+          const bool ok = left > 4 * u;
           c[m][t][u] = ok ? __ldg(ci[m] + p + 4 * u) : -1;
           a[m][t][u] = ok ? __ldg(val[m] + p + 4 * u) : T(0);
         }
@@ -715,12 +720,13 @@ __device__ __forceinline__ Acc tile_long_rows(const int *__restrict__ ci, const 
   const bool alone = re - rb > kRowAlone;
   const int se = alone ? rb : re;
   const int longest = (int)__reduce_max_sync(0xffffffffu, (unsigned)(se - rb));
-  int pos[8], end[8];
+  unsigned pos[8];
+  int left[8];
   Acc acc[8];
 #pragma unroll
   for (int t = 0; t < 8; ++t) {
     pos[t] = __shfl_sync(0xffffffffu, rb, t) + lane;
-    end[t] = __shfl_sync(0xffffffffu, se, t);
+    left[t] = (int)((unsigned)__shfl_sync(0xffffffffu, se, t) - pos[t]);
     acc[t] = Acc(0);
   }
   for (int s = 0; s < longest; s += 32) {
@@ -729,7 +735,7 @@ __device__ __forceinline__ Acc tile_long_rows(const int *__restrict__ ci, const 
     Acc p[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
-      const bool ok = pos[t] + s < end[t];
+      const bool ok = left[t] > s;
       c[t] = ok ? __ldg(ci + pos[t] + s) : -1;
       a[t] = ok ? __ldg(val + pos[t] + s) : T(0);
     }
@@ -737,7 +743,7 @@ __device__ __forceinline__ Acc tile_long_rows(const int *__restrict__ ci, const 
     for (int t = 0; t < 8; ++t) p[t] = c[t] >= 0 ? f.gather(c[t]) : Acc(0);
 #pragma unroll
     for (int t = 0; t < 8; ++t)
-      if (pos[t] - lane + s < end[t]) {  // the same for the whole warp
+      if (left[t] + lane > s) {  // the same for the whole warp
         if (c[t] >= 0) f.add(acc[t], Acc(a[t]), p[t]);
       }
   }

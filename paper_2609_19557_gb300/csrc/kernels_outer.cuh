@@ -53,7 +53,7 @@ __global__ void k_scale_csr(int nrows, const int *rp, const int *ci, double *val
   for (long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < nrows;
        i += ((long long)gridDim.x * blockDim.x) >> 5) {
     const double ri = rs[i] * mult;
-    for (int k = rp[i] + lane; k < rp[i + 1]; k += 32) val[k] = ri * val[k] * cs[ci[k]];
+    for (unsigned k = rp[i] + lane, e = rp[i + 1]; k < e; k += 32) val[k] = ri * val[k] * cs[ci[k]];
   }
 }
 

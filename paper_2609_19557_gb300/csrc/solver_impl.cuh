@@ -671,7 +671,7 @@ class Solver : public SolverBase {
   // block walked through the simplex row of 20,404 entries, 56 of the 80 us of a
   // batched trial).
   int nb_rows(int g) const {
-    return std::max(grid_for(std::max(m_, 1), tile_rows_per_block(g)), std::min(152, (d_.lr_nnz + 511) / 512));
+    return std::max(grid_for(std::max(m_, 1), tile_rows_per_block(g)), (int)std::min(152LL, (d_.lr_nnz + 511LL) / 512));
   }
   int nb_cols(int g) const { return grid_for(n_, tile_rows_per_block(g)); }
   int nb_rows() const { return nb_rows(gA_); }
