@@ -182,13 +182,17 @@ PDNQP_API int pdnqp_solve_batch(pdnqp_t *const *hs, int count, double eps_abs, d
                                 int *status);
 
 /* Failure-detection self-test (no counterpart in the paper).  Makes one kind
- * of bounded device wait (the trial loop's, or a bulk copy's) run out on purpose on
- * the current device, without a fault: kind 0 = a grid barrier that one of
- * its 4 blocks never reaches (the others poll the release up to their limit),
- * kind 1 = a bulk-copy mbarrier that expects 16 bytes nothing sends.  On
- * return *gave_up is 1 when every waiter gave up with a failure and set the
- * fault flag, and *seconds (may be NULL) is the wall time of the launch
- * (about a second or a few).  The context stays usable.  Returns 0,
+ * of bounded device wait run out on purpose on the current device, without a
+ * fault: kind 0 = the grid barrier of the solver's kernels in a grid of 4 blocks
+ * one of which never reaches it (the others poll the release up to their limit),
+ * kind 1 = an mbarrier that expects 16 bytes of a bulk copy nothing sends (no
+ * kernel of the solver waits on one), kind 2 = the same grid barrier in the
+ * launches of a solve, which has to return PDNQP_ERR_CUDA, after which the next
+ * solve of that solver succeeds.  On return *gave_up is 1 when every waiter gave
+ * up with a failure and set the fault flag (kind 2: when the two solves ended so),
+ * and *seconds (may be NULL) is the wall time (a second or a few).  The barrier
+ * inside a thread-block cluster (small problems) is a hardware wait, as the block
+ * barrier is, and has no limit.  The context stays usable.  Returns 0,
  * PDNQP_ERR_ARG or a CUDA error code. */
 PDNQP_API int pdnqp_selftest_wait(int kind, int *gave_up, double *seconds);
 

@@ -277,17 +277,8 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[NQ], double *part
   __syncthreads();
 }
 
-// Grid barrier of a cooperative (co-resident) launch.  bar[0] counts the
-// arrivals, bar[kBarGen] is the generation, bar[kBarFault] the fault flag.  The last block to
-// arrive runs lead() with all its threads before it releases the others, so
-// lead() sees every block's writes from before the barrier and every block
-// sees lead()'s writes after it.  The wait is bounded: a block that polls
-// kSpinLimit times without a release (about a second or more), or that sees
-// the fault flag, sets the flag and the call returns false; the caller then
-// leaves the kernel, so a barrier that can never complete ends the launch
-// instead of hanging it.
+// Polls of a grid barrier before it gives up (about a second or more).
 constexpr unsigned kSpinLimit = 1u << 22;
-constexpr unsigned kSpinLimitTx = 1u << 24;  // polls of a bulk-copy barrier (with a 32 ns sleep)
 
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned *p) {
   unsigned v;
@@ -296,58 +287,6 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned *p) {
 }
 __device__ __forceinline__ void st_release_gpu(unsigned *p, unsigned v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// ---------------------------------------------------------------------------
-// Shared-memory mbarriers: one thread arms a barrier with the byte count that it
-// expects, and the barrier's phase completes when the bytes have landed.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(unsigned long long *bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-// Makes barrier initialisation visible to the copy engine (async proxy).
-__device__ __forceinline__ void mbar_init_fence() {
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(unsigned long long *bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_test(unsigned long long *bar, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0u;
-}
-// Bounded wait of one warp for the phase with the given parity: lane 0 polls
-// (and every 64 polls looks at the fault flag), the result is warp-uniform,
-// and on success every lane observes the completed phase itself, which makes
-// the copied bytes visible to it.  Returns false on a timeout (the fault flag
-// is then set) or when another warp has already set the fault flag.
-__device__ __forceinline__ bool mbar_wait_warp(unsigned long long *bar, unsigned parity, unsigned *fault) {
-  int r = 0;
-  if ((threadIdx.x & 31) == 0) {
-    for (unsigned it = 0; it <= kSpinLimitTx; ++it) {
-      if (mbar_test(bar, parity)) {
-        r = 1;
-        break;
-      }
-      if ((it & 63u) == 63u && ld_acquire_gpu(fault) != 0u) break;
-      __nanosleep(32);
-    }
-    if (!r) atomicExch(fault, 1u);
-  }
-  r = __shfl_sync(0xffffffffu, r, 0);
-  if (r)
-    for (unsigned it = 0; it <= kSpinLimitTx && !mbar_test(bar, parity); ++it) {
-    }
-  __syncwarp();
-  return r != 0;
 }
 
 // Device-wide nanosecond timer (phase timing of the persistent loop).
@@ -362,48 +301,91 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // generation do not queue behind the arrival atomics.
 constexpr int kBarGen = 32, kBarFault = 64, kBarWords = 96;
 
-template <typename F>
-__device__ __forceinline__ bool grid_sync(unsigned *bar, F lead) {
-  __shared__ int role;  // 0 released, 1 leader, 2 fault
-  unsigned gen = 0;
+// Barrier of one thread-block cluster.  A hardware wait without a limit, as
+// __syncthreads is: the hardware starts the blocks of a cluster together, and
+// every block takes the same branches, on the same state, up to each barrier.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+// The barrier alone.
+template <bool CLU>
+__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen);
+
+// Grid barrier of a cooperative (co-resident) launch, the wait of every kernel
+// that spans blocks.  bar[0] counts the arrivals, bar[kBarGen] is the generation
+// with a message in its low bit, bar[kBarFault] the fault flag.  The last block to
+// arrive runs lead() with all its threads before it releases the others, so
+// lead() sees every block's writes from before the barrier and every block sees
+// lead()'s writes after it; what lead() returned (0 or 1) is the message, which
+// every block gets.  The arrivals are reset before lead() runs, and `gen` is the
+// caller's copy of the generation (thread 0), so a waiting block polls one word
+// and, every 64 polls, the fault flag (each is a round trip to L2).
+//
+// The wait is bounded: a block that polls kSpinLimit times without a release, or
+// that sees the fault flag, sets the flag and gets -1; the caller then leaves the
+// kernel, so a barrier that can never complete ends the launch instead of hanging
+// it.
+//
+// CLU: the grid is one thread-block cluster (small problems), whose hardware
+// barrier orders the blocks' memory accesses like a block barrier (about 0.3 us
+// where the grid barrier takes 1.5 to 2.5); block 0 runs lead(), and no message
+// comes back.
+template <bool CLU, typename F>
+__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, F lead) {
+  __shared__ int role;  // message, -1 fault, 2 leader
   __syncthreads();
-  if (gridDim.x == 1) {  // nobody to wait for
-    lead();
+  if (gridDim.x == 1) {
+    const int msg = lead();
     __syncthreads();
-    return true;
+    return msg;
+  }
+  if (CLU) {
+    cluster_sync();
+    if (blockIdx.x == 0) lead();
+    cluster_sync();
+    return 0;
   }
   if (threadIdx.x == 0) {
-    gen = ld_acquire_gpu(bar + kBarGen);
     __threadfence();
-    role = (atomicAdd(bar, 1u) == gridDim.x - 1) ? 1 : 0;
-  }
-  __syncthreads();
-  if (role == 1) {
-    __threadfence();
-    lead();
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    role = -2;
+    if (atomicAdd(bar, 1u) == gridDim.x - 1) {
       atomicExch(bar, 0u);
       __threadfence();
-      st_release_gpu(bar + kBarGen, gen + 1);
-    }
-  } else if (threadIdx.x == 0) {
-    unsigned it = 0;
-    while (ld_acquire_gpu(bar + kBarGen) == gen) {
-      // The fault flag every 64 polls: each of the two reads is a round trip to L2.
-      if (++it > kSpinLimit || ((it & 63u) == 0u && ld_acquire_gpu(bar + kBarFault) != 0u)) {
-        atomicExch(bar + kBarFault, 1u);
-        role = 2;
-        break;
+      role = 2;
+    } else {
+      unsigned it = 0, v;
+      while ((v = ld_acquire_gpu(bar + kBarGen)) == gen) {
+        if (++it > kSpinLimit || ((it & 63u) == 0u && ld_acquire_gpu(bar + kBarFault) != 0u)) {
+          atomicExch(bar + kBarFault, 1u);
+          role = -1;
+          break;
+        }
+      }
+      if (role != -1) {
+        gen = v;
+        role = (int)(v & 1u);
       }
     }
-    __threadfence();
   }
   __syncthreads();
-  return role != 2;
+  if (role != 2) return role;
+  const int msg = lead();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    gen = ((gen >> 1) + 1u) << 1 | (unsigned)msg;
+    __threadfence();
+    st_release_gpu(bar + kBarGen, gen);
+  }
+  return msg;
 }
-__device__ __forceinline__ bool grid_sync(unsigned *bar) {
-  return grid_sync(bar, [] {});
+
+template <bool CLU>
+__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen) {
+  if (CLU && gridDim.x > 1) {
+    cluster_sync();
+    return 0;
+  }
+  return loop_sync<CLU>(bar, gen, [] { return 0; });
 }
 
 // Single-block final reduction of NQ quantities over nb partials (fixed order):

@@ -785,81 +785,6 @@ __device__ __forceinline__ void cols_phase_tiles(const Dev<T> &d, const DevState
   }
 }
 
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
-}
-// The barrier alone.
-template <bool CLU>
-__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen);
-
-// Grid barrier of the loop with a message: bar as in grid_sync, but the
-// generation word carries, in its low bit, what the last block's lead()
-// returned; every block gets it (-1: a wait ran out).  The arrivals are reset
-// before lead() runs, and `gen` is the caller's copy of the generation (thread
-// 0), so a waiting block polls one word and nothing else.
-//
-// CLU: the grid is one thread-block cluster (small problems), whose hardware
-// barrier orders the blocks' memory accesses like a block barrier (about 0.3 us
-// where the grid barrier takes 1.5 to 2.5); block 0 runs lead(), and no message
-// comes back.
-template <bool CLU, typename F>
-__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, F lead) {
-  __shared__ int role;  // message, -1 fault, 2 leader
-  __syncthreads();
-  if (gridDim.x == 1) {
-    const int msg = lead();
-    __syncthreads();
-    return msg;
-  }
-  if (CLU) {
-    cluster_sync();
-    if (blockIdx.x == 0) lead();
-    cluster_sync();
-    return 0;
-  }
-  if (threadIdx.x == 0) {
-    __threadfence();
-    role = -2;
-    if (atomicAdd(bar, 1u) == gridDim.x - 1) {
-      atomicExch(bar, 0u);
-      __threadfence();
-      role = 2;
-    } else {
-      unsigned it = 0, v;
-      while ((v = ld_acquire_gpu(bar + kBarGen)) == gen) {
-        if (++it > kSpinLimit || ((it & 63u) == 0u && ld_acquire_gpu(bar + kBarFault) != 0u)) {
-          atomicExch(bar + kBarFault, 1u);
-          role = -1;
-          break;
-        }
-      }
-      if (role != -1) {
-        gen = v;
-        role = (int)(v & 1u);
-      }
-    }
-  }
-  __syncthreads();
-  if (role != 2) return role;
-  const int msg = lead();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    gen = ((gen >> 1) + 1u) << 1 | (unsigned)msg;
-    __threadfence();
-    st_release_gpu(bar + kBarGen, gen);
-  }
-  return msg;
-}
-
-template <bool CLU>
-__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen) {
-  if (CLU && gridDim.x > 1) {
-    cluster_sync();
-    return 0;
-  }
-  return loop_sync<CLU>(bar, gen, [] { return 0; });
-}
-
 // This block's four sums to part[0..3] (fixed order): per warp the quantities
 // are reduced together by halving (6 FP64 additions), then warp 0 adds the
 // warps' sums.  Visible to the block after its next barrier.

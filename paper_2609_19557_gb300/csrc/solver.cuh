@@ -96,6 +96,7 @@ class SolverBase {
   virtual int cluster_size(bool roomy) const = 0;  // blocks of the cluster form, 0: too large for it
   virtual double kernel_bytes(int which) const = 0;
   virtual double last_replay_ms() const = 0;
+  virtual int jam_barrier() = 0;  // failure-detection self-test: the next launches' grid barrier never completes
   virtual double gamma() const = 0;
   virtual double lambda_min() const = 0;
   virtual void set_gamma(double g) = 0;

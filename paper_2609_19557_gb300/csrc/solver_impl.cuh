@@ -200,6 +200,15 @@ class Solver : public SolverBase {
     return 0;
   }
 
+  // The arrival count of the grid barrier to a value that no arrival completes.
+  int jam_barrier() override {
+    if (!ready_) return PDNQP_ERR_STATE;
+    const unsigned many = 1u << 31;
+    PDNQP_CK(cudaMemcpyAsync(d_.ctr + kCtrBar, &many, sizeof(many), cudaMemcpyHostToDevice, s_));
+    PDNQP_CK(cudaStreamSynchronize(s_));
+    return 0;
+  }
+
   // Compulsory DRAM bytes (each array touched once, int32 indices, value size
   // sizeof(T)); gathers of x / y assumed L2-resident.
   double last_replay_ms() const override { return last_replay_ms_; }
