@@ -523,7 +523,8 @@ static int solve_batch_fused(pdnqp_t *const *hs, int count, double eps_abs, doub
     keep_tune[i] = hs[i]->prm.autotune;
     own[i] = keep[i] && hs[i]->solver->cluster_size(roomy) > 0;
     hs[i]->prm.roomy_batch = roomy;
-    if (!own[i]) hs[i]->prm.persistent = 0;  // escalated FP64 solves run the graph form: no cooperative launch beside the batch
+    hs[i]->prm.in_batch = true;              // the setup of an escalation makes no cooperative launch beside the batch
+    if (!own[i]) hs[i]->prm.persistent = 0;  // and its solve runs the graph form
     hs[i]->prm.autotune = 0;    // the per-handle tuner replays kernels on a running state: not beside the batch
   }
   struct Group {
@@ -596,7 +597,7 @@ static int solve_batch_fused(pdnqp_t *const *hs, int count, double eps_abs, doub
   for (int i = 0; i < count; ++i) {
     hs[i]->prm.persistent = keep[i];
     hs[i]->prm.autotune = keep_tune[i];
-    hs[i]->prm.roomy_batch = false;
+    hs[i]->prm.roomy_batch = hs[i]->prm.in_batch = false;
   }
   if (rc < 0) return fail(nullptr, rc, "batch: " + err);
   int worst = 0;
@@ -641,8 +642,10 @@ int pdnqp_solve_batch(pdnqp_t *const *hs, int count, double eps_abs, double eps_
       pdnqp_t *h = hs[order[k]];
       const int keep = h->prm.persistent;
       h->prm.persistent = 0;  // graph form: no concurrent cooperative launches
+      h->prm.in_batch = true;
       const int rc = pdnqp_solve(h, eps_abs, eps_rel);
       h->prm.persistent = keep;
+      h->prm.in_batch = false;
       rcs[order[k]] = rc;
       if (rc < 0) {
         std::lock_guard<std::mutex> lk(err_mu);

@@ -117,7 +117,8 @@ __global__ void k_mul_scalar(double *p, long long n, double a) {
   PDNQP_GRID_STRIDE(i, n) p[i] *= a;
 }
 // ---------------------------------------------------------------------------
-// Lanczos (Eq. R-choice): both starts in one cooperative launch.
+// Lanczos (Eq. R-choice): both starts together, in one cooperative launch or in a
+// launch per phase.
 // ---------------------------------------------------------------------------
 // i-th output of the splitmix64 generator seeded with `seed`, mapped to [-0.5, 0.5).
 __device__ __forceinline__ double splitmix_uniform(uint64_t seed, uint64_t i) {
@@ -134,39 +135,55 @@ constexpr int kLzFull = 1024;    // up to this size every step is orthogonalised
 // matrix differs from that of exact arithmetic by its square).
 constexpr double kLzOmega = 1e-10;
 
-// Runs of `steps` Lanczos steps on the symmetric matrix Q from two start
-// vectors (seeds 1 and 2) side by side: out[s][0] = steps taken, then the
-// diagonal and the off-diagonal entries (kLzMax each).  V: [2][steps + 1][n]
-// basis vectors, w: [2][n].
+// Coefficients and recurrences of the two runs: every block forms its own copy, all
+// the same, from the block partials.
+struct LzState {
+  double al[2][kLzMax], be[2][kLzMax], om[2][3][kLzMax + 2];  // om: rows j - 1, j, j + 1 by j mod 3
+  int used[2], active[2], force[2], doit[2], done[2];         // done[0]: both runs have ended
+};
+// Phases: start vectors, their norms, then for every step the product, the
+// recurrence, the loss of orthogonality with the sums of the orthogonalisation,
+// its subtraction, and its end.
+enum : int { kLzStart, kLzNorms, kLzProduct, kLzRecur, kLzLoss, kLzSubtract, kLzEnd };
+
+// Lanczos runs of `steps` steps on the symmetric matrix Q from the start vectors
+// of the seeds first + 1 .. first + ns (1 or 2 runs): out[s][0] = steps taken, then
+// the diagonal and the off-diagonal entries (kLzMax each).  V: [ns][steps + 1][n]
+// basis vectors, w: [ns][n].
 //
 // The basis is kept semi-orthogonal by partial reorthogonalisation (H. D.
 // Simon, Math. Comp. 42, 1984): the recurrence for the loss of orthogonality
 // runs along with the coefficients, and a step and the next one are
 // orthogonalised against the whole basis only when it passes kLzOmega.  Twice
 // orthogonalising every step reads the basis 4 times a step and needs 4 n j
-// FP64 multiply-adds, 8 ms at n = 300,000 for the pipe alone.  One launch
-// instead of 128 x 12 with 256 host synchronisations: the sums that a step
-// needs are formed by every block from the block partials (fixed order, the
-// same in all blocks), so a step is 3 grid barriers.  Measured (n = 300,001, 64
-// steps): see Solver::lanczos.
-template <int K>
-__global__ void __launch_bounds__(kLzThreads, 1) k_lanczos(Mat<double> Q, int steps, double *V, double *w, double *part,
-                                                           unsigned *bar, double *out) {
+// FP64 multiply-adds, 8 ms at n = 300,000 for the pipe alone.  The sums that a
+// step needs are formed by every block from the block partials (fixed order, the
+// same in all blocks).
+//
+// COOP: all phases in one cooperative launch, a step is 3 grid barriers.  Else a
+// launch is one phase (phase, step j0), the state goes from launch to launch
+// through state[2] (read from one, written to the other, by the parity of the
+// launch's number), and a phase with nothing to do returns: 5 launches a step
+// without a host synchronisation, for devices without cooperative launches and
+// beside other solves.  The same sums in the same order: the same results.
+// Measured: see Solver::lanczos.
+template <int K, bool COOP>
+__global__ void __launch_bounds__(kLzThreads, 1) k_lanczos(Mat<double> Q, int first, int ns, int steps, double *V,
+                                                           double *w, double *part, unsigned *bar, double *out,
+                                                           LzState *state, int phase, int j0, int number) {
   constexpr int NW = kLzThreads / 32;
-  __shared__ double al[2][kLzMax], be[2][kLzMax], om[2][3][kLzMax + 2];  // om: rows j - 1, j, j + 1 by j mod 3
+  __shared__ LzState S;
   __shared__ double red[NW][32], tot[2][kLzMax];
-  __shared__ int used[2], active[2], force[2], doit[2];
   extern __shared__ __align__(16) unsigned char slots[];
   const long long n = Q.nrows;
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5, nb = gridDim.x;
   Slot<double> *buf = reinterpret_cast<Slot<double> *>(slots) + wid * kTileSlots;
-  unsigned gen = t == 0 ? ld_acquire_gpu(bar + kBarGen) : 0u;
+  unsigned gen = COOP && t == 0 ? ld_acquire_gpu(bar + kBarGen) : 0u;
   const long long e0 = (long long)blockIdx.x * kLzThreads + t, es = (long long)nb * kLzThreads;
   const WarpItems it;
   constexpr int TR = TileIter<K>::TR;
   const long long tiles = (n + TR - 1) / TR;
-  auto sync = [&] { return loop_sync<false>(bar, gen) >= 0; };
-  // One sum per start: block partials to part, then after a barrier totals in tot[s][0].
+  // One sum per run: block partials to part, then after a barrier totals in tot[s][0].
   auto put2 = [&](double a, double b, double *dst) {
     double v[2] = {a, b};
     const double r = warp_halve<2, false>(v);
@@ -189,38 +206,37 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos(Mat<double> Q, int st
     __syncthreads();
   };
   double *pa = part, *pb = part + 2 * kMaxBlocks, *ph = part + 4 * kMaxBlocks;  // ph: [block][2][kLzMax]
-  if (t < 2) {
-    used[t] = 0;
-    active[t] = 1;
-    force[t] = 0;
-  }
-  // Normalised start vectors.
-  double s0 = 0.0, s1 = 0.0;
-  for (long long i = e0; i < n; i += es) {
-    const double a = splitmix_uniform(1ull, (uint64_t)i), b = splitmix_uniform(2ull, (uint64_t)i);
-    w[i] = a;
-    w[n + i] = b;
-    s0 += a * a;
-    s1 += b * b;
-  }
-  put2(s0, s1, pb);
-  if (!sync()) return;
-  get2(pb);
-  for (int s = 0; s < 2; ++s) {
-    const double f = 1.0 / sqrt(tot[s][0]);
-    for (long long i = e0; i < n; i += es) V[(size_t)s * (steps + 1) * n + i] = w[s * n + i] * f;
-  }
-  if (!sync()) return;
-  for (int j = 0; j < steps; ++j) {
-    // w = Q v_j and alpha_j = w . v_j.
-    double a[2] = {0.0, 0.0};
+  double a[2];
+  auto start = [&] {
+    if (t < 2) {
+      S.used[t] = S.force[t] = S.doit[t] = S.done[t] = 0;
+      S.active[t] = t < ns;
+    }
+    a[0] = a[1] = 0.0;
+    for (int s = 0; s < ns; ++s)
+      for (long long i = e0; i < n; i += es) {
+        const double v = splitmix_uniform((uint64_t)(first + 1 + s), (uint64_t)i);
+        w[s * n + i] = v;
+        a[s] += v * v;
+      }
+    put2(a[0], a[1], pb);
+  };
+  auto norms = [&] {  // normalised start vectors
+    get2(pb);
+    for (int s = 0; s < ns; ++s) {
+      const double f = 1.0 / sqrt(tot[s][0]);
+      for (long long i = e0; i < n; i += es) V[(size_t)s * (steps + 1) * n + i] = w[s * n + i] * f;
+    }
+  };
+  auto product = [&](int j) {  // w = Q v_j and alpha_j = w . v_j
+    a[0] = a[1] = 0.0;
     for (long long tile = it.first; tile < tiles; tile += it.step) {
       const long long i = tile * TR + lane;
       const bool ok = lane < TR && i < n;
       const int rb = ok ? __ldg(Q.rp + i) : 0, re = ok ? __ldg(Q.rp + i + 1) : 0;
 #pragma unroll
       for (int s = 0; s < 2; ++s)
-        if (active[s]) {
+        if (S.active[s]) {
           const double *v = V + ((size_t)s * (steps + 1) + j) * n;
           const MulLd<double> f{v};
           const double q = K == 16 ? tile_long_rows<false, double>(Q.ci, Q.val, rb, re, f)
@@ -232,19 +248,19 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos(Mat<double> Q, int st
         }
     }
     put2(a[0], a[1], pa);
-    if (!sync()) return;
+  };
+  auto recur = [&](int j) {  // w -= alpha_j v_j + beta_{j-1} v_{j-1}
     get2(pa);
-    if (t < 2 && active[t]) {
-      al[t][j] = tot[t][0];
-      used[t] = j + 1;
+    if (t < 2 && S.active[t]) {
+      S.al[t][j] = tot[t][0];
+      S.used[t] = j + 1;
     }
     __syncthreads();
-    // w -= alpha_j v_j + beta_{j-1} v_{j-1}.
     a[0] = a[1] = 0.0;
     for (int s = 0; s < 2; ++s)
-      if (active[s]) {
+      if (S.active[s]) {
         const double *v = V + ((size_t)s * (steps + 1) + j) * n;
-        const double aj = al[s][j], bj = j > 0 ? be[s][j - 1] : 0.0;
+        const double aj = S.al[s][j], bj = j > 0 ? S.be[s][j - 1] : 0.0;
         for (long long i = e0; i < n; i += es) {
           double x = w[s * n + i] - aj * v[i];
           if (j > 0) x -= bj * v[i - n];
@@ -253,111 +269,172 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos(Mat<double> Q, int st
         }
       }
     put2(a[0], a[1], pb);
-    if (!sync()) return;
+  };
+  // Loss of orthogonality of the new vector against v_0 .. v_{j-1}, a lane each;
+  // where it passes kLzOmega, h = V' w over 32 basis vectors at a time (a lane's 32
+  // sums are joined by halving).  True when there is any.
+  auto loss = [&](int j) {
     get2(pb);
-    // Loss of orthogonality of the new vector against v_0 .. v_{j-1}, a lane each.
-    if (wid < 2 && active[wid]) {
+    if (wid < 2 && S.active[wid]) {
       const int s = wid;
       const double b = sqrt(tot[s][0]), eps = 1.1102230246251565e-16;
-      const double *oj = om[s][j % 3], *om1 = om[s][(j + 2) % 3];
-      double *on = om[s][(j + 1) % 3];
+      const double *oj = S.om[s][j % 3], *om1 = S.om[s][(j + 2) % 3];
+      double *on = S.om[s][(j + 1) % 3];
       double worst = 0.0;
       for (int k = lane; k < j; k += 32) {
-        double x = be[s][k] * (k + 1 == j ? 1.0 : oj[k + 1]) + (al[s][k] - al[s][j]) * oj[k];
-        if (k > 0) x += be[s][k - 1] * oj[k - 1];
-        x -= be[s][j - 1] * (k + 1 == j ? 1.0 : om1[k]);
-        x = (x + copysign(eps * (be[s][k] + b), x)) / b;
+        double x = S.be[s][k] * (k + 1 == j ? 1.0 : oj[k + 1]) + (S.al[s][k] - S.al[s][j]) * oj[k];
+        if (k > 0) x += S.be[s][k - 1] * oj[k - 1];
+        x -= S.be[s][j - 1] * (k + 1 == j ? 1.0 : om1[k]);
+        x = (x + copysign(eps * (S.be[s][k] + b), x)) / b;
         on[k] = x;
         worst = fmax(worst, fabs(x));
       }
       worst = warp_max(worst);
       if (lane == 0) {
         on[j] = eps * sqrt((double)n);
-        doit[s] = n <= kLzFull || force[s] || !(worst < kLzOmega);
-        force[s] = doit[s] && !force[s];
-        be[s][j] = b;
+        S.doit[s] = n <= kLzFull || S.force[s] || !(worst < kLzOmega);
+        S.force[s] = S.doit[s] && !S.force[s];
+        S.be[s][j] = b;
       }
     } else if (wid < 2 && lane == 0) {
-      doit[wid] = 0;
+      S.doit[wid] = 0;
     }
     __syncthreads();
-    if (doit[0] | doit[1]) {
-      // h = V' w over 32 basis vectors at a time (a lane's 32 sums are joined by
-      // halving), then w -= V h.
-      for (int s = 0; s < 2; ++s)
-        if (doit[s])
-          for (int p0 = 0; p0 <= j; p0 += 32) {
-            double acc[32];
-#pragma unroll
-            for (int p = 0; p < 32; ++p) acc[p] = 0.0;
-            const double *v = V + ((size_t)s * (steps + 1) + p0) * n;
-            for (long long i = e0; i < n; i += es) {
-              const double x = w[s * n + i];
-#pragma unroll
-              for (int p = 0; p < 32; ++p)
-                if (p0 + p <= j) acc[p] += v[(size_t)p * n + i] * x;
-            }
-            const double r = warp_halve<32, false>(acc);
-            red[wid][lane] = r;
-            __syncthreads();
-            if (t < 32) {
-              double x = red[0][t];
-              for (int k = 1; k < NW; ++k) x += red[k][t];
-              if (p0 + t < kLzMax) ph[((size_t)blockIdx.x * 2 + s) * kLzMax + p0 + t] = x;
-            }
-            __syncthreads();
-          }
-      if (!sync()) return;
-      for (int s = 0; s < 2; ++s)
-        if (doit[s])
-          for (int p = t; p <= j; p += kLzThreads) {
-            double x = 0.0;
-            for (int b = 0; b < nb; ++b) x += __ldcg(ph + ((size_t)b * 2 + s) * kLzMax + p);
-            tot[s][p] = x;
-          }
-      __syncthreads();
-      a[0] = a[1] = 0.0;
-      for (int s = 0; s < 2; ++s)
-        if (doit[s]) {
-          const double *v = V + (size_t)s * (steps + 1) * n;
-          for (long long i = e0; i < n; i += es) {
-            double x = w[s * n + i];
-            for (int p = 0; p <= j; ++p) x -= tot[s][p] * v[(size_t)p * n + i];
-            w[s * n + i] = x;
-            a[s] += x * x;
-          }
-        }
-      __syncthreads();
-      put2(a[0], a[1], pa);
-      if (!sync()) return;
-      get2(pa);
-      if (t < 2 && doit[t]) be[t][j] = sqrt(tot[t][0]);
-      for (int s = 0; s < 2; ++s)
-        if (doit[s])
-          for (int k = t; k < j; k += kLzThreads) om[s][(j + 1) % 3][k] = 1.1102230246251565e-16;
-      __syncthreads();
-    }
-    if (t < 2 && active[t]) {
-      const double b = be[t][j];
-      if (b <= 1e-12 * (fabs(al[t][j]) + (j > 0 ? be[t][j - 1] : 0.0) + 1e-300)) active[t] = 0;
-    }
-    __syncthreads();
-    if (j == steps - 1 || !(active[0] | active[1])) break;
     for (int s = 0; s < 2; ++s)
-      if (active[s]) {
-        const double f = 1.0 / be[s][j];
+      if (S.doit[s])
+        for (int p0 = 0; p0 <= j; p0 += 32) {
+          double acc[32];
+#pragma unroll
+          for (int p = 0; p < 32; ++p) acc[p] = 0.0;
+          const double *v = V + ((size_t)s * (steps + 1) + p0) * n;
+          for (long long i = e0; i < n; i += es) {
+            const double x = w[s * n + i];
+#pragma unroll
+            for (int p = 0; p < 32; ++p)
+              if (p0 + p <= j) acc[p] += v[(size_t)p * n + i] * x;
+          }
+          const double r = warp_halve<32, false>(acc);
+          red[wid][lane] = r;
+          __syncthreads();
+          if (t < 32) {
+            double x = red[0][t];
+            for (int k = 1; k < NW; ++k) x += red[k][t];
+            if (p0 + t < kLzMax) ph[((size_t)blockIdx.x * 2 + s) * kLzMax + p0 + t] = x;
+          }
+          __syncthreads();
+        }
+    return (S.doit[0] | S.doit[1]) != 0;
+  };
+  auto subtract = [&](int j) {  // w -= V h
+    for (int s = 0; s < 2; ++s)
+      if (S.doit[s])
+        for (int p = t; p <= j; p += kLzThreads) {
+          double x = 0.0;
+          for (int b = 0; b < nb; ++b) x += __ldcg(ph + ((size_t)b * 2 + s) * kLzMax + p);
+          tot[s][p] = x;
+        }
+    __syncthreads();
+    a[0] = a[1] = 0.0;
+    for (int s = 0; s < 2; ++s)
+      if (S.doit[s]) {
+        const double *v = V + (size_t)s * (steps + 1) * n;
+        for (long long i = e0; i < n; i += es) {
+          double x = w[s * n + i];
+          for (int p = 0; p <= j; ++p) x -= tot[s][p] * v[(size_t)p * n + i];
+          w[s * n + i] = x;
+          a[s] += x * x;
+        }
+      }
+    __syncthreads();
+    put2(a[0], a[1], pa);
+  };
+  auto ended = [&](int j) {  // the norm and the orthogonality after the subtraction
+    get2(pa);
+    if (t < 2 && S.doit[t]) S.be[t][j] = sqrt(tot[t][0]);
+    for (int s = 0; s < 2; ++s)
+      if (S.doit[s])
+        for (int k = t; k < j; k += kLzThreads) S.om[s][(j + 1) % 3][k] = 1.1102230246251565e-16;
+    __syncthreads();
+  };
+  auto next = [&](int j) {  // v_{j+1}; false (and the coefficients in out) when the runs have ended
+    if (t < 2 && S.active[t]) {
+      const double b = S.be[t][j];
+      if (b <= 1e-12 * (fabs(S.al[t][j]) + (j > 0 ? S.be[t][j - 1] : 0.0) + 1e-300)) S.active[t] = 0;
+    }
+    __syncthreads();
+    if (j == steps - 1 || !(S.active[0] | S.active[1])) {
+      if (blockIdx.x == 0 && t < ns) {
+        double *o = out + t * (2 * kLzMax + 1);
+        o[0] = S.used[t];
+        for (int k = 0; k < S.used[t]; ++k) {
+          o[1 + k] = S.al[t][k];
+          o[1 + kLzMax + k] = S.be[t][k];
+        }
+      }
+      return false;
+    }
+    for (int s = 0; s < 2; ++s)
+      if (S.active[s]) {
+        const double f = 1.0 / S.be[s][j];
         double *v = V + ((size_t)s * (steps + 1) + j + 1) * n;
         for (long long i = e0; i < n; i += es) v[i] = w[s * n + i] * f;
       }
+    return true;
+  };
+  if (COOP) {
+    auto sync = [&] { return loop_sync<false>(bar, gen) >= 0; };
+    start();
     if (!sync()) return;
-  }
-  if (blockIdx.x == 0 && t < 2) {
-    double *o = out + t * (2 * kLzMax + 1);
-    o[0] = used[t];
-    for (int k = 0; k < used[t]; ++k) {
-      o[1 + k] = al[t][k];
-      o[1 + kLzMax + k] = be[t][k];
+    norms();
+    if (!sync()) return;
+    for (int j = 0; j < steps; ++j) {
+      product(j);
+      if (!sync()) return;
+      recur(j);
+      if (!sync()) return;
+      if (loss(j)) {
+        if (!sync()) return;
+        subtract(j);
+        if (!sync()) return;
+        ended(j);
+      }
+      if (!next(j)) return;
+      if (!sync()) return;
     }
+  } else {
+    constexpr int words = sizeof(LzState) / 4;
+    int *const mine = reinterpret_cast<int *>(&S);
+    if (phase != kLzStart) {
+      const int *src = reinterpret_cast<const int *>(state + (number & 1));
+      for (int i = t; i < words; i += kLzThreads) mine[i] = src[i];
+    }
+    __syncthreads();
+    bool more = true;
+    if (phase == kLzStart) {
+      start();
+    } else if (phase == kLzNorms) {
+      norms();
+    } else if (!S.done[0]) {
+      const bool any = (S.doit[0] | S.doit[1]) != 0;
+      __syncthreads();  // read before loss() sets them
+      if (phase == kLzProduct) {
+        product(j0);
+      } else if (phase == kLzRecur) {
+        recur(j0);
+      } else if (phase == kLzLoss) {
+        if (!loss(j0)) more = next(j0);
+      } else if (any && phase == kLzSubtract) {
+        subtract(j0);
+      } else if (any) {
+        ended(j0);
+        more = next(j0);
+      }
+    }
+    __syncthreads();
+    if (t == 0 && !more) S.done[0] = 1;
+    __syncthreads();
+    if (blockIdx.x == 0)
+      for (int i = t; i < words; i += kLzThreads) reinterpret_cast<int *>(state + ((number + 1) & 1))[i] = mine[i];
   }
 }
 

@@ -63,6 +63,7 @@ struct Params {
   int autotune = 0;            // 1: time the lanes-per-row choices of the graph form once, keep the fastest
   int escalate = 1;            // FP32-bulk: continue in FP64 after a NUMERICAL_ERROR
   int batch_fused = 1;         // pdnqp_solve_batch: 1 = one batched graph for all inner loops, 0 = thread pool
+  bool in_batch = false;       // one of the solves of a batch (set for the call): no cooperative launch beside the others
   bool roomy_batch = false;    // in a batch whose clusters all find room at once (set for the call)
   int batch_chunk = 16;        // trial slots per launch of the batched graph
 };

@@ -386,7 +386,7 @@ class Solver : public SolverBase {
     }
     PDNQP_CK(cudaGetLastError());
     // ---- gamma (Eq. R-choice): two Lanczos starts, the smaller estimate.
-    PDNQP_TRY(lanczos(prm.lanczos_steps, &lam_min_));
+    PDNQP_TRY(lanczos(prm, &lam_min_));
     gamma_ = prm.gamma_override > 0 ? prm.gamma_override
                                      : 1.0 / (std::max(0.0, -lam_min_) + prm.delta_gamma * std::max(1.0, qnorm_));
     // H = Qbar + gamma^-1 I
@@ -400,64 +400,106 @@ class Solver : public SolverBase {
   }
 
   // The smaller of the smallest Ritz values of two Lanczos runs on the scaled Q
-  // (k_lanczos; gamma is not yet added to Hd_).
-  int lanczos(int steps, double *out) {
+  // (k_lanczos; gamma is not yet added to Hd_).  One cooperative launch, or, on
+  // devices without them and beside the other solves of a batch (a grid that takes
+  // every SM at once would wait for them all, and they for it), a launch per phase.
+  // The two runs go side by side; where their two bases (1,040 bytes a variable at
+  // 64 steps) find no room, one after the other in half of that.  Measured (n =
+  // 300,001, 64 steps, the whole device setup): 8.3 ms in one launch, 57 ms with
+  // every step orthogonalised twice and a host synchronisation a sum.
+  int lanczos(const Params &prm, double *out) {
     const long long n = n_;
     if (n == 0) {
       *out = 0.0;
       return 0;
     }
-    const int k = (int)std::min<long long>(std::min(steps, kLzMax - 1), n);
-    int dev = 0, sms = 0;
+    const int k = (int)std::min<long long>(std::min(prm.lanczos_steps, kLzMax - 1), n);
+    int dev = 0, sms = 0, can = 0;
     PDNQP_CK(cudaGetDevice(&dev));
     PDNQP_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    PDNQP_CK(cudaDeviceGetAttribute(&can, cudaDevAttrCooperativeLaunch, dev));
     const int nb = (int)std::min<long long>(std::min(sms, kMaxBlocks), (n + 255) / 256);
-    // Basis and sums of this call only.
-    double *V = nullptr;
-    const size_t nV = 2 * (size_t)(k + 1) * n, nw = 2 * (size_t)n, np = 4 * (size_t)kMaxBlocks + (size_t)nb * 2 * kLzMax,
-                 no = 2 * (2 * kLzMax + 1);
-    if (cudaMalloc(&V, (nV + nw + np + no) * sizeof(double) + kBarWords * sizeof(unsigned)) != cudaSuccess) {
-      last_err_ = "cudaMalloc: Lanczos basis";
-      cudaGetLastError();
-      return PDNQP_ERR_OOM;
-    }
-    double *w = V + nV, *part = w + nw, *res = part + np;
-    unsigned *bar = (unsigned *)(res + no);
-    const int rc = lanczos_run(k, nb, V, w, part, bar, res, no, out);
-    cudaFree(V);
-    return rc;
-  }
-  int lanczos_run(int k, int nb, double *V, double *w, double *part, unsigned *bar, double *res, size_t no, double *out) {
-    PDNQP_CK(cudaMemsetAsync(bar, 0, kBarWords * sizeof(unsigned), s_));
-    int rc = 0;
-    with_G(gN_, [&](auto GG) {
-      auto fn = k_lanczos<decltype(GG)::value>;
-      const int smem = kLzThreads / 32 * kTileSlots * (int)sizeof(Slot<double>);
-      cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      void *args[] = {(void *)&Hd_, (void *)&k, (void *)&V, (void *)&w, (void *)&part, (void *)&bar, (void *)&res};
-      if (e == cudaSuccess)
-        e = cudaLaunchCooperativeKernel((const void *)fn, dim3(nb), dim3(kLzThreads), args, smem, s_);
-      if (e != cudaSuccess) {
-        last_err_ = std::string("k_lanczos: ") + cudaGetErrorString(e);
-        rc = PDNQP_ERR_CUDA;
+    LanczosArgs a;
+    a.steps = k;
+    a.nb = nb;
+    a.coop = can && !prm.in_batch;
+    for (a.ns = 2; a.ns >= 1; --a.ns) {
+      // Bases and sums of this call only.
+      const size_t nV = (size_t)a.ns * (k + 1) * n, nw = (size_t)a.ns * n,
+                   np = 4 * (size_t)kMaxBlocks + (size_t)nb * 2 * kLzMax;
+      if (cudaMalloc(&a.V, (nV + nw + np + kLzOut) * sizeof(double) + 2 * sizeof(LzState) + kBarWords * sizeof(unsigned)) !=
+          cudaSuccess) {
+        cudaGetLastError();
+        continue;
       }
+      a.w = a.V + nV;
+      a.part = a.w + nw;
+      a.res = a.part + np;
+      a.state = (LzState *)(a.res + kLzOut);
+      a.bar = (unsigned *)(a.state + 2);
+      int rc = 0;
+      *out = INFINITY;
+      for (a.first = 0; a.first < 2 && rc == 0; a.first += a.ns) rc = lanczos_run(a, out);
+      cudaFree(a.V);
+      return rc;
+    }
+    last_err_ = "cudaMalloc: Lanczos basis";
+    return PDNQP_ERR_OOM;
+  }
+  static constexpr size_t kLzOut = 2 * (2 * kLzMax + 1);
+  struct LanczosArgs {
+    int first, ns, steps, nb;
+    bool coop;
+    double *V, *w, *part, *res;
+    LzState *state;
+    unsigned *bar;
+  };
+  // One launch, or the launches of all phases, and the smallest Ritz value into *best.
+  int lanczos_run(LanczosArgs &a, double *best) {
+    PDNQP_CK(cudaMemsetAsync(a.bar, 0, kBarWords * sizeof(unsigned), s_));
+    cudaError_t e = cudaSuccess;
+    with_G(gN_, [&](auto GG) {
+      constexpr int K = decltype(GG)::value;
+      const int smem = kLzThreads / 32 * kTileSlots * (int)sizeof(Slot<double>);
+      int phase = kLzStart, j = 0, number = 0;
+      void *args[] = {(void *)&Hd_, (void *)&a.first, (void *)&a.ns,  (void *)&a.steps, (void *)&a.V,   (void *)&a.w, (void *)&a.part,
+                      (void *)&a.bar, (void *)&a.res, (void *)&a.state, (void *)&phase,   (void *)&j, (void *)&number};
+      if (a.coop) {
+        auto fn = k_lanczos<K, true>;
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess)
+          e = cudaLaunchCooperativeKernel((const void *)fn, dim3(a.nb), dim3(kLzThreads), args, smem, s_);
+        return;
+      }
+      auto fn = k_lanczos<K, false>;
+      e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      auto launch = [&](int ph) {
+        phase = ph;
+        if (e == cudaSuccess) e = cudaLaunchKernel((const void *)fn, dim3(a.nb), dim3(kLzThreads), args, smem, s_);
+        ++number;
+      };
+      launch(kLzStart);
+      launch(kLzNorms);
+      for (j = 0; j < a.steps; ++j)
+        for (int ph : {kLzProduct, kLzRecur, kLzLoss, kLzSubtract, kLzEnd}) launch(ph);
     });
-    if (rc) return rc;
-    std::vector<double> h(no);
+    if (e != cudaSuccess) {
+      last_err_ = std::string("k_lanczos: ") + cudaGetErrorString(e);
+      return PDNQP_ERR_CUDA;
+    }
+    std::vector<double> h(kLzOut);
     unsigned fault = 0;
-    PDNQP_CK(cudaMemcpyAsync(h.data(), res, no * sizeof(double), cudaMemcpyDeviceToHost, s_));
-    PDNQP_CK(cudaMemcpyAsync(&fault, bar + kBarFault, sizeof(fault), cudaMemcpyDeviceToHost, s_));
+    PDNQP_CK(cudaMemcpyAsync(h.data(), a.res, kLzOut * sizeof(double), cudaMemcpyDeviceToHost, s_));
+    PDNQP_CK(cudaMemcpyAsync(&fault, a.bar + kBarFault, sizeof(fault), cudaMemcpyDeviceToHost, s_));
     PDNQP_CK(cudaStreamSynchronize(s_));
     if (fault) {
       last_err_ = "k_lanczos: grid barrier timed out";
       return PDNQP_ERR_CUDA;
     }
-    double best = INFINITY;
-    for (int s = 0; s < 2; ++s) {
+    for (int s = 0; s < a.ns; ++s) {
       const double *o = h.data() + s * (2 * kLzMax + 1);
-      best = std::min(best, tridiag_min(o + 1, o + 1 + kLzMax, (int)o[0]));
+      *best = std::min(*best, tridiag_min(o + 1, o + 1 + kLzMax, (int)o[0]));
     }
-    *out = best;
     return 0;
   }
 
