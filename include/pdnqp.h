@@ -164,12 +164,17 @@ PDNQP_API int pdnqp_solve(pdnqp_t *h, double eps_abs, double eps_rel);
  * group), with every problem's acceptance test, periodic check, restart and
  * inner termination taken on the device; problems small enough for the cluster
  * form (see "persistent" below; up to 1,024 tiles and 700,000 gathers where the
- * GPU has 8 SMs for every problem; handles with persistent = 1) run their inner
- * loops in that form on their own streams beside the graph.  Each problem's
+ * GPU holds all clusters of 8 blocks that these limits make of the batch at once,
+ * some 16 to 18; handles with persistent = 1) run their inner loops in that form
+ * on their own streams beside the graph.  The other problems of the call so
+ * decide the form of one between the two limits, and with it the rounding of its
+ * sums; a problem within the smaller limits, or beyond the larger ones, has its
+ * form to itself.  Each problem's
  * outer iteration (Algorithm 3, Sec. 3.4's CPU side) runs on a host thread of
  * its own (one per problem; `threads` is not used), which sleeps while its inner
  * solve is in the graph.  A problem keeps its solo block partition, so its
- * results are bitwise those of its solo solve in the same form.  Thread-pool
+ * results are bitwise those of its solo solve in the same form (in the graph:
+ * persistent = 0; between the limits: of a batch of it alone).  Thread-pool
  * form (batch_fused = 0): `threads` host threads (0: min(count, 16)) run
  * pdnqp_solve on the problems, largest first, so their graph-form inner solves
  * overlap on the GPU.  The "autotune" parameter of every handle, and

@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -514,9 +515,15 @@ static int solve_batch_fused(pdnqp_t *const *hs, int count, double eps_abs, doub
   // Problems that fit the cluster form (a few SMs each, no cooperative launch) run
   // it on their own streams beside each other, at their own pace; the others
   // share the graph.
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const bool roomy = 8LL * count <= sms;  // 8 blocks a cluster, one per SM
+  // The larger limits hold where the GPU has room at once for every cluster of 8 that
+  // they would make (problems of one block and of the graph do not count).
+  int clusters = 0, room = INT_MAX;
+  for (int i = 0; i < count; ++i)
+    if (hs[i]->prm.persistent && hs[i]->solver->cluster_size(true) > 1) {
+      ++clusters;
+      room = std::min(room, hs[i]->solver->cluster_room());
+    }
+  const bool roomy = clusters <= room;
   std::vector<int> keep(count), keep_tune(count), own(count);
   for (int i = 0; i < count; ++i) {
     keep[i] = hs[i]->prm.persistent;

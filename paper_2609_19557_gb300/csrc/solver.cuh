@@ -64,7 +64,7 @@ struct Params {
   int escalate = 1;            // FP32-bulk: continue in FP64 after a NUMERICAL_ERROR
   int batch_fused = 1;         // pdnqp_solve_batch: 1 = one batched graph for all inner loops, 0 = thread pool
   bool in_batch = false;       // one of the solves of a batch (set for the call): no cooperative launch beside the others
-  bool roomy_batch = false;    // in a batch whose clusters all find room at once (set for the call)
+  bool roomy_batch = false;    // in a batch whose clusters of 8 all find room at once (set for the call)
   int batch_chunk = 16;        // trial slots per launch of the batched graph
 };
 
@@ -95,6 +95,7 @@ class SolverBase {
   virtual int replay(int which, int reps) = 0;
   virtual int tuned_g(int which) const = 0;
   virtual int cluster_size(bool roomy) const = 0;  // blocks of the cluster form, 0: too large for it
+  virtual int cluster_room() const = 0;            // its clusters of 8 blocks that the GPU holds at once
   virtual double kernel_bytes(int which) const = 0;
   virtual double last_replay_ms() const = 0;
   virtual int jam_barrier() = 0;  // failure-detection self-test: the next launches' grid barrier never completes

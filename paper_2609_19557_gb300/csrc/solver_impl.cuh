@@ -801,19 +801,34 @@ class Solver : public SolverBase {
     // cluster of 4 takes 10.1 us a trial, a block 9.9).
     return tiles <= 16 ? 1 : 8;
   }
-  template <typename... P, typename... A>
-  int launch_cluster(void (*fn)(P...), int nb, unsigned smem, A... args) {
+  // A cluster lies inside one GPC, so the GPU holds fewer of them than its SMs over 8.
+  int cluster_room() const override {
+    int room = 0;
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = cluster_config(8, trials_smem_bytes<T>(), &at);
+    if (cudaOccupancyMaxActiveClusters(&room, trials_clu_fn(), &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    return room;
+  }
+  cudaLaunchConfig_t cluster_config(int nb, unsigned smem, cudaLaunchAttribute *at) const {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nb);
     cfg.blockDim = dim3(kTrialThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s_;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = nb;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = nb;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
+    return cfg;
+  }
+  template <typename... P, typename... A>
+  int launch_cluster(void (*fn)(P...), int nb, unsigned smem, A... args) {
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = cluster_config(nb, smem, &at);
     PDNQP_CK(cudaLaunchKernelEx(&cfg, fn, args...));
     return 0;
   }
