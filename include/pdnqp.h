@@ -253,7 +253,8 @@ PDNQP_API int pdnqp_set_start(pdnqp_t *h, const double *x0, const double *y0);
  * batch_graph_seconds, batch_graph_launches, batch_kernel_launches and
  * batch_size (the last fused pdnqp_solve_batch over this handle's precision
  * group: device time of its graph launches, their number, the batched
- * kernels they ran and the group's problem count),
+ * kernels they ran and the group's problem count; all 0 for a problem that ran in
+ * the cluster form),
  * rebases (FP32-bulk: inner solves of the last solve that ended at the
  * rejection limit and were continued from the last accepted point as a new
  * FP64 base instead of ending the solve, see pdnqp_solve).

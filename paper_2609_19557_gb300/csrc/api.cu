@@ -539,6 +539,11 @@ static int solve_batch_fused(pdnqp_t *const *hs, int count, double eps_abs, doub
     std::unique_ptr<pdq::BatchBase> batch;
   };
   Group groups[2];  // FP64, FP32-bulk
+  for (int i = 0; i < count; ++i) {  // nothing of an earlier batch; a problem in the cluster form has no graph
+    hs[i]->batch_graph_seconds = 0.0;
+    hs[i]->batch_graph_launches = hs[i]->batch_kernel_launches = 0;
+    hs[i]->batch_size = 0;
+  }
   for (int i = 0; i < count; ++i)
     if (!own[i]) groups[hs[i]->precision == PDNQP_FP32_BULK ? 1 : 0].idx.push_back(i);
   std::string err;
