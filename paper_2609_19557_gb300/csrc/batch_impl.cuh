@@ -88,7 +88,7 @@ class BatchRunner : public BatchBase, public BatchHook {
     auto all = [](int) { return true; };
     BTRY(add_map(&primal_, map_of([&](int i) { return sv_[i]->grid_n(); }, all)));
     BTRY(add_map(&apply_, map_of([&](int i) { return sv_[i]->grid_nm(); }, all)));
-    for (int g : {4, 8, 16}) {
+    for (int g : {8, 16}) {
       Launch r, c;
       r.g = c.g = g;
       BTRY(add_map(&r, map_of([&](int i) { return sv_[i]->nb_rows(g); }, [&](int i) { return lanes(g_rows_[i]) == g; })));
@@ -203,8 +203,6 @@ class BatchRunner : public BatchBase, public BatchHook {
     BatchBlk *map = nullptr;
   };
 
-  // The setting that with_G makes of a lane parameter.
-  static int lanes(int g) { return g == 4 || g == 8 ? g : 16; }
   int fail(const std::string &m) {
     err_ = m;
     return PDNQP_ERR_CUDA;

@@ -784,8 +784,8 @@ struct MaxAbs {
 };
 
 // Row reduction of a warp tile (TileIter<K>); lane l gets row tile + l.  K: the
-// matrix's lane setting, 16 = long rows (8 rows, all 32 lanes on each), 4 or 8
-// = short rows (32 rows).
+// matrix's lane setting, 16 = long rows (8 rows, all 32 lanes on each), 8 = short
+// rows (32 rows).
 template <int K, bool IsMax, typename Acc, typename T, typename F>
 __device__ __forceinline__ Acc tile_reduce(const int *rp, const int *ci, const T *val, long long tile, long long nrows,
                                            const F &f, Slot<Acc> *buf) {

@@ -26,15 +26,15 @@ namespace pdq {
     if (_r < 0) return _r;    \
   } while (0)
 
-// The lane setting of a matrix (tile_reduce): 16 spreads a warp along each row,
-// 4 and 8 take tiles of 32 short rows.
+// The lane setting of a matrix (tile_reduce): 16 spreads a warp along each row, 8
+// (and the parameter's 4) takes tiles of 32 short rows.
+static int lanes(int g) { return g == 4 || g == 8 ? 8 : 16; }
 template <typename F>
 static void with_G(int g, F f) {
-  switch (g) {
-    case 4: f(std::integral_constant<int, 4>()); break;
-    case 8: f(std::integral_constant<int, 8>()); break;
-    default: f(std::integral_constant<int, 16>()); break;
-  }
+  if (lanes(g) == 8)
+    f(std::integral_constant<int, 8>());
+  else
+    f(std::integral_constant<int, 16>());
 }
 
 // From the mean row length: rounds of 8 entries a row pay until a row fills most
@@ -898,12 +898,12 @@ class Solver : public SolverBase {
 
   // Row-binning autotuner of the graph form: replays the row kernel and the
   // column kernel (each captured as a graph of kTuneReps launches, on the
-  // state of the first inner solve) for every lanes-per-row choice, and makes
+  // state of the first inner solve) for both lane settings, and makes
   // the fastest the default of this handle.  Replays write trial buffers only
   // and restore the device state.
   int autotune_g() {
     static constexpr int kTuneReps = 20;
-    const int cand[3] = {4, 8, 16};
+    const int cand[2] = {8, 16};
     const int gA = gA_, gN = gN_;
     double best[2] = {INFINITY, INFINITY};
     int pick[2] = {gA, gN};
