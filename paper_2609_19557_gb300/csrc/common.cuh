@@ -277,8 +277,12 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[NQ], double *part
   __syncthreads();
 }
 
-// Polls of a grid barrier before it gives up (about a second or more).
+// Polls of a grid barrier before it gives up (about two seconds).
 constexpr unsigned kSpinLimit = 1u << 22;
+// The same for a launch in which one warp may go through a row of `longest` entries
+// while the other blocks wait: in entry order (one_row) that takes 64 cycles an
+// entry, and a poll, a round trip to L2, takes some 250 at least.
+__host__ __device__ constexpr unsigned spin_limit(long long longest) { return kSpinLimit + (unsigned)(longest / 2); }
 
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned *p) {
   unsigned v;
@@ -309,7 +313,7 @@ __device__ __forceinline__ void cluster_sync() {
 }
 // The barrier alone.
 template <bool CLU>
-__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen);
+__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, unsigned limit);
 
 // Grid barrier of a cooperative (co-resident) launch, the wait of every kernel
 // that spans blocks.  bar[0] counts the arrivals, bar[kBarGen] is the generation
@@ -321,8 +325,7 @@ __device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen);
 // caller's copy of the generation (thread 0), so a waiting block polls one word
 // and, every 64 polls, the fault flag (each is a round trip to L2).
 //
-// The wait is bounded: a block that polls kSpinLimit times without a release, or
-// that sees the fault flag, sets the flag and gets -1; the caller then leaves the
+// The wait is bounded: a block that polls `limit` times without a release, or that sees the fault flag, sets the flag and gets -1; the caller then leaves the
 // kernel, so a barrier that can never complete ends the launch instead of hanging
 // it.
 //
@@ -331,7 +334,7 @@ __device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen);
 // where the grid barrier takes 1.5 to 2.5); block 0 runs lead(), and no message
 // comes back.
 template <bool CLU, typename F>
-__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, F lead) {
+__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, unsigned limit, F lead) {
   __shared__ int role;  // message, -1 fault, 2 leader
   __syncthreads();
   if (gridDim.x == 1) {
@@ -355,7 +358,7 @@ __device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, F lead) {
     } else {
       unsigned it = 0, v;
       while ((v = ld_acquire_gpu(bar + kBarGen)) == gen) {
-        if (++it > kSpinLimit || ((it & 63u) == 0u && ld_acquire_gpu(bar + kBarFault) != 0u)) {
+        if (++it > limit || ((it & 63u) == 0u && ld_acquire_gpu(bar + kBarFault) != 0u)) {
           atomicExch(bar + kBarFault, 1u);
           role = -1;
           break;
@@ -380,12 +383,12 @@ __device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, F lead) {
 }
 
 template <bool CLU>
-__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen) {
+__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, unsigned limit) {
   if (CLU && gridDim.x > 1) {
     cluster_sync();
     return 0;
   }
-  return loop_sync<CLU>(bar, gen, [] { return 0; });
+  return loop_sync<CLU>(bar, gen, limit, [] { return 0; });
 }
 
 // Single-block final reduction of NQ quantities over nb partials (fixed order):

@@ -291,6 +291,7 @@ class Solver : public SolverBase {
     mE_ = P.mE;
     nnzA_ = P.a_ci.size();
     nnzH_ = P.q_ci.size();
+    d_.spin = spin_limit(std::max(n_, m_));  // no row is longer
     PDNQP_TRY(dalloc(&st_, 1));
     PDNQP_CK(cudaMallocHost(&hst_, sizeof(DevState)));
     PDNQP_CK(cudaMallocHost(&hfault_, sizeof(unsigned)));
@@ -463,7 +464,8 @@ class Solver : public SolverBase {
       const int smem = kLzThreads / 32 * kTileSlots * (int)sizeof(Slot<double>);
       int phase = kLzStart, j = 0, number = 0;
       void *args[] = {(void *)&Hd_, (void *)&a.first, (void *)&a.ns,  (void *)&a.steps, (void *)&a.V,   (void *)&a.w, (void *)&a.part,
-                      (void *)&a.bar, (void *)&a.res, (void *)&a.state, (void *)&phase,   (void *)&j, (void *)&number};
+                      (void *)&a.bar, (void *)&a.res, (void *)&a.state, (void *)&phase,   (void *)&j, (void *)&number,
+                      (void *)&d_.spin};
       if (a.coop) {
         auto fn = k_lanczos<K, true>;
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
