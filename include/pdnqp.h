@@ -159,8 +159,9 @@ PDNQP_API int pdnqp_solve(pdnqp_t *h, double eps_abs, double eps_rel);
  * (Eq. outer-termination with eps_abs / eps_rel), restarts and limits.
  * Fused form (parameter batch_fused = 1 on hs[0], the default; handles on one
  * device): the inner iterations (Algorithm 4) of the problems of one precision
- * run together in one captured CUDA graph of batch_chunk trials and one periodic
- * check, one kernel launch per phase for the whole batch (per lanes-per-row
+ * run together in one captured CUDA graph of batch_chunk trials with periodic
+ * checks in between (where the smallest k_chk of the group puts them: at the
+ * defaults one at the end), one kernel launch per phase for the whole batch (per lanes-per-row
  * group), with every problem's acceptance test, periodic check, restart and
  * inner termination taken on the device; problems small enough for the cluster
  * form (see "persistent" below; up to 1,024 tiles and 700,000 gathers where the

@@ -553,14 +553,17 @@ static int solve_batch_fused(pdnqp_t *const *hs, int count, double eps_abs, doub
     if (G.idx.empty()) continue;
     std::vector<SolverBase *> sv;
     std::vector<int> gr, gc;
+    int k_chk = INT_MAX;
     for (int i : G.idx) {
       pdnqp_t *h = hs[i];
       sv.push_back(h->solver);
       gr.push_back(h->prm.g_rows > 0 ? h->prm.g_rows : h->solver->tuned_g(1));
       gc.push_back(h->prm.g_cols > 0 ? h->prm.g_cols : h->solver->tuned_g(0));
+      k_chk = std::min(k_chk, h->prm.k_chk);
     }
     const int chunk = hs[G.idx[0]]->prm.batch_chunk;
-    G.batch.reset(g ? pdq::make_batch_f32(sv, gr, gc, chunk, &err) : pdq::make_batch_f64(sv, gr, gc, chunk, &err));
+    G.batch.reset(g ? pdq::make_batch_f32(sv, gr, gc, chunk, k_chk, &err)
+                    : pdq::make_batch_f64(sv, gr, gc, chunk, k_chk, &err));
     if (!G.batch) rc = PDNQP_ERR_CUDA;
   }
   std::vector<int> rcs(count, 0);

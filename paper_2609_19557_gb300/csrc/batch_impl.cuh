@@ -3,8 +3,8 @@
 // keeps its own solver, device state and host thread for the outer
 // iteration (Algorithm 3, on the CPU as in Sec. 3.4); when its inner solve
 // is set up, its thread hands it here and sleeps.  The scheduler launches one
-// captured CUDA graph of `chunk` trials and one check over the whole batch, one
-// launch per phase (kernels.cuh, "Batched form"): every running problem takes its
+// captured CUDA graph of `chunk` trials, with checks in between, over the whole
+// batch, one launch per phase (kernels.cuh, "Batched form"): every running problem takes its
 // trial, its acceptance decision, its periodic check, restart and inner
 // termination on the device, and problems that are not running skip.  After
 // each graph launch one gather of all device states tells the scheduler
@@ -32,9 +32,27 @@ namespace pdq {
 template <typename T>
 class BatchRunner : public BatchBase, public BatchHook {
  public:
-  BatchRunner(std::vector<Solver<T> *> sv, std::vector<int> g_rows, std::vector<int> g_cols, int chunk)
+  BatchRunner(std::vector<Solver<T> *> sv, std::vector<int> g_rows, std::vector<int> g_cols, int chunk, int k_chk)
       : sv_(std::move(sv)), g_rows_(std::move(g_rows)), g_cols_(std::move(g_cols)),
-        chunk_(std::max(1, chunk)) {}
+        chunk_(std::max(1, chunk)), every_(check_spacing(chunk_, std::max(1, k_chk))) {}
+
+  // Trials between two checks of the graph: of the divisors of chunk the one with
+  // the shortest check period of k trials, which ends at the next check (the trials
+  // up to it are idle) and pays for the checks on the way, 1/16 of a trial each.
+  // That is all of them at the defaults (k_chk 64, chunk 16: one check a launch), k_chk
+  // where it divides chunk, 1 for k_chk = 1.  Measured below, at launch_check.
+  static int check_spacing(int chunk, int k) {
+    int best = 1;
+    double least = INFINITY;
+    for (int e = 1; e <= chunk; ++e) {
+      const double t = chunk % e ? INFINITY : ((k + e - 1) / e) * (e + 1.0 / 16.0);
+      if (t < least) {
+        least = t;
+        best = e;
+      }
+    }
+    return best;
+  }
 
   ~BatchRunner() override {
     for (Solver<T> *s : sv_) {
@@ -100,12 +118,14 @@ class BatchRunner : public BatchBase, public BatchHook {
     BTRY(dalloc(&dlist_, (size_t)2 * P));
     BK(cudaMallocHost(&hstates_, sizeof(DevState) * (size_t)P));
     BK(cudaMallocHost(&hlist_, sizeof(int) * (size_t)2 * P));
-    // The graph: chunk trials [primal, rows, cols (+ decisions)], then one check
-    // [rows, cols (+ decisions), apply] over the whole batch.
+    // The graph: chunk trials [primal, rows, cols (+ decisions)], after every every_
+    // of them a check [rows, cols (+ decisions), apply], over the whole batch.
     cudaGraph_t g;
     BK(cudaStreamBeginCapture(bs_, cudaStreamCaptureModeThreadLocal));
-    for (int k = 0; k < chunk_; ++k) launch_trial();
-    launch_check();
+    for (int k = 1; k <= chunk_; ++k) {
+      launch_trial();
+      if (k % every_ == 0) launch_check();
+    }
     BK(cudaStreamEndCapture(bs_, &g));
     cudaError_t e = cudaGraphInstantiate(&gexec_, g, 0);
     cudaGraphDestroy(g);
@@ -227,11 +247,11 @@ class BatchRunner : public BatchBase, public BatchHook {
     return 0;
   }
 
-  // One trial over the batch, and one check (captured into the graph).  The check
-  // comes once a graph launch: an inner solve starts with a launch and its check
-  // period is a multiple of the default chunk, so that without rejections its
-  // checks fall due at the end of one; otherwise it waits for the end.  (Checks
-  // after every trial were 5 of 10 launches of a slot, nearly all idle.)
+  // One trial over the batch, and one check (captured into the graph).  A problem
+  // whose check is due waits for the next one: an inner solve starts with a launch,
+  // so that without rejections its checks fall due where the graph has one, and
+  // after a rejection it idles up to every_ - 1 trials a period.  (Checks after every
+  // trial are 3 to 5 of 6 to 10 launches a trial, nearly all idle.)
   void launch_trial() {
     kb_primal<T><<<primal_.nblk, kBlock, 0, bs_>>>(devs_, primal_.map);
     for (const Launch &L : rows_)
@@ -252,7 +272,7 @@ class BatchRunner : public BatchBase, public BatchHook {
   }
   long long kernels_per_launch() const {
     const long long g = (long long)(rows_.size() + cols_.size());
-    return chunk_ * (1 + g) + g + 1;
+    return (chunk_ + chunk_ / every_) * (1 + g);
   }
 
   // Scheduler edits, one graph launch, one read-back of all states.
@@ -284,7 +304,7 @@ class BatchRunner : public BatchBase, public BatchHook {
 
   std::vector<Solver<T> *> sv_;
   std::vector<int> g_rows_, g_cols_;
-  int chunk_;
+  int chunk_, every_;
   cudaStream_t bs_ = nullptr;
   cudaGraphExec_t gexec_ = nullptr;
   std::vector<void *> dmem_;
@@ -308,7 +328,7 @@ class BatchRunner : public BatchBase, public BatchHook {
 
 template <typename T>
 BatchBase *make_batch_impl(const std::vector<SolverBase *> &sv, const std::vector<int> &g_rows,
-                           const std::vector<int> &g_cols, int chunk, std::string *err) {
+                           const std::vector<int> &g_cols, int chunk, int k_chk, std::string *err) {
   std::vector<Solver<T> *> s;
   for (SolverBase *b : sv) {
     Solver<T> *p = dynamic_cast<Solver<T> *>(b);
@@ -318,7 +338,7 @@ BatchBase *make_batch_impl(const std::vector<SolverBase *> &sv, const std::vecto
     }
     s.push_back(p);
   }
-  BatchRunner<T> *r = new BatchRunner<T>(std::move(s), g_rows, g_cols, chunk);
+  BatchRunner<T> *r = new BatchRunner<T>(std::move(s), g_rows, g_cols, chunk, k_chk);
   if (r->build() < 0) {
     if (err) *err = r->error();
     delete r;

@@ -132,10 +132,11 @@ class BatchBase {
   virtual long long kernel_launches() const = 0;
 };
 // g_rows[i] / g_cols[i]: lanes per row of problem i's row and column passes
-// (the values its solo graph form would use).
+// (the values its solo graph form would use); k_chk: the problems' smallest check
+// period.
 BatchBase *make_batch_f64(const std::vector<SolverBase *> &sv, const std::vector<int> &g_rows,
-                          const std::vector<int> &g_cols, int chunk, std::string *err);
+                          const std::vector<int> &g_cols, int chunk, int k_chk, std::string *err);
 BatchBase *make_batch_f32(const std::vector<SolverBase *> &sv, const std::vector<int> &g_rows,
-                          const std::vector<int> &g_cols, int chunk, std::string *err);
+                          const std::vector<int> &g_cols, int chunk, int k_chk, std::string *err);
 
 }  // namespace pdq

@@ -7,7 +7,7 @@
 namespace pdq {
 SolverBase *make_solver_f32(cudaStream_t s) { return new Solver<float>(s); }
 BatchBase *make_batch_f32(const std::vector<SolverBase *> &sv, const std::vector<int> &g_rows,
-                          const std::vector<int> &g_cols, int chunk, std::string *err) {
-  return make_batch_impl<float>(sv, g_rows, g_cols, chunk, err);
+                          const std::vector<int> &g_cols, int chunk, int k_chk, std::string *err) {
+  return make_batch_impl<float>(sv, g_rows, g_cols, chunk, k_chk, err);
 }
 }  // namespace pdq
