@@ -95,6 +95,8 @@ class BatchRunner : public BatchBase, public BatchHook {
     }
     BTRY(upload(&devs_, devs));
     BTRY(upload(&nbr_, nbr));
+    kb_idle<T><<<(P + 255) / 256, 256, 0, bs_>>>(devs_, P);
+    BK(cudaGetLastError());
     // One block map per launch: the problem's solo partition.
     auto map_of = [&](auto nb_of, auto keep) {
       std::vector<BatchBlk> m;

@@ -1553,6 +1553,15 @@ __global__ void __launch_bounds__(kBlock) kb_check_apply(const Dev<T> *devs, con
   check_apply_body<T>(d, d.st, GridCtx{e.b, e.nb});
 }
 
+// Every problem idle, before the first graph launch: the graph runs as soon as one
+// problem is set up, when the host threads of others have not reached theirs yet,
+// and a handle may come from a debug run, which leaves its state running.
+template <typename T>
+__global__ void kb_idle(const Dev<T> *devs, int count) {
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < count; k += gridDim.x * blockDim.x)
+    devs[k].st->status = ST_IDLE;
+}
+
 // Scheduler edits between graph launches: problems in `go` that are set up
 // (ST_READY) start running; problems in `stop` that still run pause (their
 // time limit passed).

@@ -293,6 +293,14 @@ class Solver : public SolverBase {
     nnzH_ = P.q_ci.size();
     d_.spin = spin_limit(std::max(n_, m_));  // no row is longer
     PDNQP_TRY(dalloc(&st_, 1));
+    {
+      // Idle from the start: kernels of a batch look at the state before the first solve has written it.
+      DevState idle;
+      memset(&idle, 0, sizeof(idle));
+      idle.status = ST_IDLE;
+      reset_buffers(&idle);
+      PDNQP_CK(cudaMemcpyAsync(st_, &idle, sizeof(idle), cudaMemcpyHostToDevice, s_));
+    }
     PDNQP_CK(cudaMallocHost(&hst_, sizeof(DevState)));
     PDNQP_CK(cudaMallocHost(&hfault_, sizeof(unsigned)));
     *hfault_ = 0u;
