@@ -603,9 +603,9 @@ __global__ void __launch_bounds__(kBlock) k_outer_rows(Dev<T> d, Mat<double> Ad,
       spv = max_abs(spv, scale_of(hi));
       q[0] = max_abs(q[0], res_of(viol));
       q[1] = max_abs(q[1], spv);
-      const double idc = recip(Dc[j]);
-      q[2] = max_abs(q[2], res_of(viol * idc));
-      q[3] = max_abs(q[3], spv * idc);
+      const double dc = Dc[j];  // divisions: these are reported, and decide termination
+      q[2] = max_abs(q[2], res_of(viol / dc));
+      q[3] = max_abs(q[3], spv / dc);
     }
   }
   block_reduce_store<kOutRows, kOutRowsMask>(q, d.part);
@@ -624,7 +624,6 @@ __global__ void __launch_bounds__(kBlock) k_outer_cols(Dev<T> d, Mat<double> Hd,
   double q[kOutCols];
 #pragma unroll
   for (int k = 0; k < kOutCols; ++k) q[k] = 0.0;
-  const double ics = 1.0 / cs;
   TileIter<G> ti;
   for (long long tile = ti.first; tile < d.n; tile += ti.step) {
     const double hx = tile_row_sum<G, double>(Hd.rp, Hd.ci, Hd.val, tile, d.n, MulLdg<double>{x});
@@ -644,7 +643,7 @@ __global__ void __launch_bounds__(kBlock) k_outer_cols(Dev<T> d, Mat<double> Hd,
       q[5] = max_abs(q[5], res_of(xi - clampv<double>(xi - g, lo, hi)));
       const double sc = max_abs(max_abs(scale_of(qx), ci), scale_of(atl));
       q[6] = max_abs(q[6], sc);
-      const double f = ics * recip(dxi);
+      const double f = 1.0 / (cs * dxi);
       const double xo = dxi * xi, loo = lo * dxi, hio = hi * dxi, go = g * f;
       q[7] = max_abs(q[7], res_of(xo - clampv<double>(xo - go, loo, hio)));
       q[2] = max_abs(q[2], res_of(less_bits(xo, loo) ? loo - xo : (less_bits(hio, xo) ? xo - hio : 0.0)));
