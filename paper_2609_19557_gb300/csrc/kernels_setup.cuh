@@ -12,18 +12,6 @@
 namespace pdq {
 namespace {  // internal linkage: each solver TU owns its kernels
 
-// Reciprocal square root in the storage precision.  FP64: two Newton steps from
-// the FP32 value (8 FP64 instructions), outside FP32's range the library's.
-__device__ __forceinline__ float rsqrt_t(float v) { return rsqrtf(v); }
-__device__ __forceinline__ double rsqrt_t(double v) {
-  const float f = (float)v;
-  if (!(f > 1e-30f && f < 1e30f)) return rsqrt(v);
-  double r = widen(rsqrtf(f));
-  const double h = 0.5 * v;
-  r = fma(r, fma(-h * r, r, 0.5), r);
-  return fma(r, fma(-h * r, r, 0.5), r);
-}
-
 // A vector that entries multiply, and how they are added.
 struct AddSquares {
   template <typename Acc>

@@ -71,6 +71,13 @@ inline int __double2loint(double v) { return (int)warp_bits<uint64_t>(v); }
 inline double __hiloint2double(int h, int l) { return warp_bits<double>((uint64_t)(unsigned)h << 32 | (unsigned)l); }
 inline unsigned __float_as_uint(float v) { return warp_bits<unsigned>(v); }
 inline double __dmul_rn(double a, double b) { return a * b; }
+inline double rsqrt(double v) { return (double)(1.0L / sqrtl((long double)v)); }
+inline int rsqrtf_off = 0;  // CUDA's rsqrtf is within 2 units in the last place: the error to take, in units
+inline float rsqrtf(float v) {
+  float r = (float)(1.0 / std::sqrt((double)v));
+  for (int k = 0; k < std::abs(rsqrtf_off); ++k) r = std::nextafter(r, rsqrtf_off < 0 ? 0.0f : 4e38f);
+  return r;
+}
 inline size_t __cvta_generic_to_shared(const void *p) { return (size_t)p; }
 inline unsigned atomicAdd(unsigned *p, unsigned v) { return __atomic_fetch_add(p, v, __ATOMIC_SEQ_CST); }
 inline unsigned atomicExch(unsigned *p, unsigned v) { return __atomic_exchange_n(p, v, __ATOMIC_SEQ_CST); }
