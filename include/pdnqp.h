@@ -122,7 +122,11 @@ typedef struct {
  * proximal step gamma (Eq. R-choice, FP64 Lanczos).  Sizes: Q is n x n, c has
  * n entries, A is m x n (m may be 0; then A may be NULL), l_c/u_c have m
  * entries, l_x/u_x n entries.  On success *out owns all device memory and 0 is
- * returned; on failure *out is NULL and a negative code is returned. */
+ * returned; on failure *out is NULL and a negative code is returned.  The Lanczos
+ * estimate takes 528 bytes a variable (64 steps) for each of its two runs during the
+ * call (one run at a time where both find no room).  Several threads
+ * may create handles at once: the estimates are cooperative launches, which CUDA
+ * starts when all their blocks find room, so they take turns. */
 PDNQP_API int pdnqp_create(pdnqp_t **out, const pdnqp_csr *Q, const double *c, const pdnqp_csr *A, const double *l_c,
                  const double *u_c, const double *l_x, const double *u_x);
 PDNQP_API int pdnqp_create_ex(pdnqp_t **out, const pdnqp_csr *Q, const double *c, const pdnqp_csr *A, const double *l_c,
@@ -226,10 +230,11 @@ PDNQP_API int pdnqp_set_start(pdnqp_t *h, const double *x0, const double *y0);
  * of 8 rows; 0 = from the mean row length), persistent (1, the default: the trials of the
  * inner loop run inside one kernel launch per check period: small problems in
  * one thread block or one cluster of 8 (at most 512 tiles of rows or columns and
- * 120,000 gathers a trial, without long-row tiles), larger ones in a cooperative
+ * 120,000 gathers a trial), larger ones in a cooperative
  * launch with bounded grid barriers between the row and column passes; where the
  * device has no cooperative launches, the graph modes below),
- * loop_blocks_per_sm (blocks per SM of that launch; 0 = as many as fit),
+ * loop_blocks_per_sm (blocks per SM of the cooperative launch at most; one fits, so
+ * every value gives one),
  * cond_graph (with persistent = 0; 1: inner loop as a device-driven CUDA
  * graph with conditional WHILE/IF nodes; 0: unrolled graph of `chunk` trial
  * slots, which profilers can inspect kernel by kernel), eps_inf (tolerance
@@ -239,7 +244,7 @@ PDNQP_API int pdnqp_set_start(pdnqp_t *h, const double *x0, const double *y0);
  * iterations; 0 = off), anderson_mem (stored outer iterates, 2..5),
  * controller / ctrl_explore / ctrl_seed (see pdnqp_set_controller),
  * autotune (1: when the graph form runs and g_rows / g_cols are 0, the first
- * inner solve times the row and column kernels for 4, 8 and 16 lanes per row
+ * inner solve times the row and column kernels for both lane settings
  * and keeps the fastest for this handle; 0, the default: the mean-row-length
  * choice), escalate (FP32-bulk handles: 1, the default, continues a solve
  * that ends in NUMERICAL_ERROR in the FP64 form, see pdnqp_solve; 0 = off),

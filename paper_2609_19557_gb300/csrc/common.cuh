@@ -1,6 +1,6 @@
-// Device helpers shared by the PDNQP kernels: sub-warp row groups for CSR
-// SpMV, deterministic block reductions, and the device-resident scalar state
-// of the inner solver.
+// Device helpers shared by the PDNQP kernels: row sums of CSR matrices by warp
+// tiles, deterministic block reductions, the grid barrier, and the device-resident
+// scalar state of the inner solver.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>

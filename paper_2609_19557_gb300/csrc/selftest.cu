@@ -127,7 +127,12 @@ extern "C" int pdnqp_selftest_wait(int kind, int *gave_up, double *seconds) {
   if (kind < 0 || kind > 2 || !gave_up) return PDNQP_ERR_ARG;
   if (kind == 2) {
     const auto t0 = std::chrono::steady_clock::now();
-    const int rc = selftest_solver(gave_up);
+    int rc;
+    try {
+      rc = selftest_solver(gave_up);
+    } catch (...) {  // host memory
+      rc = PDNQP_ERR_OOM;
+    }
     if (seconds) *seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     return rc;
   }

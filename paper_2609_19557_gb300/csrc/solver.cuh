@@ -50,10 +50,10 @@ struct Params {
   double gamma_override = 0.0;
   int chunk = 128;
   long long iter_budget = 4000000000000000000LL;
-  int g_rows = 0, g_cols = 0;  // entries per lane per CSR-stream chunk (0 = from the mean row length)
+  int g_rows = 0, g_cols = 0;  // lane setting of the row / column kernels of the graph form (0 = from the mean row length)
   int cond_graph = 1;          // 1: device-driven WHILE/IF graph; 0: unrolled slots (profilable)
-  int persistent = 1;          // 1: persistent cooperative trial loop (when supported)
-  int loop_blocks_per_sm = 0;  // blocks per SM of that loop (0: as many as fit)
+  int persistent = 1;          // 1: persistent trial loop (one block, one cluster, or cooperative where supported)
+  int loop_blocks_per_sm = 0;  // blocks per SM of the cooperative loop at most (0, or any number: the one that fits)
   int controller = 0;          // 1: the learned controller proposes rho_in and the next primal weight
   double ctrl_explore = 0.0;   // std. dev. of Gaussian noise added to the actions (trajectory generation)
   long long ctrl_seed = 0;

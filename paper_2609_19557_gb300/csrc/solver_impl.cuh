@@ -414,8 +414,9 @@ class Solver : public SolverBase {
   // every SM at once would wait for them all, and they for it), a launch per phase.
   // The two runs go side by side; where their two bases (1,040 bytes a variable at
   // 64 steps) find no room, one after the other in half of that.  Measured (n =
-  // 300,001, 64 steps, the whole device setup): 8.3 ms in one launch, 57 ms with
-  // every step orthogonalised twice and a host synchronisation a sum.
+  // 300,001, 64 steps, the whole device setup): 8.9 ms in one launch, 9.8 by
+  // phases, 57 with every step orthogonalised twice and a host synchronisation a
+  // sum.
   int lanczos(const Params &prm, double *out) {
     const long long n = n_;
     if (n == 0) {
@@ -845,8 +846,8 @@ class Solver : public SolverBase {
   // Blocks of the persistent loop (one per SM at most): a warp has a tile at a
   // time, so the grid is the tiles over 8 warps a block up to one block per SM
   // (spread over all SMs rather than packed), and a single block, whose
-  // barriers cost next to nothing, as long as that gives a warp two tiles at
-  // most.
+  // barriers cost next to nothing, as long as that gives a warp three tiles at
+  // most and no row is dense.
   int coop_grid(int bps) {
     if (coop_key_ == bps) return coop_nb_;
     coop_key_ = bps;
@@ -1633,8 +1634,8 @@ class Solver : public SolverBase {
     return 0;
   }
 
-  // Sec. "Infeasibility detection" on the scaled problem (see outer_rows_inf /
-  // outer_cols_inf): PDNQP_PRIMAL_INFEASIBLE when lambda^{k+1} - lambda^k is an
+  // Sec. "Infeasibility detection" on the scaled problem (the sums of
+  // k_outer_rows and k_outer_cols): PDNQP_PRIMAL_INFEASIBLE when lambda^{k+1} - lambda^k is an
   // approximate Farkas certificate, PDNQP_DUAL_INFEASIBLE when x^{k+1} - x^k
   // is an approximate recession direction of descent, else 0.
   static int infeasibility(const double *v, double eps) {
