@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(kBlock) k_cols(Dev<T> d, int nb_r) {
 // ===========================================================================
 // Threads of a block: 16 warps with 128 registers a thread hold the 16 gathers
 // and 11 row-local operands of a column tile without spills where rows are short
-// (the FP64 forms of tiles of 8 long rows spill 112 to 184 bytes), and saturate the
+// (the FP64 forms of tiles of 8 long rows spill 96 to 184 bytes), and saturate the
 // gathers (an SM takes about one 32-byte sector a cycle at random addresses,
 // measured with 16 to 64 warps); one block per SM makes the grid barrier and
 // the final reduction of the acceptance sums cheap.
