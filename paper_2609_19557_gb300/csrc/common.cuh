@@ -290,12 +290,12 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[NQ], double *part
   __syncthreads();
 }
 
-// Polls of a grid barrier before it gives up (about two seconds).
+// Polls of a grid barrier before it gives up (about two seconds) ...
 constexpr unsigned kSpinLimit = 1u << 22;
-// The same for a launch in which one warp may go through a row of `longest` entries
-// while the other blocks wait: in entry order (one_row) that takes 64 cycles an
-// entry, and a poll, a round trip to L2, takes some 250 at least.
-__host__ __device__ constexpr unsigned spin_limit(long long longest) { return kSpinLimit + (unsigned)(longest / 2); }
+// ... and further ones where a warp may go through a row of `longest` entries while
+// the other blocks wait: in entry order (one_row) that takes 64 cycles an entry, and a
+// poll, a round trip to L2, takes some 250 at least.
+__host__ __device__ constexpr unsigned spin_more(long long longest) { return (unsigned)(longest / 2); }
 
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned *p) {
   unsigned v;
@@ -317,6 +317,7 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // counter: each on its own 128-byte line, so that the polls of the
 // generation do not queue behind the arrival atomics.
 constexpr int kBarGen = 32, kBarFault = 64, kBarWords = 96;
+constexpr int kBarMore = kBarFault + 1;  // further polls (spin_more), read with the fault flag
 
 // Barrier of one thread-block cluster.  A hardware wait without a limit, as
 // __syncthreads is: the hardware starts the blocks of a cluster together, and
@@ -325,8 +326,8 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
 }
 // The barrier alone.
-template <bool CLU>
-__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, unsigned limit);
+template <bool CLU, bool MORE = true>
+__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen);
 
 // Grid barrier of a cooperative (co-resident) launch, the wait of every kernel
 // that spans blocks.  bar[0] counts the arrivals, bar[kBarGen] is the generation
@@ -336,18 +337,22 @@ __device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, unsigned 
 // lead()'s writes after it; what lead() returned (0 or 1) is the message, which
 // every block gets.  The arrivals are reset before lead() runs, and `gen` is the
 // caller's copy of the generation (thread 0), so a waiting block polls one word
-// and, every 64 polls, the fault flag (each is a round trip to L2).
+// and, every 64 polls, the fault flag (each is a round trip to L2) and the words
+// beside it.
 //
-// The wait is bounded: a block that polls `limit` times without a release, or that sees the fault flag, sets the flag and gets -1; the caller then leaves the
-// kernel, so a barrier that can never complete ends the launch instead of hanging
-// it.
+// The wait is bounded: a block that polls kSpinLimit times (MORE: and bar[kBarMore])
+// without a release, or that sees the fault flag, sets the flag and gets -1; the
+// caller then leaves the kernel, so a barrier that can never complete ends the launch
+// instead of hanging it.  The trial loop does without MORE: its warps take a row 256
+// entries a round, so that kSpinLimit covers some 10^8 of them, and a limit that is
+// not a constant costs its row pass 0.5 us of 24 (n = 1e6, FP32).
 //
 // CLU: the grid is one thread-block cluster (small problems), whose hardware
 // barrier orders the blocks' memory accesses like a block barrier (about 0.3 us
 // where the grid barrier takes 1.5 to 2.5); block 0 runs lead(), and no message
 // comes back.
-template <bool CLU, typename F>
-__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, unsigned limit, F lead) {
+template <bool CLU, bool MORE = true, typename F>
+__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, F lead) {
   __shared__ int role;  // message, -1 fault, 2 leader
   __syncthreads();
   if (gridDim.x == 1) {
@@ -371,7 +376,10 @@ __device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, unsigned 
     } else {
       unsigned it = 0, v;
       while ((v = ld_acquire_gpu(bar + kBarGen)) == gen) {
-        if (++it > limit || ((it & 63u) == 0u && ld_acquire_gpu(bar + kBarFault) != 0u)) {
+        ++it;
+        const bool look = (it & 63u) == 0u;
+        if (MORE ? look && (ld_acquire_gpu(bar + kBarFault) != 0u || it > kSpinLimit + ld_acquire_gpu(bar + kBarMore))
+                 : it > kSpinLimit || (look && ld_acquire_gpu(bar + kBarFault) != 0u)) {
           atomicExch(bar + kBarFault, 1u);
           role = -1;
           break;
@@ -395,13 +403,13 @@ __device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, unsigned 
   return msg;
 }
 
-template <bool CLU>
-__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen, unsigned limit) {
+template <bool CLU, bool MORE>
+__device__ __forceinline__ int loop_sync(unsigned *bar, unsigned &gen) {
   if (CLU && gridDim.x > 1) {
     cluster_sync();
     return 0;
   }
-  return loop_sync<CLU>(bar, gen, limit, [] { return 0; });
+  return loop_sync<CLU, MORE>(bar, gen, [] { return 0; });
 }
 
 // Single-block final reduction of NQ quantities over nb partials (fixed order):

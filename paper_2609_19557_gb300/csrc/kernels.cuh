@@ -98,7 +98,6 @@ struct Dev {
   double *lr_part;     // [kMaxLong][kMaxBlocks] block partial products
   double *lr_acc;      // [4] acceptance-sum terms of the long rows (added to the row sums)
   DevState *st;
-  unsigned spin;   // polls of a grid barrier (spin_limit)
   unsigned *ctr;   // arrival counters of the last-block reductions (reset by the last block)
   unsigned long long *ptime;  // persistent loop: ns spent in the primal, row and column(+decision) passes
   cudaGraphConditionalHandle hw, hc;  // device-loop handles (0 when the graph has none)
@@ -1364,7 +1363,7 @@ __global__ void __launch_bounds__(kTrialThreads, 1) k_trials(Dev<T> d, long long
     if (!S.spec) {
       primal_phase<T>(d, &S);
       lap(0);
-      if (loop_sync<CLU>(bar, gen, d.spin) < 0) return;
+      if (loop_sync<CLU, false>(bar, gen) < 0) return;
       lap(1);
     }
     if (threadIdx.x >= kTrialThreads - 2) {  // a spare lane each, before the last warp's first item
@@ -1378,12 +1377,12 @@ __global__ void __launch_bounds__(kTrialThreads, 1) k_trials(Dev<T> d, long long
     rows_phase_tiles<T, LR, RL>(d, &S, buf, ts);
     lap(2);
     if (LR) {
-      if (loop_sync<CLU>(bar, gen, d.spin, [&] {
+      if (loop_sync<CLU, false>(bar, gen, [&] {
             long_rows_finish<T>(d, &S, d.lr_nb);
             return 0;
           }) < 0)
         return;
-    } else if (loop_sync<CLU>(bar, gen, d.spin) < 0) {
+    } else if (loop_sync<CLU, false>(bar, gen) < 0) {
       return;
     }
     lap(3);
@@ -1394,10 +1393,10 @@ __global__ void __launch_bounds__(kTrialThreads, 1) k_trials(Dev<T> d, long long
     bool led = CLU;
     int go;
     if (CLU) {  // every block of a cluster decides for itself, on the same sums
-      loop_sync<CLU>(bar, gen, d.spin);
+      loop_sync<CLU, false>(bar, gen);
       go = decide_tiles<T>(d, S, nb, LR, next, blockIdx.x == 0);
     } else {
-      go = loop_sync<CLU>(bar, gen, d.spin, [&] {
+      go = loop_sync<CLU, false>(bar, gen, [&] {
         led = true;
         return decide_tiles<T>(d, S, nb, LR, next);
       });
@@ -1432,10 +1431,10 @@ __global__ void __launch_bounds__(kTrialThreads, 1) k_check(Dev<T> d) {
   const int nb = gridDim.x;
   const GridCtx g{(int)blockIdx.x, nb};
   check_rows_body<T, RL ? 16 : 8>(d, &S, g, buf);
-  if (loop_sync<CLU>(bar, gen, d.spin) < 0) return;
+  if (loop_sync<CLU>(bar, gen) < 0) return;
   check_cols_terms<T, CL ? 16 : 8>(d, &S, g, buf);
   bool led = false;
-  if (loop_sync<CLU>(bar, gen, d.spin, [&] {
+  if (loop_sync<CLU>(bar, gen, [&] {
         led = true;
         double q[16];
         check_sums(d.part, nb, nb, q);

@@ -170,8 +170,7 @@ enum : int { kLzStart, kLzNorms, kLzProduct, kLzRecur, kLzLoss, kLzSubtract, kLz
 template <int K, bool COOP>
 __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos(Mat<double> Q, int first, int ns, int steps, double *V,
                                                            double *w, double *part, unsigned *bar, double *out,
-                                                           LzState *state, int phase, int j0, int number,
-                                                           unsigned spin) {
+                                                           LzState *state, int phase, int j0, int number) {
   constexpr int NW = kLzThreads / 32;
   __shared__ LzState S;
   __shared__ double red[NW][32], tot[2][kLzMax];
@@ -383,7 +382,7 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos(Mat<double> Q, int fi
     return true;
   };
   if (COOP) {
-    auto sync = [&] { return loop_sync<false>(bar, gen, spin) >= 0; };
+    auto sync = [&] { return loop_sync<false>(bar, gen) >= 0; };
     start();
     if (!sync()) return;
     norms();

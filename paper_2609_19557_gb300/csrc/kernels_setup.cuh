@@ -453,8 +453,8 @@ __global__ void __launch_bounds__(kTrialThreads, 1) k_setup(Dev<T> d, SetupArgs<
       return 0;
     };
     if (COOP) {
-      if (((LR && ph >= 1 && ph <= S) || ph == S + 2 ? loop_sync<FORM == kCluster>(bar, gen, d.spin, lead)
-                                                     : loop_sync<FORM == kCluster>(bar, gen, d.spin)) < 0)
+      if (((LR && ph >= 1 && ph <= S) || ph == S + 2 ? loop_sync<FORM == kCluster>(bar, gen, lead)
+                                                     : loop_sync<FORM == kCluster>(bar, gen)) < 0)
         return;
     } else if ((LR && ph >= 1 && ph <= S) || ph == S + 2) {
       if (arrive_last(d.ctr + 1)) {

@@ -21,7 +21,7 @@ namespace {
 __global__ void k_selftest_barrier(unsigned *bar, int *ret) {
   if (blockIdx.x == 0) return;
   unsigned gen = threadIdx.x == 0 ? ld_acquire_gpu(bar + kBarGen) : 0u;
-  const bool ok = loop_sync<false>(bar, gen, kSpinLimit) >= 0;
+  const bool ok = loop_sync<false>(bar, gen) >= 0;
   if (threadIdx.x == 0) ret[blockIdx.x] = ok ? 1 : 0;
 }
 

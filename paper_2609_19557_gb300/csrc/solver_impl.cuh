@@ -271,6 +271,13 @@ class Solver : public SolverBase {
     return 0;
   }
 
+  // Counter words to zero, and the further polls of the grid barrier among them.
+  int clear_barrier(unsigned *words, int count, unsigned *bar) {
+    PDNQP_CK(cudaMemsetAsync(words, 0, count * sizeof(unsigned), s_));
+    PDNQP_CK(cudaMemcpyAsync(bar + kBarMore, &spin_more_, sizeof(spin_more_), cudaMemcpyHostToDevice, s_));
+    return 0;
+  }
+
   int grid_n() const { return grid_for(n_, kBlock); }
   int grid_m() const { return grid_for(m_, kBlock); }
   int grid_nm() const { return grid_for(std::max(n_, m_), kBlock); }
@@ -291,7 +298,7 @@ class Solver : public SolverBase {
     mE_ = P.mE;
     nnzA_ = P.a_ci.size();
     nnzH_ = P.q_ci.size();
-    d_.spin = spin_limit(std::max(n_, m_));  // no row is longer
+    spin_more_ = spin_more(std::max(n_, m_));  // no row is longer
     PDNQP_TRY(dalloc(&st_, 1));
     {
       // Idle from the start: kernels of a batch look at the state before the first solve has written it.
@@ -466,15 +473,14 @@ class Solver : public SolverBase {
   };
   // One launch, or the launches of all phases, and the smallest Ritz value into *best.
   int lanczos_run(LanczosArgs &a, double *best) {
-    PDNQP_CK(cudaMemsetAsync(a.bar, 0, kBarWords * sizeof(unsigned), s_));
+    PDNQP_TRY(clear_barrier(a.bar, kBarWords, a.bar));
     cudaError_t e = cudaSuccess;
     with_G(gN_, [&](auto GG) {
       constexpr int K = decltype(GG)::value;
       const int smem = kLzThreads / 32 * kTileSlots * (int)sizeof(Slot<double>);
       int phase = kLzStart, j = 0, number = 0;
       void *args[] = {(void *)&Hd_, (void *)&a.first, (void *)&a.ns,  (void *)&a.steps, (void *)&a.V,   (void *)&a.w, (void *)&a.part,
-                      (void *)&a.bar, (void *)&a.res, (void *)&a.state, (void *)&phase,   (void *)&j, (void *)&number,
-                      (void *)&d_.spin};
+                      (void *)&a.bar, (void *)&a.res, (void *)&a.state, (void *)&phase,   (void *)&j, (void *)&number};
       if (a.coop) {
         auto fn = k_lanczos<K, true>;
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -609,7 +615,7 @@ class Solver : public SolverBase {
     d.part = part_;
     d.st = st_;
     PDNQP_TRY(dalloc(&d.ctr, kCtrWords));
-    PDNQP_CK(cudaMemsetAsync(d.ctr, 0, kCtrWords * sizeof(unsigned), s_));
+    PDNQP_TRY(clear_barrier(d.ctr, kCtrWords, d.ctr + kCtrBar));
     PDNQP_TRY(dalloc(&d.ptime, 8));
     PDNQP_CK(cudaMemsetAsync(d.ptime, 0, 8 * sizeof(unsigned long long), s_));
     d.hw = 0;
@@ -1184,7 +1190,7 @@ class Solver : public SolverBase {
     if (*hfault_) {
       // A grid barrier of the persistent loop gave up waiting: the launch ended
       // early and the iterates are not usable.
-      cudaMemsetAsync(d_.ctr, 0, kCtrWords * sizeof(unsigned), s_);
+      clear_barrier(d_.ctr, kCtrWords, d_.ctr + kCtrBar);
       cudaStreamSynchronize(s_);
       last_err_ = "persistent trial loop: grid barrier timed out";
       return PDNQP_ERR_CUDA;
@@ -1741,6 +1747,7 @@ class Solver : public SolverBase {
   long long loop_trials_ = 0;  // trials they ran
   int coop_key_ = -1, coop_nb_ = 0, loop_nb_ = 0;
   unsigned *hfault_ = nullptr;
+  unsigned spin_more_ = 0;  // of the grid barriers (loop_sync)
   // learned controller
   double *xprev_ = nullptr, *lamprev_ = nullptr, *dxv_ = nullptr;  // infeasibility tests
   double *aa_u_ = nullptr, *aa_g_ = nullptr, *aa_out_ = nullptr;    // Anderson ring and step

@@ -10,7 +10,7 @@ float load_hook(const float *) { return 0; }
 
 int main() {
   for (long long n : {0LL, 1000LL, 1000000LL, 20000000LL, 100000000LL, 2147483647LL}) {
-    const unsigned polls = pdq::spin_limit(n);
+    const unsigned polls = pdq::kSpinLimit + pdq::spin_more(n);
     if (polls < pdq::kSpinLimit || 250.0 * polls < 64.0 * n) {
       printf("%lld entries: %u polls\n", n, polls);
       return 1;

@@ -1,5 +1,5 @@
 """Bound of the grid barrier against the longest row one warp goes through alone
-while the other blocks wait (csrc/common.cuh, spin_limit)."""
+while the other blocks wait (csrc/common.cuh, spin_more)."""
 from test_row_index_range import run_host_warp
 
 
